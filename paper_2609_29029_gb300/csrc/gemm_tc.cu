@@ -1,21 +1,24 @@
-// The prefill GEMMs on Blackwell's fifth-generation tensor cores (tcgen05, sm_103a).
+// The GEMMs on Blackwell's fifth-generation tensor cores (tcgen05, sm_103a).
 //
 // C[M, N] = A[M, K] . B[N, K]^T with fp16 operands (both K-major) and fp32 accumulation in
 // tensor memory, plus the fused epilogues of the decoder layer (fp16 store with RoPE on q and
-// k, fp32 residual add, SwiGLU over 16-column gate/up groups).
+// k, fp32 residual add, SwiGLU over 16-column gate/up groups).  Two kernels:
 //
-// Persistent, warp-specialised kernel, one CTA per SM (192 threads):
-//   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 4-stage shared-memory ring
-//   warp 1      allocates 512 TMEM columns; one thread issues tcgen05.mma (M = 128, N = 256, K = 16)
-//               into one of two 256-column fp32 accumulators and commits to mbarriers
+// gemm_tc_kernel (many rows: the prefill of a scene): persistent and warp-specialised on SM pairs
+// (2-CTA clusters, 256 x 256 tiles), 192 threads per CTA:
+//   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 6-stage shared-memory ring
+//   warp 1      allocates 512 TMEM columns; one thread of the even CTA issues tcgen05.mma
+//               (cta_group::2, M = 256, N = 256, K = 16) into one of two 256-column fp32
+//               accumulators and commits to mbarriers
 //   warps 2..5  epilogue: tcgen05.ld of their 32 TMEM lanes (one row per thread), fused op, store
 // Two accumulators let the epilogue of one tile overlap the main loop of the next.  Tiles are
-// visited in bands of M-tiles whose A rows fit in L2 (48 MB), so each weight tile is read from
-// DRAM once per band.
-// Split-K (for few rows, where the tiles alone would leave most SMs idle, as in the decode
-// step): the work units are (tile, K-slice) pairs, each unit stores its fp32 partial product
-// into a caller workspace, and splitk_reduce_kernel sums the slices in a fixed order and
-// applies the epilogue.
+// visited in bands whose rows of the larger operand fit in L2 (48 MB), so each tile of the other
+// operand is read from DRAM once per band.
+//
+// gemm_ck_kernel (few rows: a decode step, one tile's prefill, a shared prompt, a small scene's
+// Gram matrix): the operands swapped, K split over a thread-block cluster and the partial
+// products summed through distributed shared memory (below).
+//
 // Every mbarrier wait is bounded (RIFT_SPIN_LIMIT iterations, ~4 s of globaltimer): on timeout
 // the kernel sets RIFT_EBIT_TIMEOUT, lets every role fall through, waits for its issued copies
 // and frees its tensor memory.
@@ -39,10 +42,10 @@ unsigned int read_clear_err_gemm() {
 
 namespace tc {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int BM = 128, BN = 256, BK = 64, STAGES = 6;
 constexpr int A_BYTES = BM * BK * 2;  // 16 KB
 constexpr int THREADS = 192;
-// Instruction descriptor (per kernel instance), kind::f16: D fp32 (bits 4-5 = 1), A fp16 (bits
+// Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A fp16 (bits
 // 7-9 = 0), B fp16 (bits 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4
 // at bits 24-28.
 
@@ -291,6 +294,12 @@ __device__ __forceinline__ void epilogue_chunk(const uint32_t (&r)[32], int row,
   }
 }
 
+// x cos + partner sin, one rounding each for the product and the sum: written out, so that every
+// kernel's RoPE gives the same bits.
+__device__ __forceinline__ float rope_mul(float x, float partner, float c, float s) {
+  return fmaf(x, c, __fmul_rn(partner, s));
+}
+
 // Rotate-half RoPE on fp32 accumulators: r1 holds dims j0..j0+31 of a head, r2 the partner
 // dims j0+half..; y1 = x1 cos - x2 sin, y2 = x2 cos + x1 sin, rounded once to fp16.
 __device__ __forceinline__ void rope_chunk(const uint32_t (&r1)[32], const uint32_t (&r2)[32], int row, int col,
@@ -305,8 +314,8 @@ __device__ __forceinline__ void rope_chunk(const uint32_t (&r1)[32], const uint3
     const float2 c0 = cs[e], c1 = cs[e + 1];
     const float a0 = __uint_as_float(r1[e]), a1 = __uint_as_float(r1[e + 1]);
     const float b0 = __uint_as_float(r2[e]), b1 = __uint_as_float(r2[e + 1]);
-    p1[e / 2] = pack_half2(a0 * c0.x - b0 * c0.y, a1 * c1.x - b1 * c1.y);
-    p2[e / 2] = pack_half2(b0 * c0.x + a0 * c0.y, b1 * c1.x + a1 * c1.y);
+    p1[e / 2] = pack_half2(rope_mul(a0, b0, c0.x, -c0.y), rope_mul(a1, b1, c1.x, -c1.y));
+    p2[e / 2] = pack_half2(rope_mul(b0, a0, c0.x, c0.y), rope_mul(b1, a1, c1.x, c1.y));
   }
   uint4* o1 = reinterpret_cast<uint4*>(out);
   uint4* o2 = reinterpret_cast<uint4*>(out + half);
@@ -323,19 +332,15 @@ __device__ __forceinline__ int kblock(int mode, int D, int k) {
   return mode == 1 ? (k < D ? k : k - D) : mode == 2 ? (k < 2 * D ? k : k - 2 * D) : k;
 }
 
-// BN_ x STAGES_: 256 x 4 for the prefill on one SM; 128 x 6 for few-row products with the
-// operands swapped (weights as the 128-row operand, the few activation rows as the N side;
-// EPI_STORE_F32_T).  PAIR: 2-CTA clusters on an SM pair, 256 x 256 tiles (cta_group::2): each SM
-// stages 128 rows of A and 128 of the 256 B rows per k-block, half the B traffic of one SM per
-// tile row, and the even CTA issues the M = 256 MMAs into both SMs' tensor memory.
-template <int EPI, int BN_, int STAGES_, bool PAIR = false>
+// 2-CTA clusters on an SM pair, 256 x 256 tiles (cta_group::2): each SM stages 128 rows of A and 128
+// of the 256 B rows per k-block, half the B traffic of one SM per tile row, and the even CTA
+// issues the M = 256 MMAs into both SMs' tensor memory.
+template <int EPI>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M_cap,
-                   int N, int K, void* C, const EpiParams ep, int group_m, int splits, size_t split_stride,
-                   int a_const) {
-  constexpr int BN = BN_, STAGES = STAGES_;  // this instance's tile width and ring depth
-  constexpr int TM = PAIR ? 2 * BM : BM;     // rows of a tile (both CTAs of the pair)
-  constexpr int B_ROWS = PAIR ? BN / 2 : BN; // B rows staged by this CTA
+                   int N, int K, void* C, const EpiParams ep, int group_m) {
+  constexpr int TM = 2 * BM;      // rows of a tile (both CTAs of the pair)
+  constexpr int B_ROWS = BN / 2;  // B rows staged by this CTA
   constexpr int B_BYTES = B_ROWS * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr int ACC_COLS = BN, TMEM_COLS = 2 * ACC_COLS;
   constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
@@ -360,37 +365,26 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), PAIR ? 256 : 128);  // the epilogue threads of every CTA that drains it
+      mbar_init(tempty_bar(b), 256);  // the epilogue threads of both CTAs
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   }
-  const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
-  if constexpr (PAIR) cluster_sync();  // both CTAs' barriers initialised before any remote arrival
+  const uint32_t rank = cluster_ctarank();
+  cluster_sync();  // both CTAs' barriers initialised before any remote arrival
   if (warp == 1) {
-    if constexpr (PAIR) {
-      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                       smem_u32(tmem_slot)),
-                   "r"(TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
-    } else {
-      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                       smem_u32(tmem_slot)),
-                   "r"(TMEM_COLS)
-                   : "memory");
-      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
   }
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_trigger();
-  // The producer waits after prefetching constant A tiles; with a device row count every role
-  // waits first, since the count is written by an earlier kernel.
-  if (warp != 0 || ep.m_dev) pdl_wait();
+  pdl_wait();
   // Rows: M_cap (host), or the device count ep.m_dev clamped to it (the rows the TMA map covers).
   const int M = ep.m_dev ? max(0, min(M_cap, *ep.m_dev)) : M_cap;
 
@@ -400,92 +394,51 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (ep.symmetric) tri_coords(tile, mt, m_blk, n_blk);
     else tile_coords(tile, mt, nt, group_m, m_blk, n_blk);
   };
-  // unit u: tile u / splits, K-blocks [k0, k1) of slice u % splits (the host makes every slice
-  // non-empty)
-  const int n_units = n_tiles * splits, k_per = (kt + splits - 1) / splits;
-  auto unit_k = [&](int u, int& k0, int& k1) {
-    k0 = (u % splits) * k_per;
-    k1 = min(kt, k0 + k_per);
-  };
-
-  // the pair walks the units together, one unit per cluster
-  const int u_first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-  const int u_step = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+  // the pair walks the tiles together, one tile per cluster
+  const int u_first = (int)(blockIdx.x >> 1), u_step = (int)(gridDim.x >> 1);
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---------------- TMA producer (PAIR: both CTAs load their halves; the even CTA's full
-      // barrier counts the bytes of both)
-      // a_const: A does not depend on earlier kernels (weights), so the first ring round of this
-      // CTA's first unit takes its A tiles before waiting for the kernel before this one.
-      int n_pre = 0;
-      if (!PAIR && a_const && !ep.m_dev && u_first < n_units) {
-        int m_blk, n_blk, k0, k1;
-        coords(u_first / splits, m_blk, n_blk);
-        unit_k(u_first, k0, k1);
-        n_pre = min(STAGES, k1 - k0);
-        for (int j = 0; j < n_pre; ++j) {
-          mbar_expect_tx(full_bar(j), STAGE_BYTES);
-          tma_load_2d(smem_u32(sA + j * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k0 + j) * BK, m_blk * BM,
-                      full_bar(j));
-        }
-      }
-      pdl_wait();
+      // ---------------- TMA producer: both CTAs load their halves; the even CTA's full barrier
+      // counts the bytes of both
       int it = 0;
       bool ok = true;
-      for (int u = u_first; u < n_units && ok; u += u_step) {
-        int m_blk, n_blk, k0, k1;
-        coords(u / splits, m_blk, n_blk);
-        unit_k(u, k0, k1);
-        for (int k = k0; k < k1; ++k, ++it) {
+      for (int u = u_first; u < n_tiles && ok; u += u_step) {
+        int m_blk, n_blk;
+        coords(u, m_blk, n_blk);
+        for (int k = 0; k < kt; ++k, ++it) {
           const int s = it % STAGES;
           const uint32_t round = it / STAGES;
-          if (it < n_pre) {  // A already requested (first round: the stage is free)
-            tma_load_2d(smem_u32(sB + s * B_BYTES), &tmB, kblock(ep.kmap_b, ep.kmap_d, k) * BK, n_blk * BN,
-                        full_bar(s));
-            continue;
-          }
           if (!mbar_wait(empty_bar(s), (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          if constexpr (PAIR) {
-            const uint32_t fb = mapa_shared(full_bar(s), 0);
-            if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
-            tma_load_2d_pair(smem_u32(sA + s * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k) * BK,
-                             m_blk * TM + (int)rank * BM, fb);
-            tma_load_2d_pair(smem_u32(sB + s * B_BYTES), &tmB, kblock(ep.kmap_b, ep.kmap_d, k) * BK,
-                             n_blk * BN + (int)rank * B_ROWS, fb);
-          } else {
-            mbar_expect_tx(full_bar(s), STAGE_BYTES);
-            tma_load_2d(smem_u32(sA + s * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k) * BK, m_blk * BM, full_bar(s));
-            tma_load_2d(smem_u32(sB + s * B_BYTES), &tmB, kblock(ep.kmap_b, ep.kmap_d, k) * BK, n_blk * BN, full_bar(s));
-          }
+          const uint32_t fb = mapa_shared(full_bar(s), 0);
+          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+          tma_load_2d_pair(smem_u32(sA + s * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k) * BK,
+                           m_blk * TM + (int)rank * BM, fb);
+          tma_load_2d_pair(smem_u32(sB + s * B_BYTES), &tmB, kblock(ep.kmap_b, ep.kmap_d, k) * BK,
+                           n_blk * BN + (int)rank * B_ROWS, fb);
         }
       }
-      // Before leaving, make sure no copy this thread issued is still in flight (bounded).  PAIR:
-      // the copies are counted on the even CTA's barrier, so wait instead for the MMAs' releases
-      // of the last stages, which also keeps this CTA alive until they have all arrived.
+      // Before leaving, make sure no copy this thread issued is still in flight (bounded): the
+      // copies are counted on the even CTA's barrier, so wait instead for the MMAs' releases of
+      // the last stages, which also keeps this CTA alive until they have all arrived.
       for (int j = 1; j <= STAGES && it - j >= 0; ++j) {
         const int i2 = it - j;
-        const int s = i2 % STAGES;
-        const uint32_t round = i2 / STAGES;
-        const uint32_t bar = PAIR ? empty_bar(s) : full_bar(s);
-        for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(bar, round & 1u); ++w) {
+        for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(empty_bar(i2 % STAGES), (i2 / STAGES) & 1u); ++w) {
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
-      // ---------------- MMA issuer (PAIR: the even CTA only)
+      // ---------------- MMA issuer (the even CTA only)
       int it = 0, tl = 0;
       bool ok = true;
-      for (int u = u_first; u < n_units && ok; u += u_step, ++tl) {
-        int k0, k1;
-        unit_k(u, k0, k1);
+      for (int u = u_first; u < n_tiles && ok; u += u_step, ++tl) {
         const int b = tl & 1;
         const uint32_t use = tl >> 1;
-        if (!mbar_wait<PAIR>(tempty_bar(b), (use & 1u) ^ 1u, abort_flag)) break;
+        if (!mbar_wait<true>(tempty_bar(b), (use & 1u) ^ 1u, abort_flag)) break;
         fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(b * ACC_COLS);
-        for (int k = k0; k < k1; ++k, ++it) {
+        for (int k = 0; k < kt; ++k, ++it) {
           const int s = it % STAGES;
           const uint32_t round = it / STAGES;
           if (!mbar_wait(full_bar(s), round & 1u, abort_flag)) { ok = false; break; }
@@ -493,38 +446,25 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint64_t ad = smem_desc(smem_u32(sA + s * A_BYTES));
           const uint64_t bd = smem_desc(smem_u32(sB + s * B_BYTES));
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {  // +32 bytes along K per step (encoded >> 4)
-            if constexpr (PAIR)
-              umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != k0 || kk != 0) ? 1u : 0u);
-            else
-              umma_f16(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != k0 || kk != 0) ? 1u : 0u);
-          }
-          if constexpr (PAIR) umma_commit_pair(empty_bar(s));
-          else umma_commit(empty_bar(s));
+          for (int kk = 0; kk < BK / 16; ++kk)  // +32 bytes along K per step (encoded >> 4)
+            umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != 0 || kk != 0) ? 1u : 0u);
+          umma_commit_pair(empty_bar(s));
         }
-        if (ok) {
-          if constexpr (PAIR) umma_commit_pair(tfull_bar(b));
-          else umma_commit(tfull_bar(b));
+        if (ok) umma_commit_pair(tfull_bar(b));
+      }
+      // the last two accumulators' releases (the odd CTA's arrivals among them) have landed
+      for (int t = tl - 1; t >= 0 && t >= tl - 2; --t)
+        for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait_cluster(tempty_bar(t & 1), (t >> 1) & 1u); ++w) {
         }
-      }
-      if constexpr (PAIR) {
-        // the last two accumulators' releases (the odd CTA's arrivals among them) have landed
-        for (int t = tl - 1; t >= 0 && t >= tl - 2; --t)
-          for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait_cluster(tempty_bar(t & 1), (t >> 1) & 1u); ++w) {
-          }
-      }
     }
   } else {
     // ---------------- epilogue (warps 2..5 -> TMEM lane quarters 2, 3, 0, 1)
     const int quarter = warp & 3;
-    const uint32_t tempty_even0 = PAIR ? mapa_shared(tempty_bar(0), 0) : tempty_bar(0);
-    const uint32_t tempty_even1 = PAIR ? mapa_shared(tempty_bar(1), 0) : tempty_bar(1);
+    const uint32_t tempty_even0 = mapa_shared(tempty_bar(0), 0), tempty_even1 = mapa_shared(tempty_bar(1), 0);
     int tl = 0;
-    for (int u = u_first; u < n_units; u += u_step, ++tl) {
+    for (int u = u_first; u < n_tiles; u += u_step, ++tl) {
       int m_blk, n_blk;
-      coords(u / splits, m_blk, n_blk);
-      // split-K partials (EPI_STORE_F32 only): slice u % splits at C + slice * split_stride
-      void* Cu = splits > 1 ? static_cast<void*>(static_cast<float*>(C) + (size_t)(u % splits) * split_stride) : C;
+      coords(u, m_blk, n_blk);
       const int b = tl & 1;
       const uint32_t use = tl >> 1;
       if (!mbar_wait(tfull_bar(b), use & 1u, abort_flag)) break;
@@ -557,47 +497,298 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int c = 0; c < BN; c += 32) {
           uint32_t r[32];
           tmem_ld32(taddr + c, r);
-          if constexpr (EPI == EPI_STORE_F32_T) {  // C[col][row] (transposed), col < N, row < M
-            const int col = n_blk * BN + c;
-            if (row < M) {
-              float* out = static_cast<float*>(Cu) + row;
+          if (row < M) epilogue_chunk<EPI>(r, row, n_blk * BN + c, N, C, ep.out_scale);
+          if constexpr (EPI == EPI_STORE_F32) {
+            // symmetric product: the off-diagonal tile also fills its mirror (a warp's lanes hold
+            // consecutive rows, so each transposed store is 32 consecutive floats)
+            if (ep.symmetric && m_blk != n_blk && row < M) {
+              float* out = static_cast<float*>(C);
 #pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (col + e < N) out[(size_t)(col + e) * M] = __uint_as_float(r[e]);
-            }
-          } else {
-            if (row < M) epilogue_chunk<EPI>(r, row, n_blk * BN + c, N, Cu, ep.out_scale);
-            if constexpr (EPI == EPI_STORE_F32) {
-              // symmetric product: the off-diagonal tile also fills its mirror (a warp's lanes hold
-              // consecutive rows, so each transposed store is 32 consecutive floats)
-              if (ep.symmetric && m_blk != n_blk && row < M) {
-                float* out = static_cast<float*>(Cu);
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                  const int col = n_blk * BN + c + e;
-                  if (col < M) out[(size_t)col * N + row] = __uint_as_float(r[e]) * ep.out_scale;
-                }
+              for (int e = 0; e < 32; ++e) {
+                const int col = n_blk * BN + c + e;
+                if (col < M) out[(size_t)col * N + row] = __uint_as_float(r[e]) * ep.out_scale;
               }
             }
           }
         }
       }
       fence_before();
-      if constexpr (PAIR) mbar_arrive_cluster(b ? tempty_even1 : tempty_even0);
-      else mbar_arrive(tempty_bar(b));
+      mbar_arrive_cluster(b ? tempty_even1 : tempty_even0);
     }
   }
   fence_before();
   __syncthreads();
-  if constexpr (PAIR) cluster_sync();  // neither CTA frees its tensor memory or exits before the other is done
+  cluster_sync();  // neither CTA frees its tensor memory or exits before the other is done
   if (warp == 1) {
     fence_after();
-    if constexpr (PAIR)
-      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
-                   : "memory");
-    else
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
-                   : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
+                 : "memory");
+  }
+}
+
+// ---------------------------------------------------------------- few rows: split K over a cluster
+// C[M, N] = A[M, K] . W[N, K]^T for products with few rows (M < 1024: a decode step, one tile's
+// prefill, a shared prompt, a small scene's Gram matrix), which stream the weights once.  The
+// operands are swapped: a CTA holds 128 weight rows as the MMA's M side and bn activation rows
+// (16 .. 160, a multiple of 16) as its N side, so a few rows cost no
+// more shared memory or tensor work than they need.  A cluster of S CTAs (1 .. 8) shares a tile:
+// rank r multiplies the K-blocks [kt r / S, kt (r + 1) / S), every CTA leaves its fp32 partial
+// product in its own shared memory, and after a cluster barrier rank r adds the S partials of
+// the rows r, r + S, ... in rank order (through distributed shared memory) and applies the
+// epilogue.  No partial product goes through HBM and no reduction kernel follows.  The ring is
+// sized for two CTAs per SM, so that uneven unit counts share the memory bandwidth evenly and a
+// programmatic dependent launch finds room next to the kernel before it: its CTAs request their
+// first weight tiles (w_const) before they wait for that kernel.
+// Bound by HBM (the weights) for one row tile; measured on one GB300, weights rotating through more
+// than L2, us per launch, against one SM per 128 x 256 tile without a split (in brackets), 7B shapes:
+//   rows   QKV           W_o           gate/up       W_down
+//      1   22.8 (32.8)   12.3 (32.1)   35.8 (53.5)   21.6 (71.4)
+//    131   27.0 (35.0)   17.6 (39.0)   46.8 (64.6)   27.7 (78.2)
+// and 19.3 / 9.2 / 32.1 / 18.2 for one row as programmatic dependents, 1.2 - 1.9 times the time the
+// weights take at the HBM rate; what is left is each launch's fill and drain.  The split-K it
+// replaces in the decode step wrote its partial products to HBM and read them back in a
+// reduction launch: one 7B layer's products at one row 113 us then, 79 us now.
+namespace ck {
+constexpr int THREADS = 192, MAX_S = 8, MAX_BN = 160;
+constexpr int W_BYTES = BM * BK * 2;
+constexpr int SMEM = 232448 / 2 - 1024;  // two CTAs per SM
+constexpr int RING = SMEM - 1024 - 512;  // after alignment; the barriers at the end
+__host__ __device__ constexpr int stage_bytes(int bn) { return W_BYTES + bn * BK * 2; }
+__host__ __device__ constexpr int stages(int bn) {
+  return RING / stage_bytes(bn) < 8 ? RING / stage_bytes(bn) : 8;
+}
+static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
+
+// Row tiles: as few as MAX_BN allows, of equal height.  S: as many CTAs per tile as the GPU holds
+// at once (two per SM), each with at least 8 K-blocks (a shorter slice is all fill and drain).
+// More CTAs than fit at once cost a second round: gate/up at one row 35.8 us with 172 CTAs, 43.6
+// with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.
+struct Plan {
+  int bn, S;
+};
+inline Plan plan(int M, int N, int K, int sms) {
+  const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
+  Plan p;
+  p.bn = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16;
+  const long long tiles = (long long)m_tiles * ((N + BM - 1) / BM);
+  p.S = MAX_S;
+  while (p.S > 1 && (tiles * p.S > 2LL * sms || ((K + BK - 1) / BK) / p.S < 8)) --p.S;
+  return p;
+}
+}  // namespace ck
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(ck::THREADS, 2)
+    gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, int M_cap, int N,
+                   int K, void* C, const EpiParams ep, int bn, int m_tiles, int S, int w_const) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ck::RING);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int stage_bytes = ck::stage_bytes(bn), stages = ck::stages(bn);
+  const uint32_t smem0 = smem_u32(smem), bar0 = smem_u32(bars);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (8 + s); };
+  const uint32_t done_bar = bar0 + 8u * 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t cols = 32;  // tensor memory columns: the power of two that holds bn
+  while (cols < (uint32_t)bn) cols *= 2;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full_bar(s), 1);
+      mbar_init(empty_bar(s), 1);
+    }
+    mbar_init(done_bar, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                 "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  if (warp != 0 || ep.m_dev) pdl_wait();
+  const int M = ep.m_dev ? max(0, min(M_cap, *ep.m_dev)) : M_cap;
+  const int rank = (int)cluster_ctarank();  // blockIdx.x % S
+  const int tile = (int)blockIdx.x / S;
+  const int m0 = (tile % m_tiles) * bn, n0 = (tile / m_tiles) * BM;
+  const int mv = min(bn, M - m0);  // rows of this tile (<= 0: past the device count, nothing to do)
+  const int kt = (K + BK - 1) / BK;
+  const int k0 = kt * rank / S, k1 = kt * (rank + 1) / S;
+
+  if (warp == 0) {
+    if (lane == 0 && mv > 0) {
+      // ---------------- TMA producer: a weight tile and the activation tile per K-block
+      auto load_w = [&](int s, int k) {
+        tma_load_2d(smem0 + s * stage_bytes, &tmW, kblock(ep.kmap_b, ep.kmap_d, k) * BK, n0, full_bar(s));
+      };
+      auto load_x = [&](int s, int k) {
+        tma_load_2d(smem0 + s * stage_bytes + ck::W_BYTES, &tmX, kblock(ep.kmap_a, ep.kmap_d, k) * BK, m0, full_bar(s));
+      };
+      const int n_pre = w_const && !ep.m_dev ? min(stages, k1 - k0) : 0;
+      for (int j = 0; j < n_pre; ++j) {
+        mbar_expect_tx(full_bar(j), stage_bytes);
+        load_w(j, k0 + j);
+      }
+      pdl_wait();
+      int it = 0;
+      for (int k = k0; k < k1; ++k, ++it) {
+        const int s = it % stages;
+        if (it < n_pre) {  // the weight tile is on its way (first round: the stage is free)
+          load_x(s, k);
+          continue;
+        }
+        if (!mbar_wait(empty_bar(s), ((it / stages) & 1u) ^ 1u, abort_flag)) break;
+        mbar_expect_tx(full_bar(s), stage_bytes);
+        load_w(s, k);
+        load_x(s, k);
+      }
+      for (int j = 1; j <= stages && it - j >= 0; ++j) {  // no copy left in flight (bounded)
+        const int i2 = it - j;
+        for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(full_bar(i2 % stages), (i2 / stages) & 1u); ++w) {
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && mv > 0) {
+      // ---------------- MMA issuer
+      const uint32_t idesc = (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+      bool ok = true;
+      for (int k = k0, it = 0; k < k1; ++k, ++it) {
+        const int s = it % stages;
+        if (!mbar_wait(full_bar(s), (it / stages) & 1u, abort_flag)) { ok = false; break; }
+        fence_after();
+        const uint64_t wd = smem_desc(smem0 + s * stage_bytes), xd = smem_desc(smem0 + s * stage_bytes + ck::W_BYTES);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk)
+          umma_f16(tmem, wd + 2 * kk, xd + 2 * kk, idesc, (it != 0 || kk != 0) ? 1u : 0u);
+        umma_commit(empty_bar(s));
+      }
+      if (ok) umma_commit(done_bar);
+    }
+  } else if (mv > 0) {
+    // ---------------- the partial product to shared memory: P[row m][weight row], over the ring
+    // (every copy has been consumed by a completed MMA)
+    const int quarter = warp & 3;
+    if (mbar_wait(done_bar, 0, abort_flag)) {
+      fence_after();
+      float* P = reinterpret_cast<float*>(smem) + quarter * 32 + lane;
+      const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
+      for (int c = 0; c < mv; c += 16) {
+        uint32_t r[16];
+        tmem_ld16(taddr + c, r);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) P[(c + e) * BM] = __uint_as_float(r[e]);
+      }
+      fence_before();
+    }
+  }
+  __syncwarp();
+  cluster_sync();  // every CTA's partial product is in place
+  if (mv > 0 && !*abort_flag) {
+    uint32_t base[ck::MAX_S];
+#pragma unroll
+    for (int r = 0; r < ck::MAX_S; ++r) base[r] = r < S ? mapa_shared(smem0, r) : 0u;
+    // the sum over the ranks of four weight rows' partials (columns q .. q + 3) of row m
+    auto acc4 = [&](int m, int q) {
+      const uint32_t off = (uint32_t)(m * BM + q) * 4u;
+      float4 f[ck::MAX_S];
+#pragma unroll
+      for (int r = 0; r < ck::MAX_S; ++r)
+        if (r < S) f[r] = ld_cluster4(base[r] + off);
+      float4 v = f[0];
+#pragma unroll
+      for (int r = 1; r < ck::MAX_S; ++r)
+        if (r < S) {
+          v.x += f[r].x;
+          v.y += f[r].y;
+          v.z += f[r].z;
+          v.w += f[r].w;
+        }
+      return v;
+    };
+    auto store_h4 = [](void* dst, float a, float b, float c, float d) {
+      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_half2(a, b), pack_half2(c, d));
+    };
+    constexpr int QUADS = EPI == EPI_SWIGLU ? 16 : 32;  // outputs of a row / 4
+    const int rows = (mv - rank + S - 1) / S;           // rows rank, rank + S, ... of the tile
+    for (int i = threadIdx.x; i < rows * QUADS; i += ck::THREADS) {
+      const int m = rank + (i / QUADS) * S, q = (i % QUADS) * 4;
+      const size_t row = (size_t)(m0 + m);
+      if constexpr (EPI == EPI_SWIGLU) {  // outputs q .. q + 3 of the tile's 64: gate 32 (q / 16) + q % 16, up 16 on
+        const int gq = 32 * (q / 16) + q % 16;
+        if (n0 + gq >= N) continue;
+        const float4 g = acc4(m, gq), u = acc4(m, gq + 16);
+        store_h4(static_cast<uint16_t*>(C) + row * (N / 2) + n0 / 2 + q, silu(g.x) * u.x, silu(g.y) * u.y,
+                 silu(g.z) * u.z, silu(g.w) * u.w);
+      } else {
+        const int col = n0 + q;
+        if (col >= N) continue;
+        float4 v = acc4(m, q);
+        if constexpr (EPI == EPI_STORE_F32) {
+          *reinterpret_cast<float4*>(static_cast<float*>(C) + row * N + col) =
+              make_float4(v.x * ep.out_scale, v.y * ep.out_scale, v.z * ep.out_scale, v.w * ep.out_scale);
+        } else if constexpr (EPI == EPI_RESID_F32) {
+          float4* o = reinterpret_cast<float4*>(static_cast<float*>(C) + row * N + col);
+          float4 h = *o;
+          h.x += v.x;
+          h.y += v.y;
+          h.z += v.z;
+          h.w += v.w;
+          *o = h;
+        } else {
+          if constexpr (EPI == EPI_QKV_ROPE) {
+            if (col < ep.rope_cols) {
+              const int half = ep.head_dim >> 1, j = q % ep.head_dim;
+              const int pos = ep.positions[row] + ep.pos_offset;
+              if (pos < 0 || pos >= ep.max_len) {
+                if (j == 0) atomicOr(&g_err_gemm, RIFT_EBIT_BADID);
+                continue;  // q and k of a row without a valid position stay unwritten
+              }
+              const bool lo = j < half;
+              const float4* cs4 = reinterpret_cast<const float4*>(ep.rope + (size_t)pos * half + (lo ? j : j - half));
+              const float4 c01 = cs4[0], c23 = cs4[1];  // (cos, sin) of four dims
+              const float4 x = acc4(m, lo ? q + half : q - half);
+              const float sg = lo ? -1.f : 1.f;
+              v = make_float4(rope_mul(v.x, x.x, c01.x, sg * c01.y), rope_mul(v.y, x.y, c01.z, sg * c01.w),
+                              rope_mul(v.z, x.z, c23.x, sg * c23.y), rope_mul(v.w, x.w, c23.z, sg * c23.w));
+            }
+          }
+          store_h4(static_cast<uint16_t*>(C) + row * N + col, v.x, v.y, v.z, v.w);
+        }
+      }
+    }
+  }
+  __syncwarp();
+  cluster_sync();  // no CTA leaves while another may still read its partial product
+  if (warp == 1) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(cols) : "memory");
   }
 }
 
@@ -809,29 +1000,14 @@ static int band_group(int M, int N, int K, int tm, int tn, int lo, int hi) {
   return n_major ? -g : g;
 }
 
-// pdl: launched as a programmatic dependent of the kernel before it; a_const: A is constant weights.
-template <int EPI, int BN_ = BN, int STAGES_ = STAGES>
-static int launch(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, void* C, const EpiParams& ep,
-                  cudaStream_t st, int splits = 1, bool pdl = false, int a_const = 0) {
-  constexpr size_t smem = (size_t)STAGES_ * (A_BYTES + BN_ * BK * 2) + 1024 + 256;
-  static std::atomic<unsigned long long> smem_raised{0};
-  if (raise_smem_limit(smem_raised, gemm_tc_kernel<EPI, BN_, STAGES_>, (int)smem) != cudaSuccess) return 1;
-  const int units = ((M + BM - 1) / BM) * ((N + BN_ - 1) / BN_) * splits;
-  const int grid = units < sm_count() ? units : sm_count();
-  const int group_m = band_group(M, N, K, BM, BN_, 8, 64);
-  return launch_ex(gemm_tc_kernel<EPI, BN_, STAGES_>, dim3(grid), dim3(THREADS), smem, st, pdl, a, b, M, N, K, C, ep,
-                   group_m, splits, (size_t)M * N, a_const) != cudaSuccess;
-}
-
 // The paired kernel (2-CTA clusters, 256 x 256 tiles), persistent over as many clusters as can be
 // resident at once.  b: the B map with 128-row boxes.  Returns -1 if no cluster can be resident
-// (the caller then uses one SM per tile).
-constexpr int PAIR_STAGES = 6;
+// (the caller then takes the cluster split-K kernel).
 template <int EPI>
 static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, void* C, const EpiParams& ep,
                        cudaStream_t st) {
-  constexpr size_t smem = (size_t)PAIR_STAGES * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
-  auto kern = gemm_tc_kernel<EPI, BN, PAIR_STAGES, true>;
+  constexpr size_t smem = (size_t)STAGES * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
+  auto kern = gemm_tc_kernel<EPI>;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
@@ -869,155 +1045,32 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
   const int group_m = band_group(M, N, K, 2 * BM, BN, 4, 32);
   cfg.gridDim = dim3(2 * clusters, 1, 1);
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, kern, a, b, M, N, K, C, ep, group_m, 1, (size_t)M * N, 0) == cudaSuccess ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, a, b, M, N, K, C, ep, group_m) == cudaSuccess ? 0 : 1;
 }
 
-// Sum of the split-K slices (in slice order) and the epilogue EPI, four consecutive outputs per
-// thread and step (float4 partial reads): the same arithmetic as epilogue_chunk / rope_chunk on
-// the summed accumulator.  N % 8 == 0, so a group of four never straddles a row, a SwiGLU
-// 16-column group or a RoPE half.
+// The cluster split-K kernel: S CTAs per (128 weight rows, bn rows) tile.
 template <int EPI>
-__global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, int M, int N, void* C,
-                                     const EpiParams ep) {
-  pdl_trigger();
-  pdl_wait();
-  const size_t stride = (size_t)M * N;
-  const int n_out = EPI == EPI_SWIGLU ? N / 2 : N;
-  const int q_out = n_out / 4;
-  const size_t total = (size_t)M * q_out;
-  auto acc4 = [&](int row, int col) {
-    const float* p = part + (size_t)row * N + col;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int sp = 0; sp < splits; ++sp) {
-      const float4 f = *reinterpret_cast<const float4*>(p + sp * stride);
-      v.x += f.x;
-      v.y += f.y;
-      v.z += f.z;
-      v.w += f.w;
-    }
-    return v;
-  };
-  auto store_h4 = [](void* dst, float a, float b, float c, float d) {
-    *reinterpret_cast<uint2*>(dst) = make_uint2(pack_half2(a, b), pack_half2(c, d));
-  };
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int row = (int)(e / q_out), col = (int)(e % q_out) * 4;
-    if constexpr (EPI == EPI_STORE_F32) {
-      const float4 v = acc4(row, col);
-      *reinterpret_cast<float4*>(static_cast<float*>(C) + (size_t)row * N + col) =
-          make_float4(v.x * ep.out_scale, v.y * ep.out_scale, v.z * ep.out_scale, v.w * ep.out_scale);
-    } else if constexpr (EPI == EPI_RESID_F32) {
-      const float4 v = acc4(row, col);
-      float4* o = reinterpret_cast<float4*>(static_cast<float*>(C) + (size_t)row * N + col);
-      float4 r = *o;
-      r.x += v.x;
-      r.y += v.y;
-      r.z += v.z;
-      r.w += v.w;
-      *o = r;
-    } else if constexpr (EPI == EPI_STORE_BF16) {
-      const float4 v = acc4(row, col);
-      store_h4(static_cast<uint16_t*>(C) + (size_t)row * N + col, v.x, v.y, v.z, v.w);
-    } else if constexpr (EPI == EPI_SWIGLU) {  // outputs f..f+3: gate column 32 (f / 16) + f % 16, up 16 further
-      const int gc = 32 * (col / 16) + col % 16;
-      const float4 g = acc4(row, gc), u = acc4(row, gc + 16);
-      store_h4(static_cast<uint16_t*>(C) + (size_t)row * n_out + col, silu(g.x) * u.x, silu(g.y) * u.y,
-               silu(g.z) * u.z, silu(g.w) * u.w);
-    } else if constexpr (EPI == EPI_QKV_ROPE) {
-      float4 y = acc4(row, col);
-      if (col < ep.rope_cols) {
-        const int half = ep.head_dim >> 1, j = col % ep.head_dim;
-        const int pos = ep.positions[row] + ep.pos_offset;
-        if (pos < 0 || pos >= ep.max_len) {
-          if (j == 0) atomicOr(&g_err_gemm, RIFT_EBIT_BADID);
-          continue;  // as the fused epilogue: q and k of a row without a valid position stay unwritten
-        }
-        const float2* cs = ep.rope + (size_t)pos * half + (j < half ? j : j - half);
-        const float4 x = acc4(row, j < half ? col + half : col - half);  // the partner dims
-        const float sg = j < half ? -1.f : 1.f;  // first half: x cos - x' sin; second: x cos + x' sin
-        y = make_float4(y.x * cs[0].x + sg * x.x * cs[0].y, y.y * cs[1].x + sg * x.y * cs[1].y,
-                        y.z * cs[2].x + sg * x.z * cs[2].y, y.w * cs[3].x + sg * x.w * cs[3].y);
-      }
-      store_h4(static_cast<uint16_t*>(C) + (size_t)row * N + col, y.x, y.y, y.z, y.w);
-    }
-  }
+static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
+                     cudaStream_t st, int bn, int S, bool pdl, int w_const) {
+  CUtensorMap mw, mx;
+  if (!make_map(&mw, W, Ks, (uint64_t)N, BM) || !make_map(&mx, A, Ks, (uint64_t)M, bn)) return 1;
+  static std::atomic<unsigned long long> smem_raised{0};
+  if (raise_smem_limit(smem_raised, gemm_ck_kernel<EPI>, ck::SMEM) != cudaSuccess) return 1;
+  const int m_tiles = (M + bn - 1) / bn, n_tiles = (N + BM - 1) / BM;
+  return launch_cluster_ex(gemm_ck_kernel<EPI>, dim3(m_tiles * n_tiles * S), dim3(ck::THREADS), ck::SMEM, st, pdl, S,
+                           mw, mx, M, N, K, C, ep, bn, m_tiles, S, w_const) != cudaSuccess;
 }
 
-// The residual add of a split-K product fused with the RMSNorm that follows it: one CTA per row,
-// h[row] += sum of the slices (in slice order), then out[row] = fp16(h / sqrt(mean(h^2) + eps) g)
-// with the bf16 gain g (the arithmetic of the standalone RMSNorm kernel).  N % 4 == 0, N <= 8192.
-// The rows are few (one per sequence in a decode step), so the kernel is latency-bound: a CTA has
-// up to 1024 threads and each holds VPT float4 columns of its row (1 at N = 4096), so that all of
-// a thread's loads (its columns of h and of every slice) are independent and issue together.
-template <int VPT>
-__global__ void __launch_bounds__(1024) splitk_resid_norm_kernel(const float* __restrict__ part, int splits, int M,
-                                                                 int N, float* __restrict__ h32,
-                                                                 const uint16_t* __restrict__ gain, float eps,
-                                                                 uint16_t* __restrict__ out) {
-  __shared__ float red[32];
-  pdl_trigger();
-  pdl_wait();
-  const size_t row = blockIdx.x, stride = (size_t)M * N;
-  const int nv = N / 4;
-  float4 v[VPT];
-  float ss = 0.f;
-#pragma unroll
-  for (int q = 0; q < VPT; ++q) {
-    const int c = threadIdx.x + q * blockDim.x;
-    if (c < nv) {
-      float4 a = reinterpret_cast<const float4*>(h32 + row * N)[c];
-      const float4* p = reinterpret_cast<const float4*>(part + row * N) + c;
-#pragma unroll 4
-      for (int sp = 0; sp < splits; ++sp) {
-        const float4 f = p[sp * stride / 4];
-        a.x += f.x;
-        a.y += f.y;
-        a.z += f.z;
-        a.w += f.w;
-      }
-      reinterpret_cast<float4*>(h32 + row * N)[c] = a;
-      v[q] = a;
-      ss += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-    }
+static int launch_ck_epi(const void* A, const void* W, uint64_t Ks, int M, int N, int K, int epi, void* C,
+                         const EpiParams& ep, cudaStream_t st, const ck::Plan& p, bool pdl, int w_const) {
+  switch (epi) {
+    case EPI_STORE_BF16: return launch_ck<EPI_STORE_BF16>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_RESID_F32: return launch_ck<EPI_RESID_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_SWIGLU: return launch_ck<EPI_SWIGLU>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_QKV_ROPE: return launch_ck<EPI_QKV_ROPE>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_STORE_F32: return launch_ck<EPI_STORE_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    default: return 1;
   }
-  const float inv = rsqrtf(block_sum(ss, red) / (float)N + eps);
-#pragma unroll
-  for (int q = 0; q < VPT; ++q) {
-    const int c = threadIdx.x + q * blockDim.x;
-    if (c < nv) {
-      const uint2 gr = reinterpret_cast<const uint2*>(gain)[c];
-      const float g0 = __uint_as_float(gr.x << 16), g1 = __uint_as_float(gr.x & 0xffff0000u);
-      const float g2 = __uint_as_float(gr.y << 16), g3 = __uint_as_float(gr.y & 0xffff0000u);
-      reinterpret_cast<uint2*>(out + row * N)[c] =
-          make_uint2(pack_half2(v[q].x * inv * g0, v[q].y * inv * g1), pack_half2(v[q].z * inv * g2, v[q].w * inv * g3));
-    }
-  }
-}
-
-// Split count for an M x N x K product whose tiles leave SMs idle: the K-slice count (1..16, at
-// least 4 K-blocks a slice, partials within the workspace) that minimises the makespan, i.e. the
-// rounds of units over the SMs times the K-blocks of a slice.  1 = no split.
-// With `unit_cost` > 0 (the swapped few-row path, whose units always store partials) every slice
-// count is weighed, each unit costing its K-blocks plus unit_cost K-blocks' worth of traffic and
-// overhead; otherwise only products whose tiles leave SMs idle are split.
-static int choose_splits(int M, int N, int K, size_t ws_bytes, int bn = BN, double unit_cost = 0.0) {
-  const int sms = sm_count();
-  const int tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn), kt = (K + BK - 1) / BK;
-  if (tiles >= sms && unit_cost == 0.0) return 1;
-  int best = 1;
-  double best_cost = (double)((tiles + sms - 1) / sms) * (kt + unit_cost);
-  for (int s = 2; s <= 16 && kt / s >= 4; ++s) {
-    if ((size_t)s * M * N * sizeof(float) > ws_bytes) break;
-    const int per = (kt + s - 1) / s;
-    const int se = (kt + per - 1) / per;  // every slice non-empty
-    const double cost = (double)((tiles * se + sms - 1) / sms) * (per + unit_cost);
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = se;
-    }
-  }
-  return best;
 }
 
 // A wait that can never complete (an mbarrier nobody arrives at), through the same bounded
@@ -1031,35 +1084,6 @@ __global__ void wait_timeout_check_kernel() {
   mbar_init(smem_u32(&bar), 1);
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   mbar_wait(smem_u32(&bar), 0, reinterpret_cast<volatile int*>(&abort_flag));
-}
-
-// The slices' partial products [splits][M][N] summed in slice order with the epilogue epi (a
-// residual product with ep.norm_out also applies the following RMSNorm).
-static int reduce_slices(const float* part, int splits, int M, int N, int epi, void* C, const EpiParams& ep,
-                         cudaStream_t st, bool pdl) {
-  if (epi == EPI_RESID_F32 && ep.norm_out) {
-    float* h = static_cast<float*>(C);
-    const uint16_t* g = static_cast<const uint16_t*>(ep.norm_gain);
-    const cudaError_t e =
-        N / 4 <= 1024
-            ? launch_ex(splitk_resid_norm_kernel<1>, dim3(M), dim3((N / 4 + 31) / 32 * 32), 0, st, pdl, part, splits,
-                        M, N, h, g, ep.norm_eps, ep.norm_out)
-            : launch_ex(splitk_resid_norm_kernel<2>, dim3(M), dim3(1024), 0, st, pdl, part, splits, M, N, h, g,
-                        ep.norm_eps, ep.norm_out);
-    return e != cudaSuccess;
-  }
-  const size_t n_out = (size_t)M * (epi == EPI_SWIGLU ? N / 2 : N) / 4;
-  const dim3 grid((unsigned)((n_out + 255) / 256 < 2048 ? (n_out + 255) / 256 : 2048));
-  cudaError_t e;
-  switch (epi) {
-    case EPI_STORE_BF16: e = launch_ex(splitk_reduce_kernel<EPI_STORE_BF16>, grid, dim3(256), 0, st, pdl, part, splits, M, N, C, ep); break;
-    case EPI_RESID_F32: e = launch_ex(splitk_reduce_kernel<EPI_RESID_F32>, grid, dim3(256), 0, st, pdl, part, splits, M, N, C, ep); break;
-    case EPI_SWIGLU: e = launch_ex(splitk_reduce_kernel<EPI_SWIGLU>, grid, dim3(256), 0, st, pdl, part, splits, M, N, C, ep); break;
-    case EPI_QKV_ROPE: e = launch_ex(splitk_reduce_kernel<EPI_QKV_ROPE>, grid, dim3(256), 0, st, pdl, part, splits, M, N, C, ep); break;
-    case EPI_STORE_F32: e = launch_ex(splitk_reduce_kernel<EPI_STORE_F32>, grid, dim3(256), 0, st, pdl, part, splits, M, N, C, ep); break;
-    default: return 1;
-  }
-  return e != cudaSuccess;
 }
 
 }  // namespace tc
@@ -1087,78 +1111,38 @@ int launch_wait_timeout_check(cudaStream_t st) {
 // Requirements: K % 8 == 0 (16-byte row pitch), N % 8 == 0 (N % 32 == 0 for SwiGLU, N % 64 == 0 for
 // the RoPE epilogue), A, B and C 16-byte aligned.
 int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, void* C, const EpiParams& ep,
-                   cudaStream_t st, void* split_ws, size_t split_ws_bytes, bool pdl, bool b_const) {
+                   cudaStream_t st, bool pdl, bool b_const) {
   using namespace tc;
   if (M <= 0 || N <= 0 || K <= 0) return 0;
   if (K % 8 != 0 || N % 8 != 0 || (epi == EPI_SWIGLU && N % 32 != 0)) return 1;
-  if (ep.m_dev && split_ws) return 1;  // a device row count is for the unsplit products only
   if (epi == EPI_QKV_ROPE && (N % 64 != 0 || (ep.head_dim != 64 && ep.head_dim != 128) || !ep.positions || !ep.rope))
     return 1;
-  // Few rows (<= 128, with scratch: the decode step): the operands swapped so that the weights
-  // stream as the 128-row operand in 128-row tiles and the rows sit on the N side (128 wide); the
-  // slices' fp32 partials are stored transposed ([M, N] as the reductions below read them).
   // The operands' stored row width: K, or 2 kmap_d blocks when read through the K-block remap.
   if (ep.kmap_d && K != 3 * ep.kmap_d * BK) return 1;
   const uint64_t Ks = ep.kmap_d ? (uint64_t)2 * ep.kmap_d * BK : (uint64_t)K;
-  EpiParams kp;  // the remap alone, for the partial products
-  kp.kmap_d = ep.kmap_d;
-  kp.kmap_a = ep.kmap_a;
-  kp.kmap_b = ep.kmap_b;
-  if (split_ws && M <= 128 && (size_t)M * N * sizeof(float) <= split_ws_bytes) {
-    constexpr int SW_BN = 128, SW_STAGES = 6;
-    CUtensorMap mw, mx;
-    if (!make_map(&mw, B, Ks, (uint64_t)N, BM) || !make_map(&mx, A, Ks, (uint64_t)M, SW_BN)) return 1;
-    EpiParams ks = kp;  // the operands swapped: the kernel's A is B
-    ks.kmap_a = ep.kmap_b;
-    ks.kmap_b = ep.kmap_a;
-    // a unit's partials (M x 128 fp32, written and read back) cost M / 16 K-blocks of weight
-    // traffic; its fill and drain about 1.5 more
-    const int splits = choose_splits(N, M, K, split_ws_bytes, SW_BN, M / 16.0 + 1.5);
-    // constant weights (b_const) are requested before the wait on the kernel before this one
-    if (launch<EPI_STORE_F32_T, SW_BN, SW_STAGES>(mw, mx, N, M, K, split_ws, ks, st, splits, pdl, b_const ? 1 : 0))
-      return 1;
-    EpiParams e = ep;
-    e.symmetric = 0;
-    return reduce_slices(static_cast<const float*>(split_ws), splits, M, N, epi, C, e, st, pdl);
-  }
+  const ck::Plan plan = ck::plan(M, N, K, sm_count());
+  // The cluster split-K kernel for one row tile, or while its split tiles fit on the GPU at once:
+  // beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
+  // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777
+  // (S = 1) 42.0 : 35.4; W_down 53.9 : 63.7 and 78.1 : 65.8; QKV at 131 rows 27.0 : 31.1, at 256
+  // (S = 1) 40.8 : 31.1; gate/up 46.8 : 57.8 and 75.6 : 57.8.
+  // A device count of the logits' rows (sequences) is usually a fraction of its capacity, and
+  // row tiles past the count cost nothing there.
+  if (M <= ck::MAX_BN || plan.S >= 2 || (epi == EPI_STORE_F32 && ep.m_dev && M < 1024))
+    return launch_ck_epi(A, B, Ks, M, N, K, epi, C, ep, st, plan, pdl, b_const ? 1 : 0);
   CUtensorMap ma, mb;
-  if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN)) return 1;
-  // The residual product with a following RMSNorm (ep.norm_out) always goes through the
-  // scratch, one slice or more, into the fused reduction + norm kernel.
-  const bool fuse_norm = epi == EPI_RESID_F32 && ep.norm_out;
-  if (fuse_norm && (!split_ws || N > 8192 || (size_t)M * N * sizeof(float) > split_ws_bytes)) return 1;
-  const int splits = split_ws ? choose_splits(M, N, K, split_ws_bytes) : 1;
-  if (splits > 1 || fuse_norm) {
-    if (launch<EPI_STORE_F32>(ma, mb, M, N, K, split_ws, kp, st, splits, pdl)) return 1;
-    EpiParams e = ep;
-    e.symmetric = 0;
-    return reduce_slices(static_cast<const float*>(split_ws), splits, M, N, epi, C, e, st, pdl);
-  }
-  // Many rows: 256 x 256 tiles on SM pairs.
-  if (M >= 1024) {
-    CUtensorMap mb2;
-    if (!make_map(&mb2, B, Ks, (uint64_t)N, BN / 2)) return 1;
-    int r = -1;
-    switch (epi) {
-      case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb2, M, N, K, C, ep, st); break;
-      case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb2, M, N, K, C, ep, st); break;
-      case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb2, M, N, K, C, ep, st); break;
-      case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb2, M, N, K, C, ep, st); break;
-      case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb2, M, N, K, C, ep, st); break;
-      default: return 1;
-    }
-    if (r >= 0) return r;
-  }
-  EpiParams e1 = ep;  // one SM per tile: 128 x 256 tiles, every tile computed
-  e1.symmetric = 0;
+  if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2)) return 1;
+  int r = -1;
   switch (epi) {
-    case EPI_STORE_BF16: return launch<EPI_STORE_BF16>(ma, mb, M, N, K, C, e1, st);
-    case EPI_RESID_F32: return launch<EPI_RESID_F32>(ma, mb, M, N, K, C, e1, st);
-    case EPI_SWIGLU: return launch<EPI_SWIGLU>(ma, mb, M, N, K, C, e1, st);
-    case EPI_QKV_ROPE: return launch<EPI_QKV_ROPE>(ma, mb, M, N, K, C, e1, st);
-    case EPI_STORE_F32: return launch<EPI_STORE_F32>(ma, mb, M, N, K, C, e1, st);
+    case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, M, N, K, C, ep, st); break;
+    case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb, M, N, K, C, ep, st); break;
+    case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb, M, N, K, C, ep, st); break;
+    case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb, M, N, K, C, ep, st); break;
+    case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb, M, N, K, C, ep, st); break;
     default: return 1;
   }
+  if (r >= 0) return r;
+  return launch_ck_epi(A, B, Ks, M, N, K, epi, C, ep, st, plan, pdl, b_const ? 1 : 0);
 }
 
 }  // namespace rift

@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(NORM_THREADS, VPT <= 4 ? 8 : 4) rmsnorm_kernel
                                                                float eps, const int* __restrict__ rows_dev,
                                                                int max_rows) {
   __shared__ float red[32];
+  pdl_trigger();
+  pdl_wait();
   const int n_rows = rows_dev ? max(0, min(max_rows, *rows_dev)) : max_rows;
   for (size_t row = blockIdx.x; row < (size_t)n_rows; row += gridDim.x)
     rmsnorm_row<IN_BF16, OUT_F16, VPT>(in, h32, gain, out, d, eps, row, red);
@@ -185,9 +187,9 @@ PrefillLayout prefill_layout(const rift_model& m, int max_T, int max_seqs, int m
 }
 
 int launch_gemm(const void* A, const void* B, int M, int N, int K, int epi, void* C, cudaStream_t st,
-                const EpiParams& ep, void* split_ws, size_t split_ws_bytes, bool pdl) {
+                const EpiParams& ep, bool pdl) {
   prof_begin(RIFT_PROF_GEMM, st);
-  const int r = launch_gemm_tc(A, B, M, N, K, epi, C, ep, st, split_ws, split_ws_bytes, pdl);
+  const int r = launch_gemm_tc(A, B, M, N, K, epi, C, ep, st, pdl);
   prof_end(RIFT_PROF_GEMM, st, 1);
   return r;
 }
@@ -226,7 +228,7 @@ static int norm_resident_ctas() {
 // on the GPU at once (8 per SM at d <= 4096), each looping over rows: a CTA that finishes early
 // frees its slot for another, so the last rows spread over the SMs as with one CTA per row.
 static void norm_launch(int kind, int T, const void* in, float* h32, const void* gain, uint16_t* out, int d,
-                        float eps, cudaStream_t st, const int* rows_dev = nullptr) {
+                        float eps, cudaStream_t st, const int* rows_dev = nullptr, bool pdl = false) {
   prof_begin(RIFT_PROF_NORM, st);
   const uint16_t* g = static_cast<const uint16_t*>(gain);
   const int per_thread = (d / 4 + NORM_THREADS - 1) / NORM_THREADS;  // d <= 8192: at most 8
@@ -234,14 +236,14 @@ static void norm_launch(int kind, int T, const void* in, float* h32, const void*
     constexpr int V = decltype(vpt)::value;
     auto grid = [&](int per_sm) { return T < 4 * per_sm * sm_count() ? T : 4 * per_sm * sm_count(); };
     if (kind == 0)
-      rmsnorm_kernel<true, true, V><<<grid(norm_resident_ctas<true, true, V>()), NORM_THREADS, 0, st>>>(
-          in, h32, g, out, d, eps, rows_dev, T);
+      launch_ex(rmsnorm_kernel<true, true, V>, dim3(grid(norm_resident_ctas<true, true, V>())), dim3(NORM_THREADS), 0,
+                st, pdl, in, h32, g, out, d, eps, rows_dev, T);
     else if (kind == 1)
-      rmsnorm_kernel<false, true, V><<<grid(norm_resident_ctas<false, true, V>()), NORM_THREADS, 0, st>>>(
-          in, nullptr, g, out, d, eps, rows_dev, T);
+      launch_ex(rmsnorm_kernel<false, true, V>, dim3(grid(norm_resident_ctas<false, true, V>())), dim3(NORM_THREADS), 0,
+                st, pdl, in, (float*)nullptr, g, out, d, eps, rows_dev, T);
     else
-      rmsnorm_kernel<false, false, V><<<grid(norm_resident_ctas<false, false, V>()), NORM_THREADS, 0, st>>>(
-          in, nullptr, g, out, d, eps, rows_dev, T);
+      launch_ex(rmsnorm_kernel<false, false, V>, dim3(grid(norm_resident_ctas<false, false, V>())), dim3(NORM_THREADS),
+                0, st, pdl, in, (float*)nullptr, g, out, d, eps, rows_dev, T);
   };
   if (per_thread <= 1) go(std::integral_constant<int, 1>{});
   else if (per_thread <= 2) go(std::integral_constant<int, 2>{});
@@ -394,17 +396,6 @@ DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len) {
   L.pos_off = take(n * sizeof(int));
   // decode attention partials: (m, l, o[head_dim]) per (sequence, key chunk, head)
   L.dpart_off = take(n * (size_t)((max_len + DEC_CHUNK - 1) / DEC_CHUNK) * m.n_heads * (m.head_dim + 2) * 4);
-  // split-K partial products of the few-row GEMMs: up to 16 slices of [min(n, 128), widest
-  // output] fp32, at most 128 MB
-  const size_t rows = n < 128 ? n : 128;
-  size_t widest = (size_t)3 * m.d;
-  if ((size_t)2 * m.ffn > widest) widest = (size_t)2 * m.ffn;
-  if (m.lm_head && (size_t)m.vocab > widest) widest = (size_t)m.vocab;
-  L.split_bytes = 16 * rows * widest * 4;
-  if (L.split_bytes > (size_t)128 << 20) L.split_bytes = (size_t)128 << 20;
-  // at least one slice of the residual products, which always go through the scratch
-  if (L.split_bytes < n * m.d * 4) L.split_bytes = n * m.d * 4;
-  L.split_off = take(L.split_bytes);
   L.total = off;
   return L;
 }
@@ -579,8 +570,6 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   uint16_t* act = reinterpret_cast<uint16_t*>(ws + L.act_off);
   float2* rope = reinterpret_cast<float2*>(ws + L.rope_off);
   int* pos = reinterpret_cast<int*>(ws + L.pos_off);
-  void* split = ws + L.split_off;
-  const size_t sb = L.split_bytes;
   float* dpart = reinterpret_cast<float*>(ws + L.dpart_off);
   const int max_chunks = (max_len + DEC_CHUNK - 1) / DEC_CHUNK;
   int hg = DEC_HG;
@@ -598,22 +587,13 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   rope_ep.max_len = max_len;
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)m.head_dim);
   const uint16_t* kv = static_cast<const uint16_t*>(kv_cache);
-  // The residual products carry the RMSNorm that follows them (g_ffn after W_o; the next layer's
-  // g_attn, or g_final after the last W_down) into their split-K reduction.
-  auto resid_norm = [&](const void* gain) {
-    EpiParams e;
-    e.norm_gain = gain;
-    e.norm_out = xn;
-    e.norm_eps = m.eps;
-    return e;
-  };
   norm_launch(0, n, x0, h32, m.g_attn[0], xn, d, m.eps, st);
   // The layer's kernels are launched as programmatic dependents of the kernel before them: each
-  // starts while its predecessor drains (the GEMMs already streaming their first weight tiles)
+  // starts while its predecessor drains (the GEMMs already requesting their first weight tiles)
   // and waits for it before touching activations.
   const bool pdl = true;
   for (int l = 0; l < m.n_layers; ++l) {
-    if (launch_gemm(xn, m.w_qkv[l], n, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep, split, sb, pdl)) return 1;
+    if (launch_gemm(xn, m.w_qkv[l], n, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep, pdl)) return 1;
     if (kv_new) {
       uint16_t* kl = static_cast<uint16_t*>(kv_new) + (size_t)l * 2 * n * d;
       kv_store(qkv, n, nullptr, d, kl, kl + (size_t)n * d, st);
@@ -634,16 +614,17 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
                   cu_seqlens, (int)m.n_heads, (int)m.head_dim, max_chunks, max_len, att) != cudaSuccess)
       return 1;
     prof_end(RIFT_PROF_ATTN, st, 2);
-    if (launch_gemm(att, m.w_o[l], n, d, d, EPI_RESID_F32, h32, st, resid_norm(m.g_ffn[l]), split, sb, pdl)) return 1;
-    if (launch_gemm(xn, m.w_gate_up[l], n, 2 * m.ffn, d, EPI_SWIGLU, act, st, EpiParams(), split, sb, pdl)) return 1;
+    if (launch_gemm(att, m.w_o[l], n, d, d, EPI_RESID_F32, h32, st, EpiParams(), pdl)) return 1;
+    norm_launch(1, n, h32, nullptr, m.g_ffn[l], xn, d, m.eps, st, nullptr, pdl);
+    if (launch_gemm(xn, m.w_gate_up[l], n, 2 * m.ffn, d, EPI_SWIGLU, act, st, EpiParams(), pdl)) return 1;
+    if (launch_gemm(act, m.w_down[l], n, d, m.ffn, EPI_RESID_F32, h32, st, EpiParams(), pdl)) return 1;
     const void* next_gain = l + 1 < m.n_layers ? m.g_attn[l + 1] : m.g_final;
-    if (launch_gemm(act, m.w_down[l], n, d, m.ffn, EPI_RESID_F32, h32, st, resid_norm(next_gain), split, sb, pdl))
-      return 1;
+    norm_launch(1, n, h32, nullptr, next_gain, xn, d, m.eps, st, nullptr, pdl);
   }
   // xn now holds RMSNorm(h) g_final in fp16 (the logits operand)
   if (hidden_out) norm_launch(2, n, h32, nullptr, m.g_final, static_cast<uint16_t*>(hidden_out), d, m.eps, st);
   if (logits) {
-    if (launch_gemm(xn, m.lm_head, n, m.vocab, d, EPI_STORE_F32, logits, st, EpiParams(), split, sb, pdl)) return 1;
+    if (launch_gemm(xn, m.lm_head, n, m.vocab, d, EPI_STORE_F32, logits, st, EpiParams(), pdl)) return 1;
   }
   return 0;
 }

@@ -26,7 +26,7 @@ struct ShardLayout {
 ShardLayout shard_layout(int N, int n_v, int d);
 // The kNN smoothing of n_rows rows against all N tiles (Appendix B Step 2).
 struct SmoothLayout {
-  size_t top_off, split_off, gram_off, splitk_off, splitk_bytes, total;
+  size_t top_off, split_off, gram_off, total;
 };
 SmoothLayout smooth_layout(int N, int n_rows, int d);
 // rift_score_tiles: V [N, d], then the token pass's scratch, which the smoothing of all N rows
@@ -119,8 +119,7 @@ int launch_prefill_shared_prefix(const rift_model& m, const int* sys_ids, int S,
                                  const int* cu_seqlens, int n_seq, const int* n_seq_dev, int max_len,
                                  const int* positions, float* last_logits, char* ws, cudaStream_t st);
 struct DecodeLayout {
-  size_t h32_off, x0_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, dpart_off, split_off, split_bytes,
-      total;
+  size_t h32_off, x0_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, dpart_off, total;
 };
 DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len);
 int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* cu_seqlens, int n_seq, int max_len,
@@ -133,8 +132,7 @@ enum GemmEpilogue {
   EPI_RESID_F32 = 1,   // R fp32 [M, N] += acc
   EPI_SWIGLU = 2,      // N = 2F interleaved in 16-column groups; C fp16 [M, F] = silu(g) * u
   EPI_QKV_ROPE = 3,    // C fp16 [M, N]; columns < rope_cols get rotate-half RoPE at positions[row]
-  EPI_STORE_F32 = 4,   // C fp32 [M, N] = acc * out_scale
-  EPI_STORE_F32_T = 5  // C fp32 [N, M] = acc (transposed; the swapped few-row products)
+  EPI_STORE_F32 = 4    // C fp32 [M, N] = acc * out_scale
 };
 struct EpiParams {
   const int* positions = nullptr;  // [M] position of each row (EPI_QKV_ROPE)
@@ -144,12 +142,8 @@ struct EpiParams {
   int max_len = 0;
   int pos_offset = 0;              // added to positions[row] (rows that follow a shared prefix)
   float out_scale = 1.f;           // EPI_STORE_F32
-  // EPI_RESID_F32 with split scratch: also norm_out fp16 [M, N] = RMSNorm(C) norm_gain (bf16 [N])
-  const void* norm_gain = nullptr;
-  uint16_t* norm_out = nullptr;
-  float norm_eps = 0.f;
   // Device row count (nullable): the product covers rows min(M, *m_dev); M is then the capacity
-  // the operands and the output are sized for.  Not used with split-K.
+  // the operands and the output are sized for.
   const int* m_dev = nullptr;
   // EPI_STORE_F32 of a symmetric product (A = B's first M rows, M <= N <= M + 7: a Gram matrix):
   // only the tiles on and above the diagonal are computed, each off-diagonal one stored twice
@@ -161,17 +155,13 @@ struct EpiParams {
   int kmap_d = 0;
   int kmap_a = 0, kmap_b = 0;
 };
-// split_ws (optional): scratch for split-K partial products; with it, products whose tiles leave
-// most SMs idle run as (tile, K-slice) units plus a reduction kernel.
-// pdl: launch as a programmatic dependent of the previous kernel in the stream (decode step).
+// pdl: launch as a programmatic dependent of the previous kernel in the stream (few-row products).
 int launch_gemm(const void* A, const void* B, int M, int N, int K, int epi, void* C,
-                cudaStream_t st, const EpiParams& ep = EpiParams(), void* split_ws = nullptr,
-                size_t split_ws_bytes = 0, bool pdl = false);
+                cudaStream_t st, const EpiParams& ep = EpiParams(), bool pdl = false);
 // b_const: B does not depend on earlier kernels (constant weights), so a programmatic dependent
 // launch may request its first tiles before waiting for the kernel before it.
 int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, void* C, const EpiParams& ep,
-                   cudaStream_t st, void* split_ws = nullptr, size_t split_ws_bytes = 0, bool pdl = false,
-                   bool b_const = true);
+                   cudaStream_t st, bool pdl = false, bool b_const = true);
 int launch_wait_timeout_check(cudaStream_t st);
 // Merge screening on the tensor cores (bf16 tokens): per kept slot and 128-token block, the two
 // best merge targets (by x.t / ||t||) of every unselected non-target token.  targets: bf16

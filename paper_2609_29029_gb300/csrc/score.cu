@@ -603,8 +603,7 @@ int launch_query_prep(const void* embed, int vocab, int d, const int* phrase_ids
 }
 
 // Scratch of the kNN smoothing of rows row0 .. row0 + n_rows - 1 against all N tiles: the split
-// rows of every tile, the Gram rows, split-K partials when the product has fewer tiles than SMs (at most 16
-// slices within 16 MB), the candidate lists.
+// rows of every tile, the Gram rows, the candidate lists.
 SmoothLayout smooth_layout(int N, int n_rows, int d) {
   SmoothLayout L{};
   size_t off = 0;
@@ -612,11 +611,6 @@ SmoothLayout smooth_layout(int N, int n_rows, int d) {
   const size_t Np = ((size_t)N + 7) & ~size_t(7);
   L.top_off = take(sizeof(int) * (size_t)n_rows * RIFT_MAX_KNN);
   L.gram_off = take(sizeof(float) * (size_t)n_rows * Np);
-  const size_t slice = sizeof(float) * (size_t)n_rows * Np;
-  size_t part = ((size_t)16 << 20) / slice;
-  part = part > 16 ? 16 : part;
-  L.splitk_bytes = part >= 2 ? part * slice : 0;
-  L.splitk_off = take(L.splitk_bytes);
   L.split_off = take(sizeof(uint16_t) * Np * 2 * d);  // the split rows last
   L.total = off;
   return L;
@@ -724,11 +718,8 @@ int launch_smooth(const float* V, const float* s_raw, int N, int d, int row0, in
     // the whole scene's rows: G is symmetric (A holds the same rows as B, in the permuted parts
     // [hi | hi | lo] against [hi | lo | hi], whose product is symmetric up to the order of its sums)
     ep.symmetric = (row0 == 0 && n_rows == N) ? 1 : 0;
-    // split-K partials for products with fewer tiles than SMs (a scene up to ~2000 tiles)
-    void* part = L.splitk_bytes ? static_cast<void*>(ws + L.splitk_off) : nullptr;
     // S is written by an earlier kernel of the chain, not a constant operand
-    if (launch_gemm_tc(S16 + (size_t)row0 * 2 * d, S16, n_rows, Np, 3 * d, EPI_STORE_F32, G, ep, st, part,
-                       L.splitk_bytes, true, false))
+    if (launch_gemm_tc(S16 + (size_t)row0 * 2 * d, S16, n_rows, Np, 3 * d, EPI_STORE_F32, G, ep, st, true, false))
       return -1;
     launch_ex(knn_gram_topc_kernel, dim3((n_rows + 3) / 4), dim3(128), 0, st, true, (const float*)G, N, Np, row0,
               n_rows, C, topj);

@@ -1,0 +1,50 @@
+"""The cluster split-K product (few rows: weights as the 128-row operand, K split over a
+thread-block cluster) through rift_linear, at the edges of its row tiles (16 to 160 rows), weight
+tiles (128 rows), K-blocks (64) and cluster sizes, against fp64 products of the same operands."""
+import pytest
+import torch
+
+from synth import rng
+
+pytestmark = pytest.mark.gpu
+
+# fp16 outputs: one rounding, 2^-11 of the element, plus fp32 sums of K products of size ~0.05: K 2^-24
+# of the sum of their magnitudes at worst, sqrt(K) 2^-24 of it for random signs.  Relative to the
+# largest output both stay under these.
+F16_TOL = 6e-4
+F32_TOL = 2e-5
+
+# (rows, weight rows, K): one K-block; 1, 2, 3 and 8 slices of K (8 K-blocks each at least), uneven
+# ones, a K tail; rows around 16, 128, 160 and in two and three row tiles; a partial weight tile
+SHAPES = [(1, 128, 64), (1, 160, 520), (2, 136, 1032), (15, 264, 1600), (16, 4096, 4096), (17, 1024, 4104),
+          (127, 288, 2816), (160, 1024, 11008), (161, 1024, 4096), (203, 672, 4104), (333, 288, 11008)]
+
+
+def _rand(shape, stream, scale=1.0):
+    n = shape[0] * shape[1]
+    return (rng.normal_f32(6, rng.stream_id("few-rows", stream), n).view(*shape) * scale).to(torch.float16)
+
+
+def _rel(g, o):
+    return float((g.double().cpu() - o).abs().max() / o.abs().max())
+
+
+@pytest.mark.parametrize("M,N,K", SHAPES)
+def test_few_rows_all_epilogues(M, N, K, cuda, riftlib):
+    A, W = _rand((M, K), 1), _rand((N, K), 2, 0.05)
+    y = A.double() @ W.double().T
+    a, w = A.to(cuda), W.to(cuda)
+    out = torch.full((M, N), float("nan"), dtype=torch.float16, device=cuda)
+    riftlib.linear(a, w, M, N, K, riftlib.RIFT_EPI_STORE_F16, out)
+    R0 = rng.normal_f32(6, 78, M * N).view(M, N)
+    R = R0.to(cuda)
+    riftlib.linear(a, w, M, N, K, riftlib.RIFT_EPI_RESID_F32, R)
+    riftlib.sync_status()
+    assert _rel(out, y) < F16_TOL
+    assert _rel(R, R0.double() + y) < F32_TOL
+    if N % 32 == 0:
+        act = torch.full((M, N // 2), float("nan"), dtype=torch.float16, device=cuda)
+        riftlib.linear(a, w, M, N, K, riftlib.RIFT_EPI_SWIGLU, act)
+        riftlib.sync_status()
+        g, u = y.view(M, N // 32, 2, 16).unbind(2)
+        assert _rel(act, (g / (1 + torch.exp(-g)) * u).reshape(M, N // 2)) < F16_TOL
