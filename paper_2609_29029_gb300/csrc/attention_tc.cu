@@ -1,4 +1,5 @@
-// Varlen causal attention on Blackwell's tcgen05 tensor cores (sm_103a).
+// Varlen causal attention on Blackwell's tcgen05 tensor cores (sm_103a), and below it the decode
+// step's attention over the KV cache.
 //
 // Work item = (128-row q-block of one packed sequence, one head).  Persistent CTAs walk the
 // items; tensor memory and barriers are set up once per CTA.  Two shapes share one kernel:
@@ -118,6 +119,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   atomicOr(&g_err_attn, RIFT_EBIT_TIMEOUT);
   *abort_flag = 1;
   return false;
+}
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+  return r;
+}
+// The shared::cluster address of this CTA's shared variable at `addr` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+  uint32_t d;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(d) : "r"(addr), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
   asm volatile(
@@ -584,6 +605,248 @@ __global__ void __launch_bounds__(1024) schedule128_kernel(const int* __restrict
   if (threadIdx.x == 0) sched[n_max] = make_int4(min(base, n_max), 0, 0, 0);
 }
 
+// ---------------------------------------------------------------- decode: one new token per sequence
+// Attention of each sequence's new token over its P = L_i cached rows and itself.  CTA = (sequence,
+// group of 256 head columns, rank r of a cluster of CS): the cached keys [P r / CS, P (r + 1) / CS).
+// One thread streams the K and V rows of the column group, SK rows at a time (a 512-byte box row
+// each), through a shared-memory ring by TMA; eight warps consume them, warp = (head of the group,
+// share of the SK rows), lanes 16 bytes (8 head dims) each, so that one warp-wide load covers
+// KPL = 256 / HD keys.  Each lane group keeps its own running maximum m, sum l and output o (online
+// softmax, fp32, log2 units); the groups, then the warps, then the cluster's CTAs (through
+// distributed shared memory) are merged, and rank 0 stores o / l.  The new token's own key and
+// value come from the QKV product's output.
+// Bound by HBM (the cache, read once).  The ring and not registers holds the rows in flight, because
+// as a programmatic dependent this kernel shares its SMs with the products around it, whose
+// shared memory leaves little of the L1 for loads in flight; and the cache and cu are inputs of
+// the whole call, so the ring is filled before the wait for the QKV product.  Measured (GB300, 7B
+// shape, under ncu): 73 sequences of 131 .. 347 rows (401 MB of cache per layer) 60.9 us, 6.6 TB/s, against
+// 64.5 + 6.4 us for (sequence, 128-key chunk) CTAs that loaded through L1 and a kernel that merged
+// the chunks; one sequence of 635 rows 9.4 against 22.4 + 5.3 us.  Whole steps of 4 layers: 829 -> 718
+// and 530 -> 444 us.
+namespace da {
+constexpr int SK = 32, NST = 3, COLS = 256, WARPS = 8, THREADS = 32 * (WARPS + 1);
+constexpr int ROW = COLS * 2, TILE = SK * ROW;  // bytes of a row of the box, of a K or V tile
+constexpr int SMEM = NST * 2 * TILE + 128 + 64;
+}  // namespace da
+
+template <int HD>
+__global__ void __launch_bounds__(da::THREADS, 2)
+    decode_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                       const uint16_t* __restrict__ qkv, const int* __restrict__ cu, int H, int CS, int max_keys,
+                       float scale_log2, uint16_t* __restrict__ out) {
+  constexpr int SK = da::SK, NST = da::NST;
+  constexpr int HPC = da::COLS / HD, KG = da::WARPS / HPC;  // heads per CTA, warps per head
+  constexpr int LPK = HD / 8, KPL = 32 / LPK;               // lanes per key, keys per warp-wide load
+  constexpr int NL = SK / KG / KPL;                         // warp-wide loads of a warp per tile
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  __shared__ __align__(8) uint64_t bars[2 * NST];
+  __shared__ int abort_smem;
+  __shared__ float part_ml[da::WARPS][2], part_o[da::WARPS][HD];
+  __shared__ float cta_ml[HPC][2], cta_o[da::COLS];
+  volatile int* abort_flag = &abort_smem;
+  const uint32_t b0 = smem_u32(bars);
+  auto FULL = [&](int s) { return b0 + 8u * s; };
+  auto EMPTY = [&](int s) { return b0 + 8u * (NST + s); };
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int groups = (H + HPC - 1) / HPC, d = H * HD;
+  const int rank = (int)cluster_ctarank(), unit = (int)blockIdx.x / CS;
+  const int g = unit % groups, i = unit / groups;
+  const int s0 = cu[i], P = cu[i + 1] - s0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(FULL(s), 1);
+      mbar_init(EMPTY(s), da::WARPS);
+    }
+    abort_smem = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  }
+  __syncthreads();
+  pdl_trigger();
+  if (P < 0 || P + 1 > max_keys) {  // uniform over the cluster: zeros, reported
+    pdl_wait();
+    if (rank == 0) {
+      if (threadIdx.x == 0) atomicOr(&g_err_attn, RIFT_EBIT_CAPACITY);
+      for (int c = threadIdx.x; c < da::COLS && g * da::COLS + c < d; c += da::THREADS)
+        out[(size_t)i * d + g * da::COLS + c] = 0;
+    }
+    return;
+  }
+  const int k0 = (int)((long long)P * rank / CS), k1 = (int)((long long)P * (rank + 1) / CS);
+  const int tiles = (k1 - k0 + SK - 1) / SK;
+
+  if (warp == da::WARPS) {
+    if (lane == 0) {
+      // ---------------- producer (tile rows past k1 hold other rows or zeros, never used)
+      int t = 0;
+      for (; t < tiles; ++t) {
+        const int s = t % NST;
+        if (!mbar_wait(EMPTY(s), ((t / NST) & 1u) ^ 1u, abort_flag)) break;
+        mbar_expect_tx(FULL(s), 2 * da::TILE);
+        const uint32_t dst = smem_u32(ring + s * 2 * da::TILE);
+        tma_load_2d(dst, &tm_k, g * da::COLS, s0 + k0 + t * SK, FULL(s));
+        tma_load_2d(dst + da::TILE, &tm_v, g * da::COLS, s0 + k0 + t * SK, FULL(s));
+      }
+      for (int j = 1; j <= NST && t - j >= 0; ++j)  // no copy left in flight (bounded)
+        for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(FULL((t - j) % NST), ((t - j) / NST) & 1u); ++w) {
+        }
+      pdl_wait();
+    }
+  } else {
+    pdl_wait();
+    const int hh = warp / KG, kg = warp % KG, h = g * HPC + hh;
+    const int sub = lane / LPK, dl = (lane % LPK) * 8;  // key within a load, first head dim of the lane
+    auto unpack = [](const uint4& u, float (&x)[8]) {
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
+        x[2 * e] = f.x;
+        x[2 * e + 1] = f.y;
+      }
+    };
+    float q[8], acc[8], m = -INFINITY, l = 0.f;
+    const uint16_t* self = qkv + (size_t)i * 3 * d + (h < H ? h : 0) * HD + dl;  // q, then k at + d, v at + 2 d
+    unpack(*reinterpret_cast<const uint4*>(self), q);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      q[e] *= scale_log2;  // scores in log2 units
+      acc[e] = 0.f;
+    }
+    auto dot = [&](const uint4& u) {
+      float kx[8];
+      unpack(u, kx);
+      float v = 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v = fmaf(q[e], kx[e], v);
+#pragma unroll
+      for (int o = LPK / 2; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      return v;
+    };
+    {
+      const float sc = dot(*reinterpret_cast<const uint4*>(self + d));
+      if (rank == 0 && kg == 0 && sub == 0) {  // the token itself
+        m = sc;
+        l = 1.f;
+        unpack(*reinterpret_cast<const uint4*>(self + 2 * d), acc);
+      }
+    }
+    for (int t = 0; t < tiles; ++t) {
+      const int s = t % NST;
+      if (!mbar_wait(FULL(s), (t / NST) & 1u, abort_flag)) break;
+      const uint8_t* kt = ring + s * 2 * da::TILE + hh * HD * 2 + dl * 2;
+      const int last = k1 - 1 - (k0 + t * SK);  // last valid row of the tile
+      float sc[NL];
+      uint4 vr[NL];
+#pragma unroll
+      for (int u = 0; u < NL; ++u) {  // rows past the last valid one read that one, with weight 0
+        const int r = kg * (SK / KG) + u * KPL + sub;
+        const uint8_t* row = kt + min(r, last) * da::ROW;
+        const float v = dot(*reinterpret_cast<const uint4*>(row));
+        vr[u] = *reinterpret_cast<const uint4*>(row + da::TILE);
+        sc[u] = r <= last ? v : -INFINITY;
+      }
+      float mx = m;
+#pragma unroll
+      for (int u = 0; u < NL; ++u) mx = fmaxf(mx, sc[u]);
+      // a lane group whose keys are all past the end keeps m = -inf (mx = -inf): nothing to add
+      const float corr = mx == -INFINITY ? 1.f : exp2f(m - mx);
+      l *= corr;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] *= corr;
+#pragma unroll
+      for (int u = 0; u < NL; ++u) {
+        const float p = mx == -INFINITY ? 0.f : exp2f(sc[u] - mx);
+        float vx[8];
+        unpack(vr[u], vx);
+        l += p;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(p, vx[e], acc[e]);
+      }
+      m = mx;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(EMPTY(s));
+    }
+    // merge the KPL lane groups (lanes l, l + LPK, ... hold the same head dims)
+#pragma unroll
+    for (int o = LPK; o < 32; o <<= 1) {
+      const float mo = __shfl_xor_sync(0xffffffffu, m, o), lo = __shfl_xor_sync(0xffffffffu, l, o);
+      const float M = fmaxf(m, mo);
+      const float fa = m == -INFINITY ? 0.f : exp2f(m - M), fb = mo == -INFINITY ? 0.f : exp2f(mo - M);
+      l = l * fa + lo * fb;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] = acc[e] * fa + __shfl_xor_sync(0xffffffffu, acc[e], o) * fb;
+      m = M;
+    }
+    if (lane == 0) {
+      part_ml[warp][0] = m;
+      part_ml[warp][1] = l;
+    }
+    if (lane < LPK) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) part_o[warp][dl + e] = acc[e];
+    }
+  }
+  // sum of n parts (m_k, l_k, o_k), in order: weights 2^(m_k - M), parts without keys (m = -inf) none
+  auto merge = [](int n, auto get_m, auto get_l, auto get_o, float& M, float& L, float& o) {
+    M = -INFINITY;
+    for (int k = 0; k < n; ++k) M = fmaxf(M, get_m(k));
+    L = 0.f;
+    o = 0.f;
+    for (int k = 0; k < n; ++k) {
+      const float mk = get_m(k), f = mk == -INFINITY ? 0.f : exp2f(mk - M);
+      L += get_l(k) * f;
+      o += get_o(k) * f;
+    }
+  };
+  __syncthreads();
+  const int c = threadIdx.x, hh = c / HD;  // one column of the group per thread (the last warp idle)
+  float M = 0.f, L = 1.f, o = 0.f;
+  if (c < da::COLS) {
+    const int w0 = hh * KG;
+    merge(KG, [&](int k) { return part_ml[w0 + k][0]; }, [&](int k) { return part_ml[w0 + k][1]; },
+          [&](int k) { return part_o[w0 + k][c % HD]; }, M, L, o);
+  }
+  if (CS > 1) {
+    if (c < da::COLS) {
+      cta_o[c] = o;
+      if (c % HD == 0) {
+        cta_ml[hh][0] = M;
+        cta_ml[hh][1] = L;
+      }
+    }
+    cluster_sync();  // every CTA's part is in place
+    if (rank == 0 && c < da::COLS) {
+      const uint32_t aml = smem_u32(&cta_ml[hh][0]), ao = smem_u32(&cta_o[c]);
+      float pm[8], pl[8], po[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < CS) {
+          pm[r] = ld_cluster(mapa_shared(aml, r));
+          pl[r] = ld_cluster(mapa_shared(aml + 4, r));
+          po[r] = ld_cluster(mapa_shared(ao, r));
+        }
+      M = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < CS) M = fmaxf(M, pm[r]);
+      L = 0.f;
+      o = 0.f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < CS) {
+          const float f = pm[r] == -INFINITY ? 0.f : exp2f(pm[r] - M);
+          L += pl[r] * f;
+          o += po[r] * f;
+        }
+    }
+    cluster_sync();  // no CTA leaves while rank 0 may still read its part
+  }
+  if (rank == 0 && c < da::COLS && g * da::COLS + c < d && !*abort_flag)
+    out[(size_t)i * d + g * da::COLS + c] = __half_as_ushort(__float2half_rn(o / L));
+}
+
 static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
@@ -639,16 +902,18 @@ int launch_shape(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMa
   return 0;
 }
 
-// fp16 [rows, cols] (row-major) as a 2-D tensor map of 64-column x box_rows boxes, 128B swizzle.
-bool make_attn_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows) {
+// fp16 [rows, cols] (row-major) as a 2-D tensor map of box_cols x box_rows boxes (64 columns with 128B
+// swizzle, or more without).
+bool make_attn_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint32_t box_rows,
+                   uint32_t box_cols = 64) {
   auto fn = fa::encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {cols, rows};
   cuuint64_t strides[1] = {cols * 2};
-  cuuint32_t box[2] = {64, box_rows};
+  cuuint32_t box[2] = {box_cols, box_rows};
   cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -679,6 +944,30 @@ int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, i
   if (head_dim == 128)
     return launch_shape<128, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st);
   return launch_shape<64, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st);
+}
+
+// Decode attention of n sequences' new tokens: K, V fp16 [T, d] (one layer of the cache), qkv fp16
+// [n, 3 d], out fp16 [n, d].  The keys of a sequence are split over a cluster while the units (sequence
+// x 256 columns) leave half the CTA slots (two per SM) empty and a rank keeps at least two tiles of
+// the longest sequence (one 635-row sequence: 16 units, 8 ranks each).
+int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16_t* V, int T, const int* cu, int n,
+                            int n_heads, int head_dim, int max_keys, uint16_t* out, cudaStream_t st, bool pdl) {
+  using namespace fa;
+  const int d = n_heads * head_dim, groups = (d + da::COLS - 1) / da::COLS;
+  CUtensorMap mk, mv;  // no cached row at all: a map nothing is loaded through
+  if (!make_attn_map(&mk, K, d, T > 0 ? T : 1, da::SK, da::COLS) ||
+      !make_attn_map(&mv, V, d, T > 0 ? T : 1, da::SK, da::COLS))
+    return 1;
+  int cs = 1;
+  while (cs < 8 && n * groups * cs <= sm_count() && max_keys >= 4 * da::SK * cs) cs *= 2;
+  const float scale_log2 = 1.4426950408889634f / sqrtf((float)head_dim);
+  auto go = [&](auto kern, std::atomic<unsigned long long>& smem_raised) -> int {
+    if (raise_smem_limit(smem_raised, kern, da::SMEM) != cudaSuccess) return 1;
+    return launch_cluster_ex(kern, dim3(n * groups * cs), dim3(da::THREADS), da::SMEM, st, pdl, cs, mk, mv, qkv, cu,
+                             n_heads, cs, max_keys, scale_log2, out) != cudaSuccess;
+  };
+  static std::atomic<unsigned long long> raised128{0}, raised64{0};
+  return head_dim == 128 ? go(decode_attn_kernel<128>, raised128) : go(decode_attn_kernel<64>, raised64);
 }
 
 }  // namespace rift

@@ -302,9 +302,9 @@ __device__ __forceinline__ float rope_mul(float x, float partner, float c, float
 
 // Rotate-half RoPE on fp32 accumulators: r1 holds dims j0..j0+31 of a head, r2 the partner
 // dims j0+half..; y1 = x1 cos - x2 sin, y2 = x2 cos + x1 sin, rounded once to fp16.
-__device__ __forceinline__ void rope_chunk(const uint32_t (&r1)[32], const uint32_t (&r2)[32], int row, int col,
-                                           int half, int N, int pos, const float2* __restrict__ tab, void* C) {
-  uint16_t* out = static_cast<uint16_t*>(C) + (size_t)row * N + col;
+// `out`: the row's element of r1[0]; `copy` (nullable): a second place to store to (the KV cache).
+__device__ __forceinline__ void rope_chunk(const uint32_t (&r1)[32], const uint32_t (&r2)[32], int col, int half,
+                                           int pos, const float2* __restrict__ tab, uint16_t* out, uint16_t* copy) {
   const int head_dim = 2 * half;
   const int j0 = col % head_dim;
   const float2* cs = tab + (size_t)pos * half + j0;
@@ -317,13 +317,17 @@ __device__ __forceinline__ void rope_chunk(const uint32_t (&r1)[32], const uint3
     p1[e / 2] = pack_half2(rope_mul(a0, b0, c0.x, -c0.y), rope_mul(a1, b1, c1.x, -c1.y));
     p2[e / 2] = pack_half2(rope_mul(b0, a0, c0.x, c0.y), rope_mul(b1, a1, c1.x, c1.y));
   }
-  uint4* o1 = reinterpret_cast<uint4*>(out);
-  uint4* o2 = reinterpret_cast<uint4*>(out + half);
+  auto store = [&](uint16_t* dst) {
+    uint4* o1 = reinterpret_cast<uint4*>(dst);
+    uint4* o2 = reinterpret_cast<uint4*>(dst + half);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    o1[q] = make_uint4(p1[4 * q], p1[4 * q + 1], p1[4 * q + 2], p1[4 * q + 3]);
-    o2[q] = make_uint4(p2[4 * q], p2[4 * q + 1], p2[4 * q + 2], p2[4 * q + 3]);
-  }
+    for (int q = 0; q < 4; ++q) {
+      o1[q] = make_uint4(p1[4 * q], p1[4 * q + 1], p1[4 * q + 2], p1[4 * q + 3]);
+      o2[q] = make_uint4(p2[4 * q], p2[4 * q + 1], p2[4 * q + 2], p2[4 * q + 3]);
+    }
+  };
+  store(out);
+  if (copy) store(copy);
 }
 
 // K-block k of an operand read through EpiParams' remap (mode 1: [hi | hi | lo], 2: [hi | lo | hi]
@@ -472,7 +476,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int row = m_blk * TM + (int)rank * BM + quarter * 32 + lane;
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * ACC_COLS);
       if constexpr (EPI == EPI_QKV_ROPE) {
-        const int half = ep.head_dim >> 1;
+        const int half = ep.head_dim >> 1, kv_d = ep.rope_cols >> 1;
         const int pos = (row < M) ? ep.positions[row] + ep.pos_offset : 0;
         const bool pos_ok = pos >= 0 && pos < ep.max_len;
         if (row < M && !pos_ok) atomicOr(&g_err_gemm, RIFT_EBIT_BADID);
@@ -485,11 +489,16 @@ __global__ void __launch_bounds__(THREADS, 1)
             uint32_t r1[32], r2[32];
             tmem_ld32(taddr + c, r1);
             tmem_ld32(taddr + c + half, r2);
-            if (row < M && pos_ok) rope_chunk(r1, r2, row, col, half, N, pos, ep.rope, C);
+            if (row < M && pos_ok)
+              rope_chunk(r1, r2, col, half, pos, ep.rope, static_cast<uint16_t*>(C) + (size_t)row * N + col,
+                         ep.k_out && col >= kv_d ? ep.k_out + (size_t)row * kv_d + col - kv_d : nullptr);
           } else {
             uint32_t r[32];
             tmem_ld32(taddr + c, r);
-            if (row < M) epilogue_chunk<EPI_STORE_BF16>(r, row, col, N, C);
+            if (row < M) {
+              epilogue_chunk<EPI_STORE_BF16>(r, row, col, N, C);
+              if (ep.v_out) epilogue_chunk<EPI_STORE_BF16>(r, row, col - ep.rope_cols, kv_d, ep.v_out);
+            }
           }
         }
       } else {
@@ -780,6 +789,12 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
             }
           }
           store_h4(static_cast<uint16_t*>(C) + row * N + col, v.x, v.y, v.z, v.w);
+          if constexpr (EPI == EPI_QKV_ROPE) {
+            const int kv_d = ep.rope_cols >> 1;
+            if (ep.k_out && col >= kv_d)
+              store_h4(col < ep.rope_cols ? ep.k_out + row * kv_d + col - kv_d : ep.v_out + row * kv_d + col - ep.rope_cols,
+                       v.x, v.y, v.z, v.w);
+          }
         }
       }
     }

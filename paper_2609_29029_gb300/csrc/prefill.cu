@@ -10,7 +10,7 @@
 //   act = SiLU(xn W_g^T) * (xn W_u^T)            GEMM, SwiGLU epilogue (interleaved gate/up)
 //   h  += act W_down^T                           GEMM, fp32 residual epilogue
 // and finally hidden = RMSNorm(h) g_final in bf16.  Optional outputs: each layer's keys (after
-// RoPE) and values copied out of the QKV buffer (the KV cache), and the logits of every
+// RoPE) and values (the KV cache, stored by the QKV product's epilogue), and the logits of every
 // sequence's last token, RMSNorm(h_last) g_final times the output matrix.
 //
 // The decode step runs the same layer sequence for one new token per sequence, at position L_i,
@@ -112,31 +112,6 @@ __global__ void rope_table_kernel(float2* __restrict__ tab, int max_len, int hal
   double s, c;
   sincos((double)p * inv, &s, &c);
   tab[i] = make_float2((float)c, (float)s);
-}
-
-// KV cache rows: k_out[r] = qkv[r, d .. 2d), v_out[r] = qkv[r, 2d .. 3d) (fp16, heads contiguous),
-// for the rows below the device count rows_dev clamped to rows (all rows without one).
-__global__ void kv_store_kernel(const uint16_t* __restrict__ qkv, int rows, const int* __restrict__ rows_dev, int d,
-                                uint16_t* __restrict__ k_out, uint16_t* __restrict__ v_out) {
-  const int nv = d / 8;  // uint4 per row half
-  if (rows_dev) rows = max(0, min(rows, *rows_dev));
-  const size_t total = (size_t)rows * 2 * nv;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t r = e / (2 * nv);
-    const int c = (int)(e % (2 * nv));
-    const uint4 v = reinterpret_cast<const uint4*>(qkv + r * 3 * d + d)[c];
-    if (c < nv)
-      reinterpret_cast<uint4*>(k_out + r * d)[c] = v;
-    else
-      reinterpret_cast<uint4*>(v_out + r * d)[c - nv] = v;
-  }
-}
-
-static void kv_store(const uint16_t* qkv, int rows, const int* rows_dev, int d, uint16_t* k_out, uint16_t* v_out,
-                     cudaStream_t st) {
-  const size_t total = (size_t)rows * (d / 4);
-  const int grid = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  kv_store_kernel<<<grid, 256, 0, st>>>(qkv, rows, rows_dev, d, k_out, v_out);
 }
 
 // Rows T .. T + n_tail - 1 (clamped to the cap rows of the buffer) of an fp16 [cap, cols] buffer
@@ -288,11 +263,11 @@ int launch_prefill(const rift_model& m, void* hidden, int T, const int* T_dev, c
       norm_launch(0, T, hidden, h32, m.g_attn[0], xn, d, m.eps, st, T_dev);
     else
       norm_launch(1, T, h32, nullptr, m.g_attn[l], xn, d, m.eps, st, T_dev);
-    if (launch_gemm(xn, m.w_qkv[l], T, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep)) return 1;
     if (kv_out) {
-      uint16_t* kl = static_cast<uint16_t*>(kv_out) + (size_t)l * 2 * T * d;
-      kv_store(qkv, T, T_dev, d, kl, kl + (size_t)T * d, st);
+      rope_ep.k_out = static_cast<uint16_t*>(kv_out) + (size_t)l * 2 * T * d;
+      rope_ep.v_out = rope_ep.k_out + (size_t)T * d;
     }
+    if (launch_gemm(xn, m.w_qkv[l], T, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep)) return 1;
     prof_begin(RIFT_PROF_ATTN, st);
     const uint16_t* pk = prefix_kv ? static_cast<const uint16_t*>(prefix_kv) + (size_t)l * 2 * S_pre * d : nullptr;
     if (launch_attention(qkv, T, cu_seqlens, n_seq, m.n_heads, m.head_dim, sched, L.max_qblocks, att, st, pk,
@@ -378,9 +353,6 @@ int launch_prefill_shared_prefix(const rift_model& m, const int* sys_ids, int S,
 // Decode step: one new token per sequence
 // ------------------------------------------------------------------------------------------
 
-constexpr int DEC_CHUNK = 128;  // keys per decode-attention work unit
-constexpr int DEC_HG = 8;       // heads per decode-attention CTA (one warp each)
-
 DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len) {
   DecodeLayout L{};
   size_t off = 0;
@@ -394,8 +366,6 @@ DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len) {
   L.act_off = take(n * m.ffn * 2);
   L.rope_off = take((size_t)max_len * (m.head_dim / 2) * sizeof(float2));
   L.pos_off = take(n * sizeof(int));
-  // decode attention partials: (m, l, o[head_dim]) per (sequence, key chunk, head)
-  L.dpart_off = take(n * (size_t)((max_len + DEC_CHUNK - 1) / DEC_CHUNK) * m.n_heads * (m.head_dim + 2) * 4);
   L.total = off;
   return L;
 }
@@ -418,145 +388,6 @@ __global__ void decode_embed_kernel(const int* __restrict__ ids, const int* __re
 }
 
 
-// Attention of each sequence's new token over its P = L_i cached rows and itself, split like
-// flash decoding: CTA (sequence i, chunk c of DEC_CHUNK keys, group of hg heads: the largest of
-// 8, 4, 2, 1 that divides H), one warp per head.  A key row's hg head slices are hg * head_dim * 2
-// contiguous bytes, read together by the CTA's warps.  Lanes read 16 bytes (8 head dims) each, so
-// one warp-wide load covers KPL = 256 / head_dim keys, LPK = head_dim / 8 lanes per key; each
-// lane group keeps its own running maximum m, sum l and output o over its keys (online softmax,
-// fp32, log2 units) and the groups are merged at the end of the chunk.  (m, l, o) of the chunk go
-// to `part`, and decode_combine_kernel merges a sequence's chunks.  Units past a sequence's last
-// key exit at once.
-template <int HD>
-__global__ void __launch_bounds__(DEC_HG * 32, 3) decode_attn_kernel(const uint16_t* __restrict__ qkv,
-                                                                     const uint16_t* __restrict__ Kc,
-                                                                     const uint16_t* __restrict__ Vc,
-                                                                     const int* __restrict__ cu, int H, int hg,
-                                                                     int max_chunks, float scale_log2,
-                                                                     float* __restrict__ part) {
-  pdl_trigger();
-  pdl_wait();
-  constexpr int LPK = HD / 8, KPL = 32 / LPK;  // lanes per key, keys per warp-wide load
-  constexpr int NL = 4;                        // warp-wide loads of K (and of V) in flight
-  const int groups = H / hg;  // hg = blockDim.x / 32 heads per CTA
-  const int g = blockIdx.x % groups, c = (blockIdx.x / groups) % max_chunks, i = blockIdx.x / (groups * max_chunks);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = g * hg + warp;
-  const int d = H * HD;
-  const int s0 = cu[i], P = cu[i + 1] - s0, nk = P + 1;
-  const int j_begin = c * DEC_CHUNK, j_end = min(nk, j_begin + DEC_CHUNK);
-  if (j_begin >= nk) return;
-  const int sub = lane / LPK, dl = (lane % LPK) * 8;  // key within a load, first head dim of the lane
-  const uint16_t* self = qkv + (size_t)i * 3 * d + h * HD;  // q, then k at + d, v at + 2d
-  auto unpack = [](const uint4& u, float (&x)[8]) {
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[e]));
-      x[2 * e] = f.x;
-      x[2 * e + 1] = f.y;
-    }
-  };
-  float q[8];
-  unpack(__ldg(reinterpret_cast<const uint4*>(self + dl)), q);
-#pragma unroll
-  for (int e = 0; e < 8; ++e) q[e] *= scale_log2;  // scores in log2 units
-  float m = -INFINITY, l = 0.f, acc[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-  for (int j0 = j_begin; j0 < j_end; j0 += NL * KPL) {
-    uint4 kr[NL], vr[NL];
-#pragma unroll
-    for (int u = 0; u < NL; ++u) {  // rows past the chunk end read the last row, weight 0
-      const int j = min(j0 + u * KPL + sub, j_end - 1);
-      const size_t r = (size_t)(s0 + j) * d + h * HD + dl;
-      kr[u] = __ldg(reinterpret_cast<const uint4*>(j < P ? Kc + r : self + d + dl));
-      vr[u] = __ldg(reinterpret_cast<const uint4*>(j < P ? Vc + r : self + 2 * d + dl));
-    }
-    float sc[NL];
-#pragma unroll
-    for (int u = 0; u < NL; ++u) {
-      float kx[8];
-      unpack(kr[u], kx);
-      float dot = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) dot = fmaf(q[e], kx[e], dot);
-#pragma unroll
-      for (int o = LPK / 2; o >= 1; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      sc[u] = (j0 + u * KPL + sub < j_end) ? dot : -INFINITY;
-    }
-    float mx = m;
-#pragma unroll
-    for (int u = 0; u < NL; ++u) mx = fmaxf(mx, sc[u]);
-    // a lane group whose keys are all past the end keeps m = -inf (mx = -inf): nothing to add
-    const float corr = mx == -INFINITY ? 1.f : exp2f(m - mx);
-    l *= corr;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] *= corr;
-#pragma unroll
-    for (int u = 0; u < NL; ++u) {
-      const float p = mx == -INFINITY ? 0.f : exp2f(sc[u] - mx);
-      float vx[8];
-      unpack(vr[u], vx);
-      l += p;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] = fmaf(p, vx[e], acc[e]);
-    }
-    m = mx;
-  }
-  // merge the KPL lane groups (lanes l, l + LPK, ... hold the same head dims)
-#pragma unroll
-  for (int o = LPK; o < 32; o <<= 1) {
-    const float mo = __shfl_xor_sync(0xffffffffu, m, o), lo = __shfl_xor_sync(0xffffffffu, l, o);
-    const float M = fmaxf(m, mo);
-    const float fa = m == -INFINITY ? 0.f : exp2f(m - M), fb = mo == -INFINITY ? 0.f : exp2f(mo - M);
-    l = l * fa + lo * fb;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = acc[e] * fa + __shfl_xor_sync(0xffffffffu, acc[e], o) * fb;
-    m = M;
-  }
-  float* dst = part + (((size_t)i * max_chunks + c) * H + h) * (HD + 2);
-  if (lane == 0) {
-    dst[0] = m;
-    dst[1] = l;
-  }
-  if (lane < LPK) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) dst[2 + dl + e] = acc[e];
-  }
-}
-
-// out[i, h] = sum_c o_c 2^(m_c - M) / sum_c l_c 2^(m_c - M), chunks in order (M = max_c m_c).
-// A sequence with more than max_keys keys sets RIFT_EBIT_CAPACITY and gets zeros.
-__global__ void decode_combine_kernel(const float* __restrict__ part, const int* __restrict__ cu, int H, int HD,
-                                      int max_chunks, int max_keys, uint16_t* __restrict__ out) {
-  pdl_trigger();
-  pdl_wait();
-  const int i = blockIdx.x / H, h = blockIdx.x % H;
-  const int nk = cu[i + 1] - cu[i] + 1;
-  uint16_t* o = out + ((size_t)i * H + h) * HD;
-  if (nk > max_keys) {
-    if (threadIdx.x == 0) atomicOr(&g_err_prefill, RIFT_EBIT_CAPACITY);
-    for (int e = threadIdx.x; e < HD; e += blockDim.x) o[e] = 0;
-    return;
-  }
-  const int nch = (nk + DEC_CHUNK - 1) / DEC_CHUNK;
-  const float* p0 = part + ((size_t)i * max_chunks * H + h) * (HD + 2);
-  const size_t cstride = (size_t)H * (HD + 2);
-  float M = -INFINITY;
-  for (int c = 0; c < nch; ++c) M = fmaxf(M, p0[c * cstride]);
-  for (int e = threadIdx.x; e < HD; e += blockDim.x) {
-    float L = 0.f, v = 0.f;
-    for (int c = 0; c < nch; ++c) {
-      const float* pc = p0 + c * cstride;
-      const float f = exp2f(pc[0] - M);
-      L += pc[1] * f;
-      v += pc[2 + e] * f;
-    }
-    o[e] = __half_as_ushort(__float2half_rn(v / L));
-  }
-}
-
 int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* cu_seqlens, int n_seq, int max_len,
                   const int* token_ids, const void* embed, int vocab_embed, void* hidden_out, void* kv_new,
                   float* logits, char* ws, cudaStream_t st) {
@@ -570,10 +401,6 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   uint16_t* act = reinterpret_cast<uint16_t*>(ws + L.act_off);
   float2* rope = reinterpret_cast<float2*>(ws + L.rope_off);
   int* pos = reinterpret_cast<int*>(ws + L.pos_off);
-  float* dpart = reinterpret_cast<float*>(ws + L.dpart_off);
-  const int max_chunks = (max_len + DEC_CHUNK - 1) / DEC_CHUNK;
-  int hg = DEC_HG;
-  while (m.n_heads % hg != 0) hg /= 2;
   const int d = m.d, half = m.head_dim / 2, n = n_seq;
 
   rope_table_kernel<<<(max_len * half + 255) / 256, 256, 0, st>>>(rope, max_len, half, m.rope_theta);
@@ -585,7 +412,6 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   rope_ep.rope_cols = 2 * d;
   rope_ep.head_dim = m.head_dim;
   rope_ep.max_len = max_len;
-  const float scale_log2 = 1.4426950408889634f / sqrtf((float)m.head_dim);
   const uint16_t* kv = static_cast<const uint16_t*>(kv_cache);
   norm_launch(0, n, x0, h32, m.g_attn[0], xn, d, m.eps, st);
   // The layer's kernels are launched as programmatic dependents of the kernel before them: each
@@ -593,27 +419,16 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   // and waits for it before touching activations.
   const bool pdl = true;
   for (int l = 0; l < m.n_layers; ++l) {
-    if (launch_gemm(xn, m.w_qkv[l], n, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep, pdl)) return 1;
     if (kv_new) {
-      uint16_t* kl = static_cast<uint16_t*>(kv_new) + (size_t)l * 2 * n * d;
-      kv_store(qkv, n, nullptr, d, kl, kl + (size_t)n * d, st);
+      rope_ep.k_out = static_cast<uint16_t*>(kv_new) + (size_t)l * 2 * n * d;
+      rope_ep.v_out = rope_ep.k_out + (size_t)n * d;
     }
+    if (launch_gemm(xn, m.w_qkv[l], n, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep, pdl)) return 1;
     const uint16_t* Kc = kv + (size_t)l * 2 * T * d;
     const uint16_t* Vc = Kc + (size_t)T * d;
     prof_begin(RIFT_PROF_ATTN, st);
-    const int units = n * max_chunks * (m.n_heads / hg);
-    cudaError_t e;
-    if (m.head_dim == 128)
-      e = launch_ex(decode_attn_kernel<128>, dim3(units), dim3(hg * 32), 0, st, pdl, (const uint16_t*)qkv, Kc, Vc,
-                    cu_seqlens, (int)m.n_heads, hg, max_chunks, scale_log2, dpart);
-    else
-      e = launch_ex(decode_attn_kernel<64>, dim3(units), dim3(hg * 32), 0, st, pdl, (const uint16_t*)qkv, Kc, Vc,
-                    cu_seqlens, (int)m.n_heads, hg, max_chunks, scale_log2, dpart);
-    if (e != cudaSuccess) return 1;
-    if (launch_ex(decode_combine_kernel, dim3(n * m.n_heads), dim3(m.head_dim), 0, st, pdl, (const float*)dpart,
-                  cu_seqlens, (int)m.n_heads, (int)m.head_dim, max_chunks, max_len, att) != cudaSuccess)
-      return 1;
-    prof_end(RIFT_PROF_ATTN, st, 2);
+    if (launch_decode_attention(qkv, Kc, Vc, T, cu_seqlens, n, m.n_heads, m.head_dim, max_len, att, st, pdl)) return 1;
+    prof_end(RIFT_PROF_ATTN, st, 1);
     if (launch_gemm(att, m.w_o[l], n, d, d, EPI_RESID_F32, h32, st, EpiParams(), pdl)) return 1;
     norm_launch(1, n, h32, nullptr, m.g_ffn[l], xn, d, m.eps, st, nullptr, pdl);
     if (launch_gemm(xn, m.w_gate_up[l], n, 2 * m.ffn, d, EPI_SWIGLU, act, st, EpiParams(), pdl)) return 1;
@@ -622,7 +437,8 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
     norm_launch(1, n, h32, nullptr, next_gain, xn, d, m.eps, st, nullptr, pdl);
   }
   // xn now holds RMSNorm(h) g_final in fp16 (the logits operand)
-  if (hidden_out) norm_launch(2, n, h32, nullptr, m.g_final, static_cast<uint16_t*>(hidden_out), d, m.eps, st);
+  if (hidden_out)
+    norm_launch(2, n, h32, nullptr, m.g_final, static_cast<uint16_t*>(hidden_out), d, m.eps, st, nullptr, pdl);
   if (logits) {
     if (launch_gemm(xn, m.lm_head, n, m.vocab, d, EPI_STORE_F32, logits, st, EpiParams(), pdl)) return 1;
   }

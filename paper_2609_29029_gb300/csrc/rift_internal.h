@@ -119,7 +119,7 @@ int launch_prefill_shared_prefix(const rift_model& m, const int* sys_ids, int S,
                                  const int* cu_seqlens, int n_seq, const int* n_seq_dev, int max_len,
                                  const int* positions, float* last_logits, char* ws, cudaStream_t st);
 struct DecodeLayout {
-  size_t h32_off, x0_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, dpart_off, total;
+  size_t h32_off, x0_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, total;
 };
 DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len);
 int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* cu_seqlens, int n_seq, int max_len,
@@ -141,6 +141,10 @@ struct EpiParams {
   int head_dim = 0;
   int max_len = 0;
   int pos_offset = 0;              // added to positions[row] (rows that follow a shared prefix)
+  // EPI_QKV_ROPE, nullable: the KV cache's keys (columns rope_cols / 2 .. rope_cols, after RoPE) and
+  // values (columns rope_cols ..) of the layer, fp16 [M, rope_cols / 2] each, written beside C
+  uint16_t* k_out = nullptr;
+  uint16_t* v_out = nullptr;
   float out_scale = 1.f;           // EPI_STORE_F32
   // Device row count (nullable): the product covers rows min(M, *m_dev); M is then the capacity
   // the operands and the output are sized for.
@@ -183,6 +187,10 @@ void launch_attention_schedule(const int* cu_seqlens, int n_seq, const int* n_se
 int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, int n_heads, int head_dim,
                      const int4* sched, int n_sched_max, void* out, cudaStream_t st, const void* prefix_k = nullptr,
                      const void* prefix_v = nullptr, int S_pre = 0);
+// Decode attention: each of n sequences' new token (qkv fp16 [n, 3 d]) over its cached rows (K, V fp16
+// [T, d], one layer) and itself; a sequence with more than max_keys keys sets RIFT_EBIT_CAPACITY.
+int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16_t* V, int T, const int* cu, int n,
+                            int n_heads, int head_dim, int max_keys, uint16_t* out, cudaStream_t st, bool pdl);
 unsigned int read_clear_err_attn();
 
 }  // namespace rift

@@ -1,0 +1,56 @@
+"""The decode step's attention (keys streamed in 32-row tiles through a TMA ring, split over a
+cluster when there are few sequences) through rift_decode_step: cached lengths around the tile and
+the cluster's shares, one and many sequences, both head sizes and a head count that leaves part of
+the last 256-column group empty; against the oracle at the hidden-state tolerance."""
+import pytest
+import torch
+
+from oracle import rift_oracle as O
+from synth import rng, workloads as W
+
+import parity as P
+
+pytestmark = pytest.mark.gpu
+
+HD128 = W.DecoderShape(n_layers=1, d=640, n_heads=5, head_dim=128, ffn=688, vocab=504)   # 2.5 column groups
+HD64 = W.DecoderShape(n_layers=1, d=320, n_heads=5, head_dim=64, ffn=688, vocab=504)      # 1.25 column groups
+
+LENGTHS = {"one": [600], "one_short": [1], "edges": [0, 1, 31, 32, 33, 95, 96, 97, 128, 257],
+           "many": [(7 * i) % 70 for i in range(160)]}  # 480 units of 2-3 column groups: no cluster
+
+
+@pytest.mark.parametrize("name", list(LENGTHS))
+@pytest.mark.parametrize("dec", [HD64, HD128], ids=["hd64", "hd128"])
+def test_decode_attention_lengths(dec, name, cuda, riftlib):
+    from paper_2609_29029_gb300 import DeviceModel
+    lens = LENGTHS[name]
+    n, T, d, hd = len(lens), sum(lens), dec.d, dec.head_dim
+    layers = [W.make_layer(dec, 0, "cpu")]
+    gf = W.make_final_norm(dec, "cpu")
+    dm = DeviceModel(dec, layers, gf, cuda)
+    # rows after the last cached one hold NaN: no row of another sequence may enter a sum
+    kv = rng.normal_f32(21, rng.stream_id("dec-kv"), 2 * T * d).view(1, 2, T, d).to(torch.float16)
+    kv_d = torch.full((1, 2, T + 40, d), float("nan"), dtype=torch.float16, device=cuda)
+    kv_d[:, :, :T] = kv.to(cuda)
+    cu = [0]
+    for L in lens:
+        cu.append(cu[-1] + L)
+    embed = rng.normal_f32(22, rng.stream_id("dec-embed"), 40 * d).view(40, d).to(torch.bfloat16)
+    ids = [(5 * i + 3) % 40 for i in range(n)]
+    max_len = max(lens) + 1
+    hid = torch.empty(n, d, dtype=torch.bfloat16, device=cuda)
+    kvn = torch.empty(1, 2, n, d, dtype=torch.float16, device=cuda)
+    need = riftlib.decode_workspace_bytes(dm.struct, n, max_len)
+    ws = torch.empty(need, dtype=torch.uint8, device=cuda)
+    riftlib.decode_step(dm.struct, kv_d, T + 40, torch.tensor(cu, dtype=torch.int32, device=cuda), n, max_len,
+                        torch.tensor(ids, dtype=torch.int32, device=cuda), embed.to(cuda), 40, hid, kvn, None, ws, need)
+    riftlib.sync_status()
+    worst = 0.0
+    for i in sorted(set(range(min(n, 12))) | {n - 1}):
+        cache = [(kv[0, 0, cu[i]:cu[i + 1]].double().view(-1, dec.n_heads, hd),
+                  kv[0, 1, cu[i]:cu[i + 1]].double().view(-1, dec.n_heads, hd))]
+        ref, new = O.decode_token(embed[ids[i]], cache, lambda l: layers[l], gf, dec)
+        for got, want in ((hid[i], ref), (kvn[0, 0, i], new[0][0]), (kvn[0, 1, i], new[0][1])):
+            want = want.double().reshape(-1)
+            worst = max(worst, float((got.double().cpu().reshape(-1) - want).abs().max() / want.abs().max()))
+    assert worst < P.HIDDEN_TOL, worst
