@@ -29,6 +29,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "rift_internal.h"
@@ -299,6 +300,8 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_trigger();
+  pdl_wait();
   const int n_items = min(n_entries, sched[n_entries].x) * H;  // entries in use (the schedule's count)
   const int d = H * HD;
   const int np = (S_pre + KB - 1) / KB;  // prefix blocks ahead of every sequence's own
@@ -564,12 +567,29 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
 // sequence count is n_seq_dev's value when given (a count written by an earlier kernel), clamped
 // to n_seq; a sequence that ends past row_cap (the rows the buffers hold) and the sequences after
 // it are left out and RIFT_EBIT_CAPACITY is set.  Longer sequences' entries are not reordered:
-// items are interleaved across CTAs by the persistent loop.
+// items are interleaved across CTAs by the persistent loop.  CTA 0 builds the schedule; the others
+// (a prefill's) fill the RoPE table and zero the rows past T that the attention's last query tile
+// and key block can reach (up to 127): a masked key still meets its value row in the P V product,
+// where 0 x NaN = NaN, so those rows must hold finite values (with the row count equal to the
+// capacity they are out of bounds and read as zero instead).
 __global__ void __launch_bounds__(1024) schedule128_kernel(const int* __restrict__ cu, int n_seq,
                                                            const int* __restrict__ n_seq_dev, int row_cap,
-                                                           int4* __restrict__ sched, int n_max) {
+                                                           int4* __restrict__ sched, int n_max,
+                                                           const __grid_constant__ PrefillSetup ps) {
   __shared__ int sh[33];
   __shared__ int s_cut;
+  pdl_trigger();
+  if (blockIdx.x > 0) {
+    const size_t i0 = (size_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x, step = (size_t)(gridDim.x - 1) * blockDim.x;
+    for (size_t i = i0; i < (size_t)ps.max_len * ps.half; i += step)
+      ps.rope[i] = rope_cos_sin((double)(i / ps.half) * ps.freq.inv[i % ps.half]);
+    if (ps.T_dev) {
+      const int T = max(0, min(row_cap, *ps.T_dev)), rows = min(128, row_cap - T), nv = ps.tail_cols / 8;
+      for (size_t e = i0; e < (size_t)rows * nv; e += step)
+        reinterpret_cast<uint4*>(ps.tail + (size_t)(T + e / nv) * ps.tail_cols)[e % nv] = make_uint4(0, 0, 0, 0);
+    }
+    return;
+  }
   int n = n_seq;
   if (n_seq_dev) {
     const int nd = *n_seq_dev;
@@ -875,8 +895,15 @@ static int sm_count() {
 
 // q-block schedule of the tcgen05 attention (one entry per 128 rows of a sequence)
 void launch_attention_schedule(const int* cu_seqlens, int n_seq, const int* n_seq_dev, int row_cap, int4* sched,
-                               int n_sched_max, cudaStream_t st) {
-  fa::schedule128_kernel<<<1, 1024, 0, st>>>(cu_seqlens, n_seq, n_seq_dev, row_cap, sched, n_sched_max);
+                               int n_sched_max, cudaStream_t st, const PrefillSetup* setup) {
+  if (!setup) {
+    fa::schedule128_kernel<<<1, 1024, 0, st>>>(cu_seqlens, n_seq, n_seq_dev, row_cap, sched, n_sched_max, PrefillSetup{});
+    return;
+  }
+  // a table value per thread: 256 threads of a block keep its double operations spread over the SMs
+  const size_t work = (size_t)setup->max_len * setup->half;
+  const int blocks = (int)std::min<size_t>((work + 255) / 256, 4096);
+  fa::schedule128_kernel<<<1 + blocks, 256, 0, st>>>(cu_seqlens, n_seq, n_seq_dev, row_cap, sched, n_sched_max, *setup);
 }
 
 int attention_max_qblocks(int max_T, int max_seqs) { return (max_T + fa::BQ - 1) / fa::BQ + max_seqs; }
@@ -889,7 +916,7 @@ constexpr int kAttnKB = 64;
 template <int HD, int KB>
 int launch_shape(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMap& mpk, const CUtensorMap& mpv,
                  int S_pre, const int4* sched, int n_sched_max, int n_heads, float scale_log2, void* out,
-                 cudaStream_t st) {
+                 cudaStream_t st, bool pdl) {
   using namespace fa;
   using CF = Cfg<HD, KB>;
   static std::atomic<unsigned long long> smem_raised{0};
@@ -897,9 +924,8 @@ int launch_shape(const CUtensorMap& mq, const CUtensorMap& mkv, const CUtensorMa
   const int items = n_sched_max * n_heads;
   const int slots = CF::CTAS * sm_count();
   const int grid = items < slots ? items : slots;
-  attn_tc_kernel<HD, KB><<<grid, THREADS, CF::SMEM, st>>>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads,
-                                                          scale_log2, static_cast<uint16_t*>(out));
-  return 0;
+  return launch_ex(attn_tc_kernel<HD, KB>, dim3(grid), dim3(THREADS), CF::SMEM, st, pdl, mq, mkv, mpk, mpv, S_pre, sched,
+                   n_sched_max, n_heads, scale_log2, static_cast<uint16_t*>(out)) != cudaSuccess;
 }
 
 // fp16 [rows, cols] (row-major) as a 2-D tensor map of box_cols x box_rows boxes (64 columns with 128B
@@ -923,7 +949,7 @@ bool make_attn_map(CUtensorMap* map, const void* base, uint64_t cols, uint64_t r
 // values fp16 [S_pre, H hd] attended to by every sequence before its own rows.
 int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, int n_heads, int head_dim,
                      const int4* sched, int n_sched_max, void* out, cudaStream_t st, const void* prefix_k,
-                     const void* prefix_v, int S_pre) {
+                     const void* prefix_v, int S_pre, bool pdl) {
   using namespace fa;
   (void)n_seq;
   (void)cu_seqlens;  // the schedule entries carry the sequence bounds
@@ -942,8 +968,8 @@ int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, i
   }
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)head_dim);
   if (head_dim == 128)
-    return launch_shape<128, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st);
-  return launch_shape<64, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st);
+    return launch_shape<128, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st, pdl);
+  return launch_shape<64, kAttnKB>(mq, mkv, mpk, mpv, S_pre, sched, n_sched_max, n_heads, scale_log2, out, st, pdl);
 }
 
 // Decode attention of n sequences' new tokens: K, V fp16 [T, d] (one layer of the cache), qkv fp16

@@ -1020,7 +1020,7 @@ static int band_group(int M, int N, int K, int tm, int tn, int lo, int hi) {
 // (the caller then takes the cluster split-K kernel).
 template <int EPI>
 static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, void* C, const EpiParams& ep,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool pdl) {
   constexpr size_t smem = (size_t)STAGES * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
   auto kern = gemm_tc_kernel<EPI>;
   cudaLaunchAttribute attr[1];
@@ -1058,9 +1058,10 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
   const int units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
   const int clusters = units < max_clusters ? units : max_clusters;
   const int group_m = band_group(M, N, K, 2 * BM, BN, 4, 32);
-  cfg.gridDim = dim3(2 * clusters, 1, 1);
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, kern, a, b, M, N, K, C, ep, group_m) == cudaSuccess ? 0 : 1;
+  return launch_cluster_ex(kern, dim3(2 * clusters), dim3(THREADS), smem, st, pdl, 2, a, b, M, N, K, C, ep, group_m) ==
+                 cudaSuccess
+             ? 0
+             : 1;
 }
 
 // The cluster split-K kernel: S CTAs per (128 weight rows, bn rows) tile.
@@ -1149,11 +1150,11 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2)) return 1;
   int r = -1;
   switch (epi) {
-    case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, M, N, K, C, ep, st); break;
-    case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb, M, N, K, C, ep, st); break;
-    case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb, M, N, K, C, ep, st); break;
-    case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb, M, N, K, C, ep, st); break;
-    case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb, M, N, K, C, ep, st); break;
+    case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, M, N, K, C, ep, st, pdl); break;
+    case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb, M, N, K, C, ep, st, pdl); break;
+    case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb, M, N, K, C, ep, st, pdl); break;
+    case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb, M, N, K, C, ep, st, pdl); break;
+    case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb, M, N, K, C, ep, st, pdl); break;
     default: return 1;
   }
   if (r >= 0) return r;

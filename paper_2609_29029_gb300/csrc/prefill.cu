@@ -20,6 +20,7 @@
 // moves the final hidden states by about 3% of their largest magnitude; fp16 (3 more mantissa
 // bits, same tensor-core rate, LLaVA-1.5-7B's checkpoint dtype) keeps the whole path near 0.5%.
 #include <atomic>
+#include <cmath>
 #include <type_traits>
 
 #include "rift_internal.h"
@@ -37,11 +38,11 @@ unsigned int read_clear_err_prefill() {
 
 constexpr int NORM_THREADS = 256;
 
-// One row of the RMSNorm below.
+// One row of the RMSNorm below: row `row` of out (and h32) from row `in_row` of in (negative: zeros).
 template <bool IN_BF16, bool OUT_F16, int VPT>
 __device__ __forceinline__ void rmsnorm_row(const void* __restrict__ in, float* __restrict__ h32,
                                             const uint16_t* __restrict__ gain, uint16_t* __restrict__ out, int d,
-                                            float eps, size_t row, float* red) {
+                                            float eps, size_t row, long long in_row, float* red) {
   const int nv = d / 4;
   float4 v[VPT];
   float ss = 0.f;
@@ -50,12 +51,13 @@ __device__ __forceinline__ void rmsnorm_row(const void* __restrict__ in, float* 
     const int c = threadIdx.x + q * NORM_THREADS;
     if (c < nv) {
       if constexpr (IN_BF16) {
-        uint2 raw = reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(in) + row * d)[c];
+        const uint2 raw = in_row >= 0 ? reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(in) + in_row * d)[c]
+                                      : make_uint2(0u, 0u);
         v[q] = make_float4(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xffff0000u),
                            __uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xffff0000u));
         reinterpret_cast<float4*>(h32 + row * d)[c] = v[q];
       } else {
-        v[q] = reinterpret_cast<const float4*>(static_cast<const float*>(in) + row * d)[c];
+        v[q] = reinterpret_cast<const float4*>(static_cast<const float*>(in) + in_row * d)[c];
       }
       ss += v[q].x * v[q].x + v[q].y * v[q].y + v[q].z * v[q].z + v[q].w * v[q].w;
     }
@@ -100,33 +102,14 @@ __global__ void __launch_bounds__(NORM_THREADS, VPT <= 4 ? 8 : 4) rmsnorm_kernel
   pdl_wait();
   const int n_rows = rows_dev ? max(0, min(max_rows, *rows_dev)) : max_rows;
   for (size_t row = blockIdx.x; row < (size_t)n_rows; row += gridDim.x)
-    rmsnorm_row<IN_BF16, OUT_F16, VPT>(in, h32, gain, out, d, eps, row, red);
+    rmsnorm_row<IN_BF16, OUT_F16, VPT>(in, h32, gain, out, d, eps, row, (long long)row, red);
 }
 
-// cos/sin of pos * theta^(-2j/hd), evaluated in double and rounded once to fp32.
-__global__ void rope_table_kernel(float2* __restrict__ tab, int max_len, int half, float theta) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= max_len * half) return;
-  const int p = i / half, j = i % half;
-  const double inv = pow((double)theta, -2.0 * j / (2.0 * half));
-  double s, c;
-  sincos((double)p * inv, &s, &c);
-  tab[i] = make_float2((float)c, (float)s);
-}
-
-// Rows T .. T + n_tail - 1 (clamped to the cap rows of the buffer) of an fp16 [cap, cols] buffer
-// set to zero, T = *T_dev.  The attention's last query tile and key block may reach up to 127
-// rows past the last packed row, and a masked key still meets its value row in the P V product,
-// where 0 x NaN = NaN: so the rows past T that the tensor maps can reach must hold finite values
-// (with the row count equal to the capacity they are out of bounds and read as zero instead).
-__global__ void zero_tail_kernel(uint16_t* __restrict__ buf, int cols, const int* __restrict__ T_dev, int cap,
-                                 int n_tail) {
-  const int T = max(0, min(cap, *T_dev));
-  const int rows = min(n_tail, cap - T);
-  const int nv = cols / 8;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < (size_t)rows * nv;
-       e += (size_t)gridDim.x * blockDim.x)
-    reinterpret_cast<uint4*>(buf + (size_t)(T + e / nv) * cols)[e % nv] = make_uint4(0, 0, 0, 0);
+static RopeFreq rope_freq(const rift_model& m) {
+  RopeFreq f;
+  const int half = m.head_dim / 2;
+  for (int j = 0; j < 64; ++j) f.inv[j] = j < half ? std::pow((double)m.rope_theta, -2.0 * j / m.head_dim) : 0.0;
+  return f;
 }
 
 // out[i] = h32[cu[i + 1] - 1]: the residual stream of each sequence's last row (zeros for an
@@ -134,6 +117,8 @@ __global__ void zero_tail_kernel(uint16_t* __restrict__ buf, int cols, const int
 // below the device count n_seq_dev (all gridDim.x of them without one).
 __global__ void last_rows_kernel(const float* __restrict__ h32, const int* __restrict__ cu,
                                  const int* __restrict__ n_seq_dev, int row_cap, int d, float* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x;
   if (n_seq_dev && i >= *n_seq_dev) return;
   const bool empty = cu[i + 1] <= cu[i] || cu[i + 1] > row_cap;
@@ -241,13 +226,14 @@ int launch_prefill(const rift_model& m, void* hidden, int T, const int* T_dev, c
   int4* sched = reinterpret_cast<int4*>(ws + L.sched_off);
   const int d = m.d, half = m.head_dim / 2;
 
+  // The kernels after the first are launched as programmatic dependents of the kernel before them: with
+  // few rows their launch latencies are a good part of the time (two layers over one 131-row tile
+  // 373 -> 316 us with the setup in one launch; no difference at 23,800 rows).
+  const bool pdl = true;
   prof_begin(RIFT_PROF_ROPE, st);
-  rope_table_kernel<<<(max_len * half + 255) / 256, 256, 0, st>>>(rope, max_len, half, m.rope_theta);
+  PrefillSetup ps = {rope, max_len, half, rope_freq(m), qkv, 3 * d, T_dev};
+  launch_attention_schedule(cu_seqlens, n_seq, n_seq_dev, T, sched, L.max_qblocks, st, &ps);
   prof_end(RIFT_PROF_ROPE, st, 1);
-  prof_begin(RIFT_PROF_ATTN, st);
-  launch_attention_schedule(cu_seqlens, n_seq, n_seq_dev, T, sched, L.max_qblocks, st);
-  if (T_dev) zero_tail_kernel<<<64, 256, 0, st>>>(qkv, 3 * d, T_dev, T, 128);
-  prof_end(RIFT_PROF_ATTN, st, T_dev ? 2 : 1);
   // every product covers the rows the device count holds (T rows of capacity)
   EpiParams rows_ep;
   rows_ep.m_dev = T_dev;
@@ -260,34 +246,36 @@ int launch_prefill(const rift_model& m, void* hidden, int T, const int* T_dev, c
   rope_ep.pos_offset = S_pre;
   for (int l = 0; l < m.n_layers; ++l) {
     if (l == 0)
-      norm_launch(0, T, hidden, h32, m.g_attn[0], xn, d, m.eps, st, T_dev);
+      norm_launch(0, T, hidden, h32, m.g_attn[0], xn, d, m.eps, st, T_dev, pdl);
     else
-      norm_launch(1, T, h32, nullptr, m.g_attn[l], xn, d, m.eps, st, T_dev);
+      norm_launch(1, T, h32, nullptr, m.g_attn[l], xn, d, m.eps, st, T_dev, pdl);
     if (kv_out) {
       rope_ep.k_out = static_cast<uint16_t*>(kv_out) + (size_t)l * 2 * T * d;
       rope_ep.v_out = rope_ep.k_out + (size_t)T * d;
     }
-    if (launch_gemm(xn, m.w_qkv[l], T, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep)) return 1;
+    if (launch_gemm(xn, m.w_qkv[l], T, 3 * d, d, EPI_QKV_ROPE, qkv, st, rope_ep, pdl)) return 1;
     prof_begin(RIFT_PROF_ATTN, st);
     const uint16_t* pk = prefix_kv ? static_cast<const uint16_t*>(prefix_kv) + (size_t)l * 2 * S_pre * d : nullptr;
     if (launch_attention(qkv, T, cu_seqlens, n_seq, m.n_heads, m.head_dim, sched, L.max_qblocks, att, st, pk,
-                         pk ? pk + (size_t)S_pre * d : nullptr, prefix_kv ? S_pre : 0))
+                         pk ? pk + (size_t)S_pre * d : nullptr, prefix_kv ? S_pre : 0, pdl))
       return 1;
     prof_end(RIFT_PROF_ATTN, st, 1);
-    if (launch_gemm(att, m.w_o[l], T, d, d, EPI_RESID_F32, h32, st, rows_ep)) return 1;
-    norm_launch(1, T, h32, nullptr, m.g_ffn[l], xn, d, m.eps, st, T_dev);
-    if (launch_gemm(xn, m.w_gate_up[l], T, 2 * m.ffn, d, EPI_SWIGLU, act, st, rows_ep)) return 1;
-    if (launch_gemm(act, m.w_down[l], T, d, m.ffn, EPI_RESID_F32, h32, st, rows_ep)) return 1;
+    if (launch_gemm(att, m.w_o[l], T, d, d, EPI_RESID_F32, h32, st, rows_ep, pdl)) return 1;
+    norm_launch(1, T, h32, nullptr, m.g_ffn[l], xn, d, m.eps, st, T_dev, pdl);
+    if (launch_gemm(xn, m.w_gate_up[l], T, 2 * m.ffn, d, EPI_SWIGLU, act, st, rows_ep, pdl)) return 1;
+    if (launch_gemm(act, m.w_down[l], T, d, m.ffn, EPI_RESID_F32, h32, st, rows_ep, pdl)) return 1;
   }
-  norm_launch(2, T, h32, nullptr, m.g_final, static_cast<uint16_t*>(hidden), d, m.eps, st, T_dev);
+  norm_launch(2, T, h32, nullptr, m.g_final, static_cast<uint16_t*>(hidden), d, m.eps, st, T_dev, pdl);
   if (last_logits) {
     float* last32 = reinterpret_cast<float*>(ws + L.last32_off);
     uint16_t* last16 = reinterpret_cast<uint16_t*>(ws + L.last16_off);
-    last_rows_kernel<<<n_seq, 256, 0, st>>>(h32, cu_seqlens, n_seq_dev, T, d, last32);
-    norm_launch(1, n_seq, last32, nullptr, m.g_final, last16, d, m.eps, st, n_seq_dev);
+    if (launch_ex(last_rows_kernel, dim3(n_seq), dim3(256), 0, st, pdl, (const float*)h32, cu_seqlens, n_seq_dev, T, d,
+                  last32) != cudaSuccess)
+      return 1;
+    norm_launch(1, n_seq, last32, nullptr, m.g_final, last16, d, m.eps, st, n_seq_dev, pdl);
     EpiParams seq_ep;
     seq_ep.m_dev = n_seq_dev;
-    if (launch_gemm(last16, m.lm_head, n_seq, m.vocab, d, EPI_STORE_F32, last_logits, st, seq_ep)) return 1;
+    if (launch_gemm(last16, m.lm_head, n_seq, m.vocab, d, EPI_STORE_F32, last_logits, st, seq_ep, pdl)) return 1;
   }
   return 0;
 }
@@ -359,34 +347,43 @@ DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len) {
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
   const size_t n = (size_t)(n_seq > 0 ? n_seq : 1);
   L.h32_off = take(n * m.d * 4);
-  L.x0_off = take(n * m.d * 2);
   L.xn_off = take(n * m.d * 2);
   L.qkv_off = take(n * 3 * m.d * 2);
   L.attn_off = take(n * m.d * 2);
   L.act_off = take(n * m.ffn * 2);
-  L.rope_off = take((size_t)max_len * (m.head_dim / 2) * sizeof(float2));
+  L.rope_off = take(n * (m.head_dim / 2) * sizeof(float2));  // a row per sequence
   L.pos_off = take(n * sizeof(int));
   L.total = off;
   return L;
 }
 
-// x0[i] = embed[ids[i]] (bf16) and pos[i] = L_i = cu[i + 1] - cu[i], the new token's position.
-// An id outside [0, vocab) sets RIFT_EBIT_BADID and gives a zero row.
-__global__ void decode_embed_kernel(const int* __restrict__ ids, const int* __restrict__ cu,
-                                    const uint16_t* __restrict__ embed, int vocab, int d,
-                                    uint16_t* __restrict__ x0, int* __restrict__ pos) {
+// The start of a decode step, one CTA per sequence i: h32[i] = embed[ids[i]], xn[i] = RMSNorm(h32[i]) gain
+// (fp16), row i of the RoPE table = (cos, sin) at the new token's position L_i = cu[i + 1] - cu[i], and
+// pos[i] = i, its row of the table (-1 if L_i is not below max_len: the QKV epilogue reports it).  An
+// id outside [0, vocab) sets RIFT_EBIT_BADID and gives a zero row.
+template <int VPT>
+__global__ void __launch_bounds__(NORM_THREADS) decode_start_kernel(const int* __restrict__ ids,
+                                                                   const int* __restrict__ cu,
+                                                                   const uint16_t* __restrict__ embed, int vocab, int d,
+                                                                   int max_len, int half,
+                                                                   const __grid_constant__ RopeFreq freq,
+                                                                   const uint16_t* __restrict__ gain, float eps,
+                                                                   float* __restrict__ h32, uint16_t* __restrict__ xn,
+                                                                   float2* __restrict__ rope, int* __restrict__ pos) {
+  __shared__ float red[32];
+  pdl_trigger();
   const int i = blockIdx.x;
   const int id = ids[i];
   const bool ok = id >= 0 && id < vocab;
+  const int L = cu[i + 1] - cu[i];
   if (threadIdx.x == 0) {
-    pos[i] = cu[i + 1] - cu[i];
+    pos[i] = L >= 0 && L < max_len ? i : -1;
     if (!ok) atomicOr(&g_err_prefill, RIFT_EBIT_BADID);
   }
-  uint4* dst = reinterpret_cast<uint4*>(x0 + (size_t)i * d);
-  const uint4* src = reinterpret_cast<const uint4*>(embed + (size_t)(ok ? id : 0) * d);
-  for (int c = threadIdx.x; c < d / 8; c += blockDim.x) dst[c] = ok ? src[c] : make_uint4(0, 0, 0, 0);
+  if ((int)threadIdx.x < half)
+    rope[(size_t)i * half + threadIdx.x] = rope_cos_sin((double)max(L, 0) * freq.inv[threadIdx.x]);
+  rmsnorm_row<true, true, VPT>(embed, h32, gain, xn, d, eps, (size_t)i, ok ? (long long)id : -1, red);
 }
-
 
 int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* cu_seqlens, int n_seq, int max_len,
                   const int* token_ids, const void* embed, int vocab_embed, void* hidden_out, void* kv_new,
@@ -394,7 +391,6 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   if (n_seq == 0) return 0;
   const DecodeLayout L = decode_layout(m, n_seq, max_len);
   float* h32 = reinterpret_cast<float*>(ws + L.h32_off);
-  uint16_t* x0 = reinterpret_cast<uint16_t*>(ws + L.x0_off);
   uint16_t* xn = reinterpret_cast<uint16_t*>(ws + L.xn_off);
   uint16_t* qkv = reinterpret_cast<uint16_t*>(ws + L.qkv_off);
   uint16_t* att = reinterpret_cast<uint16_t*>(ws + L.attn_off);
@@ -403,17 +399,25 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
   int* pos = reinterpret_cast<int*>(ws + L.pos_off);
   const int d = m.d, half = m.head_dim / 2, n = n_seq;
 
-  rope_table_kernel<<<(max_len * half + 255) / 256, 256, 0, st>>>(rope, max_len, half, m.rope_theta);
-  decode_embed_kernel<<<n, 128, 0, st>>>(token_ids, cu_seqlens, static_cast<const uint16_t*>(embed), vocab_embed, d,
-                                         x0, pos);
+  prof_begin(RIFT_PROF_NORM, st);
+  auto start = [&](auto kern) {
+    kern<<<n, NORM_THREADS, 0, st>>>(token_ids, cu_seqlens, static_cast<const uint16_t*>(embed), vocab_embed, d, max_len,
+                                     half, rope_freq(m), static_cast<const uint16_t*>(m.g_attn[0]), m.eps, h32, xn, rope,
+                                     pos);
+  };
+  const int per_thread = (d / 4 + NORM_THREADS - 1) / NORM_THREADS;  // d <= 8192: at most 8
+  if (per_thread <= 1) start(decode_start_kernel<1>);
+  else if (per_thread <= 2) start(decode_start_kernel<2>);
+  else if (per_thread <= 4) start(decode_start_kernel<4>);
+  else start(decode_start_kernel<8>);
+  prof_end(RIFT_PROF_NORM, st, 1);
   EpiParams rope_ep;
   rope_ep.positions = pos;
   rope_ep.rope = rope;
   rope_ep.rope_cols = 2 * d;
   rope_ep.head_dim = m.head_dim;
-  rope_ep.max_len = max_len;
+  rope_ep.max_len = n;  // the rows of the table
   const uint16_t* kv = static_cast<const uint16_t*>(kv_cache);
-  norm_launch(0, n, x0, h32, m.g_attn[0], xn, d, m.eps, st);
   // The layer's kernels are launched as programmatic dependents of the kernel before them: each
   // starts while its predecessor drains (the GEMMs already requesting their first weight tiles)
   // and waits for it before touching activations.

@@ -87,6 +87,42 @@ static inline cudaError_t launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 bl
   return launch_cluster_ex(kernel, grid, block, smem, st, pdl, 1, args...);
 }
 
+// RoPE angular frequencies theta^(-2j / head_dim), j < head_dim / 2 <= 64, evaluated on the host in
+// double.
+struct RopeFreq {
+  double inv[64];
+};
+
+// (cos, sin) of x >= 0 (up to ~1e5), each rounded once to fp32 from a double good to ~1e-12: x reduced
+// by the nearest multiple k of pi/2 (Cody and Waite's two-part reduction, its constants the leading
+// bits of pi/2 and the rest), then the Taylor polynomials on |r| <= pi/4 (the first terms left out,
+// r^15 / 15! and r^14 / 14!, are below 4e-13).  A GB300 SM retires about two double operations a cycle,
+// so they are what a RoPE table costs: this takes about 20 a value, the library's pow and sincos
+// per value about 160 (a 131 x 64 table 11.6 us; now 4.1 us together with the attention schedule, whose own
+// launch took 3.7; a decode step's start, which needs one row per sequence, 29.6 -> 7.5 us for one
+// sequence of 635 rows).
+__device__ __forceinline__ float2 rope_cos_sin(double x) {
+  const double two_over_pi = 0.63661977236758134308, pio2 = 1.57079632679489661923, pio2_rest = 6.123233995736766e-17;
+  const double k = rint(x * two_over_pi);
+  const double r = fma(-k, pio2_rest, fma(-k, pio2, x));
+  const double z = r * r;
+  double s = fma(z, 1.0 / 6227020800.0, -1.0 / 39916800.0);
+  s = fma(z, s, 1.0 / 362880.0);
+  s = fma(z, s, -1.0 / 5040.0);
+  s = fma(z, s, 1.0 / 120.0);
+  s = fma(z, s, -1.0 / 6.0);
+  s = fma(z * r, s, r);
+  double c = fma(z, 1.0 / 479001600.0, -1.0 / 3628800.0);
+  c = fma(z, c, 1.0 / 40320.0);
+  c = fma(z, c, -1.0 / 720.0);
+  c = fma(z, c, 1.0 / 24.0);
+  c = fma(z, c, -0.5);
+  c = fma(z, c, 1.0);
+  const float cf = (float)c, sf = (float)s;
+  const int q = (int)k & 3;  // x = r + q pi/2 (mod 2 pi)
+  return make_float2(q == 0 ? cf : q == 1 ? -sf : q == 2 ? -cf : sf, q == 0 ? sf : q == 1 ? cf : q == 2 ? -sf : -cf);
+}
+
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -119,7 +119,7 @@ int launch_prefill_shared_prefix(const rift_model& m, const int* sys_ids, int S,
                                  const int* cu_seqlens, int n_seq, const int* n_seq_dev, int max_len,
                                  const int* positions, float* last_logits, char* ws, cudaStream_t st);
 struct DecodeLayout {
-  size_t h32_off, x0_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, total;
+  size_t h32_off, xn_off, qkv_off, attn_off, act_off, rope_off, pos_off, total;
 };
 DecodeLayout decode_layout(const rift_model& m, int n_seq, int max_len);
 int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* cu_seqlens, int n_seq, int max_len,
@@ -180,13 +180,24 @@ int launch_merge_screen(const uint16_t* X, int N, int n_v, int d, const int* kep
 int attention_max_qblocks(int max_T, int max_seqs);
 // The schedule holds n_sched_max + 1 entries (the last: the count in use).  n_seq_dev (nullable):
 // a device sequence count clamped to n_seq; sequences ending past row_cap rows are dropped.
+// setup (nullable): what else a prefill needs before its first layer, done by the same launch: the
+// RoPE table, and rows T .. T + 127 (T = *T_dev, clamped to the row_cap rows of the buffer) of an
+// fp16 [row_cap, tail_cols] buffer set to zero.
+struct PrefillSetup {
+  float2* rope;
+  int max_len, half;
+  RopeFreq freq;
+  uint16_t* tail;
+  int tail_cols;
+  const int* T_dev;  // nullable: no tail to zero
+};
 void launch_attention_schedule(const int* cu_seqlens, int n_seq, const int* n_seq_dev, int row_cap, int4* sched,
-                               int n_sched_max, cudaStream_t st);
+                               int n_sched_max, cudaStream_t st, const PrefillSetup* setup = nullptr);
 // prefix_k, prefix_v (optional): fp16 [S_pre, d] keys (after RoPE) and values of a prefix that every
 // sequence attends to before its own rows.
 int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, int n_heads, int head_dim,
                      const int4* sched, int n_sched_max, void* out, cudaStream_t st, const void* prefix_k = nullptr,
-                     const void* prefix_v = nullptr, int S_pre = 0);
+                     const void* prefix_v = nullptr, int S_pre = 0, bool pdl = false);
 // Decode attention: each of n sequences' new token (qkv fp16 [n, 3 d]) over its cached rows (K, V fp16
 // [T, d], one layer) and itself; a sequence with more than max_keys keys sets RIFT_EBIT_CAPACITY.
 int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16_t* V, int T, const int* cu, int n,

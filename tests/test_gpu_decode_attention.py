@@ -1,7 +1,7 @@
 """The decode step's attention (keys streamed in 32-row tiles through a TMA ring, split over a
 cluster when there are few sequences) through rift_decode_step: cached lengths around the tile and
 the cluster's shares, one and many sequences, both head sizes and a head count that leaves part of
-the last 256-column group empty; against the oracle at the hidden-state tolerance."""
+the last 256-column group empty, long sequences (RoPE at large positions); against the oracle at the hidden-state tolerance."""
 import pytest
 import torch
 
@@ -16,6 +16,7 @@ HD128 = W.DecoderShape(n_layers=1, d=640, n_heads=5, head_dim=128, ffn=688, voca
 HD64 = W.DecoderShape(n_layers=1, d=320, n_heads=5, head_dim=64, ffn=688, vocab=504)      # 1.25 column groups
 
 LENGTHS = {"one": [600], "one_short": [1], "edges": [0, 1, 31, 32, 33, 95, 96, 97, 128, 257],
+           "long": [30000, 7],  # RoPE angles up to 30000 rad
            "many": [(7 * i) % 70 for i in range(160)]}  # 480 units of 2-3 column groups: no cluster
 
 
