@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(da::THREADS, 2)
     }
     for (int t = 0; t < tiles; ++t) {
       const int s = t % NST;
-      if (!mbar_wait(FULL(s), (t / NST) & 1u, abort_flag)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(FULL(s), (t / NST) & 1u, abort_flag))) break;
       const uint8_t* kt = ring + s * 2 * da::TILE + hh * HD * 2 + dl * 2;
       const int last = k1 - 1 - (k0 + t * SK);  // last valid row of the tile
       float sc[NL];

@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
     // ---------------- the partial product to shared memory: P[row m][weight row], over the ring
     // (every copy has been consumed by a completed MMA)
     const int quarter = warp & 3;
-    if (mbar_wait(done_bar, 0, abort_flag)) {
+    if (__all_sync(0xffffffffu, mbar_wait(done_bar, 0, abort_flag))) {
       fence_after();
       float* P = reinterpret_cast<float*>(smem) + quarter * 32 + lane;
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -808,39 +808,55 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
 }
 
 // ---------------------------------------------------------------- merge screening (Stage 2)
-// Similarity of every token of a kept tile to the tile's merge targets on the tensor cores: per
-// (kept slot j, 128-token block) a 128 x 128 x d bf16 product against 128 target rows at a time,
-// one token row per epilogue thread, which keeps the two best targets by x.t / ||t|| (fp32, ties
-// to the lower target) for each unselected token that is not itself a target.  The choice
-// between the two is then made at ~fp64 accuracy outside (merge.cu).  Rows of the block past the
-// tile's tokens and target columns past the slot's m are computed and ignored.
+// Similarity of the unselected tokens of a kept tile to the tile's merge targets on the tensor cores:
+// per (kept slot j, 128 of its unselected tokens) a 128 x m x d bf16 product against up to COLS target
+// rows at a time, one token row per epilogue thread, which keeps the two best targets by
+// x.t / ||t|| (fp32, ties to the lower target) for each token that is not itself a target.  Bound by
+// HBM (the unselected tokens, read once): the four epilogue warps gather the token rows with
+// cp.async into the swizzled tiles, so the selected tokens are neither read nor multiplied (three
+// blocks a slot instead of five at 333 of 576 tokens), 48 KB a CTA in flight; TMA's gather4 form
+// took 11 cycles per 128-byte row: 65 us at 400 tiles (about 95 kept), 102 with gather4, 87 reading
+// every token.  Where the two targets are
+// closer than the product's error bound, the choice between them is made at ~fp64 accuracy outside
+// (merge.cu); the bound scales with ||x||, which the gathering threads sum from their own chunks.
+// Bound: an accumulator update adds 16 exact products, each addend cut below 2^-24 of the largest
+// (16 x 2^-24 = 2^-20 of a magnitude of at most ||x|| ||t||), so d / 16 updates err by at most d 2^-24 ||x||
+// in x.t / ||t||, and the difference of two by d 2^-23 ||x|| (about 9% of the tokens of a random tile
+// are closer, all others need no second look).
 namespace ms {
-constexpr int STAGES = 3, THREADS = 192, COLS = 128;
+constexpr int STAGES = 4, THREADS = 192, COLS = 80, TMEM_COLS = 128;
+constexpr int BROWS = 16;  // target rows per TMA box: a product is as wide as its targets need
 constexpr int A_BYTES = 128 * BK * 2, B_BYTES = COLS * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
-// kind::f16 with bf16 A and B (bits 7-9 and 10-12 = 1), fp32 D, K-major, M = N = 128
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(COLS >> 3) << 17) | ((128u >> 4) << 24);
+// kind::f16 with bf16 A and B (bits 7-9 and 10-12 = 1), fp32 D, K-major, M = 128; N >> 3 added at bit 17
+constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
 }  // namespace ms
 
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+
 __global__ void __launch_bounds__(ms::THREADS, 2)
-    merge_screen_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT, int n_v,
-                        int d, const int* __restrict__ kept, const int* __restrict__ n_kept,
+    merge_screen_kernel(const __grid_constant__ CUtensorMap tmT, const uint16_t* __restrict__ X, int n_v, int d,
+                        const int* __restrict__ kept, const int* __restrict__ n_kept,
                         const int* __restrict__ sel_off, const int* __restrict__ ctx_off, int max_ctx,
-                        const float* __restrict__ tinv, const int* __restrict__ pos, int2* __restrict__ cand) {
-  constexpr int STAGES = ms::STAGES, COLS = ms::COLS, A_BYTES = ms::A_BYTES, B_BYTES = ms::B_BYTES,
-                STAGE_BYTES = ms::STAGE_BYTES;
-  constexpr uint32_t IDESC = ms::IDESC;
+                        const float* __restrict__ tinv, const int* __restrict__ rest, int2* __restrict__ cand) {
+  constexpr int STAGES = ms::STAGES, COLS = ms::COLS, A_BYTES = ms::A_BYTES, B_BYTES = ms::B_BYTES;
+  pdl_trigger();
+  pdl_wait();
   const int j = blockIdx.y, mb = blockIdx.x;
   if (j >= *n_kept) return;
   const int co = ctx_off[j], m = ctx_off[j + 1] - co;
-  if (m == 0 || co + m > max_ctx) return;  // uniform over the CTA, before any setup
+  if (m == 0 || co + m > max_ctx) return;  // uniform over the CTA, before any setup (as the next)
   const int R = n_v - (sel_off[j + 1] - sel_off[j]);
+  if (mb * 128 >= R) return;
   const int step = R / m;
   extern __shared__ uint8_t smem_raw[];
+  __shared__ float nrm_s[128];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + STAGES * A_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + STAGES * ms::STAGE_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t bar0 = smem_u32(bars);
@@ -850,7 +866,7 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s2 = 0; s2 < STAGES; ++s2) {
-      mbar_init(full_bar(s2), 1);
+      mbar_init(full_bar(s2), 129);  // the gathering threads and the TMA thread
       mbar_init(empty_bar(s2), 1);
     }
     mbar_init(tfull, 1);
@@ -861,7 +877,7 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                 "r"(COLS)
+                 "r"(ms::TMEM_COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
@@ -869,22 +885,24 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
   __syncthreads();
   fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const int kt = d / BK, nblk = (m + COLS - 1) / COLS;
-  const int xrow = kept[j] * n_v + mb * 128;
+  const int kt = d / BK, nblk = (m + COLS - 1) / COLS, n_it = nblk * kt;
+  auto width = [&](int nb) { return min(COLS, (m - nb * COLS + ms::BROWS - 1) / ms::BROWS * ms::BROWS); };
 
   if (warp == 0) {
     if (lane == 0) {
+      // ---------------- TMA: the target rows
       int it = 0;
       bool ok = true;
-      for (int nb = 0; nb < nblk && ok; ++nb)
+      for (int nb = 0; nb < nblk && ok; ++nb) {
+        const int w = width(nb);
         for (int k = 0; k < kt; ++k, ++it) {
           const int s2 = it % STAGES;
-          const uint32_t round = it / STAGES;
-          if (!mbar_wait(empty_bar(s2), (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          mbar_expect_tx(full_bar(s2), STAGE_BYTES);
-          tma_load_2d(smem_u32(sA + s2 * A_BYTES), &tmX, k * BK, xrow, full_bar(s2));
-          tma_load_2d(smem_u32(sB + s2 * B_BYTES), &tmT, k * BK, co + nb * COLS, full_bar(s2));
+          if (!mbar_wait(empty_bar(s2), ((it / STAGES) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          mbar_expect_tx(full_bar(s2), w * BK * 2);
+          for (int b = 0; b < w; b += ms::BROWS)
+            tma_load_2d(smem_u32(sB + s2 * B_BYTES + b * BK * 2), &tmT, k * BK, co + nb * COLS + b, full_bar(s2));
         }
+      }
       for (int q = 1; q <= STAGES && it - q >= 0; ++q) {  // no copy left in flight (bounded)
         const int i2 = it - q;
         for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(full_bar(i2 % STAGES), (i2 / STAGES) & 1u); ++w) {
@@ -893,11 +911,13 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
     }
   } else if (warp == 1) {
     if (lane == 0) {
+      // ---------------- MMA issuer
       int it = 0;
       bool ok = true;
       for (int nb = 0; nb < nblk && ok; ++nb) {
         if (!mbar_wait(tempty, (nb & 1) ^ 1, abort_flag)) break;
         fence_after();
+        const uint32_t idesc = ms::IDESC | ((uint32_t)(width(nb) >> 3) << 17);
         for (int k = 0; k < kt; ++k, ++it) {
           const int s2 = it % STAGES;
           if (!mbar_wait(full_bar(s2), (it / STAGES) & 1u, abort_flag)) { ok = false; break; }
@@ -906,36 +926,97 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
           const uint64_t bd = smem_desc(smem_u32(sB + s2 * B_BYTES));
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            umma_f16(tmem_base, ad + 2 * kk, bd + 2 * kk, IDESC, (k != 0 || kk != 0) ? 1u : 0u);
+            umma_f16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc, (k != 0 || kk != 0) ? 1u : 0u);
           umma_commit(empty_bar(s2));
         }
         if (ok) umma_commit(tfull);
       }
     }
   } else {
-    // epilogue: warps 2..5 -> TMEM lane quarters 2, 3, 0, 1; thread = token row
+    // ---------------- gather and epilogue (warps 2..5)
+    // Gather: thread g takes 16-byte chunk g % 8 of rows g / 8 + 16 i (past the last unselected token: that
+    // token again), at the chunk's place in the 128-byte swizzle.
+    const int g = threadIdx.x - 64, c = g & 7;
+    const uint16_t* src[8];
+    uint32_t off[8];
+    float ss[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = (g >> 3) + 16 * i;
+      const int tok = rest[(size_t)j * n_v + min(mb * 128 + row, R - 1)];
+      src[i] = X + ((size_t)kept[j] * n_v + tok) * d + c * 8;
+      off[i] = (uint32_t)(row * 128 + ((c ^ (row & 7)) << 4));
+      ss[i] = 0.f;
+    }
+    // Epilogue: TMEM lane quarters 2, 3, 0, 1; thread = token row
     const int quarter = warp & 3, r = quarter * 32 + lane;
-    const int tok = mb * 128 + r;
-    const int a = tok < n_v ? pos[(size_t)j * n_v + tok] : -1;
-    const bool want = a >= 0 && !(a % step == 0 && a / step < m);
+    const int a = mb * 128 + r;
+    const bool want = a < R && !(a % step == 0 && a / step < m);
     float v1 = -INFINITY, v2 = -INFINITY;
     int b1 = -1, b2 = -1;
+    constexpr int LAG = STAGES - 1;  // tiles in flight behind the one being requested
     bool ok = true;
-    for (int nb = 0; nb < nblk; ++nb) {
+    // tile `it` has landed in this thread's chunks: norms (first pass over the tokens), then hand it over
+    auto finish = [&](int it) {
+      const uint8_t* tile = sA + (it % STAGES) * A_BYTES;
+      if (it < kt) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float x[8];
+          unpack_bf16x8(*reinterpret_cast<const uint4*>(tile + off[i]), x);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) ss[i] = fmaf(x[e], x[e], ss[i]);
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      mbar_arrive(full_bar(it % STAGES));
+    };
+    for (int nb = 0; nb < nblk && ok; ++nb) {
+      // request tiles up to LAG ahead of the end of this pass; hand over those that have landed
+      const int it0 = nb == 0 ? 0 : nb * kt + LAG, it1 = min(n_it, (nb + 1) * kt + LAG);
+      for (int it = it0; it < it1 || it - LAG < (nb + 1) * kt; ++it) {
+        if (it < n_it) {
+          if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(it % STAGES), ((it / STAGES) & 1u) ^ 1u, abort_flag))) {
+            ok = false;
+            break;
+          }
+          const uint32_t dst = smem_u32(sA + (it % STAGES) * A_BYTES);
+          const int k = (it % kt) * BK;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) cp_async16(dst + off[i], src[i] + k);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        if (it >= LAG) {
+          asm volatile("cp.async.wait_group %0;\n" ::"n"(LAG) : "memory");
+          finish(it - LAG);
+        }
+      }
+      if (!ok) break;
+      if (nb == 0) {  // row norms: the eight threads of a row hold its chunks' sums
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float v = ss[i];
+          v += __shfl_xor_sync(0xffffffffu, v, 1);
+          v += __shfl_xor_sync(0xffffffffu, v, 2);
+          v += __shfl_xor_sync(0xffffffffu, v, 4);
+          if (c == 0) nrm_s[(g >> 3) + 16 * i] = v;
+        }
+        asm volatile("bar.sync 1, 128;\n" ::: "memory");
+      }
       const int c0 = nb * COLS, nc = min(COLS, m - c0);
       const float* inv_n = tinv + co + c0;  // 1 / ||t|| (0 for a zero target: similarity 0)
-      if (!mbar_wait(tfull, nb & 1, abort_flag)) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull, nb & 1, abort_flag))) { ok = false; break; }
       fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-      for (int c = 0; c < nc; c += 32) {
-        uint32_t acc[32];
-        tmem_ld32(taddr + c, acc);
+      for (int cc = 0; cc < nc; cc += 16) {
+        uint32_t acc[16];
+        tmem_ld16(taddr + cc, acc);
         if (want) {
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            if (c + e < nc) {
-              const float v = __uint_as_float(acc[e]) * inv_n[c + e];
-              const int b = c0 + c + e;
+          for (int e = 0; e < 16; ++e) {
+            if (cc + e < nc) {
+              const float v = __uint_as_float(acc[e]) * inv_n[cc + e];
+              const int b = c0 + cc + e;
               if (v > v1) {
                 v2 = v1;
                 b2 = b1;
@@ -952,13 +1033,17 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
       fence_before();
       mbar_arrive(tempty);
     }
-    if (ok && want) cand[(size_t)j * n_v + a] = make_int2(b1, b2);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    if (ok && want) {
+      const bool clear = v1 - v2 > (float)d * 0x1p-23f * sqrtf(nrm_s[r]);  // false with a NaN or an infinite norm
+      cand[(size_t)j * n_v + a] = make_int2(b1, clear ? -1 : b2);
+    }
   }
   fence_before();
   __syncthreads();
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(ms::TMEM_COLS) : "memory");
   }
 }
 
@@ -1106,17 +1191,14 @@ __global__ void wait_timeout_check_kernel() {
 
 int launch_merge_screen(const uint16_t* X, int N, int n_v, int d, const int* kept, const int* n_kept,
                         const int* sel_off, const int* ctx_off, int max_ctx, const uint16_t* targets,
-                        const float* tinv, const int* pos, int2* cand, cudaStream_t st) {
+                        const float* tinv, const int* rest, int2* cand, cudaStream_t st) {
   using namespace tc;
-  CUtensorMap mx, mt;
-  if (!make_map(&mx, X, (uint64_t)d, (uint64_t)N * n_v, 128, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16) ||
-      !make_map(&mt, targets, (uint64_t)d, (uint64_t)max_ctx, ms::COLS, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16))
-    return 1;
+  CUtensorMap mt;
+  if (!make_map(&mt, targets, (uint64_t)d, (uint64_t)max_ctx, ms::BROWS, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)) return 1;
   static std::atomic<unsigned long long> smem_raised{0};
   if (raise_smem_limit(smem_raised, merge_screen_kernel, (int)ms::SMEM) != cudaSuccess) return 1;
-  merge_screen_kernel<<<dim3((n_v + 127) / 128, N), ms::THREADS, ms::SMEM, st>>>(
-      mx, mt, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, tinv, pos, cand);
-  return 0;
+  return launch_ex(merge_screen_kernel, dim3((n_v + 127) / 128, N), dim3(ms::THREADS), ms::SMEM, st, true, mt, X, n_v, d,
+                   kept, n_kept, sel_off, ctx_off, max_ctx, tinv, rest, cand) != cudaSuccess;
 }
 
 int launch_wait_timeout_check(cudaStream_t st) {

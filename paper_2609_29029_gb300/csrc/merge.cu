@@ -12,10 +12,12 @@
 //                         arithmetic (ties to the lower target)
 //   (bf16 tokens) merge_screen_kernel (gemm_tc.cu) takes the top 2 from a tcgen05 product of
 //                         each 128-token block with the slot's target rows, and
-//                         merge_decide_kernel makes the same float-float decision between them
-//   merge_groups_kernel   the groups as member lists in ascending token index (counting sort)
-//   merge_mean_kernel     per contextual token: the fp32 sum of its members' rows in that order,
-//                         divided by the group size, stored as bf16
+//                         merge_decide_kernel makes the same float-float decision between the two
+//                         where they are closer than the product's error bound
+//   merge_mean_kernel     per contextual token: its members in ascending token index, the fp32 sum
+//                         of their rows in that order, divided by the group size, stored as bf16
+#include <type_traits>
+
 #include "rift_internal.h"
 
 namespace rift {
@@ -53,63 +55,52 @@ __device__ __forceinline__ void load8(const XT* p, float (&v)[8]) {
   }
 }
 
-// Float-float accumulation of a.b over d terms (d % 256 == 0) by one warp (TwoProduct with an
-// FMA, TwoSum), eight elements per lane and step, then the lanes' pairs summed in fp64.
+// a.b += into the float-float pair (hi, lo): TwoProduct with an FMA, then TwoSum.
+__device__ __forceinline__ void ff_step(float x, float y, float& hi, float& lo) {
+  const float p = __fmul_rn(x, y);
+  const float pe = fmaf(x, y, -p);
+  const float s = __fadd_rn(hi, p);
+  const float bb = __fsub_rn(s, hi);
+  const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+  hi = s;
+  lo = __fadd_rn(lo, __fadd_rn(er, pe));
+}
+
+// The sum of the lanes' float-float pairs (TwoSum of the high parts), in every lane.
+__device__ __forceinline__ void ff_warp_sum(float& hi, float& lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+    const float s = __fadd_rn(hi, h2);
+    const float bb = __fsub_rn(s, hi);
+    const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
+    hi = s;
+    lo = __fadd_rn(__fadd_rn(lo, l2), er);
+  }
+}
+
+// Float-float accumulation of a.b over d terms by one warp, eight elements per lane and step, four
+// steps' loads ahead of the serial chain, then the lanes' pairs summed (~2^-44 relative).
 template <typename XT>
 __device__ double ff_dot(const XT* a, const XT* b, int d, int lane) {
   float hi = 0.f, lo = 0.f;
-  for (int k = lane * 8; k < d; k += 256) {
-    float x[8], y[8];
-    load8(a + k, x);
-    load8(b + k, y);
+  for (int k0 = lane * 8; k0 < d; k0 += 4 * 256) {
+    float x[4][8], y[4][8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float p = __fmul_rn(x[e], y[e]);
-      const float pe = fmaf(x[e], y[e], -p);
-      const float s = __fadd_rn(hi, p);
-      const float bb = __fsub_rn(s, hi);
-      const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-      hi = s;
-      lo = __fadd_rn(lo, __fadd_rn(er, pe));
-    }
+    for (int u = 0; u < 4; ++u)
+      if (k0 + u * 256 < d) {
+        load8(a + k0 + u * 256, x[u]);
+        load8(b + k0 + u * 256, y[u]);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k0 + u * 256 < d) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ff_step(x[u][e], y[u][e], hi, lo);
+      }
   }
-  double acc = (double)hi + (double)lo;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return acc;
-}
-
-// a.b and a.c in one pass over a, each summed as ff_dot does.
-template <typename XT>
-__device__ double2 ff_dot2(const XT* a, const XT* b, const XT* c, int d, int lane) {
-  float hb = 0.f, lb = 0.f, hc = 0.f, lc = 0.f;
-  auto step = [](float x, float y, float& hi, float& lo) {
-    const float p = __fmul_rn(x, y);
-    const float pe = fmaf(x, y, -p);
-    const float s = __fadd_rn(hi, p);
-    const float bb = __fsub_rn(s, hi);
-    const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    hi = s;
-    lo = __fadd_rn(lo, __fadd_rn(er, pe));
-  };
-  for (int k = lane * 8; k < d; k += 256) {
-    float x[8], y[8], z[8];
-    load8(a + k, x);
-    load8(b + k, y);
-    load8(c + k, z);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      step(x[e], y[e], hb, lb);
-      step(x[e], z[e], hc, lc);
-    }
-  }
-  double sb = (double)hb + (double)lb, sc = (double)hc + (double)lc;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sb += __shfl_xor_sync(0xffffffffu, sb, o);
-    sc += __shfl_xor_sync(0xffffffffu, sc, o);
-  }
-  return make_double2(sb, sc);
+  ff_warp_sum(hi, lo);
+  return (double)hi + (double)lo;
 }
 
 // m_j = min(budgets[j] - s_j, n_v - s_j) and its exclusive prefix sum over the kept slots.  If
@@ -120,6 +111,8 @@ __global__ void __launch_bounds__(1024) merge_plan_kernel(const int* __restrict_
                                                           const int* __restrict__ sel_off, int N, int n_v,
                                                           int max_ctx, int* __restrict__ ctx_off) {
   __shared__ int sh[33];
+  pdl_trigger();
+  pdl_wait();
   const int n = *n_kept;
   auto count = [&](int j) {
     const int s = sel_off[j + 1] - sel_off[j];
@@ -146,8 +139,12 @@ __global__ void __launch_bounds__(1024) merge_plan_kernel(const int* __restrict_
   for (int j = n + threadIdx.x; j <= N; j += blockDim.x) ctx_off[j] = base;
 }
 
-// One CTA per kept slot: rest[j][0 .. R) = the unselected tokens in ascending index, the targets
-// (written to ctx_target) and their norms (tnorm, fp64 from a float-float sum of squares).
+// Grid (kept slot, y): rest[j][0 .. R) = the unselected tokens in ascending index (written by y = 0),
+// the targets (written to ctx_target) and their norms (tnorm, fp64 from a float-float sum of
+// squares), one target per warp: the warps of the TY CTAs take targets y * 8 + warp, + TY * 8, ...
+// The norm is a serial float-float chain, so the targets are spread over many warps (400 tiles, about 95
+// kept, 45 targets a slot: 19 us, 73 with one CTA per slot).
+constexpr int TY = 8;
 template <typename XT>
 __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict__ X, int n_v, int d,
                                                             const int* __restrict__ kept,
@@ -156,14 +153,18 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
                                                             const int* __restrict__ sel_off,
                                                             const int* __restrict__ ctx_off, int max_ctx,
                                                             int* __restrict__ rest, int* __restrict__ ctx_target,
-                                                            double* __restrict__ tnorm, int* __restrict__ pos,
-                                                            float* __restrict__ tinv, uint16_t* __restrict__ trow) {
+                                                            double* __restrict__ tnorm, float* __restrict__ tinv,
+                                                            uint16_t* __restrict__ trow) {
   __shared__ unsigned char chosen[RIFT_MAX_NV];
+  __shared__ int rj[RIFT_MAX_NV];
   __shared__ int sh[33];
-  const int j = blockIdx.x;
+  pdl_trigger();
+  pdl_wait();
+  const int j = blockIdx.x, y = blockIdx.y;
   if (j >= *n_kept) return;
   const int so = sel_off[j], s = sel_off[j + 1] - so;
   const int co = ctx_off[j], m = ctx_off[j + 1] - co;
+  if (y > 0 && y * 8 >= m) return;
   for (int k = threadIdx.x; k < n_v; k += blockDim.x) chosen[k] = 0;
   __syncthreads();
   for (int q = threadIdx.x; q < s; q += blockDim.x) {
@@ -171,15 +172,16 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
     if (k >= 0 && k < n_v) chosen[k] = 1;
   }
   __syncthreads();
-  int* rj = rest + (size_t)j * n_v;
   int base = 0;
   for (int c0 = 0; c0 < n_v; c0 += blockDim.x) {
     const int k = c0 + threadIdx.x;
     const int f = (k < n_v && !chosen[k]) ? 1 : 0;
     int total;
     const int at = block_excl_scan(f, sh, &total);
-    if (f) rj[base + at] = k;
-    if (pos && k < n_v) pos[(size_t)j * n_v + k] = f ? base + at : -1;
+    if (f) {
+      rj[base + at] = k;
+      if (y == 0) rest[(size_t)j * n_v + base + at] = k;
+    }
     base += total;
   }
   __syncthreads();
@@ -188,7 +190,7 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
   const int step = R / m;
   const XT* Xt = X + (size_t)kept[j] * n_v * d;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int q = warp; q < m; q += blockDim.x / 32) {
+  for (int q = y * 8 + warp; q < m; q += TY * 8) {
     const int t = rj[q * step];
     const double nn = ff_dot(Xt + (size_t)t * d, Xt + (size_t)t * d, d, lane);
     if (co + q >= max_ctx) continue;
@@ -205,11 +207,14 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
   }
 }
 
-// Grid (blocks of 8 unselected positions, kept slot), 8 warps: for the position a of each warp
-// (not a target), the better of its two screened candidates cand[j][a] at ~fp64 accuracy:
-// x.t1 / ||t1|| vs x.t2 / ||t2|| from float-float dot products (ties to the lower target).
-template <typename XT>
-__global__ void __launch_bounds__(256) merge_decide_kernel(const XT* __restrict__ X, int n_v, int d,
+// Grid (blocks of 64 unselected positions, kept slot), 4 warps: assign[j][a] = the screened target where
+// the screening was clear (cand[j][a].y < 0); the others are listed and the warps take them in turn: the
+// better of the two candidates at ~fp64 accuracy, x.t1 / ||t1|| vs x.t2 / ||t2|| from float-float dot
+// products (ties to the lower target).  The lanes' pairs are summed as pairs too: two double
+// operations retire a cycle on an SM, so a shuffle sum in fp64 costs more than the dot product.  28 us
+// at 400 tiles, against 111 with a second look at every token.
+// Targets keep their own group.
+__global__ void __launch_bounds__(128) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
                                                            const int* __restrict__ kept,
                                                            const int* __restrict__ n_kept,
                                                            const int* __restrict__ sel_off,
@@ -218,32 +223,70 @@ __global__ void __launch_bounds__(256) merge_decide_kernel(const XT* __restrict_
                                                            const int* __restrict__ ctx_target,
                                                            const double* __restrict__ tnorm,
                                                            const int2* __restrict__ cand, int* __restrict__ assign) {
-  const int j = blockIdx.y;
+  __shared__ int4 open[64];  // (position, candidate 1, candidate 2) of the block's undecided tokens
+  __shared__ int n_open;
+  pdl_trigger();
+  pdl_wait();
+  const int j = blockIdx.y, a0 = blockIdx.x * 64;
   if (j >= *n_kept) return;
   const int R = n_v - (sel_off[j + 1] - sel_off[j]);
   const int co = ctx_off[j], m = ctx_off[j + 1] - co;
-  if (m == 0 || co + m > max_ctx) return;
+  if (m == 0 || co + m > max_ctx || a0 >= R) return;
   const int step = R / m;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int a = blockIdx.x * 8 + warp;
-  if (a >= R || (a % step == 0 && a / step < m)) return;  // targets keep their own group
-  int2 c = cand[(size_t)j * n_v + a];
-  if (c.x < 0 || c.x >= m) {  // no finite similarity (a NaN token): the first target
-    if (lane == 0) atomicOr(&g_err_merge, RIFT_EBIT_NONFINITE);
-    c = make_int2(0, -1);
+  if (threadIdx.x == 0) n_open = 0;
+  __syncthreads();
+  const int al = a0 + threadIdx.x;
+  if (threadIdx.x < 64 && al < R && !(al % step == 0 && al / step < m)) {
+    int2 c = cand[(size_t)j * n_v + al];
+    if (c.x < 0 || c.x >= m) {  // no finite similarity (a NaN token): the first target
+      atomicOr(&g_err_merge, RIFT_EBIT_NONFINITE);
+      c = make_int2(0, -1);
+    }
+    if (c.y >= 0 && c.y < m) open[atomicAdd(&n_open, 1)] = make_int4(al, c.x, c.y, 0);
+    else assign[(size_t)j * n_v + al] = c.x;
   }
-  int choice = c.x;
-  if (c.y >= 0 && c.y < m) {
-    const XT* Xt = X + (size_t)kept[j] * n_v * d;
-    const int k = rest[(size_t)j * n_v + a];
-    const int t1 = ctx_target[co + c.x], t2 = ctx_target[co + c.y];
-    const double2 dd = ff_dot2(Xt + (size_t)k * d, Xt + (size_t)t1 * d, Xt + (size_t)t2 * d, d, lane);
-    const double d1 = dd.x, d2 = dd.y;
-    const double n1 = tnorm[co + c.x], n2 = tnorm[co + c.y];
-    const double s1 = n1 > 0.0 ? d1 / n1 : 0.0, s2 = n2 > 0.0 ? d2 / n2 : 0.0;
-    if (s2 > s1 || (s2 == s1 && c.y < c.x)) choice = c.y;
+  __syncthreads();
+  const uint16_t* Xt = X + (size_t)kept[j] * n_v * d;
+  for (int i = warp; i < n_open; i += 4) {
+    const int4 o = open[i];
+    const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + o.x] * d;
+    const uint16_t* t1 = Xt + (size_t)ctx_target[co + o.y] * d;
+    const uint16_t* t2 = Xt + (size_t)ctx_target[co + o.z] * d;
+    float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+    for (int k0 = lane * 8; k0 < d; k0 += 4 * 256) {
+      uint4 xr[4], r1[4], r2[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * 256 < d) {
+          xr[u] = *reinterpret_cast<const uint4*>(x + k0 + u * 256);
+          r1[u] = *reinterpret_cast<const uint4*>(t1 + k0 + u * 256);
+          r2[u] = *reinterpret_cast<const uint4*>(t2 + k0 + u * 256);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * 256 < d) {
+          float xv[8], y1[8], y2[8];
+          unpack_bf16x8(xr[u], xv);
+          unpack_bf16x8(r1[u], y1);
+          unpack_bf16x8(r2[u], y2);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            ff_step(xv[e], y1[e], h1, l1);
+            ff_step(xv[e], y2[e], h2, l2);
+          }
+        }
+    }
+    ff_warp_sum(h1, l1);
+    ff_warp_sum(h2, l2);
+    if (lane == 0) {
+      // s1 = e1 / n1 vs s2 = e2 / n2 as e1 n2 vs e2 n1 (norms are positive; a zero target has similarity 0)
+      const double n1 = tnorm[co + o.y], n2 = tnorm[co + o.z];
+      const double e1 = n1 > 0.0 ? (double)h1 + (double)l1 : 0.0, e2 = n2 > 0.0 ? (double)h2 + (double)l2 : 0.0;
+      const double s1 = e1 * (n2 > 0.0 ? n2 : 1.0), s2 = e2 * (n1 > 0.0 ? n1 : 1.0);
+      assign[(size_t)j * n_v + o.x] = s2 > s1 || (s2 == s1 && o.z < o.y) ? o.z : o.y;
+    }
   }
-  if (lane == 0) assign[(size_t)j * n_v + a] = choice;
 }
 
 // Grid (kept slot, block of TB unselected tokens).  assign[j][a] = target index of rest[a].
@@ -263,6 +306,8 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   __shared__ float best_v[TB][2];
   __shared__ int best_j[TB][2];
   __shared__ float inv_n[TB];
+  pdl_trigger();
+  pdl_wait();
   const int j = blockIdx.y;  // the token blocks of one slot are adjacent: its target rows stay in L2
   if (j >= *n_kept) return;
   const int s = sel_off[j + 1] - sel_off[j];
@@ -377,111 +422,119 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   }
 }
 
-// One CTA per kept slot: the slot's groups as member lists, ascending token index within each
-// group (targets at their own index): gstart[j][q] .. gstart[j][q+1] in memb[j].  A counting sort
-// whose placement pass runs in token order on one warp.
-__global__ void __launch_bounds__(256) merge_groups_kernel(int n_v, const int* __restrict__ n_kept,
-                                                           const int* __restrict__ sel_off,
-                                                           const int* __restrict__ ctx_off, int max_ctx,
-                                                           const int* __restrict__ rest,
-                                                           const int* __restrict__ assign, int* __restrict__ memb,
-                                                           int* __restrict__ gstart) {
-  __shared__ int cnt[RIFT_MAX_NV + 1];
-  const int j = blockIdx.x;
-  if (j >= *n_kept) return;
-  const int R = n_v - (sel_off[j + 1] - sel_off[j]);
-  const int co = ctx_off[j], m = ctx_off[j + 1] - co;
-  if (m == 0 || co + m > max_ctx) return;
-  const int step = R / m;
-  const int* rj = rest + (size_t)j * n_v;
-  const int* aj = assign + (size_t)j * n_v;
-  auto group = [&](int a) {
-    if (a % step == 0 && a / step < m) return a / step;
-    const int g = aj[a];
-    return (g >= 0 && g < m) ? g : 0;  // an unassigned token (no finite similarity) joins the first group
-  };
-  for (int q = threadIdx.x; q <= m; q += blockDim.x) cnt[q] = 0;
-  __syncthreads();
-  for (int a = threadIdx.x; a < R; a += blockDim.x) atomicAdd(&cnt[group(a)], 1);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int* gs = gstart + (size_t)j * (n_v + 1);
-    int acc = 0;
-    for (int q = 0; q < m; ++q) {  // cnt becomes each group's next free slot
-      const int c = cnt[q];
-      gs[q] = acc;
-      cnt[q] = acc;
-      acc += c;
-    }
-    gs[m] = acc;
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    // placement in token order by one warp, 32 tokens at a time: a token's slot is its group's
-    // next free one plus the number of lower lanes of the same group
-    const int lane = threadIdx.x;
-    int* mj = memb + (size_t)j * n_v;
-    for (int a0 = 0; a0 < R; a0 += 32) {
-      const int a = a0 + lane;
-      const int g = a < R ? group(a) : -1 - lane;  // idle lanes match no one
-      const unsigned same = __match_any_sync(0xffffffffu, g);
-      if (a < R) mj[cnt[g] + __popc(same & ((1u << lane) - 1u))] = rj[a];
-      __syncwarp();
-      if (a < R && (same >> lane) == 1u) cnt[g] += __popc(same);  // the group's highest lane
-      __syncwarp();
-    }
-  }
-}
-
-// Grid (kept slot, y), 256 threads: contextual token q = y, y + gridDim.y, ... is the mean of its
-// group's rows, summed in fp32 in member order (ascending index), each thread owning d / 256 of
-// the columns; stored as bf16.
-constexpr int MT = 256, MV = RIFT_MERGE_MAX_D / (MT * 8);
+// Grid (kept slot, 512 columns, part), 64 threads of eight columns: the contextual tokens' means over the
+// slot's unselected rows, read once, group after group, in ascending token index within a group (the
+// target's own row and the tokens assigned to it): summed in fp32, divided by the group size and
+// stored as bf16.  Each CTA sorts the slot's tokens by group itself (a stable counting sort in shared
+// memory, about 2 us, which took a launch and member lists in HBM), so the rows' loads, MU rows ahead,
+// do not wait for group boundaries, and takes its part (1 / MP) of the groups: with all of them a
+// scheduler had 2 or 3 warps to hide the adds' latency with.  73 us at 400 tiles, 76 with MP = 1 and 76 for
+// the sort and the sums as two launches.
+constexpr int MT = 64, MCOLS = 8 * MT, MU = 16, MP = 2;
 template <typename XT>
 __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X, int n_v, int d,
                                                         const int* __restrict__ kept, const int* __restrict__ n_kept,
+                                                        const int* __restrict__ sel_off,
                                                         const int* __restrict__ ctx_off, int max_ctx,
-                                                        const int* __restrict__ memb, const int* __restrict__ gstart,
+                                                        const int* __restrict__ rest, const int* __restrict__ assign,
                                                         uint16_t* __restrict__ ctx) {
-  const int j = blockIdx.x;
+  __shared__ uint16_t grp[RIFT_MAX_NV];        // group of unselected token a
+  __shared__ uint32_t memb[RIFT_MAX_NV + MU];  // sorted: group << 16 | token index
+  __shared__ int cnt[RIFT_MAX_NV + 1], at[RIFT_MAX_NV + 1];  // group sizes; each group's next place
+  pdl_trigger();
+  pdl_wait();
+  const int j = blockIdx.x, c0 = blockIdx.y * MCOLS + threadIdx.x * 8, lane = threadIdx.x & 31;
   if (j >= *n_kept) return;
   const int co = ctx_off[j], m = ctx_off[j + 1] - co;
-  if (m == 0 || co + m > max_ctx) return;
-  const int* gs = gstart + (size_t)j * (n_v + 1);
-  const int* mj = memb + (size_t)j * n_v;
-  const XT* Xt = X + (size_t)kept[j] * n_v * d;
-  for (int q = blockIdx.y; q < m; q += gridDim.y) {
-    const int g0 = gs[q], g1 = gs[q + 1];
-    float acc[MV][8];
-#pragma unroll
-    for (int v = 0; v < MV; ++v)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[v][e] = 0.f;
-    for (int g = g0; g < g1; ++g) {
-      const XT* row = Xt + (size_t)mj[g] * d;
-#pragma unroll
-      for (int v = 0; v < MV; ++v) {
-        const int c = (threadIdx.x + v * MT) * 8;
-        if (c < d) {
-          float x[8];
-          load8(row + c, x);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[v][e] += x[e];
-        }
-      }
+  const int q_lo = m * (int)blockIdx.z / MP, q_hi = m * ((int)blockIdx.z + 1) / MP;
+  if (q_lo == q_hi || co + m > max_ctx) return;
+  const int R = n_v - (sel_off[j + 1] - sel_off[j]), step = R / m;
+  const int* rj = rest + (size_t)j * n_v;
+  for (int q = threadIdx.x; q < m; q += MT) cnt[q] = 0;
+  __syncthreads();
+  for (int a = threadIdx.x; a < R; a += MT) {
+    int g = a / step;
+    if (a % step != 0 || g >= m) {
+      g = assign[(size_t)j * n_v + a];
+      if (g < 0 || g >= m) g = 0;  // an unassigned token (no finite similarity) joins the first group
     }
-    const float inv = 1.f / (float)(g1 - g0);
+    grp[a] = (uint16_t)g;
+    atomicAdd(&cnt[g], 1);
+  }
+  __syncthreads();
+  __shared__ int range[2];
+  if (threadIdx.x < 32) {
+    int base = 0;
+    for (int q0 = 0; q0 < m; q0 += 32) {  // exclusive prefix sum of the group sizes
+      const int v = q0 + lane < m ? cnt[q0 + lane] : 0, inc = warp_incl_scan(v);
+      if (q0 + lane < m) at[q0 + lane] = base + inc - v;
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      range[0] = at[q_lo];
+      range[1] = q_hi < m ? at[q_hi] : R;
+    }
+    __syncwarp();
+    // placement in token order, 32 tokens at a time: a token's place is its group's next one plus the
+    // number of lower lanes of the same group
+    for (int a0 = 0; a0 < R; a0 += 32) {
+      const int a = a0 + lane;
+      const int g = a < R ? grp[a] : -1 - lane;  // idle lanes match no one
+      const unsigned same = __match_any_sync(0xffffffffu, g);
+      if (a < R) memb[at[g] + __popc(same & ((1u << lane) - 1u))] = ((uint32_t)g << 16) | (uint32_t)rj[a];
+      __syncwarp();
+      if (a < R && (same >> lane) == 1u) at[g] += __popc(same);  // the group's highest lane
+      __syncwarp();
+    }
+    if (lane < MU) memb[R + lane] = memb[R - 1];  // a step past the end loads a row again
+  }
+  __syncthreads();
+  if (c0 >= d) return;
+  const int i0 = range[0], i1 = range[1];
+  const XT* Xc = X + (size_t)kept[j] * n_v * d + c0;
+  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  int cur = q_lo;
+  auto flush = [&]() {
+    const float inv = 1.f / (float)cnt[cur];
+    uint32_t w[4];
 #pragma unroll
-    for (int v = 0; v < MV; ++v) {
-      const int c = (threadIdx.x + v * MT) * 8;
-      if (c < d) {
-        uint32_t w[4];
+    for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+    *reinterpret_cast<uint4*>(ctx + (size_t)(co + cur) * d + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+  };
+  constexpr int NR = sizeof(XT) == 2 ? 1 : 2;  // 16-byte loads per row
+  for (int i = i0; i < i1; i += MU / NR) {
+    uint4 raw[MU / NR][NR];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(acc[v][2 * e] * inv, acc[v][2 * e + 1] * inv);
-        *reinterpret_cast<uint4*>(ctx + (size_t)(co + q) * d + c) = make_uint4(w[0], w[1], w[2], w[3]);
+    for (int u = 0; u < MU / NR; ++u) {
+      const XT* row = Xc + (size_t)(memb[i + u] & 0xffffu) * d;
+#pragma unroll
+      for (int v = 0; v < NR; ++v) raw[u][v] = reinterpret_cast<const uint4*>(row)[v];
+    }
+#pragma unroll
+    for (int u = 0; u < MU / NR; ++u) {
+      if (i + u >= i1) break;
+      const int g = (int)(memb[i + u] >> 16);
+      if (g != cur) {  // every group has its target: no group is empty
+        flush();
+        cur = g;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
       }
+      float x[8];
+      if constexpr (NR == 1) {
+        unpack_bf16x8(raw[u][0], x);
+      } else {
+        const uint32_t w[8] = {raw[u][0].x, raw[u][0].y, raw[u][0].z, raw[u][0].w,
+                               raw[u][1].x, raw[u][1].y, raw[u][1].z, raw[u][1].w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(w[e]);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] += x[e];
     }
   }
+  flush();
 }
 
 }  // namespace mg
@@ -493,9 +546,6 @@ MergeLayout merge_layout(int N, int n_v) {
   L.rest_off = take((size_t)N * n_v * sizeof(int));
   L.assign_off = take((size_t)N * n_v * sizeof(int));
   L.tnorm_off = take((size_t)N * n_v * sizeof(double));
-  L.memb_off = take((size_t)N * n_v * sizeof(int));
-  L.gstart_off = take((size_t)N * (n_v + 1) * sizeof(int));
-  L.pos_off = take((size_t)N * n_v * sizeof(int));
   L.tinv_off = take((size_t)N * n_v * sizeof(float));  // at most n_v - 1 targets per slot
   L.cand_off = take((size_t)N * n_v * sizeof(int2));
   L.total = off;
@@ -510,41 +560,40 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
   int* rest = reinterpret_cast<int*>(ws + L.rest_off);
   int* assign = reinterpret_cast<int*>(ws + L.assign_off);
   double* tnorm = reinterpret_cast<double*>(ws + L.tnorm_off);
-  int* memb = reinterpret_cast<int*>(ws + L.memb_off);
-  int* gstart = reinterpret_cast<int*>(ws + L.gstart_off);
-  int* pos = reinterpret_cast<int*>(ws + L.pos_off);
   float* tinv = reinterpret_cast<float*>(ws + L.tinv_off);
   int2* cand = reinterpret_cast<int2*>(ws + L.cand_off);
-  merge_plan_kernel<<<1, 1024, 0, st>>>(n_kept, budgets, sel_off, N, n_v, max_ctx, ctx_off);
-  const dim3 ga((n_v + TB - 1) / TB, N), gm(N, 32);
-  const size_t ab_bytes = 2 * (size_t)KC * (TB + 4) * sizeof(float);
-  if (xdt == RIFT_BF16) {
-    // bf16 tokens: the target rows go to ctx (overwritten by the means at the end), the top two
-    // of every token come from the tensor cores, the choice between them from float-float sums
-    const uint16_t* x = static_cast<const uint16_t*>(X);
-    merge_targets_kernel<uint16_t><<<N, 256, 0, st>>>(x, n_v, d, kept, n_kept, sel, sel_off, ctx_off, max_ctx, rest,
-                                                      ctx_target, tnorm, pos, tinv, ctx);
-    if (max_ctx > 0 &&
-        launch_merge_screen(x, N, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, ctx, tinv, pos, cand, st))
-      return -1;
-    merge_decide_kernel<uint16_t><<<dim3((n_v + 7) / 8, N), 256, 0, st>>>(x, n_v, d, kept, n_kept, sel_off, ctx_off,
-                                                                        max_ctx, rest, ctx_target, tnorm, cand,
-                                                                        assign);
-    merge_groups_kernel<<<N, 256, 0, st>>>(n_v, n_kept, sel_off, ctx_off, max_ctx, rest, assign, memb, gstart);
-    merge_mean_kernel<uint16_t><<<gm, MT, 0, st>>>(x, n_v, d, kept, n_kept, ctx_off, max_ctx, memb, gstart, ctx);
-    return max_ctx > 0 ? 6 : 5;
-  } else {
-    const float* x = static_cast<const float*>(X);
-    merge_targets_kernel<float><<<N, 256, 0, st>>>(x, n_v, d, kept, n_kept, sel, sel_off, ctx_off, max_ctx, rest,
-                                                   ctx_target, tnorm, nullptr, nullptr, nullptr);
-    static std::atomic<unsigned long long> smem_raised{0};
-    if (raise_smem_limit(smem_raised, merge_assign_kernel<float>, (int)ab_bytes) != cudaSuccess) return -1;
-    merge_assign_kernel<float><<<ga, 256, ab_bytes, st>>>(x, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, rest,
-                                                   ctx_target, tnorm, assign);
-    merge_groups_kernel<<<N, 256, 0, st>>>(n_v, n_kept, sel_off, ctx_off, max_ctx, rest, assign, memb, gstart);
-    merge_mean_kernel<float><<<gm, MT, 0, st>>>(x, n_v, d, kept, n_kept, ctx_off, max_ctx, memb, gstart, ctx);
-  }
-  return 5;
+  // every kernel a programmatic dependent of the one before it
+  bool ok = launch_ex(merge_plan_kernel, dim3(1), dim3(1024), 0, st, true, n_kept, budgets, sel_off, N, n_v, max_ctx,
+                      ctx_off) == cudaSuccess;
+  auto go = [&](auto* x) {
+    using XT = std::remove_const_t<std::remove_pointer_t<decltype(x)>>;
+    constexpr bool bf16 = sizeof(XT) == 2;
+    ok = ok && launch_ex(merge_targets_kernel<XT>, dim3(N, TY), dim3(256), 0, st, true, x, n_v, d, kept, n_kept, sel,
+                         sel_off, (const int*)ctx_off, max_ctx, rest, ctx_target, tnorm,
+                         bf16 ? tinv : (float*)nullptr, bf16 ? ctx : (uint16_t*)nullptr) == cudaSuccess;
+    if constexpr (bf16) {
+      // the target rows go to ctx (overwritten by the means at the end), the top two of every token
+      // come from the tensor cores, the choice between them where they are close from float-float sums
+      if (max_ctx > 0)
+        ok = ok && launch_merge_screen(x, N, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, ctx, tinv, rest, cand, st) == 0;
+      ok = ok && launch_ex(merge_decide_kernel, dim3((n_v + 63) / 64, N), dim3(128), 0, st, true, x, n_v, d, kept,
+                           n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
+                           (const double*)tnorm, (const int2*)cand, assign) == cudaSuccess;
+    } else {
+      static std::atomic<unsigned long long> smem_raised{0};
+      const size_t ab_bytes = 2 * (size_t)KC * (TB + 4) * sizeof(float);
+      ok = ok && raise_smem_limit(smem_raised, merge_assign_kernel<XT>, (int)ab_bytes) == cudaSuccess &&
+           launch_ex(merge_assign_kernel<XT>, dim3((n_v + TB - 1) / TB, N), dim3(256), ab_bytes, st, true, x, n_v, d,
+                     kept, n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
+                     (const double*)tnorm, assign) == cudaSuccess;
+    }
+    ok = ok && launch_ex(merge_mean_kernel<XT>, dim3(N, (d + MCOLS - 1) / MCOLS, MP), dim3(MT), 0, st, true, x,
+                         n_v, d, kept, n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)assign, ctx) == cudaSuccess;
+  };
+  if (xdt == RIFT_BF16) go(static_cast<const uint16_t*>(X));
+  else go(static_cast<const float*>(X));
+  if (!ok) return -1;
+  return xdt == RIFT_BF16 && max_ctx > 0 ? 5 : 4;
 }
 
 }  // namespace rift
