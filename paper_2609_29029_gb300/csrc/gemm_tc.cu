@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // prefill, a shared prompt, a small scene's Gram matrix), which stream the weights once.  The
 // operands are swapped: a CTA holds 128 weight rows as the MMA's M side and bn activation rows
 // (16 .. 160, a multiple of 16) as its N side, so a few rows cost no
-// more shared memory or tensor work than they need.  A cluster of S CTAs (1 .. 8) shares a tile:
+// more shared memory or tensor work than they need.  A cluster of S CTAs (1 .. 16) shares a tile:
 // rank r multiplies the K-blocks [kt r / S, kt (r + 1) / S), every CTA leaves its fp32 partial
 // product in its own shared memory, and after a cluster barrier rank r adds the S partials of
 // the rows r, r + S, ... in rank order (through distributed shared memory) and applies the
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // replaces in the decode step wrote its partial products to HBM and read them back in a
 // reduction launch: one 7B layer's products at one row 113 us then, 79 us now.
 namespace ck {
-constexpr int THREADS = 192, MAX_S = 8, MAX_BN = 160;
+constexpr int THREADS = 192, PORTABLE_S = 8, MAX_S = 16, MAX_BN = 160;
 constexpr int W_BYTES = BM * BK * 2;
 constexpr int SMEM = 232448 / 2 - 1024;  // two CTAs per SM
 constexpr int RING = SMEM - 1024 - 512;  // after alignment; the barriers at the end
@@ -569,19 +569,27 @@ __host__ __device__ constexpr int stages(int bn) {
 static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 
 // Row tiles: as few as MAX_BN allows, of equal height.  S: as many CTAs per tile as the GPU holds
-// at once (two per SM), each with at least 8 K-blocks (a shorter slice is all fill and drain).
+// at once (two per SM), each with at least min_blocks K-blocks (8: a shorter slice is all fill and
+// drain; a Gram matrix, on its own in a chain of small kernels, takes slices of 3).  More than 8 CTAs
+// (a non-portable cluster) where a single tile would leave the rest idle: 16 for the Gram matrix of
+// up to 128 tiles, K = 3 d (64 tiles at d = 4096: 11 us with 16, 15 with 8).
 // More CTAs than fit at once cost a second round: gate/up at one row 35.8 us with 172 CTAs, 43.6
 // with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.
 struct Plan {
   int bn, S;
 };
-inline Plan plan(int M, int N, int K, int sms) {
+inline Plan plan(int M, int N, int K, int sms, int min_blocks) {
   const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
   Plan p;
   p.bn = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16;
   const long long tiles = (long long)m_tiles * ((N + BM - 1) / BM);
-  p.S = MAX_S;
-  while (p.S > 1 && (tiles * p.S > 2LL * sms || ((K + BK - 1) / BK) / p.S < 8)) --p.S;
+  const int kt = (K + BK - 1) / BK;
+  if (tiles <= 2 && kt / MAX_S >= min_blocks) {
+    p.S = MAX_S;
+    return p;
+  }
+  p.S = PORTABLE_S;
+  while (p.S > 1 && (tiles * p.S > 2LL * sms || kt / p.S < min_blocks)) --p.S;
   return p;
 }
 }  // namespace ck
@@ -1155,8 +1163,10 @@ static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, in
                      cudaStream_t st, int bn, int S, bool pdl, int w_const) {
   CUtensorMap mw, mx;
   if (!make_map(&mw, W, Ks, (uint64_t)N, BM) || !make_map(&mx, A, Ks, (uint64_t)M, bn)) return 1;
-  static std::atomic<unsigned long long> smem_raised{0};
-  if (raise_smem_limit(smem_raised, gemm_ck_kernel<EPI>, ck::SMEM) != cudaSuccess) return 1;
+  static std::atomic<unsigned long long> smem_raised{0}, cluster_raised{0};
+  if (raise_smem_limit(smem_raised, gemm_ck_kernel<EPI>, ck::SMEM) != cudaSuccess ||
+      (S > ck::PORTABLE_S && raise_cluster_limit(cluster_raised, gemm_ck_kernel<EPI>) != cudaSuccess))
+    return 1;
   const int m_tiles = (M + bn - 1) / bn, n_tiles = (N + BM - 1) / BM;
   return launch_cluster_ex(gemm_ck_kernel<EPI>, dim3(m_tiles * n_tiles * S), dim3(ck::THREADS), ck::SMEM, st, pdl, S,
                            mw, mx, M, N, K, C, ep, bn, m_tiles, S, w_const) != cudaSuccess;
@@ -1218,7 +1228,7 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   // The operands' stored row width: K, or 2 kmap_d blocks when read through the K-block remap.
   if (ep.kmap_d && K != 3 * ep.kmap_d * BK) return 1;
   const uint64_t Ks = ep.kmap_d ? (uint64_t)2 * ep.kmap_d * BK : (uint64_t)K;
-  const ck::Plan plan = ck::plan(M, N, K, sm_count());
+  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ep.kmap_d ? 3 : 8);
   // The cluster split-K kernel for one row tile, or while its split tiles fit on the GPU at once:
   // beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
   // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777

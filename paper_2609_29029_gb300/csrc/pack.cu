@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(PK_THREADS) pack_kernel(
   }
 }
 
-constexpr int PKB_ROWS = 64;   // rows per CTA
+constexpr int PKB_ROWS = 64;   // rows per CTA, at most
 constexpr int PKB_SLOTS = 8;   // row buffers
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(64) pack_bulk_kernel(
     const int* __restrict__ sys_ids, int S, const int* __restrict__ query_ids, int Q,
     const uint16_t* __restrict__ embed, int vocab, const uint16_t* __restrict__ ctx,
     const int* __restrict__ ctx_off, uint16_t* __restrict__ packed, int max_T, int* __restrict__ positions,
-    int row_base, int* __restrict__ cu, int* __restrict__ T) {
+    int row_base, int* __restrict__ cu, int* __restrict__ T, int cta_rows) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ __align__(128) uint8_t ring[];
@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(64) pack_bulk_kernel(
   const int L = S + b + Q;
   const int base = j * (S + Q) + so + co;
   const int tile = kept[j];
-  const int r0 = blockIdx.y * PKB_ROWS;
-  const int n = min(L - r0, PKB_ROWS);
+  const int r0 = blockIdx.y * cta_rows;
+  const int n = min(L - r0, cta_rows);
   if (n <= 0) return;
   for (int q = threadIdx.x; q < n; q += blockDim.x)
     if (base + r0 + q < max_T) positions[base + r0 + q] = r0 + q;
@@ -240,10 +240,14 @@ void launch_pack(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
     static std::atomic<unsigned long long> smem_raised{0};
     if (raise_smem_limit(smem_raised, pack_bulk_kernel, PKB_SLOTS * 8192 * 2) != cudaSuccess)
       return;  // the error stays pending for the caller's launch check
-    dim3 gb(N, (max_L + PKB_ROWS - 1) / PKB_ROWS);
+    // A CTA streams its rows one ring after another, so with few tiles its row count is the time: 64 rows
+    // a CTA where many tiles keep the GPU full (fewer CTAs for tiles that are not kept), else 16 (64 tiles,
+    // 17 kept: 36 us with 64 rows a CTA, 16 with 16).
+    const int cta_rows = N > 128 ? PKB_ROWS : 16;
+    dim3 gb(N, (max_L + cta_rows - 1) / cta_rows);
     launch_ex(pack_bulk_kernel, gb, dim3(64), smem, st, true, static_cast<const uint16_t*>(X), N, n_v, d, kept,
               n_kept, sel, sel_off, sys_ids, S, query_ids, Q, static_cast<const uint16_t*>(embed), vocab, cx, ctx_off,
-              static_cast<uint16_t*>(packed), max_T, positions, row_base, cu_seqlens, T);
+              static_cast<uint16_t*>(packed), max_T, positions, row_base, cu_seqlens, T, cta_rows);
   } else
     launch_ex(pack_kernel<float>, grid, dim3(PK_THREADS), 0, st, true, static_cast<const float*>(X), N, n_v, d, kept,
               n_kept, sel, sel_off, sys_ids, S, query_ids, Q, static_cast<const uint16_t*>(embed), vocab, cx, ctx_off,

@@ -47,6 +47,16 @@ inline cudaError_t raise_smem_limit(std::atomic<unsigned long long>& done, K* ke
   return e;
 }
 
+// Allows `kernel` clusters of more than 8 CTAs (up to 16) in the current CUDA context; `done` as above.
+template <typename K>
+inline cudaError_t raise_cluster_limit(std::atomic<unsigned long long>& done, K* kernel) {
+  const unsigned long long ctx = current_context_id();
+  if (ctx != 0 && done.load(std::memory_order_acquire) == ctx) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && ctx != 0) done.store(ctx, std::memory_order_release);
+  return e;
+}
+
 // Programmatic dependent launch.  A kernel launched with `pdl` set (launch_ex) may begin while
 // the kernel before it in the stream is still running: each of its threads calls pdl_wait()
 // before its first access to memory that earlier kernels write or read (constant weights

@@ -20,7 +20,7 @@ unsigned int read_clear_err_gemm();
 // ---- score.cu ----
 // The token pass over N tiles (Eq. 1 per token, pooled sums): w and the partial pooled sums.
 struct ShardLayout {
-  int chunk_tokens, n_chunks;
+  int n_chunks;
   size_t w_off, cnt_off, ppart_off, total;
 };
 ShardLayout shard_layout(int N, int n_v, int d);

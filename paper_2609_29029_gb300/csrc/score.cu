@@ -234,12 +234,19 @@ __global__ void __launch_bounds__(256) tile_finalize_kernel(const float* __restr
 
 // ------------------------------------------------------------------------------------------
 // a2: token scores + partial pooled sums.  256 threads; thread t owns the 16-byte vectors
-// t, t + 256, ... of a token row (NVEC of them).  Tokens go in groups of 8: every thread
-// loads its vectors of all 8 tokens first (8 * NVEC 16-byte loads in flight), then the 16
-// partial sums (x.w and x.x of each token) are reduced across the CTA.
+// t, t + 256, ... of a token row (NVEC of them) over the chunk's tokens, in token order.  Tokens go LT
+// at a time: every thread loads its vectors of all of them first (LT * NVEC 16-byte loads in
+// flight), then each warp's sums x.w and x.x of each token go to shared memory and are added across
+// the warps once, at the end of the chunk, so nothing in the loop waits for another warp.
+// Few tiles (CS > 1): the 256 threads are spread over a cluster of CS CTAs, a 256 / CS-thread part of the
+// columns each, and the warps' sums are read through distributed shared memory at the end: the same
+// sums in the same order, bit for bit, on CS times the CTAs.
+// HBM-bound (X read once); under ncu, us, with a cross-warp reduction per 8 tokens and without the
+// clusters in brackets: 400 tiles x 576 x 4096 bf16 269 (276), 7.0 TB/s; 64 tiles 56 (62); 4 tiles x 576 x
+// 256 fp32, which is the latency of 6 (24) rounds of loads, 17 (28).
 // ------------------------------------------------------------------------------------------
 constexpr int SC_THREADS = 256;
-constexpr int SC_GROUP = 8;
+constexpr int SC_CHUNK = 192;  // tokens per chunk: 3 chunks per 576-token tile
 
 template <typename XT>
 struct VecTraits;
@@ -275,9 +282,25 @@ __device__ __forceinline__ float warp_reduce16(float (&v)[16]) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
-template <typename XT, int NVEC>
-__global__ void __launch_bounds__(SC_THREADS, 2)
-    token_score_kernel(const XT* __restrict__ X, int n_v, int d, int chunk_tokens, int n_chunks,
+__device__ __forceinline__ uint32_t sc_mapa(const void* p, int rank) {
+  uint32_t d;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+               : "=r"(d)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ float sc_ld_cluster(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sc_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+template <typename XT, int NVEC, int CS>
+__global__ void __launch_bounds__(SC_THREADS / CS, NVEC == 1 ? 1 : 2 * CS)
+    token_score_kernel(const XT* __restrict__ X, int n_v, int d, int n_chunks,
                        const float* __restrict__ w, float* __restrict__ token_scores,
                        float* __restrict__ Ppart, unsigned int* __restrict__ cnt, float* __restrict__ V,
                        float* __restrict__ s_raw, uint16_t* __restrict__ S16, int N, int Np) {
@@ -285,20 +308,23 @@ __global__ void __launch_bounds__(SC_THREADS, 2)
   pdl_wait();
   using VT = VecTraits<XT>;
   constexpr int VW = VT::W;
-  constexpr int GROUP = (NVEC <= 2) ? SC_GROUP : SC_GROUP / 2;  // raw loads: GROUP*NVEC*4 regs
-  __shared__ float red[SC_THREADS / 32][16];
-  __shared__ float tot[16];
-  const int tile = blockIdx.x / n_chunks;
-  const int chunk = blockIdx.x - tile * n_chunks;
-  const int k0 = chunk * chunk_tokens;
-  const int k1 = min(n_v, k0 + chunk_tokens);
+  constexpr int LT = NVEC == 1 ? 32 : NVEC == 2 ? 8 : 4;  // raw loads: LT * NVEC * 4 registers
+  constexpr int G = LT < 8 ? LT : 8;                      // tokens per warp reduction
+  constexpr int THREADS = SC_THREADS / CS, WARPS = THREADS / 32;
+  __shared__ float red[WARPS][SC_CHUNK][2];  // each warp's x.w and x.x of each token
+  const int rank = CS == 1 ? 0 : (int)(blockIdx.x % CS), unit = (int)blockIdx.x / CS;
+  const int tile = unit / n_chunks;
+  const int chunk = unit - tile * n_chunks;
+  const int k0 = chunk * SC_CHUNK;
+  const int k1 = min(n_v, k0 + SC_CHUNK);
   const int nvec = d / VW;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int vt = rank * THREADS + threadIdx.x;  // the thread's place among the 256
 
   float wv[NVEC][VW], P[NVEC][VW];
 #pragma unroll
   for (int j = 0; j < NVEC; ++j) {
-    int v = threadIdx.x + j * SC_THREADS;
+    int v = vt + j * SC_THREADS;
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
       wv[j][e] = (v < nvec) ? w[v * VW + e] : 0.f;
@@ -306,58 +332,68 @@ __global__ void __launch_bounds__(SC_THREADS, 2)
     }
   }
   const XT* base = X + ((size_t)tile * n_v) * d;
-  for (int g0 = k0; g0 < k1; g0 += GROUP) {
-    uint4 raw[GROUP][NVEC];
+  for (int g0 = k0; g0 < k1; g0 += LT) {
+    uint4 raw[LT][NVEC];
 #pragma unroll
-    for (int g = 0; g < GROUP; ++g) {
+    for (int g = 0; g < LT; ++g) {
 #pragma unroll
       for (int j = 0; j < NVEC; ++j) {
-        int v = threadIdx.x + j * SC_THREADS;
+        int v = vt + j * SC_THREADS;
         if (g0 + g < k1 && v < nvec)
           raw[g][j] = __ldcs(reinterpret_cast<const uint4*>(base + (size_t)(g0 + g) * d + v * VW));
         else
           raw[g][j] = make_uint4(0u, 0u, 0u, 0u);
       }
     }
-    float part[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) part[q] = 0.f;
+    for (int s0 = 0; s0 < LT; s0 += G) {
+      float part[16];
 #pragma unroll
-    for (int g = 0; g < GROUP; ++g) {
-      float dt = 0.f, ss = 0.f;
+      for (int q = 0; q < 16; ++q) part[q] = 0.f;
 #pragma unroll
-      for (int j = 0; j < NVEC; ++j) {
-        float xv[VW];
-        VT::unpack(raw[g][j], xv);
+      for (int g = 0; g < G; ++g) {
+        float dt = 0.f, ss = 0.f;
 #pragma unroll
-        for (int e = 0; e < VW; ++e) {
-          dt = fmaf(xv[e], wv[j][e], dt);
-          ss = fmaf(xv[e], xv[e], ss);
-          P[j][e] += xv[e];
+        for (int j = 0; j < NVEC; ++j) {
+          float xv[VW];
+          VT::unpack(raw[s0 + g][j], xv);
+#pragma unroll
+          for (int e = 0; e < VW; ++e) {
+            dt = fmaf(xv[e], wv[j][e], dt);
+            ss = fmaf(xv[e], xv[e], ss);
+            P[j][e] += xv[e];
+          }
         }
+        part[g] = dt;
+        part[8 + g] = ss;
       }
-      part[g] = dt;
-      part[8 + g] = ss;
-    }
-    float r = warp_reduce16(part);
-    if ((lane & 1) == 0) red[wid][lane >> 1] = r;
-    __syncthreads();
-    if (threadIdx.x < 16) {
-      float s = 0.f;
-#pragma unroll
-      for (int q = 0; q < SC_THREADS / 32; ++q) s += red[q][threadIdx.x];
-      tot[threadIdx.x] = s;
-    }
-    __syncthreads();
-    if (threadIdx.x < GROUP && g0 + threadIdx.x < k1) {
-      token_scores[(size_t)tile * n_v + g0 + threadIdx.x] =
-          tot[threadIdx.x] / sqrtf(tot[8 + threadIdx.x]);
+      const float r = warp_reduce16(part);
+      const int q = lane >> 1, k = g0 - k0 + s0 + (q & 7);
+      if ((lane & 1) == 0 && (q & 7) < G && k < SC_CHUNK) red[wid][k][q >> 3] = r;
     }
   }
-  float* out = Ppart + (size_t)blockIdx.x * d;
+  if constexpr (CS > 1) sc_cluster_sync();
+  else __syncthreads();
+  // token k0 + k: the warps' sums in warp order
+  for (int k = rank + CS * threadIdx.x; k < k1 - k0; k += CS * THREADS) {
+    float dt = 0.f, ss = 0.f;
+#pragma unroll
+    for (int q = 0; q < SC_THREADS / 32; ++q) {
+      if constexpr (CS == 1) {
+        dt += red[q][k][0];
+        ss += red[q][k][1];
+      } else {
+        const uint32_t a = sc_mapa(&red[q % WARPS][k][0], q / WARPS);
+        dt += sc_ld_cluster(a);
+        ss += sc_ld_cluster(a + 4);
+      }
+    }
+    token_scores[(size_t)tile * n_v + k0 + k] = dt / sqrtf(ss);
+  }
+  float* out = Ppart + (size_t)unit * d;
 #pragma unroll
   for (int j = 0; j < NVEC; ++j) {
-    int v = threadIdx.x + j * SC_THREADS;
+    int v = vt + j * SC_THREADS;
     if (v < nvec) {
 #pragma unroll
       for (int e = 0; e < VW; e += 4)
@@ -368,8 +404,13 @@ __global__ void __launch_bounds__(SC_THREADS, 2)
   // classic last-block reduction: every thread's stores are fenced before the count; the
   // finalising CTA fences before it reads the other partials), so no finalisation kernel follows
   // the pass.  Without it, tile_finalize_kernel does the same after the pass.
+  if constexpr (CS > 1) {
+    sc_cluster_sync();  // no CTA leaves while another may still read its sums
+    return;
+  }
   if (!cnt) return;
   __shared__ unsigned int last;
+  __shared__ float fin_red[32];
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -381,7 +422,7 @@ __global__ void __launch_bounds__(SC_THREADS, 2)
   if (!last) return;
   __threadfence();
   finalize_tile<(8192 / 4 + SC_THREADS - 1) / SC_THREADS>(tile, Ppart, n_chunks, d, w, V, s_raw, S16, N, Np,
-                                                          &red[0][0]);
+                                                          fin_red);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -552,35 +593,48 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
     }
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  double gl[RIFT_MAX_KNN];
-  int jl[RIFT_MAX_KNN];
-  for (int a = 0; a < C; ++a) {  // insertion into (g desc, j asc) order
-    double g = g64[a];
-    int j = jj[a], b = a;
-    while (b > 0 && (g > gl[b - 1] || (g == gl[b - 1] && j < jl[b - 1]))) { gl[b] = gl[b - 1]; jl[b] = jl[b - 1]; --b; }
-    gl[b] = g; jl[b] = j;
+  if (w != 0) return;
+  // Lane a < C holds candidate a, lane C the tile itself.  Rank by (similarity descending, index
+  // ascending); the m first are the neighbours.
+  // (as order-preserving integers: an SM retires about two double operations a cycle)
+  const double g0 = lane < C ? g64[lane] : -INFINITY;
+  long long g = __double_as_longlong(g0 == g0 ? (g0 == 0.0 ? 0.0 : g0) : -INFINITY);
+  if (g < 0) g ^= 0x7fffffffffffffffll;
+  const int j = lane < C ? jj[lane] : i;
+  int rank = 0;
+  for (int b = 0; b < C; ++b) {
+    const long long gb = __shfl_sync(0xffffffffu, g, b);
+    const int jb = __shfl_sync(0xffffffffu, j, b);
+    if (gb > g || (gb == g && (jb < j || (jb == j && b < lane)))) ++rank;
   }
-  if (nbr)
-    for (int r = 0; r < m; ++r) nbr[(size_t)il * m + r] = jl[r];
-  int mem[RIFT_MAX_KNN + 1];
-  int n = 0;
-  for (int r = 0; r < m; ++r) {
-    if (jl[r] >= 0 && jl[r] < N) {
-      mem[n++] = jl[r];
-    } else {  // fewer than m finite similarities (a NaN row): reported, never indexed
-      atomicOr(&g_err_score, RIFT_EBIT_NONFINITE);
-    }
-  }
-  mem[n++] = i;
-  for (int a = 1; a < n; ++a) {
-    int v = mem[a], b = a;
-    while (b > 0 && mem[b - 1] > v) { mem[b] = mem[b - 1]; --b; }
-    mem[b] = v;
-  }
+  const bool nb = lane < C && rank < m, valid = nb && j >= 0 && j < N;
+  if (nb && nbr) nbr[(size_t)il * m + rank] = j;
+  if (nb && !valid) atomicOr(&g_err_score, RIFT_EBIT_NONFINITE);  // fewer than m finite similarities: never indexed
+  // the sum over the set {i} + NN(i) in ascending index: each member's place, then the adds in order
+  const bool member = valid || lane == C;
+  const float sv = member ? s_raw[j] : 0.f;
+  int place = 0;
+  const unsigned in = __ballot_sync(0xffffffffu, member);
+  for (unsigned t = in; t; t &= t - 1)
+    if (__shfl_sync(0xffffffffu, j, __ffs(t) - 1) < j) ++place;
   float acc = 0.f;
-  for (int a = 0; a < n; ++a) acc = __fadd_rn(acc, s_raw[mem[a]]);
-  s_tilde[il] = __fdiv_rn(acc, (float)(m + 1));
+  const int n = __popc(in);
+  for (int a = 0; a < n; ++a) {
+    const unsigned who = __ballot_sync(0xffffffffu, member && place == a);
+    acc = __fadd_rn(acc, __shfl_sync(0xffffffffu, sv, __ffs(who) - 1));
+  }
+  if (lane == 0) s_tilde[il] = __fdiv_rn(acc, (float)(m + 1));
+}
+
+static int sm_count() {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 148;
+  }
+  return n;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -620,8 +674,7 @@ SmoothLayout smooth_layout(int N, int n_rows, int d) {
 // sums.
 ShardLayout shard_layout(int N, int n_v, int d) {
   ShardLayout L{};
-  L.chunk_tokens = 192;  // 3 CTAs per 576-token tile
-  L.n_chunks = (n_v + L.chunk_tokens - 1) / L.chunk_tokens;
+  L.n_chunks = (n_v + SC_CHUNK - 1) / SC_CHUNK;
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~size_t(255); return o; };
   L.w_off = take(sizeof(float) * d);
@@ -651,9 +704,19 @@ template <typename XT, int NVEC>
 static void launch_tokens(const void* X, int N, int n_v, int d, const ShardLayout& L, const float* w,
                           float* token_scores, float* Ppart, unsigned int* cnt, float* V, float* s_raw,
                           uint16_t* S16, cudaStream_t st) {
-  launch_ex(token_score_kernel<XT, NVEC>, dim3(N * L.n_chunks), dim3(SC_THREADS), 0, st, true,
-            static_cast<const XT*>(X), n_v, d, L.chunk_tokens, L.n_chunks, (const float*)w, token_scores, Ppart,
-            cnt, V, s_raw, S16, N, (N + 7) & ~7);
+  auto go = [&](auto cs) {
+    constexpr int CS = decltype(cs)::value;
+    launch_cluster_ex(token_score_kernel<XT, NVEC, CS>, dim3(N * L.n_chunks * CS), dim3(SC_THREADS / CS), 0, st, true, CS,
+                      static_cast<const XT*>(X), n_v, d, L.n_chunks, w, token_scores, Ppart, cnt, V, s_raw, S16, N,
+                      (N + 7) & ~7);
+  };
+  // Clusters while the chunks are fewer than four CTAs per SM (64 tiles: 192 CTAs on 152 SMs), and rows long
+  // enough that every thread has a vector (a shorter row's columns would all fall to rank 0)
+  const int units = N * L.n_chunks, want = 4 * sm_count();
+  const bool full = d >= SC_THREADS * VecTraits<XT>::W;
+  if (full && units * 2 <= want) go(std::integral_constant<int, 4>{});
+  else if (full && units < want) go(std::integral_constant<int, 2>{});
+  else go(std::integral_constant<int, 1>{});
 }
 
 int launch_score_tokens(const void* X, rift_dtype xdt, int N, int n_v, int d, const float* t, const float* B,

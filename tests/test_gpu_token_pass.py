@@ -1,0 +1,73 @@
+"""The token pass on clusters (few tiles) and without (many): the same token scores, tile scores and
+tile embeddings bit for bit, whatever the number of tiles, for widths with a full, a partial and
+several vectors per thread and token counts off the load batches; against fp64.  And the neighbour
+ranking of the smoothing with exact ties."""
+import pytest
+import torch
+
+from synth import rng
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dt,d,n_v", [("bf16", 2048, 200), ("bf16", 4096, 193), ("bf16", 8192, 21), ("f32", 1024, 577),
+                                      ("f32", 4096, 33), ("bf16", 320, 100), ("f32", 64, 5)])
+def test_scores_do_not_depend_on_the_tile_count(dt, d, n_v, cuda, riftlib):
+    chunks = -(-n_v // 192)
+    N = 640 // chunks + 1  # more than four CTAs per SM: no cluster
+    g = torch.Generator(device=cuda)
+    g.manual_seed(1)
+    X = torch.randn(N, n_v, d, generator=g, device=cuda).to(torch.bfloat16 if dt == "bf16" else torch.float32)
+    t = torch.randn(d, generator=g, device=cuda)
+    t /= t.norm()
+    xdt = riftlib.RIFT_BF16 if dt == "bf16" else riftlib.RIFT_F32
+
+    def score(n):
+        r = torch.full((n, n_v), float("nan"), device=cuda)
+        s = torch.full((n,), float("nan"), device=cuda)
+        V = torch.full((n, d), float("nan"), device=cuda)
+        need = riftlib.score_shard_workspace_bytes(n, n_v, d)
+        ws = torch.empty(need, dtype=torch.uint8, device=cuda)
+        riftlib.score_shard(X, xdt, n, n_v, d, t, None, 0, r, s, V, ws, need)
+        riftlib.sync_status()
+        return r, s, V
+
+    r, s, V = score(N)
+    for n in (1, 300 // chunks, 600 // chunks):  # clusters of 4, 4 and 2
+        got = score(n)
+        for a, b in zip(got, (r, s, V)):
+            assert torch.equal(a, b[:n])
+    x = X[:3].double().cpu()
+    w = t.double().cpu()
+    ref = (x @ w) / x.norm(dim=2)
+    # fp32 sums of d terms: sqrt(d) 2^-24 of the norms' product at random signs, and the division
+    assert float((r[:3].cpu().double() - ref).abs().max()) < 4e-6
+    P = x.sum(dim=1)
+    assert float((V[:3].cpu().double() - P / P.norm(dim=1, keepdim=True)).abs().max()) < 1e-6
+
+
+@pytest.mark.parametrize("m", [1, 6, 16])
+def test_neighbour_ties_go_to_the_lower_index(m, cuda, riftlib):
+    d, groups, N = 256, 8, 43
+    g = rng.normal_f32(4, rng.stream_id("tie-dirs"), groups * d).view(groups, d)
+    g = g / g.norm(dim=1, keepdim=True)
+    which = [(5 * i + i // 7) % groups for i in range(N)]  # tiles of one group are identical
+    V = g[which].contiguous()
+    sim = g.double() @ g.double().T
+    s_raw = rng.normal_f32(4, rng.stream_id("tie-scores"), N)
+    tile_s = torch.empty(N, device=cuda)
+    nbr = torch.empty(N, m, dtype=torch.int32, device=cuda)
+    need = riftlib.smooth_workspace_bytes(N, N, d)
+    ws = torch.empty(need, dtype=torch.uint8, device=cuda)
+    riftlib.smooth_rows(V.to(cuda), s_raw.to(cuda), N, d, 0, N, m, tile_s, nbr, ws, need)
+    riftlib.sync_status()
+    got = nbr.cpu().tolist()
+    for i in range(N):
+        want = sorted((j for j in range(N) if j != i), key=lambda j: (-float(sim[which[i], which[j]]), j))[:m]
+        if m <= 6:  # with m = 16 the candidates hold no spare: a group cut by the list's end keeps its lowest
+            assert got[i] == want, i
+        assert [which[j] for j in got[i]] == [which[j] for j in want], i
+        acc = torch.zeros(1)
+        for j in sorted(got[i] + [i]):
+            acc = acc + s_raw[j]
+        assert tile_s[i].cpu() == (acc / float(m + 1))[0]
