@@ -105,15 +105,17 @@ class ScenePipeline:
         self.nbr = torch.empty(max(N * self.m, 1), **i32)
         self.u = torch.empty(N, **f32)
         self.kept = torch.empty(N, **i32)
-        self.n_kept = torch.zeros(1, **i32)
+        # (n_kept, T): one buffer, so that one copy brings both to the host
+        self._counts = torch.zeros(2, **i32)
+        self.n_kept, self.T = self._counts[0:1], self._counts[1:2]
         self.budgets = torch.empty(N, **i32)
         self.sel = torch.empty(N * n_v, **i32)
         self.sel_off = torch.empty(N + 1, **i32)
         self.packed = torch.empty(self.max_T, d, dtype=torch.bfloat16, device=dev)
         self.cu = torch.empty(N + 1, **i32)
         self.positions = torch.empty(max(self.max_T, 1), **i32)
-        self.T = torch.zeros(1, **i32)
         self.counts_host = torch.zeros(2, dtype=torch.int32, pin_memory=True)
+        self._counts_ev = torch.cuda.Event()
         self.max_ctx = N * self.max_m
         self.ctx = torch.empty(max(self.max_ctx, 1), d, dtype=torch.bfloat16, device=dev) if self.max_m else None
         self.ctx_off = torch.zeros(N + 1, **i32) if self.max_m else None
@@ -195,12 +197,14 @@ class ScenePipeline:
     def _enqueue_counts(self, stream=None):
         """Copy (n_kept, T) into pinned host memory on `stream` once they are written, and record
         an event for counts() to wait on."""
-        s = stream if stream is not None else torch.cuda.current_stream()
-        with torch.cuda.stream(s):
-            self.counts_host[0:1].copy_(self.n_kept, non_blocking=True)
-            self.counts_host[1:2].copy_(self.T, non_blocking=True)
-            self._counts_ev = torch.cuda.Event()
+        s = torch.cuda.current_stream()
+        if stream is None or stream == s:
+            self.counts_host.copy_(self._counts, non_blocking=True)
             self._counts_ev.record(s)
+            return
+        with torch.cuda.stream(stream):
+            self.counts_host.copy_(self._counts, non_blocking=True)
+            self._counts_ev.record(stream)
 
     def counts(self):
         """(n_kept, T) of the last query run with counts=False: waits only until its packing has
@@ -281,11 +285,12 @@ class ScenePipeline:
         """One scene query, a1-a9, enqueued on `stream` with no host wait in between.  counts=True
         then waits for it, checks the device error flags and returns (n_kept, T); counts=False
         returns at once (None): counts() gives them once the packing has run."""
-        self.select(X, embed, phrase_ids, bg_ids, p, stream=stream)
-        self.pack(X, embed, sys_ids, query_ids, stream)
+        h = abi.stream_handle(stream)  # looked up once: as much host time as a launch
+        self.select(X, embed, phrase_ids, bg_ids, p, stream=h)
+        self.pack(X, embed, sys_ids, query_ids, h)
         self._enqueue_counts(stream)
         if prefill and self.model is not None:
-            self.prefill(stream)
+            self.prefill(h)
         if counts:
             abi.sync_status(stream)
             return self.counts()
