@@ -569,22 +569,22 @@ __host__ __device__ constexpr int stages(int bn) {
 static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 
 // Row tiles: as few as MAX_BN allows, of equal height.  S: as many CTAs per tile as the GPU holds
-// at once (two per SM), each with at least min_blocks K-blocks (8: a shorter slice is all fill and
-// drain; a Gram matrix, on its own in a chain of small kernels, takes slices of 3).  More than 8 CTAs
-// (a non-portable cluster) where a single tile would leave the rest idle: 16 for the Gram matrix of
-// up to 128 tiles, K = 3 d (64 tiles at d = 4096: 11 us with 16, 15 with 8).
+// at once (two per SM), each with at least 8 K-blocks (a shorter slice is all fill and drain; a Gram
+// matrix, on its own in a chain of small kernels, takes slices of 3).  More than 8 CTAs (a
+// non-portable cluster) where one tile would leave the rest idle: 16 for the Gram matrix of up to 128 tiles, K = 3 d (64 tiles at d = 4096: 11 us with 16, 15 with 8).
 // More CTAs than fit at once cost a second round: gate/up at one row 35.8 us with 172 CTAs, 43.6
 // with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.
 struct Plan {
   int bn, S;
 };
-inline Plan plan(int M, int N, int K, int sms, int min_blocks) {
+inline Plan plan(int M, int N, int K, int sms, bool gram) {
   const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
   Plan p;
   p.bn = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16;
   const long long tiles = (long long)m_tiles * ((N + BM - 1) / BM);
   const int kt = (K + BK - 1) / BK;
-  if (tiles <= 2 && kt / MAX_S >= min_blocks) {
+  const int min_blocks = gram ? 3 : 8;
+  if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) {
     p.S = MAX_S;
     return p;
   }
@@ -611,7 +611,9 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
   return v;
 }
 
-template <int EPI>
+// MAXS: the largest cluster this instance sums over (the partial sums' loads are unrolled over it: an
+// instance for 16 costs the clusters of up to 8 12% of a decode step).
+template <int EPI, int MAXS>
 __global__ void __launch_bounds__(ck::THREADS, 2)
     gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, int M_cap, int N,
                    int K, void* C, const EpiParams ep, int bn, int m_tiles, int S, int w_const) {
@@ -728,19 +730,19 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
   __syncwarp();
   cluster_sync();  // every CTA's partial product is in place
   if (mv > 0 && !*abort_flag) {
-    uint32_t base[ck::MAX_S];
+    uint32_t base[MAXS];
 #pragma unroll
-    for (int r = 0; r < ck::MAX_S; ++r) base[r] = r < S ? mapa_shared(smem0, r) : 0u;
+    for (int r = 0; r < MAXS; ++r) base[r] = r < S ? mapa_shared(smem0, r) : 0u;
     // the sum over the ranks of four weight rows' partials (columns q .. q + 3) of row m
     auto acc4 = [&](int m, int q) {
       const uint32_t off = (uint32_t)(m * BM + q) * 4u;
-      float4 f[ck::MAX_S];
+      float4 f[MAXS];
 #pragma unroll
-      for (int r = 0; r < ck::MAX_S; ++r)
+      for (int r = 0; r < MAXS; ++r)
         if (r < S) f[r] = ld_cluster4(base[r] + off);
       float4 v = f[0];
 #pragma unroll
-      for (int r = 1; r < ck::MAX_S; ++r)
+      for (int r = 1; r < MAXS; ++r)
         if (r < S) {
           v.x += f[r].x;
           v.y += f[r].y;
@@ -1158,17 +1160,17 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
 }
 
 // The cluster split-K kernel: S CTAs per (128 weight rows, bn rows) tile.
-template <int EPI>
+template <int EPI, int MAXS = ck::PORTABLE_S>
 static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
                      cudaStream_t st, int bn, int S, bool pdl, int w_const) {
   CUtensorMap mw, mx;
   if (!make_map(&mw, W, Ks, (uint64_t)N, BM) || !make_map(&mx, A, Ks, (uint64_t)M, bn)) return 1;
   static std::atomic<unsigned long long> smem_raised{0}, cluster_raised{0};
-  if (raise_smem_limit(smem_raised, gemm_ck_kernel<EPI>, ck::SMEM) != cudaSuccess ||
-      (S > ck::PORTABLE_S && raise_cluster_limit(cluster_raised, gemm_ck_kernel<EPI>) != cudaSuccess))
+  if (raise_smem_limit(smem_raised, gemm_ck_kernel<EPI, MAXS>, ck::SMEM) != cudaSuccess ||
+      (MAXS > ck::PORTABLE_S && raise_cluster_limit(cluster_raised, gemm_ck_kernel<EPI, MAXS>) != cudaSuccess))
     return 1;
   const int m_tiles = (M + bn - 1) / bn, n_tiles = (N + BM - 1) / BM;
-  return launch_cluster_ex(gemm_ck_kernel<EPI>, dim3(m_tiles * n_tiles * S), dim3(ck::THREADS), ck::SMEM, st, pdl, S,
+  return launch_cluster_ex(gemm_ck_kernel<EPI, MAXS>, dim3(m_tiles * n_tiles * S), dim3(ck::THREADS), ck::SMEM, st, pdl, S,
                            mw, mx, M, N, K, C, ep, bn, m_tiles, S, w_const) != cudaSuccess;
 }
 
@@ -1179,7 +1181,10 @@ static int launch_ck_epi(const void* A, const void* W, uint64_t Ks, int M, int N
     case EPI_RESID_F32: return launch_ck<EPI_RESID_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
     case EPI_SWIGLU: return launch_ck<EPI_SWIGLU>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
     case EPI_QKV_ROPE: return launch_ck<EPI_QKV_ROPE>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
-    case EPI_STORE_F32: return launch_ck<EPI_STORE_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_STORE_F32:
+      return p.S > ck::PORTABLE_S
+                 ? launch_ck<EPI_STORE_F32, ck::MAX_S>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const)
+                 : launch_ck<EPI_STORE_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
     default: return 1;
   }
 }
@@ -1228,7 +1233,7 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   // The operands' stored row width: K, or 2 kmap_d blocks when read through the K-block remap.
   if (ep.kmap_d && K != 3 * ep.kmap_d * BK) return 1;
   const uint64_t Ks = ep.kmap_d ? (uint64_t)2 * ep.kmap_d * BK : (uint64_t)K;
-  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ep.kmap_d ? 3 : 8);
+  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ep.kmap_d > 0);
   // The cluster split-K kernel for one row tile, or while its split tiles fit on the GPU at once:
   // beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
   // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777
