@@ -611,8 +611,8 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr) {
   return v;
 }
 
-// MAXS: the largest cluster this instance sums over (the partial sums' loads are unrolled over it: an
-// instance for 16 costs the clusters of up to 8 12% of a decode step).
+// MAXS: the largest cluster this instance sums over (1, 4, 8 or 16; the partial sums' loads are unrolled
+// over it, so that they are all in flight: with one instance for 16, 3 us more a launch).
 template <int EPI, int MAXS>
 __global__ void __launch_bounds__(ck::THREADS, 2)
     gemm_ck_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, int M_cap, int N,
@@ -728,28 +728,33 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
     }
   }
   __syncwarp();
-  cluster_sync();  // every CTA's partial product is in place
+  if constexpr (MAXS == 1) __syncthreads();
+  else cluster_sync();  // every CTA's partial product is in place
   if (mv > 0 && !*abort_flag) {
     uint32_t base[MAXS];
 #pragma unroll
-    for (int r = 0; r < MAXS; ++r) base[r] = r < S ? mapa_shared(smem0, r) : 0u;
+    for (int r = 0; r < MAXS; ++r) base[r] = MAXS == 1 ? smem0 : r < S ? mapa_shared(smem0, r) : 0u;
     // the sum over the ranks of four weight rows' partials (columns q .. q + 3) of row m
     auto acc4 = [&](int m, int q) {
-      const uint32_t off = (uint32_t)(m * BM + q) * 4u;
-      float4 f[MAXS];
+      if constexpr (MAXS == 1) {
+        return *reinterpret_cast<const float4*>(smem + (m * BM + q) * 4);
+      } else {
+        const uint32_t off = (uint32_t)(m * BM + q) * 4u;
+        float4 f[MAXS];
 #pragma unroll
-      for (int r = 0; r < MAXS; ++r)
-        if (r < S) f[r] = ld_cluster4(base[r] + off);
-      float4 v = f[0];
+        for (int r = 0; r < MAXS; ++r)
+          if (r < S) f[r] = ld_cluster4(base[r] + off);
+        float4 v = f[0];
 #pragma unroll
-      for (int r = 1; r < MAXS; ++r)
-        if (r < S) {
-          v.x += f[r].x;
-          v.y += f[r].y;
-          v.z += f[r].z;
-          v.w += f[r].w;
-        }
-      return v;
+        for (int r = 1; r < MAXS; ++r)
+          if (r < S) {
+            v.x += f[r].x;
+            v.y += f[r].y;
+            v.z += f[r].z;
+            v.w += f[r].w;
+          }
+        return v;
+      }
     };
     auto store_h4 = [](void* dst, float a, float b, float c, float d) {
       *reinterpret_cast<uint2*>(dst) = make_uint2(pack_half2(a, b), pack_half2(c, d));
@@ -810,7 +815,7 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
     }
   }
   __syncwarp();
-  cluster_sync();  // no CTA leaves while another may still read its partial product
+  if constexpr (MAXS > 1) cluster_sync();  // no CTA leaves while another may still read its partial product
   if (warp == 1) {
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(cols) : "memory");
@@ -1160,8 +1165,8 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
 }
 
 // The cluster split-K kernel: S CTAs per (128 weight rows, bn rows) tile.
-template <int EPI, int MAXS = ck::PORTABLE_S>
-static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
+template <int EPI, int MAXS>
+static int launch_ck_instance(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
                      cudaStream_t st, int bn, int S, bool pdl, int w_const) {
   CUtensorMap mw, mx;
   if (!make_map(&mw, W, Ks, (uint64_t)N, BM) || !make_map(&mx, A, Ks, (uint64_t)M, bn)) return 1;
@@ -1174,17 +1179,25 @@ static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, in
                            mw, mx, M, N, K, C, ep, bn, m_tiles, S, w_const) != cudaSuccess;
 }
 
+template <int EPI>
+static int launch_ck(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
+                     cudaStream_t st, const ck::Plan& p, bool pdl, int w_const) {
+  if (p.S == 1) return launch_ck_instance<EPI, 1>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+  if (p.S <= 4) return launch_ck_instance<EPI, 4>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+  if constexpr (EPI == EPI_STORE_F32)  // the Gram matrix of few tiles
+    if (p.S > ck::PORTABLE_S)
+      return launch_ck_instance<EPI, ck::MAX_S>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+  return launch_ck_instance<EPI, ck::PORTABLE_S>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+}
+
 static int launch_ck_epi(const void* A, const void* W, uint64_t Ks, int M, int N, int K, int epi, void* C,
                          const EpiParams& ep, cudaStream_t st, const ck::Plan& p, bool pdl, int w_const) {
   switch (epi) {
-    case EPI_STORE_BF16: return launch_ck<EPI_STORE_BF16>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
-    case EPI_RESID_F32: return launch_ck<EPI_RESID_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
-    case EPI_SWIGLU: return launch_ck<EPI_SWIGLU>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
-    case EPI_QKV_ROPE: return launch_ck<EPI_QKV_ROPE>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
-    case EPI_STORE_F32:
-      return p.S > ck::PORTABLE_S
-                 ? launch_ck<EPI_STORE_F32, ck::MAX_S>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const)
-                 : launch_ck<EPI_STORE_F32>(A, W, Ks, M, N, K, C, ep, st, p.bn, p.S, pdl, w_const);
+    case EPI_STORE_BF16: return launch_ck<EPI_STORE_BF16>(A, W, Ks, M, N, K, C, ep, st, p, pdl, w_const);
+    case EPI_RESID_F32: return launch_ck<EPI_RESID_F32>(A, W, Ks, M, N, K, C, ep, st, p, pdl, w_const);
+    case EPI_SWIGLU: return launch_ck<EPI_SWIGLU>(A, W, Ks, M, N, K, C, ep, st, p, pdl, w_const);
+    case EPI_QKV_ROPE: return launch_ck<EPI_QKV_ROPE>(A, W, Ks, M, N, K, C, ep, st, p, pdl, w_const);
+    case EPI_STORE_F32: return launch_ck<EPI_STORE_F32>(A, W, Ks, M, N, K, C, ep, st, p, pdl, w_const);
     default: return 1;
   }
 }
