@@ -432,11 +432,6 @@ __global__ void __launch_bounds__(SC_THREADS / CS, NVEC == 1 ? 1 : 2 * CS)
 // ------------------------------------------------------------------------------------------
 constexpr int KNN_SPARE = 10;  // candidates kept beyond m for the fp64 rescoring
 
-// (g, j) beats (g2, j2): larger similarity first, then the lower index.
-__device__ __forceinline__ bool knn_better(float g, int j, float g2, int j2) {
-  return g > g2 || (g == g2 && j < j2);
-}
-
 // The Gram matrix on the tensor cores.  Each fp32 row of V (scaled by 2^10, so that the low parts
 // stay normal in fp16) is split into hi = fp16(v) and lo = fp16(v - hi), stored once as the row
 // [hi | lo] of S (2 d fp16).  The product reads S twice through a K-block remap: A = [hi | hi | lo]
@@ -475,28 +470,44 @@ __global__ void knn_split_kernel(const float* __restrict__ V, int N, int Np, int
   row[d / 8] = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// One warp per row of the materialised Gram matrix: the row's 16 best columns (larger
-// similarity, then lower index) are kept sorted across lanes 0..15, one entry per lane.  The row
-// is read 32 columns at a time; a ballot picks the columns that beat the current 16th entry, and
-// each of them (in ascending column order) is inserted at the position the entries above it
-// give, the entries below moving down a lane.  Row il of G is tile row0 + il.
+// A similarity and its column as a sortable pair: hi orders like the similarity (0 for none: a NaN, -inf
+// or a column that is not a candidate), ties go to the lower column.
+struct KnnKey {
+  uint32_t hi;
+  int j;
+};
+__device__ __forceinline__ bool knn_better(const KnnKey& a, const KnnKey& b) {
+  return a.hi > b.hi || (a.hi == b.hi && a.j < b.j);
+}
+__device__ __forceinline__ KnnKey knn_shfl_xor(const KnnKey& k, int o) {
+  return {__shfl_xor_sync(0xffffffffu, k.hi, o), __shfl_xor_sync(0xffffffffu, k.j, o)};
+}
+// One compare-exchange of a bitonic network over the lanes: the better of the pair (lane, lane ^ o) goes to
+// the lane for which `first` holds.
+__device__ __forceinline__ void knn_exchange(KnnKey& k, int o, bool first) {
+  const KnnKey p = knn_shfl_xor(k, o);
+  if (knn_better(p, k) == first) k = p;
+}
+
+// One warp per row of the materialised Gram matrix: the row's best columns (larger similarity, then lower
+// index) are kept sorted across the lanes.  The row is read 512 columns at a time, 16 loads in flight
+// per lane, and taken 32 columns at a time: none of them better than the 16th entry so far, nothing
+// is done; one or two, each is inserted at the place the entries above it give; more, the 32 are
+// sorted by a bitonic network and merged with the list (an insertion is a chain of eight shuffles
+// and ballots, and the first columns of a row would all be insertions: 64 tiles 8.7 us, this way 4.6; 400
+// tiles 14 and 10).  Row il of G is tile row0 + il.
 __global__ void knn_gram_topc_kernel(const float* __restrict__ G, int N, int ld, int row0, int n_rows, int C,
                                      int* __restrict__ top_j) {
   pdl_trigger();
   pdl_wait();
-  constexpr int K = RIFT_MAX_KNN;  // list length (C <= K)
   const int lane = threadIdx.x & 31;
   const int il = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (il >= n_rows) return;
   const int i = row0 + il;
-  float lg = -INFINITY;  // this lane's entry (lanes >= K stay empty)
-  int lj = 0x7fffffff;
-  float tg = -INFINITY;  // the 16th entry: what a column must beat
-  int tj = 0x7fffffff;
+  KnnKey list = {0u, 0x7fffffff};  // this lane's entry
+  KnnKey bar = list;               // the 16th entry: what a column must beat
   const float* row = G + (size_t)il * ld;
   bool bad = false;
-  // 16 loads in flight per lane (512 columns per step): a step is bounded by the loads' latency,
-  // not by the insertions, so fewer and wider steps finish a row sooner
   constexpr int NL = 16;
   for (int j0 = 0; j0 < N; j0 += 32 * NL) {
     float gv[NL];
@@ -508,37 +519,130 @@ __global__ void knn_gram_topc_kernel(const float* __restrict__ G, int N, int ld,
 #pragma unroll
     for (int q = 0; q < NL; ++q) {
       const int j = j0 + 32 * q + lane;
-      float g = gv[q];
-      if (!(g == g)) {
-        bad = true;
-        g = -INFINITY;
-      }
-      if (j >= N || j == i) g = -INFINITY;
-      unsigned mask = __ballot_sync(0xffffffffu, g != -INFINITY && knn_better(g, j, tg, tj));
-      while (mask) {
-        const int src = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const float cg = __shfl_sync(0xffffffffu, g, src);
-        const int cj = __shfl_sync(0xffffffffu, j, src);
-        if (!knn_better(cg, cj, tg, tj)) continue;  // the threshold rose meanwhile (uniform)
-        const int pos = __popc(__ballot_sync(0xffffffffu, lane < K && knn_better(lg, lj, cg, cj)));
-        const float ug = __shfl_up_sync(0xffffffffu, lg, 1);
-        const int uj = __shfl_up_sync(0xffffffffu, lj, 1);
-        if (lane > pos && lane < K) {
-          lg = ug;
-          lj = uj;
+      const float g = gv[q];
+      if (!(g == g)) bad = true;
+      const uint32_t u = __float_as_uint(g == 0.f ? 0.f : g);
+      KnnKey k = {(u & 0x80000000u) ? ~u : (u | 0x80000000u), j};
+      if (!(g > -INFINITY) || j >= N || j == i) k = {0u, 0x7fffffff};
+      unsigned mask = __ballot_sync(0xffffffffu, knn_better(k, bar));
+      if (mask == 0) continue;
+      if (__popc(mask) <= 2) {
+        for (; mask; mask &= mask - 1) {
+          const int src = __ffs(mask) - 1;
+          const KnnKey c = {__shfl_sync(0xffffffffu, k.hi, src), __shfl_sync(0xffffffffu, k.j, src)};
+          const int pos = __popc(__ballot_sync(0xffffffffu, knn_better(list, c)));
+          const KnnKey up = {__shfl_up_sync(0xffffffffu, list.hi, 1), __shfl_up_sync(0xffffffffu, list.j, 1)};
+          if (lane > pos) list = up;
+          if (lane == pos) list = c;
         }
-        if (lane == pos) {
-          lg = cg;
-          lj = cj;
-        }
-        tg = __shfl_sync(0xffffffffu, lg, K - 1);
-        tj = __shfl_sync(0xffffffffu, lj, K - 1);
+      } else {
+#pragma unroll
+        for (int w = 2; w <= 32; w *= 2)
+#pragma unroll
+          for (int o = w / 2; o >= 1; o /= 2) knn_exchange(k, o, ((lane & o) == 0) == ((lane & w) == 0));
+        // the 32 best of the two sorted sequences: the better of lane l's entry and the new sequence's 31 - l,
+        // a bitonic sequence, merged
+        const KnnKey r = {__shfl_sync(0xffffffffu, k.hi, 31 - lane), __shfl_sync(0xffffffffu, k.j, 31 - lane)};
+        if (knn_better(r, list)) list = r;
+#pragma unroll
+        for (int o = 16; o >= 1; o /= 2) knn_exchange(list, o, (lane & o) == 0);
       }
+      bar = {__shfl_sync(0xffffffffu, list.hi, RIFT_MAX_KNN - 1), __shfl_sync(0xffffffffu, list.j, RIFT_MAX_KNN - 1)};
     }
   }
   if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&g_err_score, RIFT_EBIT_NONFINITE);
-  if (lane < C) top_j[(size_t)il * C + lane] = (lg == -INFINITY) ? 0x7fffffff : lj;
+  if (lane < C) top_j[(size_t)il * C + lane] = list.hi == 0u ? 0x7fffffff : list.j;
+}
+
+// A lane's terms of the similarity of rows vi and vj as an unevaluated pair hi + lo of floats: the product of
+// two floats is split exactly with an FMA (Dekker's TwoProduct as rewritten by Ogita, Rump and
+// Oishi) and added with Knuth's TwoSum, so the lane sum is good to ~2^-44 relative.
+__device__ __forceinline__ void knn_ff_step4(const float4& a4, const float4& b4, float& hi, float& lo) {
+  const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float p = __fmul_rn(av[e], bv[e]);
+    const float pe = fmaf(av[e], bv[e], -p);
+    const float s = __fadd_rn(hi, p);
+    const float bb = __fsub_rn(s, hi);
+    const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(er, pe));
+  }
+}
+__device__ __forceinline__ double knn_lane_sum(float hi, float lo) {
+  double acc = (double)hi + (double)lo;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+// The similarity as an order-preserving integer (NaN as -inf): an SM retires about two double operations a
+// cycle.
+__device__ __forceinline__ long long knn_order(double g0) {
+  long long g = __double_as_longlong(g0 == g0 ? (g0 == 0.0 ? 0.0 : g0) : -INFINITY);
+  return g < 0 ? g ^ 0x7fffffffffffffffll : g;
+}
+
+// Scenes of at most KNN_PAIRS tiles: every pair's similarity at the accuracy of the rescoring below, with no
+// Gram matrix and no candidates, and the smoothing.  One CTA per tile, a warp per other tile, two at a time.
+// Up to three launches fewer than the general path, whose Gram product and candidate lists are latency at
+// this size; past 32 tiles a warp goes around more than once and the general path is as fast
+// (smoothing alone at d = 4096, us, pairs against general: 16 tiles 12.6 : 22.2, 32 tiles 13.5 : 22.7, 64 tiles
+// 25.1 : 24.0, 100 tiles 62 : 26).
+constexpr int KNN_PAIRS = 32;
+__global__ void __launch_bounds__(512) knn_pairs_smooth_kernel(const float* __restrict__ V, int d, int N, int row0, int m,
+                                                               const float* __restrict__ s_raw,
+                                                               float* __restrict__ s_tilde, int* __restrict__ nbr) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ long long g64[KNN_PAIRS];
+  __shared__ float s_sh[KNN_PAIRS];
+  __shared__ unsigned in[KNN_PAIRS / 32];
+  const int il = blockIdx.x, i = row0 + il;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x < N) s_sh[threadIdx.x] = s_raw[threadIdx.x];
+  const float4* vi = reinterpret_cast<const float4*>(V + (size_t)i * d);
+  for (int j = w; j < N && m > 0; j += 32) {
+    const int j2 = j + 16 < N ? j + 16 : j;
+    const float4* vj = reinterpret_cast<const float4*>(V + (size_t)j * d);
+    const float4* vk = reinterpret_cast<const float4*>(V + (size_t)j2 * d);
+    float hi = 0.f, lo = 0.f, hi2 = 0.f, lo2 = 0.f;
+#pragma unroll 4
+    for (int k = lane; k < d / 4; k += 32) {
+      const float4 a = vi[k], b = vj[k], c = vk[k];
+      knn_ff_step4(a, b, hi, lo);
+      knn_ff_step4(a, c, hi2, lo2);
+    }
+    const double g = knn_lane_sum(hi, lo), g2 = knn_lane_sum(hi2, lo2);
+    if (lane == 0) {
+      if (!(g == g) || !(g2 == g2)) atomicOr(&g_err_score, RIFT_EBIT_NONFINITE);
+      g64[j] = knn_order(g);
+      g64[j2] = knn_order(g2);
+    }
+  }
+  __syncthreads();
+  // rank of tile t among the others by (similarity descending, index ascending); the m first are the
+  // neighbours
+  const int t = threadIdx.x;
+  if (t < KNN_PAIRS) {
+    bool nb = false;
+    if (t < N && t != i && m > 0) {
+      const long long g = g64[t];
+      int rank = 0;
+      for (int b = 0; b < N; ++b)
+        if (b != i && (g64[b] > g || (g64[b] == g && b < t))) ++rank;
+      nb = rank < m;
+      if (nb && nbr) nbr[(size_t)il * m + rank] = t;
+    }
+    const unsigned b = __ballot_sync(0xffffffffu, nb || t == i);
+    if (lane == 0) in[w] = b;
+  }
+  __syncthreads();
+  if (t != 0) return;
+  float acc = 0.f;  // over {i} + NN(i) in ascending index
+  for (int x = 0; x < KNN_PAIRS / 32; ++x)
+    for (unsigned b = in[x]; b; b &= b - 1) acc = __fadd_rn(acc, s_sh[32 * x + __ffs(b) - 1]);
+  s_tilde[il] = __fdiv_rn(acc, (float)(m + 1));
 }
 
 // One CTA per tile, one warp per candidate: recompute the C candidates' similarities to ~fp64
@@ -558,9 +662,6 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (w < C) {
     const int j = top_j[(size_t)il * C + w];
-    // Each lane keeps its partial sum as an unevaluated pair hi + lo of floats: the product of
-    // two floats is split exactly with an FMA (Dekker's TwoProduct as rewritten by Ogita, Rump
-    // and Oishi) and added with Knuth's TwoSum, so the lane sum is good to ~2^-44 relative.
     // V_i is read by all the CTA's warps (L1 serves all but the first).  The kernel moves 16 rows
     // of V per tile from L2: its time follows those bytes, not the length of this chain (four
     // independent chains with loads ahead measured slower, at fewer resident CTAs).
@@ -569,24 +670,9 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
       const float4* vi = reinterpret_cast<const float4*>(V + (size_t)i * d);
       const float4* vj = reinterpret_cast<const float4*>(V + (size_t)j * d);
 #pragma unroll 4
-      for (int k = lane; k < d / 4; k += 32) {
-        const float4 a4 = vi[k], b4 = vj[k];
-        const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float p = __fmul_rn(av[e], bv[e]);
-          const float pe = fmaf(av[e], bv[e], -p);
-          const float s = __fadd_rn(hi, p);
-          const float bb = __fsub_rn(s, hi);
-          const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-          hi = s;
-          lo = __fadd_rn(lo, __fadd_rn(er, pe));
-        }
-      }
+      for (int k = lane; k < d / 4; k += 32) knn_ff_step4(vi[k], vj[k], hi, lo);
     }
-    double acc = (double)hi + (double)lo;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    const double acc = knn_lane_sum(hi, lo);
     if (lane == 0) {
       g64[w] = (j >= 0 && j < N) ? acc : -INFINITY;
       jj[w] = j;
@@ -596,10 +682,7 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
   if (w != 0) return;
   // Lane a < C holds candidate a, lane C the tile itself.  Rank by (similarity descending, index
   // ascending); the m first are the neighbours.
-  // (as order-preserving integers: an SM retires about two double operations a cycle)
-  const double g0 = lane < C ? g64[lane] : -INFINITY;
-  long long g = __double_as_longlong(g0 == g0 ? (g0 == 0.0 ? 0.0 : g0) : -INFINITY);
-  if (g < 0) g ^= 0x7fffffffffffffffll;
+  const long long g = knn_order(lane < C ? g64[lane] : -INFINITY);
   const int j = lane < C ? jj[lane] : i;
   int rank = 0;
   for (int b = 0; b < C; ++b) {
@@ -760,6 +843,10 @@ int launch_score_tokens(const void* X, rift_dtype xdt, int N, int n_v, int d, co
 
 int launch_smooth(const float* V, const float* s_raw, int N, int d, int row0, int n_rows, int m, float* s_tilde,
                   int* nbr, char* ws, cudaStream_t st, bool split_done) {
+  if (N <= KNN_PAIRS) {
+    launch_ex(knn_pairs_smooth_kernel, dim3(n_rows), dim3(512), 0, st, true, V, d, N, row0, m, s_raw, s_tilde, nbr);
+    return 1;
+  }
   const SmoothLayout L = smooth_layout(N, n_rows, d);
   int* topj = reinterpret_cast<int*>(ws + L.top_off);
   // candidates per row: m plus spares for the fp64 rescoring, at most the N - 1 other tiles
@@ -798,8 +885,8 @@ int launch_score(const void* X, rift_dtype xdt, int N, int n_v, int d, const flo
                  cudaStream_t st) {
   const ScoreLayout L = score_layout(N, n_v, d, M);
   float* V = reinterpret_cast<float*>(ws + L.V_off);
-  // with neighbours to find, the token pass's finalisation also writes the Gram's split rows
-  uint16_t* S16 = m > 0 ? reinterpret_cast<uint16_t*>(ws + L.smooth_off + L.S.split_off) : nullptr;
+  // with a Gram matrix to form, the token pass's finalisation also writes its split rows
+  uint16_t* S16 = m > 0 && N > KNN_PAIRS ? reinterpret_cast<uint16_t*>(ws + L.smooth_off + L.S.split_off) : nullptr;
   const int a = launch_score_tokens(X, xdt, N, n_v, d, t, B, M, token_scores, s_raw, V, ws + L.tokens_off, st, S16);
   const int b = launch_smooth(V, s_raw, N, d, 0, N, m, s_tilde, nbr, ws + L.smooth_off, st, m > 0);
   return b < 0 ? -1 : a + b;
