@@ -6,18 +6,25 @@
 //   KB = 64   keys per block, two CTAs per SM (96 KB shared memory, 256 TMEM columns each): while
 //             one CTA waits on a load, a product or its softmax, the other keeps the SM busy
 //   KB = 128  keys per block, one CTA per SM, 3-stage rings and two O buffers
-// Per CTA, 192 threads:
-//   warp 0      TMA, two threads: lane 0 loads K tiles (KB keys) into a ring, lane 1 loads the
-//               item's Q tile and the V tiles into their own ring (fp16, 128B swizzle; a 64-column
-//               box per 64 head dims)
-//   warp 1      one thread issues S_j = Q K_j^T (M = 128, N = KB) into one of two TMEM S buffers,
-//               and O += P_j V_j with P_j read from tensor memory (the A operand of the TS form) and
-//               V_j from shared memory as an MN-major operand
+// Per CTA, 256 threads:
+//   warps 0, 7  TMA, a thread each: warp 0 loads K tiles (KB keys) into a ring, warp 7 the item's Q tile
+//               and the V tiles into their own ring (fp16, 128B swizzle; a 64-column box per 64 head
+//               dims)
+//   warp 1      one thread issues S_j = Q K_j^T (M = 128, N = KB) into one of two TMEM S buffers
+//   warp 6      one thread issues O += P_j V_j with P_j read from tensor memory (the A operand of the
+//               TS form) and V_j from shared memory as an MN-major operand
 //   warps 2..5  softmax, one query row per thread (TMEM lane = row): scale, causal and
 //               sequence-end mask, online softmax with a stale maximum (O is rescaled in TMEM
 //               only when a row's maximum grows by more than 2^8), P_j written back as packed fp16
 //               over the first KB / 2 columns of its own S buffer; at the end of an item O / l is
 //               stored as fp16.
+// Every role that waits has a warp of its own: a wait costs about 110 cycles even on a ready barrier and an
+// MMA about 70 to issue, so one thread issuing both products took 1,985 cycles per 64-key block, as
+// long as the block, and two loading threads of one warp hold each other up.  Packed 7B-width batches,
+// us, against five warps with one issuer and one loading warp (in brackets): 68 x 347 rows 144 (152), 23 x 1024
+// 219 (235), 5 x 4096 567 (616); head size 64, 5 x 4096 429 (537).  What is left at long sequences: the
+// tensor pipe, about 85% busy with two CTAs (S at N = 64 keys reads 192 bytes of shared memory a
+// cycle where 128 are to be had); at the query's lengths the Q, K and V latency at each item's start.
 // K is released as soon as its S product completes and V after its PV product; S/P is
 // double-buffered, so the softmax of block j overlaps S_{j+1} and PV_{j-1}.  S_{j+2} is issued
 // only once PV_j (the reader of P_j in the same columns) has completed.  Every mbarrier wait is
@@ -47,7 +54,7 @@ unsigned int read_clear_err_attn() {
 
 namespace fa {
 
-constexpr int BQ = 128, THREADS = 192;
+constexpr int BQ = 128, THREADS = 256;
 constexpr float STALE = 8.f;  // log2 units: P <= 2^8 before a rescale is forced
 
 template <int HD, int KB>
@@ -329,9 +336,10 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
   // uses K/V stage g % NST (phase (g / NST) & 1) and S/P buffer g & 1 (phase (g >> 1) & 1); item t
   // uses O buffer t % NO (phase (t / NO) & 1).
 
-  if (warp == 0) {
-    if (lane < 2) {
-      // ---------------- TMA producers: lane 0 K tiles; lane 1 Q and V tiles
+  if (warp == 0 || warp == 7) {
+    if (lane == 0) {
+      // ---------------- TMA producers: warp 0 K tiles; warp 7 Q and V tiles
+      const bool is_k = warp == 0;
       uint32_t g = 0, t = 0;
       bool ok = true;
       int4 nxt = fetch_item(blockIdx.x);
@@ -339,7 +347,7 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
         const Item cur = decode_item(nxt, item);
         nxt = fetch_item(item + gridDim.x);
         if (cur.nkv == 0) continue;
-        if (lane == 1) {
+        if (!is_k) {
           if (!mbar_wait(Q_EMPTY, (t & 1u) ^ 1u, abort_flag)) { ok = false; break; }
           mbar_expect_tx(Q_FULL, CF::Q_BYTES);
           for (int c = 0; c < HD / 64; ++c)
@@ -348,16 +356,16 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
         for (int j = 0; j < cur.nkv; ++j, ++g) {
           const int s = g % NST;
           const uint32_t ph = (g / NST) & 1u;
-          const int base = lane == 0 ? K_EMPTY : V_EMPTY;
+          const int base = is_k ? K_EMPTY : V_EMPTY;
           if (!mbar_wait(BAR(base, s), ph ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t full = BAR(lane == 0 ? K_FULL : V_FULL, s);
+          const uint32_t full = BAR(is_k ? K_FULL : V_FULL, s);
           mbar_expect_tx(full, CF::K_BYTES);
-          uint8_t* dst = (lane == 0 ? sK + s * CF::K_BYTES : sV + s * CF::V_BYTES);
+          uint8_t* dst = (is_k ? sK + s * CF::K_BYTES : sV + s * CF::V_BYTES);
           // prefix blocks from the prefix's [S_pre, d] K / V maps (rows past S_pre read as zero),
           // then the sequence's own rows of the qkv map
           const bool pre = j < np;
-          const CUtensorMap* map = pre ? (lane == 0 ? &tm_pk : &tm_pv) : &tm_kv;
-          const int col = (pre ? 0 : (lane == 0 ? d : 2 * d)) + cur.h * HD;
+          const CUtensorMap* map = pre ? (is_k ? &tm_pk : &tm_pv) : &tm_kv;
+          const int col = (pre ? 0 : (is_k ? d : 2 * d)) + cur.h * HD;
           const int row = pre ? j * KB : cur.seq0 + (j - np) * KB;
           for (int c = 0; c < HD / 64; ++c) tma_load_2d(smem_u32(dst + c * KB * 128), map, col + c * 64, row, full);
         }
@@ -366,54 +374,59 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
     }
   } else if (warp == 1) {
     if (lane == 0) {
-      // ---------------- MMA issuer
+      // ---------------- S issuer: S_g = Q K_g^T
+      const uint64_t qd0 = desc_kmajor(smem_u32(sQ)), kd0 = desc_kmajor(smem_u32(sK));
       uint32_t g = 0, t = 0;
       bool ok = true;
-      auto issue_s = [&](uint32_t gg) -> bool {
-        const int st = gg % NST, sb = gg & 1;
-        if (!mbar_wait(BAR(K_FULL, st), (gg / NST) & 1u, abort_flag)) return false;
-        // S/P buffer sb is free once PV_{gg-2}, the reader of P_{gg-2}, has completed
-        if (gg >= 2 && !mbar_wait(BAR(PV_DONE, sb), ((gg - 2) >> 1) & 1u, abort_flag)) return false;
-        fence_after();
-        const uint32_t kb = smem_u32(sK + st * CF::K_BYTES);
-        const uint32_t qb = smem_u32(sQ);
+      int4 nxt = fetch_item(blockIdx.x);
+      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+        const int nkv = decode_item(nxt, item).nkv;
+        nxt = fetch_item(item + gridDim.x);
+        if (nkv == 0) continue;
+        if (!mbar_wait(Q_FULL, t & 1u, abort_flag)) break;
+        for (int j = 0; j < nkv; ++j, ++g) {
+          const int st = g % NST, sb = g & 1;
+          if (!mbar_wait(BAR(K_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+          // S/P buffer sb is free once PV_{g-2}, the reader of P_{g-2}, has completed
+          if (g >= 2 && !mbar_wait(BAR(PV_DONE, sb), ((g - 2) >> 1) & 1u, abort_flag)) { ok = false; break; }
+          fence_after();
+          const uint64_t kd = kd0 + (uint32_t)(st * (CF::K_BYTES >> 4));
+          const uint32_t s_col = tmem + S_COL0 + (uint32_t)KB * sb;
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {  // 16 of the head dims per step
-          const uint32_t koff = (kk & 3) * 32;
-          umma(tmem + S_COL0 + (uint32_t)KB * sb, desc_kmajor(qb + (kk >> 2) * (BQ * 128) + koff),
-               desc_kmajor(kb + (kk >> 2) * (KB * 128) + koff), CF::IDESC_S, kk > 0);
+          for (int kk = 0; kk < HD / 16; ++kk)  // 16 of the head dims per step
+            umma(s_col, qd0 + (uint32_t)(((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
+                 kd + (uint32_t)(((kk >> 2) * (KB * 128) + (kk & 3) * 32) >> 4), CF::IDESC_S, kk > 0);
+          umma_commit(BAR(S_FULL, sb));
+          umma_commit(BAR(K_EMPTY, st));
         }
-        umma_commit(BAR(S_FULL, sb));
-        umma_commit(BAR(K_EMPTY, st));
-        return true;
-      };
+        if (!ok) break;
+        umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
+        ++t;
+      }
+    }
+  } else if (warp == 6) {
+    if (lane == 0) {
+      // ---------------- PV issuer: O += P_g V_g
+      const uint64_t vd0 = desc_mnmajor(smem_u32(sV), KB * 128);
+      uint32_t g = 0, t = 0;
+      bool ok = true;
       int4 nxt = fetch_item(blockIdx.x);
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
         const int nkv = decode_item(nxt, item).nkv;
         nxt = fetch_item(item + gridDim.x);
         if (nkv == 0) continue;
         const int ob = t % NO;
-        if (!mbar_wait(Q_FULL, t & 1u, abort_flag)) break;
-        fence_after();
-        if (!issue_s(g)) break;
         for (int j = 0; j < nkv; ++j, ++g) {
-          if (j + 1 < nkv) {
-            if (!issue_s(g + 1)) { ok = false; break; }
-          } else {
-            umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
-          }
           const int st = g % NST, sb = g & 1;
-          if (!mbar_wait(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
-          if (j == 0 && !mbar_wait(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
           if (!mbar_wait(BAR(V_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+          if (j == 0 && !mbar_wait(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
           fence_after();
-          const uint32_t vb = smem_u32(sV + st * CF::V_BYTES);
+          const uint64_t vd = vd0 + (uint32_t)(st * (CF::V_BYTES >> 4));
+          const uint32_t o_col = tmem + 128u * ob, p_col = tmem + S_COL0 + (uint32_t)KB * sb;
 #pragma unroll
-          for (int kk = 0; kk < KB / 16; ++kk) {  // 16 keys (8 TMEM columns of P) per step
-            const uint64_t bdesc = desc_mnmajor(vb + kk * 2048, KB * 128);
-            umma_ts(tmem + 128u * ob, tmem + S_COL0 + (uint32_t)KB * sb + 8u * kk, bdesc, CF::IDESC_O,
-                    (j > 0 || kk > 0) ? 1u : 0u);
-          }
+          for (int kk = 0; kk < KB / 16; ++kk)  // 16 keys (8 TMEM columns of P) per step
+            umma_ts(o_col, p_col + 8u * kk, vd + (uint32_t)(kk * (2048 >> 4)), CF::IDESC_O, (j > 0 || kk > 0) ? 1u : 0u);
           umma_commit(BAR(PV_DONE, sb));
           umma_commit(BAR(V_EMPTY, st));
         }
