@@ -392,6 +392,10 @@ __global__ void __launch_bounds__(THREADS, 1)
   // Rows: M_cap (host), or the device count ep.m_dev clamped to it (the rows the TMA map covers).
   const int M = ep.m_dev ? max(0, min(M_cap, *ep.m_dev)) : M_cap;
 
+  // The first K-block, as a value the compiler does not know: with a constant it peels the K loops and the
+  // products of 23,800 rows take 0.5% longer.
+  int kb0;
+  asm volatile("mov.s32 %0, 0;" : "=r"(kb0));
   const int mt = (M + TM - 1) / TM, nt = (N + BN - 1) / BN, kt = (K + BK - 1) / BK;
   const int n_tiles = ep.symmetric ? mt * (mt + 1) / 2 : mt * nt;
   auto coords = [&](int tile, int& m_blk, int& n_blk) {
@@ -410,7 +414,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       for (int u = u_first; u < n_tiles && ok; u += u_step) {
         int m_blk, n_blk;
         coords(u, m_blk, n_blk);
-        for (int k = 0; k < kt; ++k, ++it) {
+        for (int k = kb0; k < kt; ++k, ++it) {
           const int s = it % STAGES;
           const uint32_t round = it / STAGES;
           if (!mbar_wait(empty_bar(s), (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
@@ -442,7 +446,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!mbar_wait<true>(tempty_bar(b), (use & 1u) ^ 1u, abort_flag)) break;
         fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(b * ACC_COLS);
-        for (int k = 0; k < kt; ++k, ++it) {
+        for (int k = kb0; k < kt; ++k, ++it) {
           const int s = it % STAGES;
           const uint32_t round = it / STAGES;
           if (!mbar_wait(full_bar(s), round & 1u, abort_flag)) { ok = false; break; }
@@ -451,7 +455,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint64_t bd = smem_desc(smem_u32(sB + s * B_BYTES));
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)  // +32 bytes along K per step (encoded >> 4)
-            umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != 0 || kk != 0) ? 1u : 0u);
+            umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != kb0 || kk != 0) ? 1u : 0u);
           umma_commit_pair(empty_bar(s));
         }
         if (ok) umma_commit_pair(tfull_bar(b));
