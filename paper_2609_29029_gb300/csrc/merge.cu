@@ -422,15 +422,15 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   }
 }
 
-// Grid (kept slot, 512 columns, part), 64 threads of eight columns: the contextual tokens' means over the
-// slot's unselected rows, read once, group after group, in ascending token index within a group (the
-// target's own row and the tokens assigned to it): summed in fp32, divided by the group size and
-// stored as bf16.  Each CTA sorts the slot's tokens by group itself (a stable counting sort in shared
+// Grid (kept slot, 4096 columns, part), 256 threads of two groups of eight columns: the contextual tokens'
+// means over the slot's unselected rows, read once, group after group, in ascending token index within a
+// group (the target's own row and the tokens assigned to it): summed in fp32, divided by the group size
+// and stored as bf16.  Each CTA sorts the slot's tokens by group itself (a stable counting sort in shared
 // memory, about 2 us, which took a launch and member lists in HBM), so the rows' loads, MU rows ahead,
-// do not wait for group boundaries, and takes its part (1 / MP) of the groups: with all of them a
-// scheduler had 2 or 3 warps to hide the adds' latency with.  73 us at 400 tiles, 76 with MP = 1 and 76 for
-// the sort and the sums as two launches.
-constexpr int MT = 64, MCOLS = 8 * MT, MU = 16, MP = 2;
+// do not wait for group boundaries, and takes its part (1 / MP) of the groups.  A CTA reads whole 8 KB rows:
+// in 1 KB pieces by 16 CTAs a slot they came at 3.5 TB/s (400 tiles, about 95 kept: 63 us, 73 in pieces, 60 + 16
+// as two launches with a member at a time).
+constexpr int MT = 256, MCOLS = 16 * MT, MU = 4, MP = 8;
 template <typename XT>
 __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X, int n_v, int d,
                                                         const int* __restrict__ kept, const int* __restrict__ n_kept,
@@ -493,45 +493,57 @@ __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X
   if (c0 >= d) return;
   const int i0 = range[0], i1 = range[1];
   const XT* Xc = X + (size_t)kept[j] * n_v * d + c0;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  constexpr int GAP = 8 * MT;  // columns between a thread's two groups
+  const bool two = c0 + GAP < d;
+  float acc[2][8] = {};
   int cur = q_lo;
   auto flush = [&]() {
     const float inv = 1.f / (float)cnt[cur];
-    uint32_t w[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(acc[2 * e] * inv, acc[2 * e + 1] * inv);
-    *reinterpret_cast<uint4*>(ctx + (size_t)(co + cur) * d + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+    for (int v = 0; v < 2; ++v) {
+      uint32_t w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(acc[v][2 * e] * inv, acc[v][2 * e + 1] * inv);
+      if (v == 0 || two)
+        *reinterpret_cast<uint4*>(ctx + (size_t)(co + cur) * d + c0 + v * GAP) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
   };
-  constexpr int NR = sizeof(XT) == 2 ? 1 : 2;  // 16-byte loads per row
-  for (int i = i0; i < i1; i += MU / NR) {
-    uint4 raw[MU / NR][NR];
+  constexpr int NR = sizeof(XT) == 2 ? 1 : 2;  // 16-byte loads per group of a row
+  for (int i = i0; i < i1; i += MU) {
+    uint4 raw[MU][2][NR];
 #pragma unroll
-    for (int u = 0; u < MU / NR; ++u) {
+    for (int u = 0; u < MU; ++u) {
       const XT* row = Xc + (size_t)(memb[i + u] & 0xffffu) * d;
 #pragma unroll
-      for (int v = 0; v < NR; ++v) raw[u][v] = reinterpret_cast<const uint4*>(row)[v];
+      for (int v = 0; v < 2; ++v)
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (v == 0 || two) raw[u][v][r] = reinterpret_cast<const uint4*>(row + v * GAP)[r];
     }
 #pragma unroll
-    for (int u = 0; u < MU / NR; ++u) {
+    for (int u = 0; u < MU; ++u) {
       if (i + u >= i1) break;
       const int g = (int)(memb[i + u] >> 16);
       if (g != cur) {  // every group has its target: no group is empty
         flush();
         cur = g;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-      }
-      float x[8];
-      if constexpr (NR == 1) {
-        unpack_bf16x8(raw[u][0], x);
-      } else {
-        const uint32_t w[8] = {raw[u][0].x, raw[u][0].y, raw[u][0].z, raw[u][0].w,
-                               raw[u][1].x, raw[u][1].y, raw[u][1].z, raw[u][1].w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(w[e]);
+        for (int e = 0; e < 8; ++e) acc[0][e] = acc[1][e] = 0.f;
       }
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += x[e];
+      for (int v = 0; v < 2; ++v) {
+        float x[8];
+        if constexpr (NR == 1) {
+          unpack_bf16x8(raw[u][v][0], x);
+        } else {
+          const uint4 a = raw[u][v][0], b = raw[u][v][NR - 1];
+          const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(w[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[v][e] += x[e];
+      }
     }
   }
   flush();
