@@ -10,21 +10,22 @@
 //   warps 0, 7  TMA, a thread each: warp 0 loads K tiles (KB keys) into a ring, warp 7 the item's Q tile
 //               and the V tiles into their own ring (fp16, 128B swizzle; a 64-column box per 64 head
 //               dims)
-//   warp 1      one thread issues S_j = Q K_j^T (M = 128, N = KB) into one of two TMEM S buffers
-//   warp 6      one thread issues O += P_j V_j with P_j read from tensor memory (the A operand of the
+//   warp 1      issues S_j = Q K_j^T (M = 128, N = KB) into one of two TMEM S buffers
+//   warp 6      issues O += P_j V_j with P_j read from tensor memory (the A operand of the
 //               TS form) and V_j from shared memory as an MN-major operand
 //   warps 2..5  softmax, one query row per thread (TMEM lane = row): scale, causal and
 //               sequence-end mask, online softmax with a stale maximum (O is rescaled in TMEM
 //               only when a row's maximum grows by more than 2^8), P_j written back as packed fp16
 //               over the first KB / 2 columns of its own S buffer; at the end of an item O / l is
 //               stored as fp16.
-// Every role that waits has a warp of its own: a wait costs about 110 cycles even on a ready barrier and an
-// MMA about 70 to issue, so one thread issuing both products took 1,985 cycles per 64-key block, as
-// long as the block, and two loading threads of one warp hold each other up.  Packed 7B-width batches,
-// us, against five warps with one issuer and one loading warp (in brackets): 68 x 347 rows 144 (152), 23 x 1024
-// 219 (235), 5 x 4096 567 (616); head size 64, 5 x 4096 429 (537).  What is left at long sequences: the
-// tensor pipe, about 85% busy with two CTAs (S at N = 64 keys reads 192 bytes of shared memory a
-// cycle where 128 are to be had); at the query's lengths the Q, K and V latency at each item's start.
+// Every role that waits has a warp of its own: a wait costs about 110 cycles even on a ready barrier, so one
+// thread issuing both products took 1,985 cycles per 64-key block, as long as the block, and two loading
+// threads of one warp hold each other up.  The issuing warps run their loops with all lanes and issue under
+// elect_one().  Packed 7B-width batches, us, against one lane issuing from a branch of its own, and against
+// five warps with one issuer and one loading warp: 68 x 347 rows 138 : 144 : 152, 23 x 1024 204 : 219 : 235,
+// 5 x 4096 508 : 567 : 616; head size 64, 5 x 4096 394 : 429 : 537.  What is left at long sequences: the
+// tensor pipe (S at N = 64 keys reads 192 bytes of shared memory a cycle where 128 are to be had); at the
+// query's lengths the Q, K and V latency at each item's start.
 // K is released as soon as its S product completes and V after its PV product; S/P is
 // double-buffered, so the softmax of block j overlaps S_{j+1} and PV_{j-1}.  S_{j+2} is issued
 // only once PV_j (the reader of P_j in the same columns) has completed.  Every mbarrier wait is
@@ -127,6 +128,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   atomicOr(&g_err_attn, RIFT_EBIT_TIMEOUT);
   *abort_flag = 1;
   return false;
+}
+// The same wait by a whole warp, one answer for all its lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -274,7 +279,7 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
          P_FULL = S_FULL + 2, PV_DONE = P_FULL + 2, O_FULL = PV_DONE + 2, O_EMPTY = O_FULL + NO, N_BARS = O_EMPTY + NO };
   static_assert(N_BARS <= 32, "barrier slots");
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(Q_FULL, 1);
     mbar_init(Q_EMPTY, 1);
@@ -306,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(*tmem_slot);
   pdl_trigger();
   pdl_wait();
   const int n_items = min(n_entries, sched[n_entries].x) * H;  // entries in use (the schedule's count)
@@ -373,65 +378,73 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       // ---------------- S issuer: S_g = Q K_g^T
       const uint64_t qd0 = desc_kmajor(smem_u32(sQ)), kd0 = desc_kmajor(smem_u32(sK));
       uint32_t g = 0, t = 0;
       bool ok = true;
       int4 nxt = fetch_item(blockIdx.x);
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const int nkv = decode_item(nxt, item).nkv;
+        const int nkv = warp_uniform(decode_item(nxt, item).nkv);
         nxt = fetch_item(item + gridDim.x);
         if (nkv == 0) continue;
-        if (!mbar_wait(Q_FULL, t & 1u, abort_flag)) break;
+        if (!mbar_wait_warp(Q_FULL, t & 1u, abort_flag)) break;
         for (int j = 0; j < nkv; ++j, ++g) {
           const int st = g % NST, sb = g & 1;
-          if (!mbar_wait(BAR(K_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(BAR(K_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
           // S/P buffer sb is free once PV_{g-2}, the reader of P_{g-2}, has completed
-          if (g >= 2 && !mbar_wait(BAR(PV_DONE, sb), ((g - 2) >> 1) & 1u, abort_flag)) { ok = false; break; }
+          if (g >= 2 && !mbar_wait_warp(BAR(PV_DONE, sb), ((g - 2) >> 1) & 1u, abort_flag)) { ok = false; break; }
           fence_after();
           const uint64_t kd = kd0 + (uint32_t)(st * (CF::K_BYTES >> 4));
           const uint32_t s_col = tmem + S_COL0 + (uint32_t)KB * sb;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk)  // 16 of the head dims per step
-            umma(s_col, qd0 + (uint32_t)(((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
-                 kd + (uint32_t)(((kk >> 2) * (KB * 128) + (kk & 3) * 32) >> 4), CF::IDESC_S, kk > 0);
-          umma_commit(BAR(S_FULL, sb));
-          umma_commit(BAR(K_EMPTY, st));
+            for (int kk = 0; kk < HD / 16; ++kk)  // 16 of the head dims per step
+              umma(s_col, qd0 + (uint32_t)(((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
+                   kd + (uint32_t)(((kk >> 2) * (KB * 128) + (kk & 3) * 32) >> 4), CF::IDESC_S, kk > 0);
+            umma_commit(BAR(S_FULL, sb));
+            umma_commit(BAR(K_EMPTY, st));
+          }
+          __syncwarp();
         }
         if (!ok) break;
-        umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
+        if (elect_one()) umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
+        __syncwarp();
         ++t;
       }
     }
   } else if (warp == 6) {
-    if (lane == 0) {
+    {
       // ---------------- PV issuer: O += P_g V_g
       const uint64_t vd0 = desc_mnmajor(smem_u32(sV), KB * 128);
       uint32_t g = 0, t = 0;
       bool ok = true;
       int4 nxt = fetch_item(blockIdx.x);
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const int nkv = decode_item(nxt, item).nkv;
+        const int nkv = warp_uniform(decode_item(nxt, item).nkv);
         nxt = fetch_item(item + gridDim.x);
         if (nkv == 0) continue;
         const int ob = t % NO;
         for (int j = 0; j < nkv; ++j, ++g) {
           const int st = g % NST, sb = g & 1;
-          if (!mbar_wait(BAR(V_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
-          if (j == 0 && !mbar_wait(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          if (!mbar_wait(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(BAR(V_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+          if (j == 0 && !mbar_wait_warp(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
           fence_after();
           const uint64_t vd = vd0 + (uint32_t)(st * (CF::V_BYTES >> 4));
           const uint32_t o_col = tmem + 128u * ob, p_col = tmem + S_COL0 + (uint32_t)KB * sb;
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < KB / 16; ++kk)  // 16 keys (8 TMEM columns of P) per step
-            umma_ts(o_col, p_col + 8u * kk, vd + (uint32_t)(kk * (2048 >> 4)), CF::IDESC_O, (j > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(BAR(PV_DONE, sb));
-          umma_commit(BAR(V_EMPTY, st));
+            for (int kk = 0; kk < KB / 16; ++kk)  // 16 keys (8 TMEM columns of P) per step
+              umma_ts(o_col, p_col + 8u * kk, vd + (uint32_t)(kk * (2048 >> 4)), CF::IDESC_O, (j > 0 || kk > 0) ? 1u : 0u);
+            umma_commit(BAR(PV_DONE, sb));
+            umma_commit(BAR(V_EMPTY, st));
+          }
+          __syncwarp();
         }
         if (!ok) break;
-        umma_commit(BAR(O_FULL, ob));
+        if (elect_one()) umma_commit(BAR(O_FULL, ob));
+        __syncwarp();
         ++t;
       }
     }

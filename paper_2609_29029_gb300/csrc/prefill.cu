@@ -229,7 +229,7 @@ int launch_prefill(const rift_model& m, void* hidden, int T, const int* T_dev, c
   // With few rows the kernels after the first are launched as programmatic dependents of the kernel before
   // them: launch latencies are a good part of the time (two layers over one 131-row tile 373 -> 316 us
   // with the setup in one launch).  At 28,000 rows the early launches cost more than they hide: a
-  // 32-layer query 256.5 ms with them, 254.1 without (start 255).
+  // 32-layer query 256.5 ms with them, 254.1 without.
   const bool pdl = T <= 8192;
   prof_begin(RIFT_PROF_ROPE, st);
   PrefillSetup ps = {rope, max_len, half, rope_freq(m), qkv, 3 * d, T_dev};

@@ -57,6 +57,22 @@ inline cudaError_t raise_cluster_limit(std::atomic<unsigned long long>& done, K*
   return e;
 }
 
+// A warp's value known to be the same in all lanes: it can be held in uniform registers.
+template <typename T>
+__device__ __forceinline__ T warp_uniform(T v) {
+  return __shfl_sync(0xffffffffu, v, 0);
+}
+
+// True in one lane of a converged warp, the same one each time.  A warp whose lanes all run a loop of
+// tcgen05 instructions and issue them under elect_one() pays ~15 cycles per instruction; one lane of its
+// own branch pays ~70, because its operands (descriptors, addresses) have to be moved into uniform registers
+// for each instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 // Programmatic dependent launch.  A kernel launched with `pdl` set (launch_ex) may begin while
 // the kernel before it in the stream is still running: each of its threads calls pdl_wait()
 // before its first access to memory that earlier kernels write or read (constant weights
