@@ -7,7 +7,7 @@
 //             one CTA waits on a load, a product or its softmax, the other keeps the SM busy
 //   KB = 128  keys per block, one CTA per SM, 3-stage rings and two O buffers
 // Per CTA, 256 threads:
-//   warps 0, 7  TMA, a thread each: warp 0 loads K tiles (KB keys) into a ring, warp 7 the item's Q tile
+//   warps 0, 7  TMA: warp 0 loads K tiles (KB keys) into a ring, warp 7 the item's Q tile
 //               and the V tiles into their own ring (fp16, 128B swizzle; a 64-column box per 64 head
 //               dims)
 //   warp 1      issues S_j = Q K_j^T (M = 128, N = KB) into one of two TMEM S buffers
@@ -20,10 +20,10 @@
 //               stored as fp16.
 // Every role that waits has a warp of its own: a wait costs about 110 cycles even on a ready barrier, so one
 // thread issuing both products took 1,985 cycles per 64-key block, as long as the block, and two loading
-// threads of one warp hold each other up.  The issuing warps run their loops with all lanes and issue under
-// elect_one().  Packed 7B-width batches, us, against one lane issuing from a branch of its own, and against
-// five warps with one issuer and one loading warp: 68 x 347 rows 138 : 144 : 152, 23 x 1024 204 : 219 : 235,
-// 5 x 4096 508 : 567 : 616; head size 64, 5 x 4096 394 : 429 : 537.  What is left at long sequences: the
+// threads of one warp hold each other up.  The loading and issuing warps run their loops with all
+// lanes and issue under elect_one().  Packed 7B-width batches, us, against one lane issuing from a branch of its own, and against
+// five warps with one issuer and one loading warp: 68 x 347 rows 136 : 144 : 152, 23 x 1024 202 : 219 : 235,
+// 5 x 4096 508-518 : 567 : 616; head size 64, 5 x 4096 383 : 429 : 537.  What is left at long sequences: the
 // tensor pipe (S at N = 64 keys reads 192 bytes of shared memory a cycle where 128 are to be had); at the
 // query's lengths the Q, K and V latency at each item's start.
 // K is released as soon as its S product completes and V after its PV product; S/P is
@@ -342,29 +342,34 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
   // uses O buffer t % NO (phase (t / NO) & 1).
 
   if (warp == 0 || warp == 7) {
-    if (lane == 0) {
+    {
       // ---------------- TMA producers: warp 0 K tiles; warp 7 Q and V tiles
       const bool is_k = warp == 0;
       uint32_t g = 0, t = 0;
       bool ok = true;
       int4 nxt = fetch_item(blockIdx.x);
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const Item cur = decode_item(nxt, item);
+        Item cur = decode_item(nxt, item);
+        cur.seq0 = warp_uniform(cur.seq0);
+        cur.q0 = warp_uniform(cur.q0);
+        cur.nkv = warp_uniform(cur.nkv);
         nxt = fetch_item(item + gridDim.x);
         if (cur.nkv == 0) continue;
         if (!is_k) {
-          if (!mbar_wait(Q_EMPTY, (t & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          mbar_expect_tx(Q_FULL, CF::Q_BYTES);
-          for (int c = 0; c < HD / 64; ++c)
-            tma_load_2d(smem_u32(sQ + c * BQ * 128), &tm_q, cur.h * HD + c * 64, cur.seq0 + cur.q0, Q_FULL);
+          if (!mbar_wait_warp(Q_EMPTY, (t & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          if (elect_one()) {
+            mbar_expect_tx(Q_FULL, CF::Q_BYTES);
+            for (int c = 0; c < HD / 64; ++c)
+              tma_load_2d(smem_u32(sQ + c * BQ * 128), &tm_q, cur.h * HD + c * 64, cur.seq0 + cur.q0, Q_FULL);
+          }
+          __syncwarp();
         }
         for (int j = 0; j < cur.nkv; ++j, ++g) {
           const int s = g % NST;
           const uint32_t ph = (g / NST) & 1u;
           const int base = is_k ? K_EMPTY : V_EMPTY;
-          if (!mbar_wait(BAR(base, s), ph ^ 1u, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(BAR(base, s), ph ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t full = BAR(is_k ? K_FULL : V_FULL, s);
-          mbar_expect_tx(full, CF::K_BYTES);
           uint8_t* dst = (is_k ? sK + s * CF::K_BYTES : sV + s * CF::V_BYTES);
           // prefix blocks from the prefix's [S_pre, d] K / V maps (rows past S_pre read as zero),
           // then the sequence's own rows of the qkv map
@@ -372,7 +377,11 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
           const CUtensorMap* map = pre ? (is_k ? &tm_pk : &tm_pv) : &tm_kv;
           const int col = (pre ? 0 : (is_k ? d : 2 * d)) + cur.h * HD;
           const int row = pre ? j * KB : cur.seq0 + (j - np) * KB;
-          for (int c = 0; c < HD / 64; ++c) tma_load_2d(smem_u32(dst + c * KB * 128), map, col + c * 64, row, full);
+          if (elect_one()) {
+            mbar_expect_tx(full, CF::K_BYTES);
+            for (int c = 0; c < HD / 64; ++c) tma_load_2d(smem_u32(dst + c * KB * 128), map, col + c * 64, row, full);
+          }
+          __syncwarp();
         }
         ++t;
       }

@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
   const int k0 = kt * rank / S, k1 = kt * (rank + 1) / S;
 
   if (warp == 0) {
-    if (lane == 0 && mv > 0) {
+    if (mv > 0) {
       // ---------------- TMA producer: a weight tile and the activation tile per K-block
       auto load_w = [&](int s, int k) {
         tma_load_2d(smem0 + s * stage_bytes, &tmW, kblock(ep.kmap_b, ep.kmap_d, k) * BK, n0, full_bar(s));
@@ -688,22 +688,27 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
         tma_load_2d(smem0 + s * stage_bytes + ck::W_BYTES, &tmX, kblock(ep.kmap_a, ep.kmap_d, k) * BK, m0, full_bar(s));
       };
       const int n_pre = w_const && !ep.m_dev ? min(stages, k1 - k0) : 0;
-      for (int j = 0; j < n_pre; ++j) {
-        mbar_expect_tx(full_bar(j), stage_bytes);
-        load_w(j, k0 + j);
+      if (elect_one()) {
+        for (int j = 0; j < n_pre; ++j) {
+          mbar_expect_tx(full_bar(j), stage_bytes);
+          load_w(j, k0 + j);
+        }
       }
+      __syncwarp();
       pdl_wait();
       int it = 0;
       for (int k = k0; k < k1; ++k, ++it) {
         const int s = it % stages;
-        if (it < n_pre) {  // the weight tile is on its way (first round: the stage is free)
+        // (it < n_pre: the weight tile is on its way, and in the first round the stage is free)
+        if (it >= n_pre && !mbar_wait_warp(empty_bar(s), ((it / stages) & 1u) ^ 1u, abort_flag)) break;
+        if (elect_one()) {
+          if (it >= n_pre) {
+            mbar_expect_tx(full_bar(s), stage_bytes);
+            load_w(s, k);
+          }
           load_x(s, k);
-          continue;
         }
-        if (!mbar_wait(empty_bar(s), ((it / stages) & 1u) ^ 1u, abort_flag)) break;
-        mbar_expect_tx(full_bar(s), stage_bytes);
-        load_w(s, k);
-        load_x(s, k);
+        __syncwarp();
       }
       for (int j = 1; j <= stages && it - j >= 0; ++j) {  // no copy left in flight (bounded)
         const int i2 = it - j;
