@@ -142,8 +142,9 @@ __global__ void __launch_bounds__(1024) merge_plan_kernel(const int* __restrict_
 // Grid (kept slot, y): rest[j][0 .. R) = the unselected tokens in ascending index (written by y = 0),
 // the targets (written to ctx_target) and their norms (tnorm, fp64 from a float-float sum of
 // squares), one target per warp: the warps of the TY CTAs take targets y * 8 + warp, + TY * 8, ...
-// The norm is a serial float-float chain, so the targets are spread over many warps (400 tiles, about 95
-// kept, 45 targets a slot: 19 us, 73 with one CTA per slot).
+// The norm is a serial float-float chain, so the targets are spread over many warps, and a row is read
+// once for its norm and its copy (400 tiles, about 95 kept, 45 targets a slot: 16 us; 20 with the copy
+// in a loop of its own, 73 with one CTA per slot).
 constexpr int TY = 8;
 template <typename XT>
 __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict__ X, int n_v, int d,
@@ -192,29 +193,57 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int q = y * 8 + warp; q < m; q += TY * 8) {
     const int t = rj[q * step];
-    const double nn = ff_dot(Xt + (size_t)t * d, Xt + (size_t)t * d, d, lane);
+    const XT* tr = Xt + (size_t)t * d;
+    // the row's norm and, for the tensor-core screening (bf16 tokens), its copy, in one pass of eight
+    // 16-byte loads ahead
+    constexpr int U = sizeof(XT) == 2 ? 8 : 4;
+    uint16_t* copy = trow && co + q < max_ctx ? trow + (size_t)(co + q) * d : nullptr;
+    float hi = 0.f, lo = 0.f;
+    for (int k0 = lane * 8; k0 < d; k0 += U * 256) {
+      uint4 raw[U][sizeof(XT) / 2];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k0 + u * 256 < d)
+#pragma unroll
+          for (int r = 0; r < (int)sizeof(XT) / 2; ++r)
+            raw[u][r] = reinterpret_cast<const uint4*>(tr + k0 + u * 256)[r];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k0 + u * 256 < d) {
+          float x[8];
+          if constexpr (sizeof(XT) == 2) {
+            if (copy) *reinterpret_cast<uint4*>(copy + k0 + u * 256) = raw[u][0];
+            unpack_bf16x8(raw[u][0], x);
+          } else {
+            const uint4 a = raw[u][0], b = raw[u][sizeof(XT) / 2 - 1];
+            const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(w[e]);
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) ff_step(x[e], x[e], hi, lo);
+        }
+    }
+    ff_warp_sum(hi, lo);
+    const double nn = (double)hi + (double)lo;
     if (co + q >= max_ctx) continue;
     if (lane == 0) {
       ctx_target[co + q] = t;
       tnorm[co + q] = sqrt(nn);
       if (tinv) tinv[co + q] = nn > 0.0 ? (float)(1.0 / sqrt(nn)) : 0.f;  // a zero target has similarity 0
     }
-    if (trow) {  // the target's row, for the tensor-core screening (bf16 tokens only)
-      const uint4* src = reinterpret_cast<const uint4*>(Xt + (size_t)t * d);
-      uint4* dst = reinterpret_cast<uint4*>(trow + (size_t)(co + q) * d);
-      for (int c = lane; c < d / 8; c += 32) dst[c] = src[c];
-    }
   }
 }
 
-// Grid (blocks of 64 unselected positions, kept slot), 4 warps: assign[j][a] = the screened target where
+// Grid (blocks of 64 unselected positions, kept slot), 8 warps: assign[j][a] = the screened target where
 // the screening was clear (cand[j][a].y < 0); the others are listed and the warps take them in turn: the
 // better of the two candidates at ~fp64 accuracy, x.t1 / ||t1|| vs x.t2 / ||t2|| from float-float dot
 // products (ties to the lower target).  The lanes' pairs are summed as pairs too: two double
-// operations retire a cycle on an SM, so a shuffle sum in fp64 costs more than the dot product.  28 us
-// at 400 tiles, against 111 with a second look at every token.
+// operations retire a cycle on an SM, so a shuffle sum in fp64 costs more than the dot product.  23 us
+// at 400 tiles (28 with four warps, which take two turns), against 111 with a second look at every token.
 // Targets keep their own group.
-__global__ void __launch_bounds__(128) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
+constexpr int DT = 256;
+__global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
                                                            const int* __restrict__ kept,
                                                            const int* __restrict__ n_kept,
                                                            const int* __restrict__ sel_off,
@@ -248,7 +277,7 @@ __global__ void __launch_bounds__(128) merge_decide_kernel(const uint16_t* __res
   }
   __syncthreads();
   const uint16_t* Xt = X + (size_t)kept[j] * n_v * d;
-  for (int i = warp; i < n_open; i += 4) {
+  for (int i = warp; i < n_open; i += DT / 32) {
     const int4 o = open[i];
     const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + o.x] * d;
     const uint16_t* t1 = Xt + (size_t)ctx_target[co + o.y] * d;
@@ -425,12 +454,12 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
 // Grid (kept slot, 4096 columns, part), 256 threads of two groups of eight columns: the contextual tokens'
 // means over the slot's unselected rows, read once, group after group, in ascending token index within a
 // group (the target's own row and the tokens assigned to it): summed in fp32, divided by the group size
-// and stored as bf16.  Each CTA sorts the slot's tokens by group itself (a stable counting sort in shared
-// memory, about 2 us, which took a launch and member lists in HBM), so the rows' loads, MU rows ahead,
-// do not wait for group boundaries, and takes its part (1 / MP) of the groups.  A CTA reads whole 8 KB rows:
-// in 1 KB pieces by 16 CTAs a slot they came at 3.5 TB/s (400 tiles, about 95 kept: 63 us, 73 in pieces, 60 + 16
-// as two launches with a member at a time).
-constexpr int MT = 256, MCOLS = 16 * MT, MU = 4, MP = 8;
+// and stored as bf16.  Each CTA takes its part (1 / MP) of the groups and sorts their tokens itself, a warp
+// per group over the slot's groups in shared memory, so the rows' loads, MU rows ahead, do not wait for
+// group boundaries.  A CTA reads whole 8 KB rows.  400 tiles, about 95 kept: 46 us; 61 with the slot's whole
+// order placed by one warp and eight parts, which left a tile of few selected tokens to long CTAs (56 with the
+// order alone, 48 in 16 parts); 73 in 1 KB pieces; 60 + 16 as two launches with a member at a time.
+constexpr int MT = 256, MCOLS = 16 * MT, MU = 4, MP = 12;
 template <typename XT>
 __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X, int n_v, int d,
                                                         const int* __restrict__ kept, const int* __restrict__ n_kept,
@@ -438,9 +467,9 @@ __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X
                                                         const int* __restrict__ ctx_off, int max_ctx,
                                                         const int* __restrict__ rest, const int* __restrict__ assign,
                                                         uint16_t* __restrict__ ctx) {
-  __shared__ uint16_t grp[RIFT_MAX_NV];        // group of unselected token a
-  __shared__ uint32_t memb[RIFT_MAX_NV + MU];  // sorted: group << 16 | token index
-  __shared__ int cnt[RIFT_MAX_NV + 1], at[RIFT_MAX_NV + 1];  // group sizes; each group's next place
+  __shared__ uint16_t grp[RIFT_MAX_NV], tok[RIFT_MAX_NV];  // group and token index of unselected token a
+  __shared__ uint32_t memb[RIFT_MAX_NV + MU];  // this part's members, sorted: group << 16 | token index
+  __shared__ int cnt[RIFT_MAX_NV + 1], at[RIFT_MAX_NV + 1];  // group sizes; each group's first place
   pdl_trigger();
   pdl_wait();
   const int j = blockIdx.x, c0 = blockIdx.y * MCOLS + threadIdx.x * 8, lane = threadIdx.x & 31;
@@ -459,39 +488,34 @@ __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X
       if (g < 0 || g >= m) g = 0;  // an unassigned token (no finite similarity) joins the first group
     }
     grp[a] = (uint16_t)g;
+    tok[a] = (uint16_t)rj[a];
     atomicAdd(&cnt[g], 1);
   }
   __syncthreads();
-  __shared__ int range[2];
   if (threadIdx.x < 32) {
     int base = 0;
-    for (int q0 = 0; q0 < m; q0 += 32) {  // exclusive prefix sum of the group sizes
-      const int v = q0 + lane < m ? cnt[q0 + lane] : 0, inc = warp_incl_scan(v);
-      if (q0 + lane < m) at[q0 + lane] = base + inc - v;
+    for (int q0 = q_lo; q0 < q_hi; q0 += 32) {  // exclusive prefix sum of this part's group sizes
+      const int v = q0 + lane < q_hi ? cnt[q0 + lane] : 0, inc = warp_incl_scan(v);
+      if (q0 + lane < q_hi) at[q0 + lane] = base + inc - v;
       base += __shfl_sync(0xffffffffu, inc, 31);
     }
-    __syncwarp();
-    if (lane == 0) {
-      range[0] = at[q_lo];
-      range[1] = q_hi < m ? at[q_hi] : R;
-    }
-    __syncwarp();
-    // placement in token order, 32 tokens at a time: a token's place is its group's next one plus the
-    // number of lower lanes of the same group
-    for (int a0 = 0; a0 < R; a0 += 32) {
-      const int a = a0 + lane;
-      const int g = a < R ? grp[a] : -1 - lane;  // idle lanes match no one
-      const unsigned same = __match_any_sync(0xffffffffu, g);
-      if (a < R) memb[at[g] + __popc(same & ((1u << lane) - 1u))] = ((uint32_t)g << 16) | (uint32_t)rj[a];
-      __syncwarp();
-      if (a < R && (same >> lane) == 1u) at[g] += __popc(same);  // the group's highest lane
-      __syncwarp();
-    }
-    if (lane < MU) memb[R + lane] = memb[R - 1];  // a step past the end loads a row again
+    if (lane == 0) at[q_hi] = base;
   }
   __syncthreads();
+  // placement in token order, a warp per group, 32 tokens at a time
+  for (int q = q_lo + (int)(threadIdx.x >> 5); q < q_hi; q += MT / 32) {
+    int base = at[q];
+    for (int a0 = 0; a0 < R; a0 += 32) {
+      const bool in = a0 + lane < R && grp[a0 + lane] == q;
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (in) memb[base + __popc(b & ((1u << lane) - 1u))] = ((uint32_t)q << 16) | tok[a0 + lane];
+      base += __popc(b);
+    }
+  }
+  if (threadIdx.x < MU) memb[at[q_hi] + threadIdx.x] = tok[0];  // a step past the end loads a row all the same
+  __syncthreads();
   if (c0 >= d) return;
-  const int i0 = range[0], i1 = range[1];
+  const int i1 = at[q_hi];
   const XT* Xc = X + (size_t)kept[j] * n_v * d + c0;
   constexpr int GAP = 8 * MT;  // columns between a thread's two groups
   const bool two = c0 + GAP < d;
@@ -509,7 +533,7 @@ __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X
     }
   };
   constexpr int NR = sizeof(XT) == 2 ? 1 : 2;  // 16-byte loads per group of a row
-  for (int i = i0; i < i1; i += MU) {
+  for (int i = 0; i < i1; i += MU) {
     uint4 raw[MU][2][NR];
 #pragma unroll
     for (int u = 0; u < MU; ++u) {
@@ -588,7 +612,7 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
       // come from the tensor cores, the choice between them where they are close from float-float sums
       if (max_ctx > 0)
         ok = ok && launch_merge_screen(x, N, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, ctx, tinv, rest, cand, st) == 0;
-      ok = ok && launch_ex(merge_decide_kernel, dim3((n_v + 63) / 64, N), dim3(128), 0, st, true, x, n_v, d, kept,
+      ok = ok && launch_ex(merge_decide_kernel, dim3((n_v + 63) / 64, N), dim3(DT), 0, st, true, x, n_v, d, kept,
                            n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
                            (const double*)tnorm, (const int2*)cand, assign) == cudaSuccess;
     } else {
