@@ -5,7 +5,7 @@
 // k, fp32 residual add, SwiGLU over 16-column gate/up groups).  Two kernels:
 //
 // gemm_tc_kernel (many rows: the prefill of a scene): persistent and warp-specialised on SM pairs
-// (2-CTA clusters, 256 x 256 tiles), 192 threads per CTA:
+// (2-CTA clusters, 256 x 256 tiles, or 256 x 192: tile_width), 192 threads per CTA:
 //   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 6-stage shared-memory ring
 //   warp 1      allocates 512 TMEM columns; the even CTA's issues tcgen05.mma (cta_group::2, M = 256,
 //               N = 256, K = 16) into one of two 256-column fp32 accumulators and commits to
@@ -46,7 +46,7 @@ unsigned int read_clear_err_gemm() {
 
 namespace tc {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 6;
+constexpr int BM = 128, BN = 256, NARROW_BN = 192, BK = 64, STAGES = 6;
 constexpr int A_BYTES = BM * BK * 2;  // 16 KB
 constexpr int THREADS = 192;
 // Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A fp16 (bits
@@ -346,18 +346,31 @@ __device__ __forceinline__ int kblock(int mode, int D, int k) {
   return mode == 1 ? (k < D ? k : k - D) : mode == 2 ? (k < 2 * D ? k : k - 2 * D) : k;
 }
 
-// 2-CTA clusters on an SM pair, 256 x 256 tiles (cta_group::2): each SM stages 128 rows of A and 128
-// of the 256 B rows per k-block, half the B traffic of one SM per tile row, and the even CTA
-// issues the M = 256 MMAs into both SMs' tensor memory.
+// Width of the SM pairs' tiles: NARROW_BN where that takes no more waves of tiles than BN and there is
+// more than one.  The narrower tiles' K-blocks take 0.89-0.92 of the time (not 0.75: they are bound by the
+// supply from L2, ~14 TB/s), so the width pays where the last wave would leave SMs idle and nowhere else.
+// us, 256 against 192: W_o at 1,500 rows (2 waves each) 57 : 53, at 2,448 (3) 78 : 70, W_down 119 : 107 and
+// 179 : 160, gate/up at 203 (2) 70 : 60; at 3,000 rows (3 waves, 4) W_o 78 : 88, W_down 182 : 213.  In one wave
+// W_o at 600 rows takes 35 both ways.
+__device__ __forceinline__ int tile_width(int mt, int N, int pairs) {
+  const int wide = (mt * ((N + BN - 1) / BN) + pairs - 1) / pairs;
+  const int narrow = (mt * ((N + NARROW_BN - 1) / NARROW_BN) + pairs - 1) / pairs;
+  return wide > 1 && narrow <= wide ? NARROW_BN : BN;
+}
+
+// 2-CTA clusters on an SM pair, 256 x 256 tiles (cta_group::2; 256 x 192 by tile_width): each SM stages 128
+// rows of A and half of the tile's B rows per k-block, half the B traffic of one SM per tile row, and
+// the even CTA issues the M = 256 MMAs into both SMs' tensor memory.  tmN: the B map with boxes of the
+// narrower tile's half.
 template <int EPI>
 __global__ void __launch_bounds__(THREADS, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M_cap,
-                   int N, int K, void* C, const EpiParams ep, int group_m) {
+    gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                   const __grid_constant__ CUtensorMap tmN, int M_cap, int N, int K, void* C, const EpiParams ep,
+                   int group_m) {
   constexpr int TM = 2 * BM;      // rows of a tile (both CTAs of the pair)
   constexpr int B_ROWS = BN / 2;  // B rows staged by this CTA
   constexpr int B_BYTES = B_ROWS * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr int ACC_COLS = BN, TMEM_COLS = 2 * ACC_COLS;
-  constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -406,7 +419,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   // products of 23,800 rows take 0.5% longer.
   int kb0;
   asm volatile("mov.s32 %0, 0;" : "=r"(kb0));
-  const int mt = (M + TM - 1) / TM, nt = (N + BN - 1) / BN, kt = (K + BK - 1) / BK;
+  const int mt = (M + TM - 1) / TM, kt = (K + BK - 1) / BK;
+  int bn = BN;  // the RoPE epilogue wants whole heads in a tile, the symmetric product square tiles
+  if constexpr (EPI != EPI_QKV_ROPE)
+    if (!ep.symmetric) bn = tile_width(mt, N, (int)(gridDim.x >> 1));
+  const int nt = (N + bn - 1) / bn;
   const int n_tiles = ep.symmetric ? mt * (mt + 1) / 2 : mt * nt;
   auto coords = [&](int tile, int& m_blk, int& n_blk) {
     if (ep.symmetric) tri_coords(tile, mt, m_blk, n_blk);
@@ -429,11 +446,11 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t round = it / STAGES;
           if (!mbar_wait(empty_bar(s), (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t fb = mapa_shared(full_bar(s), 0);
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + bn * BK * 2);
           tma_load_2d_pair(smem_u32(sA + s * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k) * BK,
                            m_blk * TM + (int)rank * BM, fb);
-          tma_load_2d_pair(smem_u32(sB + s * B_BYTES), &tmB, kblock(ep.kmap_b, ep.kmap_d, k) * BK,
-                           n_blk * BN + (int)rank * B_ROWS, fb);
+          tma_load_2d_pair(smem_u32(sB + s * B_BYTES), EPI == EPI_QKV_ROPE || bn == BN ? &tmB : &tmN,
+                           kblock(ep.kmap_b, ep.kmap_d, k) * BK, n_blk * bn + (int)rank * (bn >> 1), fb);
         }
       }
       // Before leaving, make sure no copy this thread issued is still in flight (bounded): the
@@ -450,6 +467,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       // ---------------- MMA issuer (the even CTA only)
       int it = 0, tl = 0;
       bool ok = true;
+      const uint32_t idesc = (1u << 4) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
       for (int u = u_first; u < n_tiles && ok; u += u_step, ++tl) {
         const int b = tl & 1;
         const uint32_t use = tl >> 1;
@@ -466,7 +484,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)  // +32 bytes along K per step (encoded >> 4)
-              umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, IDESC_T, (k != kb0 || kk != 0) ? 1u : 0u);
+              umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, (k != kb0 || kk != 0) ? 1u : 0u);
             umma_commit_pair(empty_bar(s));
           }
           __syncwarp();
@@ -521,10 +539,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       } else {
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = 0; c < bn; c += 32) {
           uint32_t r[32];
           tmem_ld32(taddr + c, r);
-          if (row < M) epilogue_chunk<EPI>(r, row, n_blk * BN + c, N, C, ep.out_scale);
+          if (row < M) epilogue_chunk<EPI>(r, row, n_blk * bn + c, N, C, ep.out_scale);
           if constexpr (EPI == EPI_STORE_F32) {
             // symmetric product: the off-diagonal tile also fills its mirror (a warp's lanes hold
             // consecutive rows, so each transposed store is 32 consecutive floats)
@@ -1146,12 +1164,12 @@ static int band_group(int M, int N, int K, int tm, int tn, int lo, int hi) {
   return n_major ? -g : g;
 }
 
-// The paired kernel (2-CTA clusters, 256 x 256 tiles), persistent over as many clusters as can be
-// resident at once.  b: the B map with 128-row boxes.  Returns -1 if no cluster can be resident
-// (the caller then takes the cluster split-K kernel).
+// The paired kernel (2-CTA clusters), persistent over as many clusters as can be resident at once.
+// b, bn: the B map with boxes of half a wide and half a narrow tile.  Returns -1 if no cluster can be
+// resident (the caller then takes the cluster split-K kernel).
 template <int EPI>
-static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, void* C, const EpiParams& ep,
-                       cudaStream_t st, bool pdl) {
+static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& bn, int M, int N, int K, void* C,
+                       const EpiParams& ep, cudaStream_t st, bool pdl) {
   constexpr size_t smem = (size_t)STAGES * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
   auto kern = gemm_tc_kernel<EPI>;
   cudaLaunchAttribute attr[1];
@@ -1189,7 +1207,7 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, int M, int N,
   const int units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
   const int clusters = units < max_clusters ? units : max_clusters;
   const int group_m = band_group(M, N, K, 2 * BM, BN, 4, 32);
-  return launch_cluster_ex(kern, dim3(2 * clusters), dim3(THREADS), smem, st, pdl, 2, a, b, M, N, K, C, ep, group_m) ==
+  return launch_cluster_ex(kern, dim3(2 * clusters), dim3(THREADS), smem, st, pdl, 2, a, b, bn, M, N, K, C, ep, group_m) ==
                  cudaSuccess
              ? 0
              : 1;
@@ -1282,20 +1300,23 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   // beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
   // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777
   // (S = 1) 42.0 : 35.4; W_down 53.9 : 63.7 and 78.1 : 65.8; QKV at 131 rows 27.0 : 31.1, at 256
-  // (S = 1) 40.8 : 31.1; gate/up 46.8 : 57.8 and 75.6 : 57.8.
+  // (S = 1) 40.8 : 31.1; gate/up 46.8 : 57.8 and 75.6 : 57.8 (wide tiles; the pairs' narrow ones, 14%
+  // less, leave the order as it is).
   // A device count of the logits' rows (sequences) is usually a fraction of its capacity, and
   // row tiles past the count cost nothing there.
   if (M <= ck::MAX_BN || plan.S >= 2 || (epi == EPI_STORE_F32 && ep.m_dev && M < 1024))
     return launch_ck_epi(A, B, Ks, M, N, K, epi, C, ep, st, plan, pdl, b_const ? 1 : 0);
-  CUtensorMap ma, mb;
-  if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2)) return 1;
+  CUtensorMap ma, mb, mn;
+  if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2) ||
+      !make_map(&mn, B, Ks, (uint64_t)N, NARROW_BN / 2))
+    return 1;
   int r = -1;
   switch (epi) {
-    case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, M, N, K, C, ep, st, pdl); break;
-    case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb, M, N, K, C, ep, st, pdl); break;
-    case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb, M, N, K, C, ep, st, pdl); break;
-    case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb, M, N, K, C, ep, st, pdl); break;
-    case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb, M, N, K, C, ep, st, pdl); break;
+    case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;
+    case EPI_RESID_F32: r = launch_pair<EPI_RESID_F32>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;
+    case EPI_SWIGLU: r = launch_pair<EPI_SWIGLU>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;
+    case EPI_QKV_ROPE: r = launch_pair<EPI_QKV_ROPE>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;
+    case EPI_STORE_F32: r = launch_pair<EPI_STORE_F32>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;
     default: return 1;
   }
   if (r >= 0) return r;
