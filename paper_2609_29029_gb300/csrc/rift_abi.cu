@@ -234,9 +234,9 @@ rift_status rift_select_budgeted_tokens(const float* token_scores, const float* 
       select_args_check(token_scores, tile_s, N, n_v, policy, u, kept, n_kept, budgets, sel, sel_off);
   if (chk != RIFT_OK) return chk;
   prof_begin(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream));
-  launch_select(token_scores, tile_s, N, n_v, p, *policy, u, kept, n_kept, budgets, sel, sel_off,
-                static_cast<cudaStream_t>(stream));
-  prof_end(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream), 2);
+  const int launches = launch_select(token_scores, tile_s, N, n_v, p, *policy, u, kept, n_kept, budgets, sel, sel_off,
+                                     static_cast<cudaStream_t>(stream));
+  prof_end(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream), launches);
   RIFT_LAUNCH_CHECK();
   return RIFT_OK;
 }
@@ -305,9 +305,9 @@ rift_status rift_select_budgeted_tokens_ranged(const float* token_scores, const 
       select_args_check(token_scores, tile_s, N, n_v, policy, u, kept, n_kept, budgets, sel, sel_off);
   if (chk != RIFT_OK) return chk;
   prof_begin(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream));
-  launch_select(token_scores, tile_s, N, n_v, p, *policy, u, kept, n_kept, budgets, sel, sel_off,
-                static_cast<cudaStream_t>(stream), s_range);
-  prof_end(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream), 2);
+  const int launches = launch_select(token_scores, tile_s, N, n_v, p, *policy, u, kept, n_kept, budgets, sel, sel_off,
+                                     static_cast<cudaStream_t>(stream), s_range);
+  prof_end(RIFT_PROF_SELECT, static_cast<cudaStream_t>(stream), launches);
   RIFT_LAUNCH_CHECK();
   return RIFT_OK;
 }

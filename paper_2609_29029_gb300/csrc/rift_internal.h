@@ -64,9 +64,9 @@ void launch_score_range(const float* s, int n, float* range, cudaStream_t st);
 
 // ---- select.cu ----
 // s_range (nullable): the scene's (min, max) of tile_s, when the N tiles are a shard of it.
-void launch_select(const float* token_scores, const float* tile_s, int N, int n_v, const float* p,
-                   const rift_policy& pol, float* u, int* kept, int* n_kept, int* budgets, int* sel,
-                   int* sel_off, cudaStream_t st, const float* s_range = nullptr);
+int launch_select(const float* token_scores, const float* tile_s, int N, int n_v, const float* p,
+                  const rift_policy& pol, float* u, int* kept, int* n_kept, int* budgets, int* sel,
+                  int* sel_off, cudaStream_t st, const float* s_range = nullptr);
 
 // ---- features.cu ----
 struct FeaturesLayout {
