@@ -645,25 +645,27 @@ __global__ void __launch_bounds__(512) knn_pairs_smooth_kernel(const float* __re
   s_tilde[il] = __fdiv_rn(acc, (float)(m + 1));
 }
 
-// One CTA per tile, one warp per candidate: recompute the C candidates' similarities to ~fp64
+// One CTA (or CS of them, a cluster) per tile, one warp per candidate: recompute the C candidates' similarities to ~fp64
 // accuracy (the fp32 pass errs by ~sqrt(d) ulp for nearly parallel tiles, and fp32 cannot even
 // separate similarities closer to 1 than 6e-8), keep the m best by those values (ties to the
 // lower index), then s~_i = (sum over the ascending set {i} + NN(i) of s_raw) / (m + 1) with
 // correctly rounded fp32 adds and divide.
 // CTA il smooths tile i = row0 + il and writes s_tilde[il], nbr[il].
-// U: float4 pairs of loads ahead per lane: an unrolled loop of 4, or batches of 8 where a CTA has an SM to
-// itself (64 tiles 14.8 -> 12.1 us; with several CTAs on an SM batches cost residency: 400 tiles 19 us
-// with the loop, 24 with batches of 4).
-template <int U>
-__global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
+// U: float4 pairs of loads ahead per lane: an unrolled loop of 4, or batches of 8 while the tiles are no more
+// than the SMs (64 tiles 14.8 -> 12.1 us; with several CTAs on an SM batches cost residency: 400 tiles 19
+// us with the loop, 24 with batches of 4).  CS: up to as many tiles as SMs a tile's candidates are spread over
+// four SMs, since one issues the 16 chains' float-float steps for 3 us: 64 tiles 9.6 us (12.1 with one CTA, 9.9
+// with two), 140 tiles 10.7 (11.1 with two); 400 tiles 27 us in clusters of four, 19 without.
+template <int U, int CS>
+__global__ void __launch_bounds__(32 * RIFT_MAX_KNN / CS) knn_rescore_smooth_kernel(
     const float* __restrict__ V, int d, const int* __restrict__ top_j, int N, int row0, int C, int m,
     const float* __restrict__ s_raw, float* __restrict__ s_tilde, int* __restrict__ nbr) {
   pdl_trigger();
   pdl_wait();
   __shared__ double g64[RIFT_MAX_KNN];
   __shared__ int jj[RIFT_MAX_KNN];
-  const int il = blockIdx.x, i = row0 + il;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int il = blockIdx.x / CS, i = row0 + il, cta = blockIdx.x % CS;
+  const int w = cta * (RIFT_MAX_KNN / CS) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w < C) {
     const int j = top_j[(size_t)il * C + w];
     // V_i is read by all the CTA's warps (L1 serves all but the first).  The kernel moves 16 rows
@@ -697,7 +699,23 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN) knn_rescore_smooth_kernel(
       jj[w] = j;
     }
   }
-  __syncthreads();
+  if constexpr (CS > 1) {
+    // the first CTA's warp 0 fetches the others' similarities; they stay until it has
+    __syncwarp();
+    sc_cluster_sync();
+    if (w == 0 && lane < C && lane >= RIFT_MAX_KNN / CS) {
+      const int src = lane / (RIFT_MAX_KNN / CS);
+      const uint32_t g_at = sc_mapa(g64 + lane, src);
+      const float g_lo = sc_ld_cluster(g_at), g_hi = sc_ld_cluster(g_at + 4);
+      jj[lane] = __float_as_int(sc_ld_cluster(sc_mapa(jj + lane, src)));
+      g64[lane] = __hiloint2double(__float_as_int(g_hi), __float_as_int(g_lo));
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    if (cta != 0) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  } else {
+    __syncthreads();
+  }
   if (w != 0) return;
   // Lane a < C holds candidate a, lane C the tile itself.  Rank by (similarity descending, index
   // ascending); the m first are the neighbours.
@@ -894,8 +912,12 @@ int launch_smooth(const float* V, const float* s_raw, int N, int d, int row0, in
               n_rows, C, topj);
     launched += split_done ? 3 : 4;
   }
-  launch_ex(N <= sm_count() ? knn_rescore_smooth_kernel<8> : knn_rescore_smooth_kernel<4>, dim3(n_rows),
-            dim3(32 * RIFT_MAX_KNN), 0, st, true, V, d, (const int*)topj, N, row0, C, m, s_raw, s_tilde, nbr);
+  auto rescore = [&](auto kern, int cs) {
+    launch_cluster_ex(kern, dim3(n_rows * cs), dim3(32 * RIFT_MAX_KNN / cs), 0, st, true, cs, V, d, (const int*)topj, N,
+                      row0, C, m, s_raw, s_tilde, nbr);
+  };
+  if (n_rows <= sm_count()) rescore(knn_rescore_smooth_kernel<8, 4>, 4);
+  else rescore(knn_rescore_smooth_kernel<4, 1>, 1);
   return launched;
 }
 
