@@ -36,14 +36,6 @@ namespace mg {
 constexpr int TB = 64;     // tokens and targets per block of the similarity pass
 constexpr int KC = 32;     // d-chunk staged per step (summed in 32-term sub-chunks)
 
-template <typename XT>
-__device__ __forceinline__ float load_x(const XT* p) {
-  if constexpr (sizeof(XT) == 2)
-    return bf16_bits_to_float(*reinterpret_cast<const uint16_t*>(p));
-  else
-    return *p;
-}
-
 // Eight consecutive elements of a row (16-byte aligned) as floats.
 template <typename XT>
 __device__ __forceinline__ void load8(const XT* p, float (&v)[8]) {
