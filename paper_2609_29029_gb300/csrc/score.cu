@@ -294,7 +294,10 @@ __device__ __forceinline__ float sc_ld_cluster(uint32_t addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
   return v;
 }
+// The .aligned forms want the whole warp together: it may arrive from a loop whose trip count differs
+// between its lanes.
 __device__ __forceinline__ void sc_cluster_sync() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
@@ -701,7 +704,6 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN / CS) knn_rescore_smooth_ker
   }
   if constexpr (CS > 1) {
     // the first CTA's warp 0 fetches the others' similarities; they stay until it has
-    __syncwarp();
     sc_cluster_sync();
     if (w == 0 && lane < C && lane >= RIFT_MAX_KNN / CS) {
       const int src = lane / (RIFT_MAX_KNN / CS);
