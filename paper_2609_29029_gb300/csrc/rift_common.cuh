@@ -170,11 +170,12 @@ __device__ __forceinline__ float warp_min(float v) {
 }
 
 // Inclusive prefix sum over the 32 lanes of a warp.
-__device__ __forceinline__ int warp_incl_scan(int v) {
+template <typename T>
+__device__ __forceinline__ T warp_incl_scan(T v) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    int n = __shfl_up_sync(0xffffffffu, v, o);
+    const T n = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += n;
   }
   return v;
@@ -192,22 +193,23 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return r;
 }
 
-// Block-wide exclusive prefix sum of one int per thread (in thread order); *total gets the
+// Block-wide exclusive prefix sum of one integer per thread (in thread order); *total gets the
 // sum.  `sh` holds >= 33 ints.
-__device__ __forceinline__ int block_excl_scan(int v, int* sh, int* total) {
+template <typename T>
+__device__ __forceinline__ T block_excl_scan(T v, T* sh, T* total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  int inc = warp_incl_scan(v);
+  const T inc = warp_incl_scan(v);
   __syncthreads();
   if (lane == 31) sh[wid] = inc;
   __syncthreads();
   if (wid == 0) {
-    int x = (lane < nw) ? sh[lane] : 0;
-    int xi = warp_incl_scan(x);
+    const T x = (lane < nw) ? sh[lane] : T(0);
+    const T xi = warp_incl_scan(x);
     if (lane < nw) sh[lane] = xi - x;
     if (lane == nw - 1) sh[32] = xi;
   }
   __syncthreads();
-  int res = sh[wid] + inc - v;
+  const T res = sh[wid] + inc - v;
   *total = sh[32];
   return res;
 }

@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(TB_THREADS) topb_kernel(const float* __restric
 // tiles 47 -> 45.5.  The results are those of prune_budget_kernel and topb_kernel, the same operations
 // for every tile.
 constexpr int SELECT_TPT = 4, SELECT_ONE = SELECT_TPT * TB_THREADS;  // tiles at most
+// (the last tile's 1 << 21 carries into bit 31: the scan is over unsigned values)
 static_assert(SELECT_ONE <= 1024 && RIFT_MAX_NV <= 1024, "the scan packs the kept tiles above 21 bits of tokens");
 template <int TPT>
 __global__ void __launch_bounds__(TB_THREADS) select_kernel(
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(TB_THREADS) select_kernel(
   pdl_wait();
   constexpr int NW = TB_THREADS / 32;
   __shared__ float rmin[NW], rmax[NW];
-  __shared__ int sh[33];
+  __shared__ unsigned sh[33];
   __shared__ int own[4];  // this CTA's tile: kept, its place, its tokens' place, its tokens
   const int tid = threadIdx.x, tile = blockIdx.x, i0 = tid * TPT;
   float f[TB_KPT], v[TPT], p[TPT];
@@ -311,9 +312,9 @@ __global__ void __launch_bounds__(TB_THREADS) select_kernel(
       loc += (1u << 21) + (unsigned)tok[e];
     }
   }
-  int all;
-  const unsigned at = (unsigned)block_excl_scan((int)loc, sh, &all);
-  const int n = (int)((unsigned)all >> 21), total = all & ((1 << 21) - 1);
+  unsigned all;
+  const unsigned at = block_excl_scan(loc, sh, &all);
+  const int n = (int)(all >> 21), total = (int)(all & ((1u << 21) - 1u));
   int place = (int)(at >> 21), off = (int)(at & ((1u << 21) - 1));
 #pragma unroll
   for (int e = 0; e < TPT; ++e) {

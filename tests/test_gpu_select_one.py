@@ -39,3 +39,25 @@ def test_selection_matches_the_oracle(N, n_v, ext_p, cuda, riftlib):
     g = sel.cpu().tolist()
     for j, i in enumerate(ok):
         assert g[o[j]:o[j + 1]] == O.top_b(r32[i], ob[j])
+
+
+@pytest.mark.parametrize("N,n_v,C", [(1024, 1024, 1024), (1024, 576, 72), (1023, 1024, 1024), (256, 64, 64)])
+def test_every_tile_kept(N, n_v, C, cuda, riftlib):
+    """Equal scores keep every tile (u = 1): the largest tile count the scan over kept tiles and their
+    tokens has to hold, at the largest token count and at a smaller one."""
+    pol = W.Policy(1.0, (C,), (0.9,), (0.2,), (0.1,), 0.2)
+    r = (torch.arange(N * n_v) * 7919 % 1009).view(N, n_v).float()
+    dev = dict(dtype=torch.int32, device=cuda)
+    u = torch.empty(N, device=cuda)
+    kept, n_kept, bud = torch.empty(N, **dev), torch.empty(1, **dev), torch.empty(N, **dev)
+    sel, off = torch.full((N * n_v,), -1, **dev), torch.empty(N + 1, **dev)
+    riftlib.select_budgeted_tokens(r.to(cuda), torch.full((N,), 0.25, device=cuda), N, n_v, None, riftlib.make_policy(pol),
+                                   u, kept, n_kept, bud, sel, off, None, 0)
+    riftlib.sync_status()
+    assert int(n_kept.item()) == N and bool((u == 1).all()) and bool((bud == C).all())
+    assert torch.equal(kept.cpu(), torch.arange(N, dtype=torch.int32))
+    assert torch.equal(off.cpu(), torch.arange(N + 1, dtype=torch.int32) * C)
+    got = sel.view(-1)[:N * C].view(N, C).cpu()
+    for i in (0, 1, N // 2, N - 1):
+        assert got[i].tolist() == O.top_b(r[i].numpy(), C)
+    assert bool((got[:, 1:] > got[:, :-1]).all())
