@@ -238,12 +238,11 @@ __global__ void __launch_bounds__(256) tile_finalize_kernel(const float* __restr
 // at a time: every thread loads its vectors of all of them first (LT * NVEC 16-byte loads in
 // flight), then each warp's sums x.w and x.x of each token go to shared memory and are added across
 // the warps once, at the end of the chunk, so nothing in the loop waits for another warp.
-// Few tiles (CS > 1): the 256 threads are spread over a cluster of CS CTAs, a 256 / CS-thread part of the
-// columns each, and the warps' sums are read through distributed shared memory at the end: the same
-// sums in the same order, bit for bit, on CS times the CTAs.
-// HBM-bound (X read once); under ncu, us, with a cross-warp reduction per 8 tokens and without the
-// clusters in brackets: 400 tiles x 576 x 4096 bf16 269 (276), 7.0 TB/s; 64 tiles 56 (62); 4 tiles x 576 x
-// 256 fp32, which is the latency of 6 (24) rounds of loads, 17 (28).
+// CS = 2 spreads the 256 threads over a cluster of two CTAs, half of the columns each, and reads the
+// warps' sums through distributed shared memory at the end: the same sums in the same order, bit for
+// bit, on twice the CTAs (launch_tokens has the rule).
+// HBM-bound (X read once): 400 tiles x 576 x 4096 bf16 269 us under ncu, 7.0 TB/s of X (276 with a cross-warp
+// reduction per 8 tokens).  Few tokens or short rows: the latency of the rounds of loads.
 // ------------------------------------------------------------------------------------------
 constexpr int SC_THREADS = 256;
 constexpr int SC_CHUNK = 192;  // tokens per chunk: 3 chunks per 576-token tile
@@ -301,8 +300,8 @@ __device__ __forceinline__ void sc_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-template <typename XT, int NVEC, int CS>
-__global__ void __launch_bounds__(SC_THREADS / CS, NVEC == 1 ? 1 : 2 * CS)
+template <typename XT, int NVEC, int CS, int LT>
+__global__ void __launch_bounds__(SC_THREADS / CS, LT * NVEC > 16 ? 1 : 2 * CS)
     token_score_kernel(const XT* __restrict__ X, int n_v, int d, int n_chunks,
                        const float* __restrict__ w, float* __restrict__ token_scores,
                        float* __restrict__ Ppart, unsigned int* __restrict__ cnt, float* __restrict__ V,
@@ -311,8 +310,8 @@ __global__ void __launch_bounds__(SC_THREADS / CS, NVEC == 1 ? 1 : 2 * CS)
   pdl_wait();
   using VT = VecTraits<XT>;
   constexpr int VW = VT::W;
-  constexpr int LT = NVEC == 1 ? 32 : NVEC == 2 ? 8 : 4;  // raw loads: LT * NVEC * 4 registers
-  constexpr int G = LT < 8 ? LT : 8;                      // tokens per warp reduction
+  constexpr int G = LT < 8 ? LT : 8;  // tokens per warp reduction (raw loads: LT * NVEC * 4 registers)
+  static_assert(SC_CHUNK % LT == 0 && LT % G == 0, "whole batches of tokens");
   constexpr int THREADS = SC_THREADS / CS, WARPS = THREADS / 32;
   __shared__ float red[WARPS][SC_CHUNK][2];  // each warp's x.w and x.x of each token
   const int rank = CS == 1 ? 0 : (int)(blockIdx.x % CS), unit = (int)blockIdx.x / CS;
@@ -826,19 +825,40 @@ template <typename XT, int NVEC>
 static void launch_tokens(const void* X, int N, int n_v, int d, const ShardLayout& L, const float* w,
                           float* token_scores, float* Ppart, unsigned int* cnt, float* V, float* s_raw,
                           uint16_t* S16, cudaStream_t st) {
-  auto go = [&](auto cs) {
-    constexpr int CS = decltype(cs)::value;
-    launch_cluster_ex(token_score_kernel<XT, NVEC, CS>, dim3(N * L.n_chunks * CS), dim3(SC_THREADS / CS), 0, st, true, CS,
-                      static_cast<const XT*>(X), n_v, d, L.n_chunks, w, token_scores, Ppart, cnt, V, s_raw, S16, N,
+  auto go = [&](auto cs, auto lt) {
+    constexpr int CS = decltype(cs)::value, LT = decltype(lt)::value;
+    launch_cluster_ex(token_score_kernel<XT, NVEC, CS, LT>, dim3(N * L.n_chunks * CS), dim3(SC_THREADS / CS), 0, st, true,
+                      CS, static_cast<const XT*>(X), n_v, d, L.n_chunks, w, token_scores, Ppart, cnt, V, s_raw, S16, N,
                       (N + 7) & ~7);
   };
-  // Clusters while the chunks are fewer than four CTAs per SM (64 tiles: 192 CTAs on 152 SMs), and rows long
-  // enough that every thread has a vector (a shorter row's columns would all fall to rank 0)
-  const int units = N * L.n_chunks, want = 4 * sm_count();
-  const bool full = d >= SC_THREADS * VecTraits<XT>::W;
-  if (full && units * 2 <= want) go(std::integral_constant<int, 4>{});
-  else if (full && units < want) go(std::integral_constant<int, 2>{});
-  else go(std::integral_constant<int, 1>{});
+  using C1 = std::integral_constant<int, 1>;
+  using C2 = std::integral_constant<int, 2>;
+  // u: CTAs of whole chunks.  Clusters of two only for bf16 rows of at most two vectors a thread that give
+  // every thread of both CTAs one (a shorter row's columns would all fall to the first CTA).
+  const int u = N * L.n_chunks, sms = sm_count();
+  const bool can_split = sizeof(XT) == 2 && d >= SC_THREADS * VecTraits<XT>::W;
+  if constexpr (NVEC == 1) {
+    // 32 tokens' loads ahead take an SM's registers for one CTA: right while a CTA is all that an SM gets,
+    // beyond that two CTAs of 16.  us, 32 against 16 (576 tokens): bf16 d = 2048, 16 tiles (48 CTAs) 34 : 38, 50
+    // (150) 38 : 41, 64 (192) 60 : 48, 400 216 : 169; fp32 d = 256, 50 tiles 26 : 28, 64 40 : 34, 400 132 : 99.
+    // Two CTAs of 32 on a cluster while every half has an SM of its own: 4 tiles at d = 2048 34 -> 30, 16 tiles
+    // 34 -> 32; four CTAs (34 -> 30, 34 -> 32) are no faster.
+    using L32 = std::integral_constant<int, 32>;
+    if constexpr (sizeof(XT) == 2)
+      if (can_split && 2 * u <= sms) return go(C2{}, L32{});
+    if (u <= sms) go(C1{}, L32{});
+    else go(C1{}, std::integral_constant<int, 16>{});
+  } else {
+    // The pass takes as long as the busiest SM: half chunks where they leave it less than whole ones do, in
+    // the first rounds.  bf16 d = 4096, us, whole chunks : halves : quarters: 4 tiles 50 : 48 : 48, 38 54 : 56 : 56, 64
+    // 70 : 66 : 67, 76 73 : 71 : 75, 90 81 : 83 : 83, 100 89 : 89 : 118, 120 130 : 127 : 129, 150 139 : 141 : 142, 210 189 : 193 :
+    // 194.  Not for fp32 (64 tiles at d = 2048 60 : 60, 120 116 : 120) and not for four vectors a thread (bf16 d = 8192,
+    // 4 tiles 97 : 106, 64 126 : 134).
+    using LT = std::integral_constant<int, NVEC == 2 ? 8 : 4>;
+    if constexpr (sizeof(XT) == 2 && NVEC == 2)
+      if (can_split && u < 4 * sms && (2 * u + sms - 1) / sms < 2 * ((u + sms - 1) / sms)) return go(C2{}, LT{});
+    go(C1{}, LT{});
+  }
 }
 
 int launch_score_tokens(const void* X, rift_dtype xdt, int N, int n_v, int d, const float* t, const float* B,

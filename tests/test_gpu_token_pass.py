@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
                                       ("f32", 4096, 33), ("bf16", 320, 100), ("f32", 64, 5)])
 def test_scores_do_not_depend_on_the_tile_count(dt, d, n_v, cuda, riftlib):
     chunks = -(-n_v // 192)
-    N = 640 // chunks + 1  # more than four CTAs per SM: no cluster
+    N = 640 // chunks + 1  # more than four CTAs per SM: no cluster, the fewest tokens ahead
     g = torch.Generator(device=cuda)
     g.manual_seed(1)
     X = torch.randn(N, n_v, d, generator=g, device=cuda).to(torch.bfloat16 if dt == "bf16" else torch.float32)
@@ -33,7 +33,9 @@ def test_scores_do_not_depend_on_the_tile_count(dt, d, n_v, cuda, riftlib):
         return r, s, V
 
     r, s, V = score(N)
-    for n in (1, 300 // chunks, 600 // chunks):  # clusters of 4, 4 and 2
+    # chunks below half the SMs and below them (more tokens ahead; clusters for bf16), a cluster of two where it
+    # evens out the SMs' load, and beyond
+    for n in (1, 76 // chunks, 150 // chunks, 190 // chunks, 300 // chunks, 600 // chunks):
         got = score(n)
         for a, b in zip(got, (r, s, V)):
             assert torch.equal(a, b[:n])
