@@ -1,6 +1,6 @@
 // Stage 1 pruning and Stage 2 budgets and token selection on sm_103a.
 //
-//   select_kernel        (up to 1024 tiles, one CTA per tile) both steps below: every CTA normalises all
+//   select_kernel        (up to 512 tiles, one CTA per tile) both steps below: every CTA normalises all
 //                        scores, takes the budgets and scans them for its own tile's place, and selects
 //                        its tile's tokens
 //   prune_budget_kernel  (more tiles; one CTA) per-scene min-max of the smoothed scores, u_i >= tau,
@@ -243,12 +243,13 @@ __global__ void __launch_bounds__(TB_THREADS) topb_kernel(const float* __restric
 }
 
 // Both steps in one launch, CTA i = tile i: bound by latency, and a launch in the chain costs more than
-// every CTA's own pass over the scores, TPT tiles a thread.  64 tiles 6.6 us against 4.9 + 5.5, the scene 134
-// -> 132 us (136 with four tiles a thread: their budgets are a serial loop); 400 tiles 434 -> 430, four small
-// tiles 47 -> 45.5.  The results are those of prune_budget_kernel and topb_kernel, the same operations
-// for every tile.
-constexpr int SELECT_TPT = 4, SELECT_ONE = SELECT_TPT * TB_THREADS;  // tiles at most
-// (the last tile's 1 << 21 carries into bit 31: the scan is over unsigned values)
+// every CTA's own pass over the scores, TPT tiles a thread, while that is short: us alone, one launch against two,
+// 64 tiles 8.3 : 12.3, 400 10.2 : 12.3, 512 12.3 : 14, 700 14-16 : 14, 1024 18.4 : 14-16; a scene's whole selection with
+// small tokens, 512 tiles 160 : 161, 640 197 : 196, 1024 279 : 277.  The scene of 64 tiles went from 134 to 132 us (136
+// with four tiles a thread: their budgets are a serial loop), 400 434 -> 430, four small tiles 47 -> 45.5.
+// The results are those of prune_budget_kernel and topb_kernel, the same operations for every tile.
+constexpr int SELECT_TPT = 2, SELECT_ONE = SELECT_TPT * TB_THREADS;  // tiles at most
+// (unsigned, so that a sum past bit 31 would still be defined)
 static_assert(SELECT_ONE <= 1024 && RIFT_MAX_NV <= 1024, "the scan packs the kept tiles above 21 bits of tokens");
 template <int TPT>
 __global__ void __launch_bounds__(TB_THREADS) select_kernel(

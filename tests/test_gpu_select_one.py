@@ -1,4 +1,4 @@
-"""The selection in one launch (up to 1024 tiles) at the edges of its range and of a thread's four tiles, and the
+"""The selection in one launch (up to 512 tiles) at the edges of its range and of a thread's tiles, and the
 two launches above it, against the oracle on shared fp32 inputs: integers and normalised scores exactly."""
 import numpy as np
 import pytest
@@ -14,7 +14,7 @@ POLICY = W.Policy(0.3, (1, 8, 16, 64), (0.9, 0.9, 0.9, 0.9), (0.2, 0.5, 0.7, 0.9
 
 
 @pytest.mark.parametrize("ext_p", [False, True], ids=["own", "ext_p"])
-@pytest.mark.parametrize("N,n_v", [(1, 64), (4, 65), (5, 576), (257, 100), (1023, 64), (1024, 70), (1025, 64)])
+@pytest.mark.parametrize("N,n_v", [(1, 64), (4, 65), (5, 576), (256, 64), (257, 100), (511, 65), (512, 64), (513, 64), (1023, 64), (1024, 70), (1025, 64)])
 def test_selection_matches_the_oracle(N, n_v, ext_p, cuda, riftlib):
     r = rng.normal_f32(8, rng.stream_id("select-one", N), N * n_v).view(N, n_v)
     r = torch.floor(r * 16) / 16  # ties
@@ -41,7 +41,7 @@ def test_selection_matches_the_oracle(N, n_v, ext_p, cuda, riftlib):
         assert g[o[j]:o[j + 1]] == O.top_b(r32[i], ob[j])
 
 
-@pytest.mark.parametrize("N,n_v,C", [(1024, 1024, 1024), (1024, 576, 72), (1023, 1024, 1024), (256, 64, 64)])
+@pytest.mark.parametrize("N,n_v,C", [(512, 1024, 1024), (512, 576, 72), (1024, 1024, 1024), (1024, 576, 72), (1023, 1024, 1024), (256, 64, 64)])
 def test_every_tile_kept(N, n_v, C, cuda, riftlib):
     """Equal scores keep every tile (u = 1): the largest tile count the scan over kept tiles and their
     tokens has to hold, at the largest token count and at a smaller one."""
