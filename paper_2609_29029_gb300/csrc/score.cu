@@ -585,13 +585,15 @@ __device__ __forceinline__ long long knn_order(double g0) {
   return g < 0 ? g ^ 0x7fffffffffffffffll : g;
 }
 
-// Scenes of at most KNN_PAIRS tiles: every pair's similarity at the accuracy of the rescoring below, with no
-// Gram matrix and no candidates, and the smoothing.  One CTA per tile, a warp per other tile, two at a time.
-// Up to three launches fewer than the general path, whose Gram product and candidate lists are latency at
-// this size; past 32 tiles a warp goes around more than once and the general path is as fast
-// (smoothing alone at d = 4096, us, pairs against general: 16 tiles 12.6 : 22.2, 32 tiles 13.5 : 22.7, 64 tiles
-// 25.1 : 24.0, 100 tiles 62 : 26).
-constexpr int KNN_PAIRS = 32;
+// Scenes of at most KNN_PAIRS tiles and rows of up to KNN_PAIRS_D: every pair's similarity at the accuracy of
+// the rescoring below, with no Gram matrix and no candidates, and the smoothing.  One CTA per tile, a warp per
+// other tile, two at a time.  Up to three launches fewer than the general path, whose Gram product and candidate
+// lists are latency at this size; past 32 tiles a warp goes around more than once, and past 4096 columns its serial
+// chain is the longer one.  Smoothing alone, us, pairs against general: d = 4096, 4 tiles 24.6 : 23.6, 16 tiles 22.6 :
+// 23.6, 32 26.6 : 25.6 (two launches fewer for the host), d = 1024 12-14 : 17-20; d = 8192, 4 tiles 39 : 30, 16 37 : 32, 32 41 : 32;
+// d = 4096 at 64 tiles 25.1 : 24.0, at 100 62 : 26 (warm).
+constexpr int KNN_PAIRS = 32, KNN_PAIRS_D = 4096;
+static bool smooth_by_pairs(int N, int d) { return N <= KNN_PAIRS && d <= KNN_PAIRS_D; }
 __global__ void __launch_bounds__(512) knn_pairs_smooth_kernel(const float* __restrict__ V, int d, int N, int row0, int m,
                                                                const float* __restrict__ s_raw,
                                                                float* __restrict__ s_tilde, int* __restrict__ nbr) {
@@ -902,7 +904,7 @@ int launch_score_tokens(const void* X, rift_dtype xdt, int N, int n_v, int d, co
 
 int launch_smooth(const float* V, const float* s_raw, int N, int d, int row0, int n_rows, int m, float* s_tilde,
                   int* nbr, char* ws, cudaStream_t st, bool split_done) {
-  if (N <= KNN_PAIRS) {
+  if (smooth_by_pairs(N, d)) {
     launch_ex(knn_pairs_smooth_kernel, dim3(n_rows), dim3(512), 0, st, true, V, d, N, row0, m, s_raw, s_tilde, nbr);
     return 1;
   }
@@ -949,7 +951,7 @@ int launch_score(const void* X, rift_dtype xdt, int N, int n_v, int d, const flo
   const ScoreLayout L = score_layout(N, n_v, d, M);
   float* V = reinterpret_cast<float*>(ws + L.V_off);
   // with a Gram matrix to form, the token pass's finalisation also writes its split rows
-  uint16_t* S16 = m > 0 && N > KNN_PAIRS ? reinterpret_cast<uint16_t*>(ws + L.smooth_off + L.S.split_off) : nullptr;
+  uint16_t* S16 = m > 0 && !smooth_by_pairs(N, d) ? reinterpret_cast<uint16_t*>(ws + L.smooth_off + L.S.split_off) : nullptr;
   const int a = launch_score_tokens(X, xdt, N, n_v, d, t, B, M, token_scores, s_raw, V, ws + L.tokens_off, st, S16);
   const int b = launch_smooth(V, s_raw, N, d, 0, N, m, s_tilde, nbr, ws + L.smooth_off, st, m > 0);
   return b < 0 ? -1 : a + b;

@@ -48,12 +48,13 @@ def test_scores_do_not_depend_on_the_tile_count(dt, d, n_v, cuda, riftlib):
     assert float((V[:3].cpu().double() - P / P.norm(dim=1, keepdim=True)).abs().max()) < 1e-6
 
 
-# up to 32 tiles: every pair; more: Gram, candidates (whole groups of 32 columns sorted or inserted) and
-# rescoring
-@pytest.mark.parametrize("N", [2, 17, 31, 32, 33, 64, 65, 97, 600])
+# up to 32 tiles of up to 4096 columns: every pair; more: Gram, candidates (whole groups of 32 columns sorted or
+# inserted) and rescoring
+@pytest.mark.parametrize("N,d", [(N, 256) for N in (2, 17, 31, 32, 33, 64, 65, 97, 600)] +
+                         [(2, 4096), (32, 4096), (2, 4160), (17, 8192), (32, 8192)])
 @pytest.mark.parametrize("m", [1, 6, 16])
-def test_neighbour_ties_go_to_the_lower_index(N, m, cuda, riftlib):
-    d, groups, m = 256, 8, min(m, N - 1)
+def test_neighbour_ties_go_to_the_lower_index(N, d, m, cuda, riftlib):
+    groups, m = 8, min(m, N - 1)
     g = rng.normal_f32(4, rng.stream_id("tie-dirs"), groups * d).view(groups, d)
     g = g / g.norm(dim=1, keepdim=True)
     which = [(5 * i + i // 7) % groups for i in range(N)]  # tiles of one group are identical
