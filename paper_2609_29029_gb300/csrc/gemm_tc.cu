@@ -605,28 +605,38 @@ __host__ __device__ constexpr int stages(int bn) {
 static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 
 // Row tiles: as few as MAX_BN allows, of equal height.  S: as many CTAs per tile as the GPU holds
-// at once (two per SM), each with at least 8 K-blocks (a shorter slice is all fill and drain; a Gram
+// at once, each with at least 8 K-blocks (a shorter slice is all fill and drain; a Gram
 // matrix, on its own in a chain of small kernels, takes slices of 3).  More than 8 CTAs (a
 // non-portable cluster) where one tile would leave the rest idle: 16 for the Gram matrix of up to 128 tiles, K = 3 d (64 tiles at d = 4096: 11 us with 16, 15 with 8).
 // More CTAs than fit at once cost a second round: gate/up at one row 35.8 us with 172 CTAs, 43.6
-// with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.
+// with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.  Two CTAs fit on an SM, but a cluster has to
+// fit in one GPC: resident[S] clusters at once (asked from the driver), fewer than 2 SMs / S for most S.  100 rows,
+// us, by the count of CTAs alone against resident[S]: N = 5120 x K = 4096 28.7 (S = 7) : 20.7 (6), 6144 x 4096
+// 30.7 (6) : 22.5 (5).
+// K too short to split (fewer than 16 K-blocks): row tiles of at most SHORT_BN instead, as long as they fit at
+// once; what a CTA takes is then its epilogue, a serial chain over its rows.  us, tiles of 160 rows, 48, and the
+// SM pairs, 300 rows: 256 x 256 + residual 22.5 : 12.3 : 20.5, 768 x 256 10.2 : 8.2 : 14.3, SwiGLU 1376 x 256
+// 14.3 : 10.2 : 16.4; 1,500 rows of the last (too many to fit) 14.3 : 14.3 : 16.4.
+constexpr int SHORT_BN = 48;
 struct Plan {
   int bn, S;
+  bool one_round;  // all its CTAs are resident at once, or the K slices are
 };
-inline Plan plan(int M, int N, int K, int sms, bool gram) {
-  const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
-  Plan p;
-  p.bn = ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16;
-  const long long tiles = (long long)m_tiles * ((N + BM - 1) / BM);
+inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram) {
+  const long long n_tiles = (N + BM - 1) / BM;
   const int kt = (K + BK - 1) / BK;
   const int min_blocks = gram ? 3 : 8;
-  if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) {
-    p.S = MAX_S;
-    return p;
+  auto height = [&](int m_tiles) { return ((M + m_tiles - 1) / m_tiles + 15) / 16 * 16; };
+  if (!gram && kt < 2 * min_blocks) {
+    const int m_tiles = (M + SHORT_BN - 1) / SHORT_BN;
+    if (m_tiles * n_tiles <= 2LL * sms) return {height(m_tiles), 1, true};
   }
-  p.S = PORTABLE_S;
-  while (p.S > 1 && (tiles * p.S > 2LL * sms || kt / p.S < min_blocks)) --p.S;
-  return p;
+  const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
+  const long long tiles = m_tiles * n_tiles;
+  if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) return {height(m_tiles), MAX_S, true};
+  int S = PORTABLE_S;
+  while (S > 1 && (tiles > resident[S] || kt / S < min_blocks)) --S;
+  return {height(m_tiles), S, S >= 2};
 }
 }  // namespace ck
 
@@ -1213,6 +1223,47 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtenso
              : 1;
 }
 
+// Stands for gemm_ck_kernel in the question below: the driver counts a kernel with tcgen05.alloc as one CTA an SM,
+// whatever it allocates.
+__global__ void __launch_bounds__(ck::THREADS, 2) ck_shape_kernel() {}
+
+// resident[S], S = 1 .. 8: the clusters of S CTAs of the cluster split-K kernel that the current device holds at once
+// (asked once per device; 2 SMs / S where the query fails).
+static const int* ck_resident() {
+  struct Table {
+    std::once_flag once;
+    int n[ck::PORTABLE_S + 1];
+  };
+  static Table tables[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  Table& t = tables[dev];
+  std::call_once(t.once, [&] {
+    const bool raised = cudaFuncSetAttribute(ck_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ck::SMEM) ==
+                        cudaSuccess;
+    for (int S = 1; S <= ck::PORTABLE_S; ++S) {
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = S;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(S);
+      cfg.blockDim = dim3(ck::THREADS);
+      cfg.dynamicSmemBytes = ck::SMEM;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (!raised || cudaOccupancyMaxActiveClusters(&n, ck_shape_kernel, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        n = 2 * sm_count() / S;
+      }
+      t.n[S] = n;
+    }
+  });
+  return t.n;
+}
+
 // The cluster split-K kernel: S CTAs per (128 weight rows, bn rows) tile.
 template <int EPI, int MAXS>
 static int launch_ck_instance(const void* A, const void* W, uint64_t Ks, int M, int N, int K, void* C, const EpiParams& ep,
@@ -1295,16 +1346,16 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   // The operands' stored row width: K, or 2 kmap_d blocks when read through the K-block remap.
   if (ep.kmap_d && K != 3 * ep.kmap_d * BK) return 1;
   const uint64_t Ks = ep.kmap_d ? (uint64_t)2 * ep.kmap_d * BK : (uint64_t)K;
-  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ep.kmap_d > 0);
-  // The cluster split-K kernel for one row tile, or while its split tiles fit on the GPU at once:
-  // beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
+  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ck_resident(), ep.kmap_d > 0);
+  // The cluster split-K kernel for one row tile, or while its tiles fit on the GPU at once, split or, where K is
+  // short, low: beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
   // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777
   // (S = 1) 42.0 : 35.4; W_down 53.9 : 63.7 and 78.1 : 65.8; QKV at 131 rows 27.0 : 31.1, at 256
   // (S = 1) 40.8 : 31.1; gate/up 46.8 : 57.8 and 75.6 : 57.8 (wide tiles; the pairs' narrow ones, 14%
   // less, leave the order as it is).
   // A device count of the logits' rows (sequences) is usually a fraction of its capacity, and
   // row tiles past the count cost nothing there.
-  if (M <= ck::MAX_BN || plan.S >= 2 || (epi == EPI_STORE_F32 && ep.m_dev && M < 1024))
+  if (M <= ck::MAX_BN || plan.one_round || (epi == EPI_STORE_F32 && ep.m_dev && M < 1024))
     return launch_ck_epi(A, B, Ks, M, N, K, epi, C, ep, st, plan, pdl, b_const ? 1 : 0);
   CUtensorMap ma, mb, mn;
   if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2) ||

@@ -1,6 +1,7 @@
 """The cluster split-K product (few rows: weights as the 128-row operand, K split over a
-thread-block cluster) through rift_linear, at the edges of its row tiles (16 to 160 rows), weight
-tiles (128 rows), K-blocks (64) and cluster sizes, against fp64 products of the same operands."""
+thread-block cluster) through rift_linear, at the edges of its row tiles (16 to 160 rows; at most 48
+where K is too short to split), weight tiles (128 rows), K-blocks (64) and cluster sizes, and of the rows it
+takes before the SM pairs' kernel does, against fp64 products of the same operands."""
 import pytest
 import torch
 
@@ -18,6 +19,13 @@ F32_TOL = 2e-5
 # ones, a K tail; rows around 16, 128, 160 and in two and three row tiles; a partial weight tile
 SHAPES = [(1, 128, 64), (1, 160, 520), (2, 136, 1032), (15, 264, 1600), (16, 4096, 4096), (17, 1024, 4104),
           (127, 288, 2816), (160, 1024, 11008), (161, 1024, 4096), (203, 672, 4104), (333, 288, 11008)]
+# short K: 48 and 49 rows, a K tail, the last K-block count that is short and the first that is not
+SHAPES += [(48, 128, 200), (49, 136, 64), (300, 256, 256), (1000, 264, 72), (1023, 768, 960), (161, 96, 1016), (161, 96, 1024)]
+# as many short tiles as fit on 152 SMs at once (16 x 19), one row more (SM pairs, K tail), and SM pairs with tails in
+# rows, weight rows and K
+SHAPES += [(768, 2432, 200), (769, 2432, 200), (4400, 2056, 1032)]
+# tiles whose count times the cluster size fits while the clusters do not (40 tiles: 38 clusters of 7 fit, 46 of 6)
+SHAPES += [(100, 5120, 4096), (777, 1024, 4104)]
 
 
 def _rand(shape, stream, scale=1.0):
