@@ -608,6 +608,9 @@ static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 // at once, each with at least 8 K-blocks (a shorter slice is all fill and drain; a Gram
 // matrix, on its own in a chain of small kernels, takes slices of 3).  More than 8 CTAs (a
 // non-portable cluster) where one tile would leave the rest idle: 16 for the Gram matrix of up to 128 tiles, K = 3 d (64 tiles at d = 4096: 11 us with 16, 15 with 8).
+// A Gram matrix of more than 32 tiles takes 4 at most: it starts while the kernel before it drains, and larger
+// clusters then wait for a GPC.  Whole smoothing, us, S = 4 : 5: 1,024 scene tiles at d = 1024 59 : 69, 4096 93 : 101,
+// 8192 150 : 162; 832 at 4096 79 : 84 (6: 84), 8192 123 : 122 (6: 121); up to 32 tiles 8 wins (700 at 8192 108, with 4 118).
 // More CTAs than fit at once cost a second round: gate/up at one row 35.8 us with 172 CTAs, 43.6
 // with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.  Two CTAs fit on an SM, but a cluster has to
 // fit in one GPC: resident[S] clusters at once (asked from the driver), fewer than 2 SMs / S for most S.  100 rows,
@@ -634,7 +637,7 @@ inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram) {
   const int m_tiles = (M + MAX_BN - 1) / MAX_BN;
   const long long tiles = m_tiles * n_tiles;
   if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) return {height(m_tiles), MAX_S, true};
-  int S = PORTABLE_S;
+  int S = gram && tiles > 32 ? 4 : PORTABLE_S;
   while (S > 1 && (tiles > resident[S] || kt / S < min_blocks)) --S;
   return {height(m_tiles), S, S >= 2};
 }
