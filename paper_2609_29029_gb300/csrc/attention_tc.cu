@@ -682,13 +682,19 @@ namespace da {
 constexpr int SK = 32, NST = 3, COLS = 256, WARPS = 8, THREADS = 32 * (WARPS + 1);
 constexpr int ROW = COLS * 2, TILE = SK * ROW;  // bytes of a row of the box, of a K or V tile
 constexpr int SMEM = NST * 2 * TILE + 128 + 64;
+
+// A sequence of P cached rows is long among the batch's if it is more than `factor` / 1024 of rows x groups (of
+// columns): fewer than 1024 / (factor x groups) of them are.
+__device__ __forceinline__ bool is_long(int P, int rows, int groups, int factor) {
+  return (long long)P * 1024 > (long long)rows * groups * factor;
+}
 }  // namespace da
 
 template <int HD>
 __global__ void __launch_bounds__(da::THREADS, 2)
     decode_attn_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                       const uint16_t* __restrict__ qkv, const int* __restrict__ cu, int H, int CS, int max_keys,
-                       float scale_log2, uint16_t* __restrict__ out) {
+                       const uint16_t* __restrict__ qkv, const int* __restrict__ cu, int n, int H, int CS, int part,
+                       int long_factor, int max_keys, float scale_log2, uint16_t* __restrict__ out) {
   constexpr int SK = da::SK, NST = da::NST;
   constexpr int HPC = da::COLS / HD, KG = da::WARPS / HPC;  // heads per CTA, warps per head
   constexpr int LPK = HD / 8, KPL = 32 / LPK;               // lanes per key, keys per warp-wide load
@@ -706,7 +712,33 @@ __global__ void __launch_bounds__(da::THREADS, 2)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int groups = (H + HPC - 1) / HPC, d = H * HD;
   const int rank = (int)cluster_ctarank(), unit = (int)blockIdx.x / CS;
-  const int g = unit % groups, i = unit / groups;
+  const int g = unit % groups;
+  // A ragged batch in two launches, uniform over the cluster.  part 1: sequence i = unit / groups, the long ones left
+  // out; 2: the (unit / groups)-th long one.
+  auto is_long = [&](int j) {
+    const int len = cu[j + 1] - cu[j];
+    return len >= 0 && len + 1 <= max_keys && da::is_long(len, cu[n] - cu[0], groups, long_factor);
+  };
+  int i = unit / groups;
+  if (part == 2) {
+    __shared__ int scan[33], found;
+    const int slot = i;
+    if (threadIdx.x == 0) found = -1;
+    for (int j0 = 0, seen = 0; j0 < n && seen <= slot; j0 += da::THREADS) {
+      const int j = j0 + threadIdx.x, f = j < n && is_long(j) ? 1 : 0;
+      int total;
+      const int at = block_excl_scan(f, scan, &total);
+      if (f && seen + at == slot) found = j;
+      seen += total;
+    }
+    __syncthreads();
+    i = found;
+  }
+  if (part == 2 ? i < 0 : part == 1 && is_long(i)) {
+    pdl_trigger();
+    pdl_wait();
+    return;
+  }
   const int s0 = cu[i], P = cu[i + 1] - s0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < NST; ++s) {
@@ -1008,9 +1040,15 @@ int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, i
 }
 
 // Decode attention of n sequences' new tokens: K, V fp16 [T, d] (one layer of the cache), qkv fp16
-// [n, 3 d], out fp16 [n, d].  The keys of a sequence are split over a cluster while the units (sequence
-// x 256 columns) leave half the CTA slots (two per SM) empty and a rank keeps at least two tiles of
-// the longest sequence (one 635-row sequence: 16 units, 8 ranks each).
+// [n, 3 d], out fp16 [n, d].  Returns the number of launches, or -1.  The keys of a sequence are split over a
+// cluster while the units (sequence x 256 columns) leave half the CTA slots (two per SM) empty and a rank keeps at
+// least two tiles of the longest sequence (one 635-row sequence: 16 units, 8 ranks each).
+// A batch that may hold a sequence of more than twice an SM's even share (long max_keys, and not every sequence of
+// it) takes a second launch with clusters of 8 for such sequences alone: one CTA streams 60 rows a us, and clusters
+// for all sequences leave slots empty (10 x 4,096 rows 174 us -> 264).
+// us of a one-layer step in one launch and now: 30,000 + 15 x 300 rows at d = 4096 538 : 185, 32,000 + 39 x 131
+// 812 : 189, 8,000 + 72 x 300 286 : 164; d = 1024, 32,000 + 39 x 131 525 : 117; with nothing long after all (max_len 8192,
+// 73 of up to 347 rows) 137 : 142.
 int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16_t* V, int T, const int* cu, int n,
                             int n_heads, int head_dim, int max_keys, uint16_t* out, cudaStream_t st, bool pdl) {
   using namespace fa;
@@ -1018,14 +1056,23 @@ int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16
   CUtensorMap mk, mv;  // no cached row at all: a map nothing is loaded through
   if (!make_attn_map(&mk, K, d, T > 0 ? T : 1, da::SK, da::COLS) ||
       !make_attn_map(&mv, V, d, T > 0 ? T : 1, da::SK, da::COLS))
-    return 1;
+    return -1;
+  const long long sms = sm_count();
   int cs = 1;
-  while (cs < 8 && n * groups * cs <= sm_count() && max_keys >= 4 * da::SK * cs) cs *= 2;
+  while (cs < 8 && (long long)n * groups * cs <= sms && max_keys >= 4 * da::SK * cs) cs *= 2;
+  constexpr int MAX_CS = 8, MIN_LONG = 2048;  // rows below which one CTA is done in about 30 us
+  const bool ragged = cs < MAX_CS && n > 1 && max_keys > MIN_LONG && T != (long long)n * (max_keys - 1);
+  const int long_factor = std::max(1, (int)(2048LL * cs / sms));  // twice the share of cs CTAs
+  const int max_long = std::min(n, 1024 / (long_factor * groups) + 1);
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)head_dim);
   auto go = [&](auto kern, std::atomic<unsigned long long>& smem_raised) -> int {
-    if (raise_smem_limit(smem_raised, kern, da::SMEM) != cudaSuccess) return 1;
-    return launch_cluster_ex(kern, dim3(n * groups * cs), dim3(da::THREADS), da::SMEM, st, pdl, cs, mk, mv, qkv, cu,
-                             n_heads, cs, max_keys, scale_log2, out) != cudaSuccess;
+    if (raise_smem_limit(smem_raised, kern, da::SMEM) != cudaSuccess) return -1;
+    auto one = [&](int seqs, int cluster, int part) {
+      return launch_cluster_ex(kern, dim3(seqs * groups * cluster), dim3(da::THREADS), da::SMEM, st, pdl, cluster, mk, mv, qkv,
+                               cu, n, n_heads, cluster, part, long_factor, max_keys, scale_log2, out) == cudaSuccess;
+    };
+    if (!one(n, cs, ragged ? 1 : 0) || (ragged && !one(max_long, MAX_CS, 2))) return -1;
+    return ragged ? 2 : 1;
   };
   static std::atomic<unsigned long long> raised128{0}, raised64{0};
   return head_dim == 128 ? go(decode_attn_kernel<128>, raised128) : go(decode_attn_kernel<64>, raised64);

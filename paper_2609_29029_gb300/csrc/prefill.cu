@@ -432,8 +432,9 @@ int launch_decode(const rift_model& m, const void* kv_cache, int T, const int* c
     const uint16_t* Kc = kv + (size_t)l * 2 * T * d;
     const uint16_t* Vc = Kc + (size_t)T * d;
     prof_begin(RIFT_PROF_ATTN, st);
-    if (launch_decode_attention(qkv, Kc, Vc, T, cu_seqlens, n, m.n_heads, m.head_dim, max_len, att, st, pdl)) return 1;
-    prof_end(RIFT_PROF_ATTN, st, 1);
+    const int nk = launch_decode_attention(qkv, Kc, Vc, T, cu_seqlens, n, m.n_heads, m.head_dim, max_len, att, st, pdl);
+    if (nk < 0) return 1;
+    prof_end(RIFT_PROF_ATTN, st, nk);
     if (launch_gemm(att, m.w_o[l], n, d, d, EPI_RESID_F32, h32, st, EpiParams(), pdl)) return 1;
     norm_launch(1, n, h32, nullptr, m.g_ffn[l], xn, d, m.eps, st, nullptr, pdl);
     if (launch_gemm(xn, m.w_gate_up[l], n, 2 * m.ffn, d, EPI_SWIGLU, act, st, EpiParams(), pdl)) return 1;

@@ -199,7 +199,8 @@ int launch_attention(const void* qkv, int T, const int* cu_seqlens, int n_seq, i
                      const int4* sched, int n_sched_max, void* out, cudaStream_t st, const void* prefix_k = nullptr,
                      const void* prefix_v = nullptr, int S_pre = 0, bool pdl = false);
 // Decode attention: each of n sequences' new token (qkv fp16 [n, 3 d]) over its cached rows (K, V fp16
-// [T, d], one layer) and itself; a sequence with more than max_keys keys sets RIFT_EBIT_CAPACITY.
+// [T, d], one layer) and itself; a sequence with more than max_keys keys sets RIFT_EBIT_CAPACITY.  Returns the
+// number of launches, or -1.
 int launch_decode_attention(const uint16_t* qkv, const uint16_t* K, const uint16_t* V, int T, const int* cu, int n,
                             int n_heads, int head_dim, int max_keys, uint16_t* out, cudaStream_t st, bool pdl);
 unsigned int read_clear_err_attn();

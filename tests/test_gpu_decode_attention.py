@@ -17,7 +17,10 @@ HD64 = W.DecoderShape(n_layers=1, d=320, n_heads=5, head_dim=64, ffn=688, vocab=
 
 LENGTHS = {"one": [600], "one_short": [1], "edges": [0, 1, 31, 32, 33, 95, 96, 97, 128, 257],
            "long": [30000, 7],  # RoPE angles up to 30000 rad
-           "many": [(7 * i) % 70 for i in range(160)]}  # 480 units of 2-3 column groups: no cluster
+           "many": [(7 * i) % 70 for i in range(160)],  # 480 units of 2-3 column groups: no cluster
+           # a few sequences far longer than the rest: a launch of their own, clusters for these alone
+           "ragged": [20] * 20 + [4000] + [33] * 20 + [3000] + [0] * 5 + [64] * 13,
+           "ragged_wide": [3] * 290 + [2500, 1] + [5] * 27 + [2300]}  # found past the first 288 sequences
 
 
 @pytest.mark.parametrize("name", list(LENGTHS))
@@ -47,7 +50,7 @@ def test_decode_attention_lengths(dec, name, cuda, riftlib):
                         torch.tensor(ids, dtype=torch.int32, device=cuda), embed.to(cuda), 40, hid, kvn, None, ws, need)
     riftlib.sync_status()
     worst = 0.0
-    for i in sorted(set(range(min(n, 12))) | {n - 1}):
+    for i in sorted(set(range(min(n, 12))) | {n - 1} | {i for i in range(n) if lens[i] > 2000}):
         cache = [(kv[0, 0, cu[i]:cu[i + 1]].double().view(-1, dec.n_heads, hd),
                   kv[0, 1, cu[i]:cu[i + 1]].double().view(-1, dec.n_heads, hd))]
         ref, new = O.decode_token(embed[ids[i]], cache, lambda l: layers[l], gf, dec)
@@ -55,3 +58,32 @@ def test_decode_attention_lengths(dec, name, cuda, riftlib):
             want = want.double().reshape(-1)
             worst = max(worst, float((got.double().cpu().reshape(-1) - want).abs().max() / want.abs().max()))
     assert worst < P.HIDDEN_TOL, worst
+
+
+def test_one_long_sequence_does_not_hold_up_a_batch(cuda, riftlib):
+    """A 30,000-row sequence among fifteen of 300 rows costs about what the same rows cost spread evenly (1.1 times
+    measured); streamed by one CTA per 256 columns it took 3.3 times that."""
+    from paper_2609_29029_gb300 import DeviceModel
+    dec = W.DecoderShape(n_layers=1, d=4096, n_heads=32, head_dim=128, ffn=64, vocab=504)
+    dm = DeviceModel(dec, [W.make_layer(dec, 0, "cpu")], W.make_final_norm(dec, "cpu"), cuda)
+    T, n = 30000 + 15 * 300, 16
+    kv = torch.randn(1, 2, T, dec.d, device=cuda).to(torch.float16)
+    embed = torch.randn(40, dec.d, device=cuda).to(torch.bfloat16)
+    ids = torch.arange(n, dtype=torch.int32, device=cuda)
+    hid = torch.empty(n, dec.d, dtype=torch.bfloat16, device=cuda)
+
+    def best(lens):
+        cu = torch.tensor([sum(lens[:i]) for i in range(n + 1)], dtype=torch.int32, device=cuda)
+        need = riftlib.decode_workspace_bytes(dm.struct, n, max(lens) + 1)
+        ws = torch.empty(need, dtype=torch.uint8, device=cuda)
+        times = []
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            riftlib.decode_step(dm.struct, kv, T, cu, n, max(lens) + 1, ids, embed, 40, hid, None, None, ws, need)
+            b.record()
+            riftlib.sync_status()
+            times.append(a.elapsed_time(b))
+        return min(times)
+
+    assert best([30000] + [300] * 15) < 2 * best([T // n] * n)
