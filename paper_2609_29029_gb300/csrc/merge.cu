@@ -58,17 +58,24 @@ __device__ __forceinline__ void ff_step(float x, float y, float& hi, float& lo) 
   lo = __fadd_rn(lo, __fadd_rn(er, pe));
 }
 
-// The sum of the lanes' float-float pairs (TwoSum of the high parts), in every lane.
-__device__ __forceinline__ void ff_warp_sum(float& hi, float& lo) {
+// The sum of the lanes' float-float pairs in fp64, in every lane.
+__device__ __forceinline__ double ff_warp_sum(float hi, float lo) {
+  double acc = (double)hi + (double)lo;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    const float s = __fadd_rn(hi, h2);
-    const float bb = __fsub_rn(s, hi);
-    const float er = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
-    hi = s;
-    lo = __fadd_rn(__fadd_rn(lo, l2), er);
-  }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+
+// Two such sums at once (both in every lane): the halves of the warp take one each after the first step, so that
+// the pair costs as many fp64 additions a lane as one sum does (an SM retires about two a cycle).
+__device__ __forceinline__ double2 ff_warp_sum2(float h1, float l1, float h2, float l2) {
+  const double a = (double)h1 + (double)l1, b = (double)h2 + (double)l2;
+  const bool upper = (threadIdx.x & 16) != 0;
+  double acc = upper ? b : a;
+  acc += __shfl_xor_sync(0xffffffffu, upper ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return make_double2(__shfl_sync(0xffffffffu, acc, 0), __shfl_sync(0xffffffffu, acc, 16));
 }
 
 // Float-float accumulation of a.b over d terms by one warp, eight elements per lane and step, four
@@ -91,8 +98,7 @@ __device__ double ff_dot(const XT* a, const XT* b, int d, int lane) {
         for (int e = 0; e < 8; ++e) ff_step(x[u][e], y[u][e], hi, lo);
       }
   }
-  ff_warp_sum(hi, lo);
-  return (double)hi + (double)lo;
+  return ff_warp_sum(hi, lo);
 }
 
 // m_j = min(budgets[j] - s_j, n_v - s_j) and its exclusive prefix sum over the kept slots.  If
@@ -135,7 +141,7 @@ __global__ void __launch_bounds__(1024) merge_plan_kernel(const int* __restrict_
 // the targets (written to ctx_target) and their norms (tnorm, fp64 from a float-float sum of
 // squares), one target per warp: the warps of the TY CTAs take targets y * 8 + warp, + TY * 8, ...
 // The norm is a serial float-float chain, so the targets are spread over many warps, and a row is read
-// once for its norm and its copy (400 tiles, about 95 kept, 45 targets a slot: 16 us; 20 with the copy
+// once for its norm and its copy (400 tiles, about 95 kept, 45 targets a slot: 17 us; 20 with the copy
 // in a loop of its own, 73 with one CTA per slot).
 constexpr int TY = 8;
 template <typename XT>
@@ -216,8 +222,7 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
           for (int e = 0; e < 8; ++e) ff_step(x[e], x[e], hi, lo);
         }
     }
-    ff_warp_sum(hi, lo);
-    const double nn = (double)hi + (double)lo;
+    const double nn = ff_warp_sum(hi, lo);
     if (co + q >= max_ctx) continue;
     if (lane == 0) {
       ctx_target[co + q] = t;
@@ -230,9 +235,8 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
 // Grid (blocks of 64 unselected positions, kept slot), 8 warps: assign[j][a] = the screened target where
 // the screening was clear (cand[j][a].y < 0); the others are listed and the warps take them in turn: the
 // better of the two candidates at ~fp64 accuracy, x.t1 / ||t1|| vs x.t2 / ||t2|| from float-float dot
-// products (ties to the lower target).  The lanes' pairs are summed as pairs too: two double
-// operations retire a cycle on an SM, so a shuffle sum in fp64 costs more than the dot product.  23 us
-// at 400 tiles (28 with four warps, which take two turns), against 111 with a second look at every token.
+// products (ties to the lower target), the lanes' pairs summed in fp64.  24 us
+// at 400 tiles, against 111 with a second look at every token.
 // Targets keep their own group.
 constexpr int DT = 256;
 __global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
@@ -298,12 +302,11 @@ __global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __rest
           }
         }
     }
-    ff_warp_sum(h1, l1);
-    ff_warp_sum(h2, l2);
+    const double2 dots = ff_warp_sum2(h1, l1, h2, l2);
     if (lane == 0) {
       // s1 = e1 / n1 vs s2 = e2 / n2 as e1 n2 vs e2 n1 (norms are positive; a zero target has similarity 0)
       const double n1 = tnorm[co + o.y], n2 = tnorm[co + o.z];
-      const double e1 = n1 > 0.0 ? (double)h1 + (double)l1 : 0.0, e2 = n2 > 0.0 ? (double)h2 + (double)l2 : 0.0;
+      const double e1 = n1 > 0.0 ? dots.x : 0.0, e2 = n2 > 0.0 ? dots.y : 0.0;
       const double s1 = e1 * (n2 > 0.0 ? n2 : 1.0), s2 = e2 * (n1 > 0.0 ? n1 : 1.0);
       assign[(size_t)j * n_v + o.x] = s2 > s1 || (s2 == s1 && o.z < o.y) ? o.z : o.y;
     }
