@@ -889,13 +889,19 @@ __global__ void __launch_bounds__(ck::THREADS, 2)
 // cp.async into the swizzled tiles, so the selected tokens are neither read nor multiplied (three
 // blocks a slot instead of five at 333 of 576 tokens), 48 KB a CTA in flight; TMA's gather4 form
 // took 11 cycles per 128-byte row: 65 us at 400 tiles (about 95 kept), 102 with gather4, 87 reading
-// every token.  Where the two targets are
-// closer than the product's error bound, the choice between them is made at ~fp64 accuracy outside
-// (merge.cu); the bound scales with ||x||, which the gathering threads sum from their own chunks.
-// Bound: an accumulator update adds 16 exact products, each addend cut below 2^-24 of the largest
-// (16 x 2^-24 = 2^-20 of a magnitude of at most ||x|| ||t||), so d / 16 updates err by at most d 2^-24 ||x||
-// in x.t / ||t||, and the difference of two by d 2^-23 ||x|| (about 9% of the tokens of a random tile
-// are closer, all others need no second look).
+// every token.  A target is within the screening's error if x.t / ||t|| is less than the bound below the best one's;
+// where others than the best are, the choice among them is made at ~fp64 accuracy outside (merge.cu).  The bound
+// scales with ||x||, which the gathering threads sum from their own chunks.
+// Bound.  An accumulator update adds 16 exact products to the accumulator: the 17 addends aligned to the largest and cut,
+// the result cut to fp32.  Measured on this unit (a test holds it to that) an addend loses less than 2^-25 of the
+// largest one's power of two, the result less than 2^-23 of its own, and no addend or result is larger than ||x|| ||t||:
+// (16 / 4 + 1) 2^-23 an update, d / 16 of them (5 / 16) d 2^-23 ||x|| in x.t / ||t||, plus 2^-23 for the roundings of
+// 1 / ||t|| and of the product with it; the difference of two twice that, (0.625 d + 2) 2^-23 ||x||.  Twice this is taken,
+// (1.25 d + 8) 2^-23 ||x|| rounded up, which leaves room for the norm's own rounding and would cover a cut at 2^-24.  About
+// 12% of the tokens of a random tile have a second target within it, 0.6% a third.  Where squares or products
+// could underflow (||x|| < 2^-30, a target's norm < 2^-40) every target counts as within it.  Up to seven targets are
+// listed for a token, from a second look at its products where more than two are within; more than seven, or more
+// than two beyond one block of COLS targets, and all are candidates.
 namespace ms {
 constexpr int STAGES = 4, THREADS = 192, COLS = 80, TMEM_COLS = 128;
 constexpr int BROWS = 16;  // target rows per TMA box: a product is as wide as its targets need
@@ -913,7 +919,7 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
     merge_screen_kernel(const __grid_constant__ CUtensorMap tmT, const uint16_t* __restrict__ X, int n_v, int d,
                         const int* __restrict__ kept, const int* __restrict__ n_kept,
                         const int* __restrict__ sel_off, const int* __restrict__ ctx_off, int max_ctx,
-                        const float* __restrict__ tinv, const int* __restrict__ rest, int2* __restrict__ cand) {
+                        const float* __restrict__ tinv, const int* __restrict__ rest, MergeCand* __restrict__ cand) {
   constexpr int STAGES = ms::STAGES, COLS = ms::COLS, A_BYTES = ms::A_BYTES, B_BYTES = ms::B_BYTES;
   pdl_trigger();
   pdl_wait();
@@ -1029,7 +1035,7 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
     const int quarter = warp & 3, r = quarter * 32 + lane;
     const int a = mb * 128 + r;
     const bool want = a < R && !(a % step == 0 && a / step < m);
-    float v1 = -INFINITY, v2 = -INFINITY;
+    float v1 = -INFINITY, v2 = -INFINITY, v3 = -INFINITY, tinv_max = 0.f;
     int b1 = -1, b2 = -1;
     constexpr int LAG = STAGES - 1;  // tiles in flight behind the one being requested
     bool ok = true;
@@ -1092,29 +1098,62 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             if (cc + e < nc) {
-              const float v = __uint_as_float(acc[e]) * inv_n[cc + e];
+              // the three highest and the lower indices of the first two (ties keep the lower), without branches: the
+              // lanes of a warp hardly ever agree on them; a NaN counts as -inf
+              const float ti = inv_n[cc + e], v = fmaxf(__uint_as_float(acc[e]) * ti, -INFINITY);
               const int b = c0 + cc + e;
-              if (v > v1) {
-                v2 = v1;
-                b2 = b1;
-                v1 = v;
-                b1 = b;
-              } else if (v > v2) {
-                v2 = v;
-                b2 = b;
-              }
+              tinv_max = fmaxf(tinv_max, ti);
+              b2 = v > v1 ? b1 : v > v2 ? b : b2;
+              b1 = v > v1 ? b : b1;
+              v3 = fmaxf(v3, fminf(v, v2));
+              v2 = fmaxf(v2, fminf(v, v1));
+              v1 = fmaxf(v1, v);
             }
           }
         }
+      }
+      if (nb == nblk - 1) {
+        // the best, and the targets within the product's error of it
+        const float x2 = nrm_s[r];
+        const float bound =
+            x2 > 0x1p-60f && tinv_max <= 0x1p40f ? (1.25f * (float)d + 8.f) * 0x1p-23f * sqrtf(x2) : INFINITY;
+        auto within = [&](float v) { return !(v1 - v > bound); };  // true with a NaN or an infinite norm
+        const bool more = want && within(v3);
+        MergeCand mc;
+        mc.c[0] = (uint16_t)b1;
+        mc.c[1] = (uint16_t)(within(v2) ? b2 : -1);
+#pragma unroll
+        for (int k = 2; k < MergeCand::MAX; ++k) mc.c[k] = MergeCand::NONE;
+        mc.all = more ? 1 : 0;
+        if (nblk == 1 && __any_sync(0xffffffffu, more)) {  // the products are still there: list the rest
+          int n = 1;
+          uint64_t lo = mc.c[0] | 0xffffffffffff0000ull, hi = ~0ull;
+          for (int cc = 0; cc < nc; cc += 16) {
+            uint32_t acc[16];
+            tmem_ld16(taddr + cc, acc);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              const int b = cc + e;
+              if (b < nc && b != b1 && within(__uint_as_float(acc[e]) * inv_n[b])) {
+                const uint64_t keep = ~(0xffffull << (16 * (n & 3))), put = (uint64_t)b << (16 * (n & 3));
+                if (n < 4) lo = (lo & keep) | put;
+                else if (n < MergeCand::MAX) hi = (hi & keep) | put;
+                ++n;
+              }
+            }
+          }
+          if (more && n <= MergeCand::MAX) {
+#pragma unroll
+            for (int k = 0; k < MergeCand::MAX; ++k) mc.c[k] = (uint16_t)((k < 4 ? lo : hi) >> (16 * (k & 3)));
+            mc.all = 0;
+          }
+        }
+        if (want) cand[(size_t)j * n_v + a] = mc;
       }
       fence_before();
       mbar_arrive(tempty);
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
-    if (ok && want) {
-      const bool clear = v1 - v2 > (float)d * 0x1p-23f * sqrtf(nrm_s[r]);  // false with a NaN or an infinite norm
-      cand[(size_t)j * n_v + a] = make_int2(b1, clear ? -1 : b2);
-    }
   }
   fence_before();
   __syncthreads();
@@ -1322,7 +1361,7 @@ __global__ void wait_timeout_check_kernel() {
 
 int launch_merge_screen(const uint16_t* X, int N, int n_v, int d, const int* kept, const int* n_kept,
                         const int* sel_off, const int* ctx_off, int max_ctx, const uint16_t* targets,
-                        const float* tinv, const int* rest, int2* cand, cudaStream_t st) {
+                        const float* tinv, const int* rest, MergeCand* cand, cudaStream_t st) {
   using namespace tc;
   CUtensorMap mt;
   if (!make_map(&mt, targets, (uint64_t)d, (uint64_t)max_ctx, ms::BROWS, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16)) return 1;

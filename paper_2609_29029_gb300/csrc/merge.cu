@@ -9,11 +9,11 @@
 //                         32-term chunks, a running top 2 per token; the two are recomputed as
 //                         float-float sums (good to ~2^-44) and compared as x.t1 / ||t1|| vs
 //                         x.t2 / ||t2|| in fp64, so the decision is the cosine argmax of the exact
-//                         arithmetic (ties to the lower target)
-//   (bf16 tokens) merge_screen_kernel (gemm_tc.cu) takes the top 2 from a tcgen05 product of
-//                         each 128-token block with the slot's target rows, and
-//                         merge_decide_kernel makes the same float-float decision between the two
-//                         where they are closer than the product's error bound
+//                         arithmetic (ties to the lower target) unless three targets are closer to each
+//                         other than the fp32 sums' error, when the best may not be among the two
+//   (bf16 tokens) merge_screen_kernel (gemm_tc.cu) lists the targets whose tcgen05 product is
+//                         within its error bound of the best one's, for each 128 tokens of a slot, and
+//                         merge_decide_kernel makes the same float-float decision among them
 //   merge_mean_kernel     per contextual token: its members in ascending token index, the fp32 sum
 //                         of their rows in that order, divided by the group size, stored as bf16
 #include <type_traits>
@@ -232,14 +232,60 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
   }
 }
 
-// Grid (blocks of 64 unselected positions, kept slot), 8 warps: assign[j][a] = the screened target where
-// the screening was clear (cand[j][a].y < 0); the others are listed and the warps take them in turn: the
-// better of the two candidates at ~fp64 accuracy, x.t1 / ||t1|| vs x.t2 / ||t2|| from float-float dot
-// products (ties to the lower target), the lanes' pairs summed in fp64.  24 us
-// at 400 tiles, against 111 with a second look at every token.
+// Grid (blocks of 64 unselected positions, kept slot), 8 warps: assign[j][a] = the screened target where no other is
+// within the screening's error of it; the other tokens are listed and the warps take them in turn: the
+// best of the candidates at ~fp64 accuracy, x.t / ||t|| from float-float dot products with the lanes' pairs
+// summed in fp64 (ties to the lower target).  Candidates: the screening's list, or, where it is longer than that
+// (near-duplicate targets, tokens next to zero), all targets of the slot but those whose row is
+// a copy of an earlier target's (blank parts of a tile), which a tie never chooses; the warps share these.  34 us
+// at 400 tiles (about 12% of the tokens have a list, most of two), against 111 with a second look at every token.
 // Targets keep their own group.
 constexpr int DT = 256;
-__global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
+
+// Whether two rows hold the same bits (b null: whether the row is all zeros, of either sign), by one warp.
+__device__ __forceinline__ bool same_row(const uint16_t* a, const uint16_t* b, int d, int lane) {
+  for (int k = lane * 8; k < (d + 255) / 256 * 256; k += 256) {
+    uint32_t differ = 0u;
+    if (k < d) {
+      const uint4 x = *reinterpret_cast<const uint4*>(a + k);
+      const uint4 y = b ? *reinterpret_cast<const uint4*>(b + k) : make_uint4(0u, 0u, 0u, 0u);
+      differ = ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) & (b ? 0xffffffffu : 0x7fff7fffu);
+    }
+    if (__any_sync(0xffffffffu, differ != 0u)) return false;
+  }
+  return true;
+}
+
+// x.t1 and x.t2 by one warp, four steps' loads ahead of the serial chains.
+__device__ __forceinline__ double2 ff_dots(const uint16_t* x, const uint16_t* t1, const uint16_t* t2, int d, int lane) {
+  float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
+  for (int k0 = lane * 8; k0 < d; k0 += 4 * 256) {
+    uint4 xr[4], r1[4], r2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k0 + u * 256 < d) {
+        xr[u] = *reinterpret_cast<const uint4*>(x + k0 + u * 256);
+        r1[u] = *reinterpret_cast<const uint4*>(t1 + k0 + u * 256);
+        r2[u] = *reinterpret_cast<const uint4*>(t2 + k0 + u * 256);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (k0 + u * 256 < d) {
+        float xv[8], y1[8], y2[8];
+        unpack_bf16x8(xr[u], xv);
+        unpack_bf16x8(r1[u], y1);
+        unpack_bf16x8(r2[u], y2);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          ff_step(xv[e], y1[e], h1, l1);
+          ff_step(xv[e], y2[e], h2, l2);
+        }
+      }
+  }
+  return ff_warp_sum2(h1, l1, h2, l2);
+}
+
+__global__ void __launch_bounds__(DT, 2) merge_decide_kernel(const uint16_t* __restrict__ X, int n_v, int d,
                                                            const int* __restrict__ kept,
                                                            const int* __restrict__ n_kept,
                                                            const int* __restrict__ sel_off,
@@ -247,9 +293,13 @@ __global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __rest
                                                            const int* __restrict__ rest,
                                                            const int* __restrict__ ctx_target,
                                                            const double* __restrict__ tnorm,
-                                                           const int2* __restrict__ cand, int* __restrict__ assign) {
-  __shared__ int4 open[64];  // (position, candidate 1, candidate 2) of the block's undecided tokens
-  __shared__ int n_open;
+                                                           const MergeCand* __restrict__ cand, int* __restrict__ assign) {
+  __shared__ int open[64];        // the block's undecided tokens: those with a list from the front, those with all
+  __shared__ MergeCand list[64];  // targets for candidates from the back, and their lists
+  __shared__ int n_open, n_all;
+  __shared__ unsigned char dup[RIFT_MAX_NV];  // target q's row is an earlier target's
+  __shared__ double part_e[DT / 32], part_n[DT / 32];  // the warps' best among their share of all targets
+  __shared__ int part_q[DT / 32];
   pdl_trigger();
   pdl_wait();
   const int j = blockIdx.y, a0 = blockIdx.x * 64;
@@ -259,57 +309,89 @@ __global__ void __launch_bounds__(DT) merge_decide_kernel(const uint16_t* __rest
   if (m == 0 || co + m > max_ctx || a0 >= R) return;
   const int step = R / m;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) n_open = 0;
+  if (threadIdx.x == 0) n_open = n_all = 0;
   __syncthreads();
   const int al = a0 + threadIdx.x;
   if (threadIdx.x < 64 && al < R && !(al % step == 0 && al / step < m)) {
-    int2 c = cand[(size_t)j * n_v + al];
-    if (c.x < 0 || c.x >= m) {  // no finite similarity (a NaN token): the first target
+    const MergeCand c = cand[(size_t)j * n_v + al];
+    if (c.c[0] >= m) {  // no finite similarity (a NaN token): the first target
       atomicOr(&g_err_merge, RIFT_EBIT_NONFINITE);
-      c = make_int2(0, -1);
+      assign[(size_t)j * n_v + al] = 0;
+    } else if (c.c[1] >= m && !c.all) {
+      assign[(size_t)j * n_v + al] = c.c[0];
+    } else {
+      const int at = c.all ? 63 - atomicAdd(&n_all, 1) : atomicAdd(&n_open, 1);
+      open[at] = al;
+      list[at] = c;
     }
-    if (c.y >= 0 && c.y < m) open[atomicAdd(&n_open, 1)] = make_int4(al, c.x, c.y, 0);
-    else assign[(size_t)j * n_v + al] = c.x;
   }
   __syncthreads();
   const uint16_t* Xt = X + (size_t)kept[j] * n_v * d;
+  const int* target = ctx_target + co;
+  const double* norm = tnorm + co;
+  auto row = [&](int q) { return Xt + (size_t)target[q] * d; };
+  // s1 = e1 / n1 vs s2 = e2 / n2 as e1 n2 vs e2 n1 (norms are positive; a zero target has similarity 0)
+  struct Best {
+    int q;
+    double e, n;
+    __device__ void offer(double e2, double norm2, int q2) {
+      const double e0 = norm2 > 0.0 ? e2 : 0.0, n0 = norm2 > 0.0 ? norm2 : 1.0;
+      const double s = e0 * n, s_best = e * n0;
+      if (e0 == e0 && (q < 0 || s > s_best || (s == s_best && q2 < q))) {
+        q = q2;
+        e = e0;
+        n = n0;
+      }
+    }
+  };
   for (int i = warp; i < n_open; i += DT / 32) {
-    const int4 o = open[i];
-    const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + o.x] * d;
-    const uint16_t* t1 = Xt + (size_t)ctx_target[co + o.y] * d;
-    const uint16_t* t2 = Xt + (size_t)ctx_target[co + o.z] * d;
-    float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
-    for (int k0 = lane * 8; k0 < d; k0 += 4 * 256) {
-      uint4 xr[4], r1[4], r2[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (k0 + u * 256 < d) {
-          xr[u] = *reinterpret_cast<const uint4*>(x + k0 + u * 256);
-          r1[u] = *reinterpret_cast<const uint4*>(t1 + k0 + u * 256);
-          r2[u] = *reinterpret_cast<const uint4*>(t2 + k0 + u * 256);
-        }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (k0 + u * 256 < d) {
-          float xv[8], y1[8], y2[8];
-          unpack_bf16x8(xr[u], xv);
-          unpack_bf16x8(r1[u], y1);
-          unpack_bf16x8(r2[u], y2);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            ff_step(xv[e], y1[e], h1, l1);
-            ff_step(xv[e], y2[e], h2, l2);
-          }
-        }
+    const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + open[i]] * d;
+    Best best = {-1, 0.0, 1.0};
+    for (int k = 0; k < MergeCand::MAX; k += 2) {
+      const int t1 = list[i].c[k], t2 = k + 1 < MergeCand::MAX && list[i].c[k + 1] < m ? list[i].c[k + 1] : t1;
+      if (t1 >= m) break;
+      const double2 e = ff_dots(x, row(t1), row(t2), d, lane);
+      best.offer(e.x, norm[t1], t1);
+      best.offer(e.y, norm[t2], t2);
     }
-    const double2 dots = ff_warp_sum2(h1, l1, h2, l2);
+    if (lane == 0) assign[(size_t)j * n_v + open[i]] = best.q < 0 ? list[i].c[0] : best.q;
+  }
+  if (n_all == 0) return;
+  for (int q = warp; q < m; q += DT / 32) {  // a copy has its original's norm, bit for bit
+    bool copy = false;
+    const long long nq = __double_as_longlong(norm[q]);
+    for (int p0 = 0; p0 < q && !copy; p0 += 32) {
+      const int p = p0 + lane;
+      unsigned eq = __ballot_sync(0xffffffffu, p < q && __double_as_longlong(norm[p < q ? p : q]) == nq);
+      for (; eq && !copy; eq &= eq - 1) copy = same_row(row(p0 + __ffs(eq) - 1), row(q), d, lane);
+    }
+    if (lane == 0) dup[q] = copy;
+  }
+  __syncthreads();
+  for (int i = 0; i < n_all; ++i) {  // the warps share the targets, two at a time
+    const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + open[63 - i]] * d;
+    const bool zero = same_row(x, nullptr, d, lane);  // all similarities are 0: the first target
+    Best best = {-1, 0.0, 1.0};
+    for (int q = 2 * warp; q < m && !zero; q += 2 * (DT / 32)) {
+      const bool u1 = !dup[q], u2 = q + 1 < m && !dup[q + 1];
+      if (!u1 && !u2) continue;
+      const int t1 = u1 ? q : q + 1, t2 = u2 ? q + 1 : q;
+      const double2 e = ff_dots(x, row(t1), row(t2), d, lane);
+      best.offer(e.x, norm[t1], t1);
+      best.offer(e.y, norm[t2], t2);
+    }
     if (lane == 0) {
-      // s1 = e1 / n1 vs s2 = e2 / n2 as e1 n2 vs e2 n1 (norms are positive; a zero target has similarity 0)
-      const double n1 = tnorm[co + o.y], n2 = tnorm[co + o.z];
-      const double e1 = n1 > 0.0 ? dots.x : 0.0, e2 = n2 > 0.0 ? dots.y : 0.0;
-      const double s1 = e1 * (n2 > 0.0 ? n2 : 1.0), s2 = e2 * (n1 > 0.0 ? n1 : 1.0);
-      assign[(size_t)j * n_v + o.x] = s2 > s1 || (s2 == s1 && o.z < o.y) ? o.z : o.y;
+      part_q[warp] = best.q;
+      part_e[warp] = best.e;
+      part_n[warp] = best.n;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < DT / 32; ++w)
+        if (part_q[w] >= 0) best.offer(part_e[w], part_n[w], part_q[w]);
+      assign[(size_t)j * n_v + open[63 - i]] = best.q < 0 ? list[63 - i].c[0] : best.q;
+    }
+    __syncthreads();
   }
 }
 
@@ -578,7 +660,7 @@ MergeLayout merge_layout(int N, int n_v) {
   L.assign_off = take((size_t)N * n_v * sizeof(int));
   L.tnorm_off = take((size_t)N * n_v * sizeof(double));
   L.tinv_off = take((size_t)N * n_v * sizeof(float));  // at most n_v - 1 targets per slot
-  L.cand_off = take((size_t)N * n_v * sizeof(int2));
+  L.cand_off = take((size_t)N * n_v * sizeof(MergeCand));
   L.total = off;
   return L;
 }
@@ -592,7 +674,7 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
   int* assign = reinterpret_cast<int*>(ws + L.assign_off);
   double* tnorm = reinterpret_cast<double*>(ws + L.tnorm_off);
   float* tinv = reinterpret_cast<float*>(ws + L.tinv_off);
-  int2* cand = reinterpret_cast<int2*>(ws + L.cand_off);
+  MergeCand* cand = reinterpret_cast<MergeCand*>(ws + L.cand_off);
   // every kernel a programmatic dependent of the one before it
   bool ok = launch_ex(merge_plan_kernel, dim3(1), dim3(1024), 0, st, true, n_kept, budgets, sel_off, N, n_v, max_ctx,
                       ctx_off) == cudaSuccess;
@@ -609,7 +691,7 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
         ok = ok && launch_merge_screen(x, N, n_v, d, kept, n_kept, sel_off, ctx_off, max_ctx, ctx, tinv, rest, cand, st) == 0;
       ok = ok && launch_ex(merge_decide_kernel, dim3((n_v + 63) / 64, N), dim3(DT), 0, st, true, x, n_v, d, kept,
                            n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
-                           (const double*)tnorm, (const int2*)cand, assign) == cudaSuccess;
+                           (const double*)tnorm, (const MergeCand*)cand, assign) == cudaSuccess;
     } else {
       static std::atomic<unsigned long long> smem_raised{0};
       const size_t ab_bytes = 2 * (size_t)KC * (TB + 4) * sizeof(float);

@@ -166,14 +166,18 @@ int launch_gemm(const void* A, const void* B, int M, int N, int K, int epi, void
 int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, void* C, const EpiParams& ep,
                    cudaStream_t st, bool pdl = false, bool b_const = true);
 int launch_wait_timeout_check(cudaStream_t st);
-// Merge screening on the tensor cores (bf16 tokens): per kept slot and 128 of its unselected tokens, the
-// two best merge targets (by x.t / ||t||) of every non-target token, the second -1 where the first
-// is clear of it by more than the product's error bound.  targets: bf16 [max_ctx, d] target rows;
-// tinv [max_ctx] = 1 / ||t||; rest [N, n_v] = the slot's unselected tokens (ascending); cand [N, n_v]
-// out, indexed as rest.
+// Merge screening on the tensor cores (bf16 tokens): per kept slot and 128 of its unselected tokens, the merge targets
+// that may be the best of every non-target token.  cand [N, n_v] out, indexed as rest.  targets: bf16 [max_ctx, d]
+// target rows; tinv [max_ctx] = 1 / ||t||; rest [N, n_v] = the slot's unselected tokens (ascending).
+struct alignas(16) MergeCand {
+  static constexpr int MAX = 7;
+  static constexpr uint16_t NONE = 0xffff;
+  uint16_t c[MAX];  // the best target by the product (NONE: no finite similarity), then those within its error; NONE
+  uint16_t all;     // 1: every target is a candidate
+};
 int launch_merge_screen(const uint16_t* X, int N, int n_v, int d, const int* kept, const int* n_kept,
                         const int* sel_off, const int* ctx_off, int max_ctx, const uint16_t* targets,
-                        const float* tinv, const int* rest, int2* cand, cudaStream_t st);
+                        const float* tinv, const int* rest, MergeCand* cand, cudaStream_t st);
 
 // Varlen causal attention (attention_tc.cu): q-block schedule built once per prefill from
 // cu_seqlens, then one launch per layer.  qkv fp16 [T, 3 d], out fp16 [T, d].

@@ -1,8 +1,8 @@
 """The merge's choice between close targets (bf16 tokens): the tensor-core screening decides alone only
-where its best target is clear of the second by more than its error bound, everything else is
+where its best target is clear of the others by more than its error bound, everything else is
 decided by float-float sums.  Tiles of near-duplicate tokens (cosine gaps from 1e-2 down to 1e-8) and
-exact duplicates (ties to the lower target), one, few and more than 128 targets per slot, against
-the oracle's groups: a wrong choice moves a group's mean far outside one bf16 spacing."""
+exact duplicates (ties to the lower target), one, few and more than 128 targets per slot: every token's
+assignment, as the call leaves it in its workspace, against the oracle's groups, and the groups' means."""
 import pytest
 import torch
 
@@ -51,7 +51,14 @@ def test_close_targets(n_v, d, m, protos, bits, cuda, riftlib):
                              torch.tensor(off, **i32), ctx, 2 * m, ctx_off, ctx_target, ws, need)
     riftlib.sync_status()
     assert ctx_off.cpu().tolist() == [0, m, 2 * m]
-    for t, (targets, _, mean) in enumerate(ref):
+    off = (2 * n_v * 4 + 255) // 256 * 256  # the unselected tokens' lists, then the assignments
+    assign = ws[off:off + 2 * n_v * 4].view(torch.int32).view(2, n_v).cpu()
+    for t, (targets, groups, mean) in enumerate(ref):
+        rest = [k for k in range(n_v) if k not in set(dom[t])]
+        want = {k: q for q, gr in enumerate(groups) for k in gr[1:]}
+        assert len(want) == len(rest) - m
+        wrong = [(k, int(assign[t, a]), want[k]) for a, k in enumerate(rest) if k in want and int(assign[t, a]) != want[k]]
+        assert not wrong, (t, len(wrong), wrong[:5])
         assert ctx_target[t * m:(t + 1) * m].cpu().tolist() == targets
         got = ctx[t * m:(t + 1) * m].cpu().double()
         assert bool(((got - mean).abs() <= mean.abs().clamp_min(1e-30) * 2.0 ** -7).all()), t
