@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <cmath>
 
 #include "rift.h"
 
@@ -119,34 +120,41 @@ struct RopeFreq {
   double inv[64];
 };
 
-// (cos, sin) of x >= 0 (up to ~1e5), each rounded once to fp32 from a double good to ~1e-12: x reduced
+// (cos, sin) of x >= 0 in double, good to ~2e-16 for x up to 2^31 and beyond: x reduced
 // by the nearest multiple k of pi/2 (Cody and Waite's two-part reduction, its constants the leading
 // bits of pi/2 and the rest), then the Taylor polynomials on |r| <= pi/4 (the first terms left out,
-// r^15 / 15! and r^14 / 14!, are below 4e-13).  A GB300 SM retires about two double operations a cycle,
-// so they are what a RoPE table costs: this takes about 20 a value, the library's pow and sincos
-// per value about 160 (a 131 x 64 table 11.6 us; now 4.1 us together with the attention schedule, whose own
-// launch took 3.7; a decode step's start, which needs one row per sequence, 29.6 -> 7.5 us for one
-// sequence of 635 rows).
-__device__ __forceinline__ float2 rope_cos_sin(double x) {
+// r^17 / 17! and r^18 / 18!, are below 5e-17).
+__host__ __device__ __forceinline__ double2 rope_cos_sin_f64(double x) {
   const double two_over_pi = 0.63661977236758134308, pio2 = 1.57079632679489661923, pio2_rest = 6.123233995736766e-17;
   const double k = rint(x * two_over_pi);
   const double r = fma(-k, pio2_rest, fma(-k, pio2, x));
   const double z = r * r;
-  double s = fma(z, 1.0 / 6227020800.0, -1.0 / 39916800.0);
+  double s = fma(z, -1.0 / 1307674368000.0, 1.0 / 6227020800.0);
+  s = fma(z, s, -1.0 / 39916800.0);
   s = fma(z, s, 1.0 / 362880.0);
   s = fma(z, s, -1.0 / 5040.0);
   s = fma(z, s, 1.0 / 120.0);
   s = fma(z, s, -1.0 / 6.0);
   s = fma(z * r, s, r);
-  double c = fma(z, 1.0 / 479001600.0, -1.0 / 3628800.0);
+  double c = fma(z, 1.0 / 20922789888000.0, -1.0 / 87178291200.0);
+  c = fma(z, c, 1.0 / 479001600.0);
+  c = fma(z, c, -1.0 / 3628800.0);
   c = fma(z, c, 1.0 / 40320.0);
   c = fma(z, c, -1.0 / 720.0);
   c = fma(z, c, 1.0 / 24.0);
   c = fma(z, c, -0.5);
   c = fma(z, c, 1.0);
-  const float cf = (float)c, sf = (float)s;
-  const int q = (int)k & 3;  // x = r + q pi/2 (mod 2 pi)
-  return make_float2(q == 0 ? cf : q == 1 ? -sf : q == 2 ? -cf : sf, q == 0 ? sf : q == 1 ? cf : q == 2 ? -sf : -cf);
+  const int q = (int)((long long)k & 3);  // x = r + q pi/2 (mod 2 pi)
+  return make_double2(q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s, q == 0 ? s : q == 1 ? c : q == 2 ? -s : -c);
+}
+// The same, each rounded once to fp32.  A GB300 SM retires about two double operations a cycle,
+// so they are what a RoPE table costs: this takes about 23 a value, the library's pow and sincos
+// per value about 160 (a 131 x 64 table 11.6 us; now 4.3 us together with the attention schedule, whose own
+// launch took 3.7; a decode step's start, which needs one row per sequence, 29.6 -> 8.0 us for one
+// sequence of 635 rows).
+__device__ __forceinline__ float2 rope_cos_sin(double x) {
+  const double2 v = rope_cos_sin_f64(x);
+  return make_float2((float)v.x, (float)v.y);
 }
 
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
