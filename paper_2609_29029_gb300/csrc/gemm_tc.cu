@@ -5,7 +5,8 @@
 // k, fp32 residual add, SwiGLU over 16-column gate/up groups).  Two kernels:
 //
 // gemm_tc_kernel (many rows: the prefill of a scene): persistent and warp-specialised on SM pairs
-// (2-CTA clusters, 256 x 256 tiles, or 256 x 192: tile_width), 192 threads per CTA:
+// (2-CTA clusters, 256 x 256 tiles, or 256 x 192: tile_width), or on single SMs where 128 x 256 tiles take
+// fewer waves (one_sm_tiles), 192 threads per CTA:
 //   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 6-stage shared-memory ring
 //   warp 1      allocates 512 TMEM columns; the even CTA's issues tcgen05.mma (cta_group::2, M = 256,
 //               N = 256, K = 16) into one of two 256-column fp32 accumulators and commits to
@@ -29,6 +30,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "rift_internal.h"
@@ -46,9 +48,11 @@ unsigned int read_clear_err_gemm() {
 
 namespace tc {
 
-constexpr int BM = 128, BN = 256, NARROW_BN = 192, BK = 64, STAGES = 6;
+constexpr int BM = 128, BN = 256, NARROW_BN = 192, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;  // 16 KB
 constexpr int THREADS = 192;
+// Depth of the ring of K-blocks: as deep as shared memory allows, 32 KB a CTA of a pair (cg = 2), 48 KB a CTA alone.
+__host__ __device__ constexpr int ring_stages(int cg) { return cg == 2 ? 6 : 4; }
 // Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A fp16 (bits
 // 7-9 = 0), B fp16 (bits 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4
 // at bits 24-28.
@@ -362,13 +366,16 @@ __device__ __forceinline__ int tile_width(int mt, int N, int pairs) {
 // rows of A and half of the tile's B rows per k-block, half the B traffic of one SM per tile row, and
 // the even CTA issues the M = 256 MMAs into both SMs' tensor memory.  tmN: the B map with boxes of the
 // narrower tile's half.
-template <int EPI>
+// CG = 1 (one_sm_tiles): one SM a tile, 128 x 256, all of the tile's B rows staged by its CTA; no clusters, no
+// narrower tiles, tmB with boxes of a whole tile.
+template <int EPI, int CG>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmN, int M_cap, int N, int K, void* C, const EpiParams ep,
                    int group_m) {
-  constexpr int TM = 2 * BM;      // rows of a tile (both CTAs of the pair)
-  constexpr int B_ROWS = BN / 2;  // B rows staged by this CTA
+  constexpr int TM = CG * BM;      // rows of a tile (both CTAs of the pair)
+  constexpr int B_ROWS = BN / CG;  // B rows staged by this CTA
+  constexpr int STAGES = ring_stages(CG);
   constexpr int B_BYTES = B_ROWS * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
   constexpr int ACC_COLS = BN, TMEM_COLS = 2 * ACC_COLS;
   extern __shared__ uint8_t smem_raw[];
@@ -392,19 +399,26 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull_bar(b), 1);
-      mbar_init(tempty_bar(b), 256);  // the epilogue threads of both CTAs
+      mbar_init(tempty_bar(b), 128 * CG);  // the epilogue threads of the tile's CTAs
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   }
-  const uint32_t rank = cluster_ctarank();
-  cluster_sync();  // both CTAs' barriers initialised before any remote arrival
+  const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
+  if constexpr (CG == 2) cluster_sync();  // both CTAs' barriers initialised before any remote arrival
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                 "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+    if constexpr (CG == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                   "r"(TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
   }
   fence_before();
   __syncthreads();
@@ -421,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   asm volatile("mov.s32 %0, 0;" : "=r"(kb0));
   const int mt = (M + TM - 1) / TM, kt = (K + BK - 1) / BK;
   int bn = BN;  // the RoPE epilogue wants whole heads in a tile, the symmetric product square tiles
-  if constexpr (EPI != EPI_QKV_ROPE)
+  if constexpr (EPI != EPI_QKV_ROPE && CG == 2)
     if (!ep.symmetric) bn = tile_width(mt, N, (int)(gridDim.x >> 1));
   const int nt = (N + bn - 1) / bn;
   const int n_tiles = ep.symmetric ? mt * (mt + 1) / 2 : mt * nt;
@@ -430,7 +444,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     else tile_coords(tile, mt, nt, group_m, m_blk, n_blk);
   };
   // the pair walks the tiles together, one tile per cluster
-  const int u_first = (int)(blockIdx.x >> 1), u_step = (int)(gridDim.x >> 1);
+  const int u_first = (int)blockIdx.x / CG, u_step = (int)gridDim.x / CG;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -445,12 +459,17 @@ __global__ void __launch_bounds__(THREADS, 1)
           const int s = it % STAGES;
           const uint32_t round = it / STAGES;
           if (!mbar_wait(empty_bar(s), (round & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t fb = mapa_shared(full_bar(s), 0);
-          if (rank == 0) mbar_expect_tx(full_bar(s), 2 * A_BYTES + bn * BK * 2);
-          tma_load_2d_pair(smem_u32(sA + s * A_BYTES), &tmA, kblock(ep.kmap_a, ep.kmap_d, k) * BK,
-                           m_blk * TM + (int)rank * BM, fb);
-          tma_load_2d_pair(smem_u32(sB + s * B_BYTES), EPI == EPI_QKV_ROPE || bn == BN ? &tmB : &tmN,
-                           kblock(ep.kmap_b, ep.kmap_d, k) * BK, n_blk * bn + (int)rank * (bn >> 1), fb);
+          const int ka = kblock(ep.kmap_a, ep.kmap_d, k) * BK, kb = kblock(ep.kmap_b, ep.kmap_d, k) * BK;
+          if (rank == 0) mbar_expect_tx(full_bar(s), CG * A_BYTES + bn * BK * 2);
+          if constexpr (CG == 2) {
+            const uint32_t fb = mapa_shared(full_bar(s), 0);
+            tma_load_2d_pair(smem_u32(sA + s * A_BYTES), &tmA, ka, m_blk * TM + (int)rank * BM, fb);
+            tma_load_2d_pair(smem_u32(sB + s * B_BYTES), EPI == EPI_QKV_ROPE || bn == BN ? &tmB : &tmN, kb,
+                             n_blk * bn + (int)rank * (bn >> 1), fb);
+          } else {
+            tma_load_2d(smem_u32(sA + s * A_BYTES), &tmA, ka, m_blk * TM, full_bar(s));
+            tma_load_2d(smem_u32(sB + s * B_BYTES), &tmB, kb, n_blk * BN, full_bar(s));
+          }
         }
       }
       // Before leaving, make sure no copy this thread issued is still in flight (bounded): the
@@ -484,12 +503,17 @@ __global__ void __launch_bounds__(THREADS, 1)
           if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)  // +32 bytes along K per step (encoded >> 4)
-              umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, (k != kb0 || kk != 0) ? 1u : 0u);
-            umma_commit_pair(empty_bar(s));
+              if constexpr (CG == 2) umma_f16_pair(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, (k != kb0 || kk != 0) ? 1u : 0u);
+              else umma_f16(tmem_d, ad + 2 * kk, bd + 2 * kk, idesc, (k != kb0 || kk != 0) ? 1u : 0u);
+            if constexpr (CG == 2) umma_commit_pair(empty_bar(s));
+            else umma_commit(empty_bar(s));
           }
           __syncwarp();
         }
-        if (ok && elect_one()) umma_commit_pair(tfull_bar(b));
+        if (ok && elect_one()) {
+          if constexpr (CG == 2) umma_commit_pair(tfull_bar(b));
+          else umma_commit(tfull_bar(b));
+        }
         __syncwarp();
       }
       // the last two accumulators' releases (the odd CTA's arrivals among them) have landed
@@ -500,7 +524,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else {
     // ---------------- epilogue (warps 2..5 -> TMEM lane quarters 2, 3, 0, 1)
     const int quarter = warp & 3;
-    const uint32_t tempty_even0 = mapa_shared(tempty_bar(0), 0), tempty_even1 = mapa_shared(tempty_bar(1), 0);
+    const uint32_t tempty_even0 = CG == 2 ? mapa_shared(tempty_bar(0), 0) : tempty_bar(0);
+    const uint32_t tempty_even1 = CG == 2 ? mapa_shared(tempty_bar(1), 0) : tempty_bar(1);
     int tl = 0;
     for (int u = u_first; u < n_tiles; u += u_step, ++tl) {
       int m_blk, n_blk;
@@ -558,16 +583,21 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       fence_before();
-      mbar_arrive_cluster(b ? tempty_even1 : tempty_even0);
+      if constexpr (CG == 2) mbar_arrive_cluster(b ? tempty_even1 : tempty_even0);
+      else mbar_arrive(b ? tempty_even1 : tempty_even0);
     }
   }
   fence_before();
   __syncthreads();
-  cluster_sync();  // neither CTA frees its tensor memory or exits before the other is done
+  if constexpr (CG == 2) cluster_sync();  // neither CTA frees its tensor memory or exits before the other is done
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
-                 : "memory");
+    if constexpr (CG == 2)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
+                   : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(TMEM_COLS)
+                   : "memory");
   }
 }
 
@@ -1222,8 +1252,8 @@ static int band_group(int M, int N, int K, int tm, int tn, int lo, int hi) {
 template <int EPI>
 static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& bn, int M, int N, int K, void* C,
                        const EpiParams& ep, cudaStream_t st, bool pdl) {
-  constexpr size_t smem = (size_t)STAGES * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
-  auto kern = gemm_tc_kernel<EPI>;
+  constexpr size_t smem = (size_t)ring_stages(2) * (A_BYTES + (BN / 2) * BK * 2) + 1024 + 256;
+  auto kern = gemm_tc_kernel<EPI, 2>;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
@@ -1263,6 +1293,31 @@ static int launch_pair(const CUtensorMap& a, const CUtensorMap& b, const CUtenso
                  cudaSuccess
              ? 0
              : 1;
+}
+
+// Whether 128 x 256 tiles on one SM each are the faster ones for fewer than 1024 rows: where they take fewer waves than the
+// pairs' tiles by more than their waves are slower, a third (a pair shares its B tile).  257 .. 384 rows fill one and a
+// half of the pairs' row tiles, 769 .. 896 three and a half.  us, pairs against one SM: 300 rows QKV (2 waves, 1) 49.2 : 45.1,
+// gate/up (3, 2) 78.2 : 71.7, 24576 x 8192 (3, 2) 135 : 125; 777 x 5120 x 4096 (2, 1) 45.1 : 38.9; 600 rows of gate/up (4, 3)
+// 94.2 : 94.2, which stays with the pairs.
+static bool one_sm_tiles(int M, int N, int sms) {
+  if (M >= 1024) return false;
+  const long long nt = (N + BN - 1) / BN;
+  const long long one = ((M + BM - 1) / BM * nt + sms - 1) / sms;
+  const long long pair = ((M + 2 * BM - 1) / (2 * BM) * nt + sms / 2 - 1) / (sms / 2);
+  return 4 * one < 3 * pair;
+}
+
+// One SM a tile, persistent.  b: the B map with boxes of a whole tile.
+template <int EPI>
+static int launch_single(const CUtensorMap& a, const CUtensorMap& b, int M, int N, int K, void* C, const EpiParams& ep,
+                         cudaStream_t st, bool pdl) {
+  constexpr size_t smem = (size_t)ring_stages(1) * (A_BYTES + BN * BK * 2) + 1024 + 256;
+  static std::atomic<unsigned long long> smem_raised{0};
+  if (raise_smem_limit(smem_raised, gemm_tc_kernel<EPI, 1>, (int)smem) != cudaSuccess) return 1;
+  const int units = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+  return launch_ex(gemm_tc_kernel<EPI, 1>, dim3(std::min(units, sm_count())), dim3(THREADS), smem, st, pdl, a, b, b, M, N, K, C,
+                   ep, band_group(M, N, K, BM, BN, 4, 32)) != cudaSuccess;
 }
 
 // Stands for gemm_ck_kernel in the question below: the driver counts a kernel with tcgen05.alloc as one CTA an SM,
@@ -1400,9 +1455,19 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   if (M <= ck::MAX_BN || plan.one_round || (epi == EPI_STORE_F32 && ep.m_dev && M < 1024))
     return launch_ck_epi(A, B, Ks, M, N, K, epi, C, ep, st, plan, pdl, b_const ? 1 : 0);
   CUtensorMap ma, mb, mn;
-  if (!make_map(&ma, A, Ks, (uint64_t)M, BM) || !make_map(&mb, B, Ks, (uint64_t)N, BN / 2) ||
-      !make_map(&mn, B, Ks, (uint64_t)N, NARROW_BN / 2))
-    return 1;
+  if (!make_map(&ma, A, Ks, (uint64_t)M, BM)) return 1;
+  if (!ep.symmetric && one_sm_tiles(M, N, sm_count())) {
+    if (!make_map(&mb, B, Ks, (uint64_t)N, BN)) return 1;
+    switch (epi) {
+      case EPI_STORE_BF16: return launch_single<EPI_STORE_BF16>(ma, mb, M, N, K, C, ep, st, pdl);
+      case EPI_RESID_F32: return launch_single<EPI_RESID_F32>(ma, mb, M, N, K, C, ep, st, pdl);
+      case EPI_SWIGLU: return launch_single<EPI_SWIGLU>(ma, mb, M, N, K, C, ep, st, pdl);
+      case EPI_QKV_ROPE: return launch_single<EPI_QKV_ROPE>(ma, mb, M, N, K, C, ep, st, pdl);
+      case EPI_STORE_F32: return launch_single<EPI_STORE_F32>(ma, mb, M, N, K, C, ep, st, pdl);
+      default: return 1;
+    }
+  }
+  if (!make_map(&mb, B, Ks, (uint64_t)N, BN / 2) || !make_map(&mn, B, Ks, (uint64_t)N, NARROW_BN / 2)) return 1;
   int r = -1;
   switch (epi) {
     case EPI_STORE_BF16: r = launch_pair<EPI_STORE_BF16>(ma, mb, mn, M, N, K, C, ep, st, pdl); break;

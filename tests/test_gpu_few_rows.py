@@ -26,6 +26,8 @@ SHAPES += [(48, 128, 200), (49, 136, 64), (300, 256, 256), (1000, 264, 72), (102
 SHAPES += [(768, 2432, 200), (769, 2432, 200), (4400, 2056, 1032)]
 # tiles whose count times the cluster size fits while the clusters do not (40 tiles: 38 clusters of 7 fit, 46 of 6)
 SHAPES += [(100, 5120, 4096), (777, 1024, 4104)]
+# 128 x 256 tiles of one SM (fewer waves than the pairs'): one and several tiles a CTA, tails in rows, weight rows and K
+SHAPES += [(257, 12288, 1032), (300, 12296, 1096), (384, 22016, 1032), (777, 5128, 1032)]
 
 
 def _rand(shape, stream, scale=1.0):
@@ -56,3 +58,30 @@ def test_few_rows_all_epilogues(M, N, K, cuda, riftlib):
         riftlib.sync_status()
         g, u = y.view(M, N // 32, 2, 16).unbind(2)
         assert _rel(act, (g / (1 + torch.exp(-g)) * u).reshape(M, N // 2)) < F16_TOL
+
+
+def test_one_sm_tiles_with_rope_and_cache(cuda, riftlib):
+    """The QKV product of 300 rows at d = 4096 runs on tiles of one SM, that of 600 rows on SM pairs: the same keys,
+    values and hidden states for the rows the two batches share."""
+    from paper_2609_29029_gb300 import DeviceModel
+    from synth import workloads as W
+    dec = W.DecoderShape(n_layers=1, d=4096, n_heads=32, head_dim=128, ffn=64, vocab=504)
+    dm = DeviceModel(dec, [W.make_layer(dec, 0, "cpu")], W.make_final_norm(dec, "cpu"), cuda)
+    rows = torch.randn(600, dec.d, device=cuda).to(torch.bfloat16)
+
+    def prefill(lens):
+        T, n = sum(lens), len(lens)
+        cu = torch.tensor([sum(lens[:i]) for i in range(n + 1)], dtype=torch.int32, device=cuda)
+        pos = torch.cat([torch.arange(L, dtype=torch.int32, device=cuda) for L in lens])
+        hid = rows[:T].clone()
+        kv = torch.full((1, 2, T, dec.d), float("nan"), dtype=torch.float16, device=cuda)
+        need = riftlib.prefill_workspace_bytes(dm.struct, T, n, max(lens))
+        ws = torch.empty(need, dtype=torch.uint8, device=cuda)
+        riftlib.prefill_layers(dm.struct, hid, T, cu, n, max(lens), pos, ws, need, kv_out=kv)
+        riftlib.sync_status()
+        return hid.float(), kv.float()
+
+    h1, kv1 = prefill([100, 31, 169])
+    h2, kv2 = prefill([100, 31, 169, 300])
+    assert float((kv1 - kv2[:, :, :300]).abs().max()) <= 2.0 ** -10 * float(kv1.abs().max())
+    assert float((h1 - h2[:300]).abs().max()) <= 2.0 ** -7 * float(h1.abs().max())
