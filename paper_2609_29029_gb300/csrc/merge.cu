@@ -78,21 +78,21 @@ __device__ __forceinline__ double2 ff_warp_sum2(float h1, float l1, float h2, fl
   return make_double2(__shfl_sync(0xffffffffu, acc, 0), __shfl_sync(0xffffffffu, acc, 16));
 }
 
-// Float-float accumulation of a.b over d terms by one warp, eight elements per lane and step, four
-// steps' loads ahead of the serial chain, then the lanes' pairs summed (~2^-44 relative).
-template <typename XT>
+// Float-float accumulation of a.b over d terms by one warp, eight elements per lane and step, U steps' loads ahead of
+// the serial chain, then the lanes' pairs summed (~2^-44 relative).
+template <int U, typename XT>
 __device__ double ff_dot(const XT* a, const XT* b, int d, int lane) {
   float hi = 0.f, lo = 0.f;
-  for (int k0 = lane * 8; k0 < d; k0 += 4 * 256) {
-    float x[4][8], y[4][8];
+  for (int k0 = lane * 8; k0 < d; k0 += U * 256) {
+    float x[U][8], y[U][8];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < U; ++u)
       if (k0 + u * 256 < d) {
         load8(a + k0 + u * 256, x[u]);
         load8(b + k0 + u * 256, y[u]);
       }
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < U; ++u)
       if (k0 + u * 256 < d) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) ff_step(x[u][e], y[u][e], hi, lo);
@@ -395,8 +395,14 @@ __global__ void __launch_bounds__(DT, 2) merge_decide_kernel(const uint16_t* __r
   }
 }
 
-// Grid (kept slot, block of TB unselected tokens).  assign[j][a] = target index of rest[a].
-template <typename XT>
+// Grid (block of TB unselected tokens, kept slot).  assign[j][a] = target index of rest[a].
+// U: steps of loads ahead in the float-float dot products.  Four hide their latency where a CTA has an SM to itself, but
+// take the registers of two more CTAs (164 against 80).  Launched without overlap: as a programmatic dependent its few
+// CTAs with work land on the SMs that the kernel before it leaves first, several to one.  us of an fp32 scene with
+// the merge at d = 4096, U = 4 : 1 (dependent launch, 1): 20 tiles of 100 tokens 378 : 429 (674), 64 of 576 722 : 726
+// (883), 250 of 200 569 : 744 (893), 150 of 576 925 : 1015 (1037), 300 of 576 1481 : 1306 (1331); 700 of 576 at d = 1024
+// 1101 : 1007 (1005).
+template <typename XT, int U>
 __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict__ X, int n_v, int d,
                                                            const int* __restrict__ kept,
                                                            const int* __restrict__ n_kept,
@@ -412,7 +418,6 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   __shared__ float best_v[TB][2];
   __shared__ int best_j[TB][2];
   __shared__ float inv_n[TB];
-  pdl_trigger();
   pdl_wait();
   const int j = blockIdx.y;  // the token blocks of one slot are adjacent: its target rows stay in L2
   if (j >= *n_kept) return;
@@ -518,8 +523,8 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
     const int j2 = best_j[row][1];
     if (j2 >= 0) {
       const int t1 = ctx_target[co + choice], t2 = ctx_target[co + j2];
-      const double d1 = ff_dot(Xt + (size_t)k * d, Xt + (size_t)t1 * d, d, lane);
-      const double d2 = ff_dot(Xt + (size_t)k * d, Xt + (size_t)t2 * d, d, lane);
+      const double d1 = ff_dot<U>(Xt + (size_t)k * d, Xt + (size_t)t1 * d, d, lane);
+      const double d2 = ff_dot<U>(Xt + (size_t)k * d, Xt + (size_t)t2 * d, d, lane);
       const double n1 = tnorm[co + choice], n2 = tnorm[co + j2];
       const double s1 = n1 > 0.0 ? d1 / n1 : 0.0, s2 = n2 > 0.0 ? d2 / n2 : 0.0;
       if (s2 > s1 || (s2 == s1 && j2 < choice)) choice = j2;
@@ -652,6 +657,17 @@ __global__ void __launch_bounds__(MT) merge_mean_kernel(const XT* __restrict__ X
 
 }  // namespace mg
 
+static int sm_count() {
+  static int n = 0;
+  if (n == 0) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 148;
+  }
+  return n;
+}
+
 MergeLayout merge_layout(int N, int n_v) {
   MergeLayout L{};
   size_t off = 0;
@@ -675,7 +691,7 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
   double* tnorm = reinterpret_cast<double*>(ws + L.tnorm_off);
   float* tinv = reinterpret_cast<float*>(ws + L.tinv_off);
   MergeCand* cand = reinterpret_cast<MergeCand*>(ws + L.cand_off);
-  // every kernel a programmatic dependent of the one before it
+  // every kernel but the fp32 tokens' assignment a programmatic dependent of the one before it
   bool ok = launch_ex(merge_plan_kernel, dim3(1), dim3(1024), 0, st, true, n_kept, budgets, sel_off, N, n_v, max_ctx,
                       ctx_off) == cudaSuccess;
   auto go = [&](auto* x) {
@@ -693,12 +709,18 @@ int launch_merge(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
                            n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
                            (const double*)tnorm, (const MergeCand*)cand, assign) == cudaSuccess;
     } else {
-      static std::atomic<unsigned long long> smem_raised{0};
       const size_t ab_bytes = 2 * (size_t)KC * (TB + 4) * sizeof(float);
-      ok = ok && raise_smem_limit(smem_raised, merge_assign_kernel<XT>, (int)ab_bytes) == cudaSuccess &&
-           launch_ex(merge_assign_kernel<XT>, dim3((n_v + TB - 1) / TB, N), dim3(256), ab_bytes, st, true, x, n_v, d,
-                     kept, n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target,
-                     (const double*)tnorm, assign) == cudaSuccess;
+      const int blocks = (n_v + TB - 1) / TB;
+      auto assign_by = [&](auto kern, std::atomic<unsigned long long>& smem_raised) {
+        return raise_smem_limit(smem_raised, kern, (int)ab_bytes) == cudaSuccess &&
+               launch_ex(kern, dim3(blocks, N), dim3(256), ab_bytes, st, false, x, n_v, d, kept, n_kept, sel_off,
+                         (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)ctx_target, (const double*)tnorm,
+                         assign) == cudaSuccess;
+      };
+      static std::atomic<unsigned long long> raised4{0}, raised1{0};
+      // (about a fifth of the tiles are kept: up to two CTAs with work an SM, or so)
+      if (blocks * N <= 12 * sm_count()) ok = ok && assign_by(merge_assign_kernel<XT, 4>, raised4);
+      else ok = ok && assign_by(merge_assign_kernel<XT, 1>, raised1);
     }
     ok = ok && launch_ex(merge_mean_kernel<XT>, dim3(N, (d + MCOLS - 1) / MCOLS, MP), dim3(MT), 0, st, true, x,
                          n_v, d, kept, n_kept, sel_off, (const int*)ctx_off, max_ctx, (const int*)rest, (const int*)assign, ctx) == cudaSuccess;

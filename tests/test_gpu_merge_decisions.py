@@ -8,25 +8,29 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-def assigned(riftlib, cuda, X, m):
+def assigned(riftlib, cuda, X, m, N=1):
     """The target index (0 .. m - 1) of every unselected token of one tile X [n_v, d] whose token 0 is selected, with m
-    targets: tokens 1, 1 + R // m, ...  A target's own entry is left as it was (-1)."""
+    targets: tokens 1, 1 + R // m, ...  A target's own entry is left as it was (-1).  The tile is the last of N."""
     n_v, d = X.shape
     i32 = dict(dtype=torch.int32, device=cuda)
     sel = torch.zeros(n_v, **i32)
     ctx = torch.zeros(m, d, dtype=torch.bfloat16, device=cuda)
-    ctx_off, ctx_target = torch.zeros(2, **i32), torch.zeros(m, **i32)
-    need = riftlib.merge_workspace_bytes(1, n_v)
+    ctx_target = torch.zeros(m, **i32)
+    need = riftlib.merge_workspace_bytes(N, n_v)
     ws = torch.full((need,), 255, dtype=torch.uint8, device=cuda)
     xdt = riftlib.RIFT_BF16 if X.dtype == torch.bfloat16 else riftlib.RIFT_F32
-    riftlib.merge_contextual(X[None].contiguous().to(cuda), xdt, 1, n_v, d, torch.zeros(1, **i32), torch.ones(1, **i32),
-                             torch.tensor([1 + m], **i32), sel, torch.tensor([0, 1], **i32), ctx, m, ctx_off, ctx_target,
-                             ws, need)
+    tiles = torch.zeros(N, n_v, d, dtype=X.dtype, device=cuda)
+    tiles[N - 1] = X.to(cuda)
+    sel_off, kept = torch.ones(N + 1, **i32), torch.full((N,), N - 1, **i32)
+    sel_off[0] = 0
+    ctx_off = torch.zeros(N + 1, **i32)
+    riftlib.merge_contextual(tiles, xdt, N, n_v, d, kept, torch.ones(1, **i32), torch.full((N,), 1 + m, **i32), sel, sel_off,
+                             ctx, m, ctx_off, ctx_target, ws, need)
     riftlib.sync_status()
     R = n_v - 1
     step = R // m
     assert ctx_target.cpu().tolist() == [1 + q * step for q in range(m)]
-    off = (n_v * 4 + 255) // 256 * 256  # the unselected tokens' list, then the assignment
+    off = (N * n_v * 4 + 255) // 256 * 256  # the unselected tokens' list, then the assignment
     return ws[off:off + 4 * R].view(torch.int32).cpu().tolist()
 
 
@@ -138,6 +142,26 @@ def test_blank_tokens_and_copies_of_targets(cuda, riftlib):
     assert want[0] == 1 and want[1] == 0 and want[2] == 4
     got = assigned(riftlib, cuda, X, m)
     assert [got[a] for a in at] == want
+
+
+def test_fp32_assignment_does_not_depend_on_the_tile_count(cuda, riftlib):
+    """fp32 tokens: the forms for few and for many tiles (204 tiles of 9 token blocks) choose alike, tokens between
+    two near-duplicate targets among them."""
+    n_v, d, m = 576, 320, 37
+    g = torch.Generator()
+    g.manual_seed(5)
+    X = torch.randn(n_v, d, generator=g)
+    X[16] = X[1] + 1e-3 * torch.randn(d, generator=g)  # the first two targets
+    X[2::5] = X[1] + 1e-3 * torch.randn(len(X[2::5]), d, generator=g)
+    few, many = (assigned(riftlib, cuda, X, m, N) for N in (1, 204))
+    assert few == many
+    x = X.double()
+    step = (n_v - 1) // m
+    unit = x[1:1 + m * step:step] / x[1:1 + m * step:step].norm(dim=1, keepdim=True)
+    want = (x[1:] @ unit.T).argmax(dim=1).tolist()
+    for a in range(n_v - 1):
+        if a % step or a // step >= m:
+            assert few[a] == want[a], a
 
 
 @pytest.mark.parametrize("K", [64, 256, 4096])
