@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(256) tile_finalize_kernel(const float* __restr
 // t, t + 256, ... of a token row (NVEC of them) over the chunk's tokens, in token order.  Tokens go LT
 // at a time: every thread loads its vectors of all of them first (LT * NVEC 16-byte loads in
 // flight), then each warp's sums x.w and x.x of each token go to shared memory and are added across
-// the warps once, at the end of the chunk, so nothing in the loop waits for another warp.
+// the warps once, at the end of the chunk, so no sum in the loop waits for another warp.
 // CS = 2 spreads the 256 threads over a cluster of two CTAs, half of the columns each, and reads the
 // warps' sums through distributed shared memory at the end: the same sums in the same order, bit for
 // bit, on twice the CTAs (launch_tokens has the rule).
@@ -300,7 +300,7 @@ __device__ __forceinline__ void sc_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 
-template <typename XT, int NVEC, int CS, int LT>
+template <typename XT, int NVEC, int CS, int LT, int TG>
 __global__ void __launch_bounds__(SC_THREADS / CS, LT * NVEC > 16 ? 1 : 2 * CS)
     token_score_kernel(const XT* __restrict__ X, int n_v, int d, int n_chunks,
                        const float* __restrict__ w, float* __restrict__ token_scores,
@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(SC_THREADS / CS, LT * NVEC > 16 ? 1 : 2 * CS)
   }
   const XT* base = X + ((size_t)tile * n_v) * d;
   for (int g0 = k0; g0 < k1; g0 += LT) {
+    if (TG > 0 && (g0 - k0) % (TG > 0 ? TG : 1) == 0) __syncthreads();
     uint4 raw[LT][NVEC];
 #pragma unroll
     for (int g = 0; g < LT; ++g) {
@@ -827,18 +828,24 @@ template <typename XT, int NVEC>
 static void launch_tokens(const void* X, int N, int n_v, int d, const ShardLayout& L, const float* w,
                           float* token_scores, float* Ppart, unsigned int* cnt, float* V, float* s_raw,
                           uint16_t* S16, cudaStream_t st) {
-  auto go = [&](auto cs, auto lt) {
-    constexpr int CS = decltype(cs)::value, LT = decltype(lt)::value;
-    launch_cluster_ex(token_score_kernel<XT, NVEC, CS, LT>, dim3(N * L.n_chunks * CS), dim3(SC_THREADS / CS), 0, st, true,
-                      CS, static_cast<const XT*>(X), n_v, d, L.n_chunks, w, token_scores, Ppart, cnt, V, s_raw, S16, N,
-                      (N + 7) & ~7);
+  auto go = [&](auto cs, auto lt, auto tg) {
+    constexpr int CS = decltype(cs)::value, LT = decltype(lt)::value, TG = decltype(tg)::value;
+    launch_cluster_ex(token_score_kernel<XT, NVEC, CS, LT, TG>, dim3(N * L.n_chunks * CS), dim3(SC_THREADS / CS), 0, st,
+                      true, CS, static_cast<const XT*>(X), n_v, d, L.n_chunks, w, token_scores, Ppart, cnt, V, s_raw, S16,
+                      N, (N + 7) & ~7);
   };
   using C1 = std::integral_constant<int, 1>;
   using C2 = std::integral_constant<int, 2>;
-  // u: CTAs of whole chunks.  Clusters of two only for bf16 rows of at most two vectors a thread that give
+  using Apart = std::integral_constant<int, 0>;
+  const int u = N * L.n_chunks, sms = sm_count();  // u: CTAs of whole chunks
+  // Clusters of two only for bf16 rows of at most two vectors a thread that give
   // every thread of both CTAs one (a shorter row's columns would all fall to the first CTA).
-  const int u = N * L.n_chunks, sms = sm_count();
   const bool can_split = sizeof(XT) == 2 && d >= SC_THREADS * VecTraits<XT>::W;
+  // TG: once HBM is the bound, the warps are brought together every TG tokens: nothing else holds them to the same
+  // rows, and spread over many they cost 2% of its rate (bf16 d = 4096, 100 tiles 89.1 : 87.0 us with the barriers, 400 300 :
+  // 294; d = 2048, 400 tiles 169 : 163; fp32 d = 4096, 300 tiles of 192 tokens 157 : 153, 400 of 576 570 : 557 with one per
+  // batch, 563 with one per four).  With few CTAs they only wait (fp32 d = 4096, 4 tiles 65 : 69), and so do the four
+  // vectors of a bf16 row beyond 4096 columns (700 tiles of 300 573 : 578).
   if constexpr (NVEC == 1) {
     // 32 tokens' loads ahead take an SM's registers for one CTA: right while a CTA is all that an SM gets,
     // beyond that two CTAs of 16.  us, 32 against 16 (576 tokens): bf16 d = 2048, 16 tiles (48 CTAs) 34 : 38, 50
@@ -847,9 +854,9 @@ static void launch_tokens(const void* X, int N, int n_v, int d, const ShardLayou
     // 34 -> 32; four CTAs (34 -> 30, 34 -> 32) are no faster.
     using L32 = std::integral_constant<int, 32>;
     if constexpr (sizeof(XT) == 2)
-      if (can_split && 2 * u <= sms) return go(C2{}, L32{});
-    if (u <= sms) go(C1{}, L32{});
-    else go(C1{}, std::integral_constant<int, 16>{});
+      if (can_split && 2 * u <= sms) return go(C2{}, L32{}, Apart{});
+    if (u <= sms) go(C1{}, L32{}, Apart{});
+    else go(C1{}, std::integral_constant<int, 16>{}, std::integral_constant<int, 64>{});
   } else {
     // The pass takes as long as the busiest SM: half chunks where they leave it less than whole ones do, in
     // the first rounds.  bf16 d = 4096, us, whole chunks : halves : quarters: 4 tiles 50 : 48 : 48, 38 54 : 56 : 56, 64
@@ -857,9 +864,13 @@ static void launch_tokens(const void* X, int N, int n_v, int d, const ShardLayou
     // 194.  Not for fp32 (64 tiles at d = 2048 60 : 60, 120 116 : 120) and not for four vectors a thread (bf16 d = 8192,
     // 4 tiles 97 : 106, 64 126 : 134).
     using LT = std::integral_constant<int, NVEC == 2 ? 8 : 4>;
+    using Together = std::integral_constant<int, NVEC == 2 ? 32 : sizeof(XT) == 4 ? 4 : 0>;
+    const bool apart = 3 * u <= 4 * sms;
     if constexpr (sizeof(XT) == 2 && NVEC == 2)
-      if (can_split && u < 4 * sms && (2 * u + sms - 1) / sms < 2 * ((u + sms - 1) / sms)) return go(C2{}, LT{});
-    go(C1{}, LT{});
+      if (can_split && u < 4 * sms && (2 * u + sms - 1) / sms < 2 * ((u + sms - 1) / sms))
+        return apart ? go(C2{}, LT{}, Apart{}) : go(C2{}, LT{}, Together{});
+    if (apart) go(C1{}, LT{}, Apart{});
+    else go(C1{}, LT{}, Together{});
   }
 }
 
