@@ -247,6 +247,9 @@ __global__ void __launch_bounds__(TB_THREADS) topb_kernel(const float* __restric
 // 64 tiles 8.3 : 12.3, 400 10.2 : 12.3, 512 12.3 : 14, 700 14-16 : 14, 1024 18.4 : 14-16; a scene's whole selection with
 // small tokens, 512 tiles 160 : 161, 640 197 : 196, 1024 279 : 277.  The scene of 64 tiles went from 134 to 132 us (136
 // with four tiles a thread: their budgets are a serial loop), 400 434 -> 430, four small tiles 47 -> 45.5.
+// No early trigger: the next kernel's CTAs would take their SMs while these still wait for the smoothing, and those
+// with work to do (the kept tiles' rows) then share few of them: a scene of 300 fp32 tiles at d = 4096 596 us with it,
+// 562 without, 64 at 4096 215 : 200, 150 bf16 at 256 157 : 133.
 // The results are those of prune_budget_kernel and topb_kernel, the same operations for every tile.
 constexpr int SELECT_TPT = 2, SELECT_ONE = SELECT_TPT * TB_THREADS;  // tiles at most
 // (unsigned, so that a sum past bit 31 would still be defined)
@@ -256,7 +259,6 @@ __global__ void __launch_bounds__(TB_THREADS) select_kernel(
     const float* __restrict__ r, const float* __restrict__ s, int N, int n_v, const float* __restrict__ p_ext,
     rift_policy pol, const float* __restrict__ s_range, float* __restrict__ u, int* __restrict__ kept,
     int* __restrict__ n_kept, int* __restrict__ budgets, int* __restrict__ sel, int* __restrict__ sel_off) {
-  pdl_trigger();
   pdl_wait();
   constexpr int NW = TB_THREADS / 32;
   __shared__ float rmin[NW], rmax[NW];
