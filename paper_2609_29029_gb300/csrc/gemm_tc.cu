@@ -645,7 +645,11 @@ static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 // with 344; W_o 12.3 us with 256 (S = 8), 13.7 with 128, 28.9 with 32.  Two CTAs fit on an SM, but a cluster has to
 // fit in one GPC: resident[S] clusters at once (asked from the driver), fewer than 2 SMs / S for most S.  100 rows,
 // us, by the count of CTAs alone against resident[S]: N = 5120 x K = 4096 28.7 (S = 7) : 20.7 (6), 6144 x 4096
-// 30.7 (6) : 22.5 (5).
+// 30.7 (6) : 22.5 (5).  A programmatic dependent launch (pdl) is placed around the CTAs of the kernel before it, and
+// where all clusters of 3 or more would only just fit, some wait for a second round: a sixteenth is left free then
+// (two layers over 347 rows, whose W_o takes 96 tiles, 507 us with S = 3, of which 97 fit, 466 with S = 2; 20 decoded
+// tokens 472 : 459).  A quarter free is too much (524 rows 536 : 575), pairs need none (2,970 rows at d = 1024, 152 of
+// 152 pairs, 298 : 321), nor does a launch of its own (W_o at 384 rows 26.6 : 32.8).
 // K too short to split (fewer than 16 K-blocks): row tiles of at most SHORT_BN instead, as long as they fit at
 // once; what a CTA takes is then its epilogue, a serial chain over its rows.  us, tiles of 160 rows, 48, and the
 // SM pairs, 300 rows: 256 x 256 + residual 22.5 : 12.3 : 20.5, 768 x 256 10.2 : 8.2 : 14.3, SwiGLU 1376 x 256
@@ -655,7 +659,7 @@ struct Plan {
   int bn, S;
   bool one_round;  // all its CTAs are resident at once, or the K slices are
 };
-inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram) {
+inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram, bool pdl) {
   const long long n_tiles = (N + BM - 1) / BM;
   const int kt = (K + BK - 1) / BK;
   const int min_blocks = gram ? 3 : 8;
@@ -668,7 +672,8 @@ inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram) {
   const long long tiles = m_tiles * n_tiles;
   if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) return {height(m_tiles), MAX_S, true};
   int S = gram && tiles > 32 ? 4 : PORTABLE_S;
-  while (S > 1 && (tiles > resident[S] || kt / S < min_blocks)) --S;
+  auto fit = [&](int s) { return pdl && s > 2 ? resident[s] * 15 / 16 : resident[s]; };
+  while (S > 1 && (tiles > fit(S) || kt / S < min_blocks)) --S;
   return {height(m_tiles), S, S >= 2};
 }
 }  // namespace ck
@@ -1443,7 +1448,7 @@ int launch_gemm_tc(const void* A, const void* B, int M, int N, int K, int epi, v
   // The operands' stored row width: K, or 2 kmap_d blocks when read through the K-block remap.
   if (ep.kmap_d && K != 3 * ep.kmap_d * BK) return 1;
   const uint64_t Ks = ep.kmap_d ? (uint64_t)2 * ep.kmap_d * BK : (uint64_t)K;
-  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ck_resident(), ep.kmap_d > 0);
+  const ck::Plan plan = ck::plan(M, N, K, sm_count(), ck_resident(), ep.kmap_d > 0, pdl);
   // The cluster split-K kernel for one row tile, or while its tiles fit on the GPU at once, split or, where K is
   // short, low: beyond that its 128-row tiles are bound by the L2 traffic of their operands and the SM pairs'
   // 256 x 256 tiles win.  us, cluster against pairs: W_o at 512 rows (S = 2) 27.4 : 35.0, at 777
