@@ -9,8 +9,8 @@
 //                         32-term chunks, a running top 2 per token; the two are recomputed as
 //                         float-float sums (good to ~2^-44) and compared as x.t1 / ||t1|| vs
 //                         x.t2 / ||t2|| in fp64, so the decision is the cosine argmax of the exact
-//                         arithmetic (ties to the lower target) unless three targets are closer to each
-//                         other than the fp32 sums' error, when the best may not be among the two
+//                         arithmetic (ties to the lower target); where a third is within the fp32 sums' error
+//                         of the best, all are compared
 //   (bf16 tokens) merge_screen_kernel (gemm_tc.cu) lists the targets whose tcgen05 product is
 //                         within its error bound of the best one's, for each 128 tokens of a slot, and
 //                         merge_decide_kernel makes the same float-float decision among them
@@ -99,6 +99,23 @@ __device__ double ff_dot(const XT* a, const XT* b, int d, int lane) {
       }
   }
   return ff_warp_sum(hi, lo);
+}
+
+// Whether two rows hold the same bits (b null: whether the row is all zeros, of either sign), by one warp.
+template <typename XT>
+__device__ __forceinline__ bool same_row(const XT* a, const XT* b, int d, int lane) {
+  constexpr int W = 16 / sizeof(XT);  // elements of a 16-byte load
+  constexpr uint32_t ABS = sizeof(XT) == 2 ? 0x7fff7fffu : 0x7fffffffu;
+  for (int k = lane * W; k < (d + 32 * W - 1) / (32 * W) * (32 * W); k += 32 * W) {
+    uint32_t differ = 0u;
+    if (k < d) {
+      const uint4 x = *reinterpret_cast<const uint4*>(a + k);
+      const uint4 y = b ? *reinterpret_cast<const uint4*>(b + k) : make_uint4(0u, 0u, 0u, 0u);
+      differ = ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) & (b ? 0xffffffffu : ABS);
+    }
+    if (__any_sync(0xffffffffu, differ != 0u)) return false;
+  }
+  return true;
 }
 
 // m_j = min(budgets[j] - s_j, n_v - s_j) and its exclusive prefix sum over the kept slots.  If
@@ -242,20 +259,6 @@ __global__ void __launch_bounds__(256) merge_targets_kernel(const XT* __restrict
 // Targets keep their own group.
 constexpr int DT = 256;
 
-// Whether two rows hold the same bits (b null: whether the row is all zeros, of either sign), by one warp.
-__device__ __forceinline__ bool same_row(const uint16_t* a, const uint16_t* b, int d, int lane) {
-  for (int k = lane * 8; k < (d + 255) / 256 * 256; k += 256) {
-    uint32_t differ = 0u;
-    if (k < d) {
-      const uint4 x = *reinterpret_cast<const uint4*>(a + k);
-      const uint4 y = b ? *reinterpret_cast<const uint4*>(b + k) : make_uint4(0u, 0u, 0u, 0u);
-      differ = ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) & (b ? 0xffffffffu : 0x7fff7fffu);
-    }
-    if (__any_sync(0xffffffffu, differ != 0u)) return false;
-  }
-  return true;
-}
-
 // x.t1 and x.t2 by one warp, four steps' loads ahead of the serial chains.
 __device__ __forceinline__ double2 ff_dots(const uint16_t* x, const uint16_t* t1, const uint16_t* t2, int d, int lane) {
   float h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f;
@@ -370,7 +373,7 @@ __global__ void __launch_bounds__(DT, 2) merge_decide_kernel(const uint16_t* __r
   __syncthreads();
   for (int i = 0; i < n_all; ++i) {  // the warps share the targets, two at a time
     const uint16_t* x = Xt + (size_t)rest[(size_t)j * n_v + open[63 - i]] * d;
-    const bool zero = same_row(x, nullptr, d, lane);  // all similarities are 0: the first target
+    const bool zero = same_row<uint16_t>(x, nullptr, d, lane);  // all similarities are 0: the first target
     Best best = {-1, 0.0, 1.0};
     for (int q = 2 * warp; q < m && !zero; q += 2 * (DT / 32)) {
       const bool u1 = !dup[q], u2 = q + 1 < m && !dup[q + 1];
@@ -395,6 +398,30 @@ __global__ void __launch_bounds__(DT, 2) merge_decide_kernel(const uint16_t* __r
   }
 }
 
+// The best target for token k of a tile among `choice` and every `step`-th of the m from `first` on, by one warp:
+// copies of the best so far are passed over, and a zero token (all similarities are 0) keeps its choice.
+template <typename XT>
+__device__ __noinline__ int best_of_all(const XT* Xt, int k, const int* target, const double* norm, int m, int d, int lane,
+                                        int choice, int first, int step, double& best) {
+  const XT* x = Xt + (size_t)k * d;
+  best = 0.0;
+  if (same_row<XT>(x, nullptr, d, lane)) return choice;
+  auto row = [&](int q) { return Xt + (size_t)target[q] * d; };
+  const int given = choice;
+  for (int i = first - step; i < m; i += step) {  // the given choice first
+    const int q = i < first ? given : i;
+    if (i == given || (i > choice && __double_as_longlong(norm[q]) == __double_as_longlong(norm[choice]) &&
+                       same_row(row(q), row(choice), d, lane)))
+      continue;
+    const double dt = ff_dot<1>(x, row(q), d, lane), s = norm[q] > 0.0 ? dt / norm[q] : 0.0;
+    if (i < first || s > best || (s == best && q < choice)) {
+      choice = q;
+      best = s;
+    }
+  }
+  return choice;
+}
+
 // Grid (block of TB unselected tokens, kept slot).  assign[j][a] = target index of rest[a].
 // U: steps of loads ahead in the float-float dot products.  Four hide their latency where a CTA has an SM to itself, but
 // take the registers of two more CTAs (164 against 80).  Launched without overlap: as a programmatic dependent its few
@@ -415,9 +442,13 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   extern __shared__ float ab_sm[];  // As[KC][TB + 4], Bs[KC][TB + 4]
   float (*As)[TB + 4] = reinterpret_cast<float (*)[TB + 4]>(ab_sm);
   float (*Bs)[TB + 4] = reinterpret_cast<float (*)[TB + 4]>(ab_sm + KC * (TB + 4));
-  __shared__ float best_v[TB][2];
+  __shared__ float best_v[TB][3];  // the three highest similarities, the first two targets
   __shared__ int best_j[TB][2];
-  __shared__ float inv_n[TB];
+  __shared__ float inv_n[TB], row_ss[TB];
+  __shared__ int far;              // a target's norm is below 2^-40
+  __shared__ int n_all, all[TB];   // rows with all targets for candidates
+  __shared__ double part_s[8];
+  __shared__ int part_q[8];
   pdl_wait();
   const int j = blockIdx.y;  // the token blocks of one slot are adjacent: its target rows stay in L2
   if (j >= *n_kept) return;
@@ -430,13 +461,17 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   const XT* Xt = X + (size_t)kept[j] * n_v * d;
   const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
   if (tid < TB) {
-    best_v[tid][0] = best_v[tid][1] = -INFINITY;
+    best_v[tid][0] = best_v[tid][1] = best_v[tid][2] = -INFINITY;
     best_j[tid][0] = best_j[tid][1] = -1;
   }
+  if (tid == 0) far = n_all = 0;
+  __syncthreads();
+  float ss = 0.f;  // of this thread's part of its token row
   for (int b0 = 0; b0 < m; b0 += TB) {
     if (tid < TB) {
       const double nn = b0 + tid < m ? tnorm[co + b0 + tid] : 0.0;
       inv_n[tid] = nn > 0.0 ? (float)(1.0 / nn) : 0.f;  // a zero target has similarity 0
+      if (inv_n[tid] > 0x1p40f) far = 1;
     }
     float acc[4][4] = {};
     // 64 rows x KC columns per operand and chunk: four 8-column groups per thread and operand,
@@ -464,6 +499,7 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
         for (int e = 0; e < 8; ++e) {
           As[32 * g + scol + e][srow] = va[g][e];
           Bs[32 * g + scol + e][srow] = vb[g][e];
+          if (b0 == 0) ss = fmaf(va[g][e], va[g][e], ss);
         }
       __syncthreads();
       if (k0 + KC < d) fetch(k0 + KC);
@@ -487,7 +523,12 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
       }
       __syncthreads();
     }
-    // running top 2 per token: thread (ti, tj) offers its 4 x 4 candidates row by row
+    if (b0 == 0) {  // a row's four threads
+      ss += __shfl_xor_sync(0xffffffffu, ss, 1);
+      ss += __shfl_xor_sync(0xffffffffu, ss, 2);
+      if ((tid & 3) == 0) row_ss[tid >> 2] = ss;
+    }
+    // running top 2, and the third value, per token: thread (ti, tj) offers its 4 x 4 candidates row by row
     for (int w = 0; w < 16; ++w) {
       if (tj == w) {
 #pragma unroll
@@ -499,13 +540,17 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
             if (b >= m) continue;
             const float v = acc[r][c] * inv_n[tj * 4 + c];
             if (v > best_v[row][0] || (v == best_v[row][0] && b < best_j[row][0])) {
+              best_v[row][2] = best_v[row][1];
               best_v[row][1] = best_v[row][0];
               best_j[row][1] = best_j[row][0];
               best_v[row][0] = v;
               best_j[row][0] = b;
             } else if (v > best_v[row][1] || (v == best_v[row][1] && b < best_j[row][1])) {
+              best_v[row][2] = best_v[row][1];
               best_v[row][1] = v;
               best_j[row][1] = b;
+            } else {
+              best_v[row][2] = fmaxf(best_v[row][2], v);
             }
           }
         }
@@ -513,7 +558,10 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
       __syncthreads();
     }
   }
-  // decide between the top two at ~fp64 accuracy: x.t1 / ||t1|| vs x.t2 / ||t2||
+  // Decide between the top two at ~fp64 accuracy: x.t1 / ||t1|| vs x.t2 / ||t2||; where a third target is within the
+  // product's error of the best, among all of them.  An fp32 similarity errs by at most
+  // (32 + d / 32) 2^-24 ||x|| (chains of 32 products, then d / 32 sums, each rounded) and 2^-23 ||x|| from 1 / ||t|| and its
+  // product; the difference of two by twice that.
   const int warp = tid >> 5, lane = tid & 31;
   for (int row = warp; row < TB; row += 8) {
     const int a = a0 + row;
@@ -528,8 +576,32 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
       const double n1 = tnorm[co + choice], n2 = tnorm[co + j2];
       const double s1 = n1 > 0.0 ? d1 / n1 : 0.0, s2 = n2 > 0.0 ? d2 / n2 : 0.0;
       if (s2 > s1 || (s2 == s1 && j2 < choice)) choice = j2;
+      const float bound =
+          row_ss[row] > 0x1p-60f && !far ? (48.f + (float)d / 32.f) * 0x1p-23f * sqrtf(row_ss[row]) : INFINITY;
+      if (m > 2 && !(best_v[row][0] - best_v[row][2] > bound) && lane == 0) {
+        best_j[row][0] = choice;
+        all[atomicAdd(&n_all, 1)] = row;
+      }
     }
     if (lane == 0) assign[(size_t)j * n_v + a] = choice;
+  }
+  __syncthreads();
+  for (int i = 0; i < n_all; ++i) {  // the warps share the targets
+    const int row = all[i], choice = best_j[row][0];
+    double s;
+    const int q = best_of_all(Xt, rj[a0 + row], ctx_target + co, tnorm + co, m, d, lane, choice, warp, 8, s);
+    if (lane == 0) {
+      part_q[warp] = q;
+      part_s[warp] = s;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      int w = 0;
+      for (int o = 1; o < 8; ++o)
+        if (part_s[o] > part_s[w] || (part_s[o] == part_s[w] && part_q[o] < part_q[w])) w = o;
+      assign[(size_t)j * n_v + a0 + row] = part_q[w];
+    }
+    __syncthreads();
   }
 }
 

@@ -81,10 +81,12 @@ def one_hot(d, **at):
 
 # targets that differ from 1 by a product of 2^-26 or less with their token, which an accumulation with 1 drops: the
 # screening sees them as equal.  Up to 7: the candidates are listed; more, or more than 2 beyond the 80 targets of
-# one block: all targets are looked at; d above and off a warp's 256-column steps
+# one block: all targets are looked at; d above and off a warp's 256-column steps.  fp32 tokens, whose sums drop the
+# products too: a third near target has all looked at
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
 @pytest.mark.parametrize("near,m", [(2, 2), (3, 6), (4, 6), (7, 9), (8, 9), (7, 80), (80, 80), (2, 81), (3, 81), (100, 100)])
 @pytest.mark.parametrize("d", [320, 4096])
-def test_best_of_several_near_targets(near, m, d, cuda, riftlib):
+def test_best_of_several_near_targets(near, m, d, dtype, cuda, riftlib):
     targets = [one_hot(d, c0=1.0, **{f"c{2 + q}": 2.0 ** -14}) if q < near else one_hot(d, **{f"c{2 + q}": 1.0})
                for q in range(m)]
     wins = sorted({0, 1, near // 2, near - 1})
@@ -95,7 +97,7 @@ def test_best_of_several_near_targets(near, m, d, cuda, riftlib):
             x[2 + q] = 2.0 ** -13 if q == w else 2.0 ** -14
         tokens.append(x)
     tokens.append(one_hot(d, c0=1.0))  # an exact tie: the lowest
-    X, at = tile(d, targets, tokens, torch.bfloat16)
+    X, at = tile(d, targets, tokens, dtype)
     got = assigned(riftlib, cuda, X, m)
     assert [got[a] for a in at] == wins + [0]
 
@@ -123,7 +125,8 @@ def test_dropped_products_do_not_decide(d, scale, cuda, riftlib):
     assert [got[k] for k in at] == [1, 1]
 
 
-def test_blank_tokens_and_copies_of_targets(cuda, riftlib):
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+def test_blank_tokens_and_copies_of_targets(dtype, cuda, riftlib):
     """Blank rows (all alike, or zero) make many targets copies of one: a blank token goes to the first of them, a zero
     one to the first target."""
     d, m = 256, 9
@@ -133,8 +136,8 @@ def test_blank_tokens_and_copies_of_targets(cuda, riftlib):
     other = [torch.randn(d, generator=g) for _ in range(4)]
     targets = [other[0], blank, blank, zero, other[1], blank, other[2], zero, blank]
     tokens = [blank, zero, other[1], -blank, blank, zero, other[2], blank + 0, other[0]]
-    X, at = tile(d, targets, tokens, torch.bfloat16)
-    x64, t64 = X.double(), torch.stack(targets).to(torch.bfloat16).double()
+    X, at = tile(d, targets, tokens, dtype)
+    x64, t64 = X.double(), torch.stack(targets).to(dtype).double()
     nrm = t64.norm(dim=1, keepdim=True)
     unit = torch.where(nrm > 0, t64 / nrm.clamp_min(1e-300), t64)
     want = [int((unit @ x64[1 + a]).argmax()) for a in at]
@@ -146,13 +149,12 @@ def test_blank_tokens_and_copies_of_targets(cuda, riftlib):
 
 def test_fp32_assignment_does_not_depend_on_the_tile_count(cuda, riftlib):
     """fp32 tokens: the forms for few and for many tiles (204 tiles of 9 token blocks) choose alike, tokens between
-    two near-duplicate targets among them."""
+    many near-duplicate targets among them."""
     n_v, d, m = 576, 320, 37
     g = torch.Generator()
     g.manual_seed(5)
     X = torch.randn(n_v, d, generator=g)
-    X[16] = X[1] + 1e-3 * torch.randn(d, generator=g)  # the first two targets
-    X[2::5] = X[1] + 1e-3 * torch.randn(len(X[2::5]), d, generator=g)
+    X[1::3] = X[1] + 1e-3 * torch.randn(len(X[1::3]), d, generator=g)  # all targets among them
     few, many = (assigned(riftlib, cuda, X, m, N) for N in (1, 204))
     assert few == many
     x = X.double()
