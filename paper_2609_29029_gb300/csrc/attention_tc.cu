@@ -342,120 +342,122 @@ __global__ void __launch_bounds__(THREADS, Cfg<HD, KB>::CTAS)
   // uses O buffer t % NO (phase (t / NO) & 1).
 
   if (warp == 0 || warp == 7) {
-    {
-      // ---------------- TMA producers: warp 0 K tiles; warp 7 Q and V tiles
-      const bool is_k = warp == 0;
-      uint32_t g = 0, t = 0;
-      bool ok = true;
-      int4 nxt = fetch_item(blockIdx.x);
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        Item cur = decode_item(nxt, item);
-        cur.seq0 = warp_uniform(cur.seq0);
-        cur.q0 = warp_uniform(cur.q0);
-        cur.nkv = warp_uniform(cur.nkv);
-        nxt = fetch_item(item + gridDim.x);
-        if (cur.nkv == 0) continue;
-        if (!is_k) {
-          if (!mbar_wait_warp(Q_EMPTY, (t & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          if (elect_one()) {
-            mbar_expect_tx(Q_FULL, CF::Q_BYTES);
-            for (int c = 0; c < HD / 64; ++c)
-              tma_load_2d(smem_u32(sQ + c * BQ * 128), &tm_q, cur.h * HD + c * 64, cur.seq0 + cur.q0, Q_FULL);
-          }
-          __syncwarp();
+    // ---------------- TMA producers: warp 0 K tiles; warp 7 Q and V tiles
+    const bool is_k = warp == 0;
+    uint32_t g = 0, t = 0, q_loads = 0;
+    bool ok = true;
+    int4 nxt = fetch_item(blockIdx.x);
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      Item cur = decode_item(nxt, item);
+      cur.seq0 = warp_uniform(cur.seq0);
+      cur.q0 = warp_uniform(cur.q0);
+      cur.nkv = warp_uniform(cur.nkv);
+      nxt = fetch_item(item + gridDim.x);
+      if (cur.nkv == 0) continue;
+      if (!is_k) {
+        if (!mbar_wait_warp(Q_EMPTY, (t & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+        ++q_loads;
+        if (elect_one()) {
+          mbar_expect_tx(Q_FULL, CF::Q_BYTES);
+          for (int c = 0; c < HD / 64; ++c)
+            tma_load_2d(smem_u32(sQ + c * BQ * 128), &tm_q, cur.h * HD + c * 64, cur.seq0 + cur.q0, Q_FULL);
         }
-        for (int j = 0; j < cur.nkv; ++j, ++g) {
-          const int s = g % NST;
-          const uint32_t ph = (g / NST) & 1u;
-          const int base = is_k ? K_EMPTY : V_EMPTY;
-          if (!mbar_wait_warp(BAR(base, s), ph ^ 1u, abort_flag)) { ok = false; break; }
-          const uint32_t full = BAR(is_k ? K_FULL : V_FULL, s);
-          uint8_t* dst = (is_k ? sK + s * CF::K_BYTES : sV + s * CF::V_BYTES);
-          // prefix blocks from the prefix's [S_pre, d] K / V maps (rows past S_pre read as zero),
-          // then the sequence's own rows of the qkv map
-          const bool pre = j < np;
-          const CUtensorMap* map = pre ? (is_k ? &tm_pk : &tm_pv) : &tm_kv;
-          const int col = (pre ? 0 : (is_k ? d : 2 * d)) + cur.h * HD;
-          const int row = pre ? j * KB : cur.seq0 + (j - np) * KB;
-          if (elect_one()) {
-            mbar_expect_tx(full, CF::K_BYTES);
-            for (int c = 0; c < HD / 64; ++c) tma_load_2d(smem_u32(dst + c * KB * 128), map, col + c * 64, row, full);
-          }
-          __syncwarp();
-        }
-        ++t;
-      }
-    }
-  } else if (warp == 1) {
-    {
-      // ---------------- S issuer: S_g = Q K_g^T
-      const uint64_t qd0 = desc_kmajor(smem_u32(sQ)), kd0 = desc_kmajor(smem_u32(sK));
-      uint32_t g = 0, t = 0;
-      bool ok = true;
-      int4 nxt = fetch_item(blockIdx.x);
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const int nkv = warp_uniform(decode_item(nxt, item).nkv);
-        nxt = fetch_item(item + gridDim.x);
-        if (nkv == 0) continue;
-        if (!mbar_wait_warp(Q_FULL, t & 1u, abort_flag)) break;
-        for (int j = 0; j < nkv; ++j, ++g) {
-          const int st = g % NST, sb = g & 1;
-          if (!mbar_wait_warp(BAR(K_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
-          // S/P buffer sb is free once PV_{g-2}, the reader of P_{g-2}, has completed
-          if (g >= 2 && !mbar_wait_warp(BAR(PV_DONE, sb), ((g - 2) >> 1) & 1u, abort_flag)) { ok = false; break; }
-          fence_after();
-          const uint64_t kd = kd0 + (uint32_t)(st * (CF::K_BYTES >> 4));
-          const uint32_t s_col = tmem + S_COL0 + (uint32_t)KB * sb;
-          if (elect_one()) {
-#pragma unroll
-            for (int kk = 0; kk < HD / 16; ++kk)  // 16 of the head dims per step
-              umma(s_col, qd0 + (uint32_t)(((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
-                   kd + (uint32_t)(((kk >> 2) * (KB * 128) + (kk & 3) * 32) >> 4), CF::IDESC_S, kk > 0);
-            umma_commit(BAR(S_FULL, sb));
-            umma_commit(BAR(K_EMPTY, st));
-          }
-          __syncwarp();
-        }
-        if (!ok) break;
-        if (elect_one()) umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
         __syncwarp();
-        ++t;
       }
+      for (int j = 0; j < cur.nkv; ++j, ++g) {
+        const int s = g % NST;
+        const uint32_t ph = (g / NST) & 1u;
+        const int base = is_k ? K_EMPTY : V_EMPTY;
+        if (!mbar_wait_warp(BAR(base, s), ph ^ 1u, abort_flag)) { ok = false; break; }
+        const uint32_t full = BAR(is_k ? K_FULL : V_FULL, s);
+        uint8_t* dst = (is_k ? sK + s * CF::K_BYTES : sV + s * CF::V_BYTES);
+        // prefix blocks from the prefix's [S_pre, d] K / V maps (rows past S_pre read as zero),
+        // then the sequence's own rows of the qkv map
+        const bool pre = j < np;
+        const CUtensorMap* map = pre ? (is_k ? &tm_pk : &tm_pv) : &tm_kv;
+        const int col = (pre ? 0 : (is_k ? d : 2 * d)) + cur.h * HD;
+        const int row = pre ? j * KB : cur.seq0 + (j - np) * KB;
+        if (elect_one()) {
+          mbar_expect_tx(full, CF::K_BYTES);
+          for (int c = 0; c < HD / 64; ++c) tma_load_2d(smem_u32(dst + c * KB * 128), map, col + c * 64, row, full);
+        }
+        __syncwarp();
+      }
+      ++t;
+    }
+    // No copy left in flight (bounded): the last of each stage, and of Q, whose item may have been left half way.
+    auto landed = [&](uint32_t bar, uint32_t parity) {
+      for (uint32_t w = 0; w < (1u << 22) && !mbar_try_wait(bar, parity); ++w) {
+      }
+    };
+    for (uint32_t j = 1; j <= NST && j <= g; ++j) landed(BAR(is_k ? K_FULL : V_FULL, (g - j) % NST), ((g - j) / NST) & 1u);
+    if (!is_k && q_loads > 0) landed(Q_FULL, (q_loads - 1) & 1u);
+  } else if (warp == 1) {
+    // ---------------- S issuer: S_g = Q K_g^T
+    const uint64_t qd0 = desc_kmajor(smem_u32(sQ)), kd0 = desc_kmajor(smem_u32(sK));
+    uint32_t g = 0, t = 0;
+    bool ok = true;
+    int4 nxt = fetch_item(blockIdx.x);
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      const int nkv = warp_uniform(decode_item(nxt, item).nkv);
+      nxt = fetch_item(item + gridDim.x);
+      if (nkv == 0) continue;
+      if (!mbar_wait_warp(Q_FULL, t & 1u, abort_flag)) break;
+      for (int j = 0; j < nkv; ++j, ++g) {
+        const int st = g % NST, sb = g & 1;
+        if (!mbar_wait_warp(BAR(K_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        // S/P buffer sb is free once PV_{g-2}, the reader of P_{g-2}, has completed
+        if (g >= 2 && !mbar_wait_warp(BAR(PV_DONE, sb), ((g - 2) >> 1) & 1u, abort_flag)) { ok = false; break; }
+        fence_after();
+        const uint64_t kd = kd0 + (uint32_t)(st * (CF::K_BYTES >> 4));
+        const uint32_t s_col = tmem + S_COL0 + (uint32_t)KB * sb;
+        if (elect_one()) {
+#pragma unroll
+          for (int kk = 0; kk < HD / 16; ++kk)  // 16 of the head dims per step
+            umma(s_col, qd0 + (uint32_t)(((kk >> 2) * (BQ * 128) + (kk & 3) * 32) >> 4),
+                 kd + (uint32_t)(((kk >> 2) * (KB * 128) + (kk & 3) * 32) >> 4), CF::IDESC_S, kk > 0);
+          umma_commit(BAR(S_FULL, sb));
+          umma_commit(BAR(K_EMPTY, st));
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      if (elect_one()) umma_commit(Q_EMPTY);  // Q is free once the item's S products complete
+      __syncwarp();
+      ++t;
     }
   } else if (warp == 6) {
-    {
-      // ---------------- PV issuer: O += P_g V_g
-      const uint64_t vd0 = desc_mnmajor(smem_u32(sV), KB * 128);
-      uint32_t g = 0, t = 0;
-      bool ok = true;
-      int4 nxt = fetch_item(blockIdx.x);
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const int nkv = warp_uniform(decode_item(nxt, item).nkv);
-        nxt = fetch_item(item + gridDim.x);
-        if (nkv == 0) continue;
-        const int ob = t % NO;
-        for (int j = 0; j < nkv; ++j, ++g) {
-          const int st = g % NST, sb = g & 1;
-          if (!mbar_wait_warp(BAR(V_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
-          if (j == 0 && !mbar_wait_warp(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          if (!mbar_wait_warp(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
-          fence_after();
-          const uint64_t vd = vd0 + (uint32_t)(st * (CF::V_BYTES >> 4));
-          const uint32_t o_col = tmem + 128u * ob, p_col = tmem + S_COL0 + (uint32_t)KB * sb;
-          if (elect_one()) {
+    // ---------------- PV issuer: O += P_g V_g
+    const uint64_t vd0 = desc_mnmajor(smem_u32(sV), KB * 128);
+    uint32_t g = 0, t = 0;
+    bool ok = true;
+    int4 nxt = fetch_item(blockIdx.x);
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      const int nkv = warp_uniform(decode_item(nxt, item).nkv);
+      nxt = fetch_item(item + gridDim.x);
+      if (nkv == 0) continue;
+      const int ob = t % NO;
+      for (int j = 0; j < nkv; ++j, ++g) {
+        const int st = g % NST, sb = g & 1;
+        if (!mbar_wait_warp(BAR(V_FULL, st), (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        if (j == 0 && !mbar_wait_warp(BAR(O_EMPTY, ob), ((t / NO) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(BAR(P_FULL, sb), (g >> 1) & 1u, abort_flag)) { ok = false; break; }
+        fence_after();
+        const uint64_t vd = vd0 + (uint32_t)(st * (CF::V_BYTES >> 4));
+        const uint32_t o_col = tmem + 128u * ob, p_col = tmem + S_COL0 + (uint32_t)KB * sb;
+        if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < KB / 16; ++kk)  // 16 keys (8 TMEM columns of P) per step
-              umma_ts(o_col, p_col + 8u * kk, vd + (uint32_t)(kk * (2048 >> 4)), CF::IDESC_O, (j > 0 || kk > 0) ? 1u : 0u);
-            umma_commit(BAR(PV_DONE, sb));
-            umma_commit(BAR(V_EMPTY, st));
-          }
-          __syncwarp();
+          for (int kk = 0; kk < KB / 16; ++kk)  // 16 keys (8 TMEM columns of P) per step
+            umma_ts(o_col, p_col + 8u * kk, vd + (uint32_t)(kk * (2048 >> 4)), CF::IDESC_O, (j > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(BAR(PV_DONE, sb));
+          umma_commit(BAR(V_EMPTY, st));
         }
-        if (!ok) break;
-        if (elect_one()) umma_commit(BAR(O_FULL, ob));
         __syncwarp();
-        ++t;
       }
+      if (!ok) break;
+      if (elect_one()) umma_commit(BAR(O_FULL, ob));
+      __syncwarp();
+      ++t;
     }
   } else {
     // ---------------- softmax and output: thread = query row (TMEM lane)

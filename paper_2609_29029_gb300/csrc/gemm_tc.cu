@@ -1024,31 +1024,29 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
       }
     }
   } else if (warp == 1) {
-    {
-      // ---------------- MMA issuer
-      int it = 0;
-      bool ok = true;
-      for (int nb = 0; nb < nblk && ok; ++nb) {
-        if (!mbar_wait_warp(tempty, (nb & 1) ^ 1, abort_flag)) break;
+    // ---------------- MMA issuer
+    int it = 0;
+    bool ok = true;
+    for (int nb = 0; nb < nblk && ok; ++nb) {
+      if (!mbar_wait_warp(tempty, (nb & 1) ^ 1, abort_flag)) break;
+      fence_after();
+      const uint32_t idesc = ms::IDESC | ((uint32_t)(width(nb) >> 3) << 17);
+      for (int k = 0; k < kt; ++k, ++it) {
+        const int s2 = it % STAGES;
+        if (!mbar_wait_warp(full_bar(s2), (it / STAGES) & 1u, abort_flag)) { ok = false; break; }
         fence_after();
-        const uint32_t idesc = ms::IDESC | ((uint32_t)(width(nb) >> 3) << 17);
-        for (int k = 0; k < kt; ++k, ++it) {
-          const int s2 = it % STAGES;
-          if (!mbar_wait_warp(full_bar(s2), (it / STAGES) & 1u, abort_flag)) { ok = false; break; }
-          fence_after();
-          const uint64_t ad = smem_desc(smem_u32(sA + s2 * A_BYTES));
-          const uint64_t bd = smem_desc(smem_u32(sB + s2 * B_BYTES));
-          if (elect_one()) {
+        const uint64_t ad = smem_desc(smem_u32(sA + s2 * A_BYTES));
+        const uint64_t bd = smem_desc(smem_u32(sB + s2 * B_BYTES));
+        if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              umma_f16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc, (k != 0 || kk != 0) ? 1u : 0u);
-            umma_commit(empty_bar(s2));
-          }
-          __syncwarp();
+          for (int kk = 0; kk < BK / 16; ++kk)
+            umma_f16(tmem_base, ad + 2 * kk, bd + 2 * kk, idesc, (k != 0 || kk != 0) ? 1u : 0u);
+          umma_commit(empty_bar(s2));
         }
-        if (ok && elect_one()) umma_commit(tfull);
         __syncwarp();
       }
+      if (ok && elect_one()) umma_commit(tfull);
+      __syncwarp();
     }
   } else {
     // ---------------- gather and epilogue (warps 2..5)
