@@ -954,7 +954,8 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
     merge_screen_kernel(const __grid_constant__ CUtensorMap tmT, const uint16_t* __restrict__ X, int n_v, int d,
                         const int* __restrict__ kept, const int* __restrict__ n_kept,
                         const int* __restrict__ sel_off, const int* __restrict__ ctx_off, int max_ctx,
-                        const float* __restrict__ tinv, const int* __restrict__ rest, MergeCand* __restrict__ cand) {
+                        const uint16_t* __restrict__ targets, const float* __restrict__ tinv,
+                        const int* __restrict__ rest, MergeCand* __restrict__ cand) {
   constexpr int STAGES = ms::STAGES, COLS = ms::COLS, A_BYTES = ms::A_BYTES, B_BYTES = ms::B_BYTES;
   pdl_trigger();
   pdl_wait();
@@ -966,7 +967,9 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
   if (mb * 128 >= R) return;
   const int step = R / m;
   extern __shared__ uint8_t smem_raw[];
-  __shared__ float nrm_s[128];
+  __shared__ float nrm_s[128], inv_s[RIFT_MAX_NV];  // the tokens' ||x||^2; the targets' 1 / ||t||
+  __shared__ uint16_t twin[RIFT_MAX_NV];            // an earlier target of the same norm, or NONE
+  __shared__ int any_twin;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + STAGES * A_BYTES;
@@ -1107,8 +1110,8 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
           finish(it - LAG);
         }
       }
-      if (!ok) break;
-      if (nb == 0) {  // row norms: the eight threads of a row hold its chunks' sums
+      if (nb == 0) {  // (also on an abort, so that no warp waits here for another)
+        // row norms: the eight threads of a row hold its chunks' sums
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           float v = ss[i];
@@ -1117,10 +1120,31 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
           v += __shfl_xor_sync(0xffffffffu, v, 4);
           if (c == 0) nrm_s[(g >> 3) + 16 * i] = v;
         }
+        // 1 / ||t|| (0 for a zero target: similarity 0); NaN, which is no candidate, for a target whose row is a copy of an
+        // earlier one's (blank parts of a tile): a tie never chooses it
+        for (int q = g; q < m; q += 128) inv_s[q] = tinv[co + q];
+        if (g == 0) any_twin = 0;
         asm volatile("bar.sync 1, 128;\n" ::: "memory");
+        for (int q = g; q < m; q += 128) {
+          int p = 0;
+          while (p < q && inv_s[p] != inv_s[q]) ++p;
+          twin[q] = p < q ? (uint16_t)p : MergeCand::NONE;
+          if (p < q) any_twin = 1;
+        }
+        asm volatile("bar.sync 1, 128;\n" ::: "memory");
+        if (any_twin) {
+          for (int q = quarter; q < m; q += 4) {
+            const int p = twin[q];
+            if (p != MergeCand::NONE && same_row(targets + (size_t)(co + p) * d, targets + (size_t)(co + q) * d, d, lane) &&
+                lane == 0)
+              inv_s[q] = __int_as_float(0x7fffffff);
+          }
+          asm volatile("bar.sync 1, 128;\n" ::: "memory");
+        }
       }
+      if (!ok) break;
       const int c0 = nb * COLS, nc = min(COLS, m - c0);
-      const float* inv_n = tinv + co + c0;  // 1 / ||t|| (0 for a zero target: similarity 0)
+      const float* inv_n = inv_s + c0;
       if (!__all_sync(0xffffffffu, mbar_wait(tfull, nb & 1, abort_flag))) { ok = false; break; }
       fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16);
@@ -1167,7 +1191,7 @@ __global__ void __launch_bounds__(ms::THREADS, 2)
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
               const int b = cc + e;
-              if (b < nc && b != b1 && within(__uint_as_float(acc[e]) * inv_n[b])) {
+              if (b < nc && b != b1 && within(fmaxf(__uint_as_float(acc[e]) * inv_n[b], -INFINITY))) {
                 const uint64_t keep = ~(0xffffull << (16 * (n & 3))), put = (uint64_t)b << (16 * (n & 3));
                 if (n < 4) lo = (lo & keep) | put;
                 else if (n < MergeCand::MAX) hi = (hi & keep) | put;
@@ -1426,7 +1450,7 @@ int launch_merge_screen(const uint16_t* X, int N, int n_v, int d, const int* kep
   static std::atomic<unsigned long long> smem_raised{0};
   if (raise_smem_limit(smem_raised, merge_screen_kernel, (int)ms::SMEM) != cudaSuccess) return 1;
   return launch_ex(merge_screen_kernel, dim3((n_v + 127) / 128, N), dim3(ms::THREADS), ms::SMEM, st, true, mt, X, n_v, d,
-                   kept, n_kept, sel_off, ctx_off, max_ctx, tinv, rest, cand) != cudaSuccess;
+                   kept, n_kept, sel_off, ctx_off, max_ctx, targets, tinv, rest, cand) != cudaSuccess;
 }
 
 int launch_wait_timeout_check(cudaStream_t st) {

@@ -101,23 +101,6 @@ __device__ double ff_dot(const XT* a, const XT* b, int d, int lane) {
   return ff_warp_sum(hi, lo);
 }
 
-// Whether two rows hold the same bits (b null: whether the row is all zeros, of either sign), by one warp.
-template <typename XT>
-__device__ __forceinline__ bool same_row(const XT* a, const XT* b, int d, int lane) {
-  constexpr int W = 16 / sizeof(XT);  // elements of a 16-byte load
-  constexpr uint32_t ABS = sizeof(XT) == 2 ? 0x7fff7fffu : 0x7fffffffu;
-  for (int k = lane * W; k < (d + 32 * W - 1) / (32 * W) * (32 * W); k += 32 * W) {
-    uint32_t differ = 0u;
-    if (k < d) {
-      const uint4 x = *reinterpret_cast<const uint4*>(a + k);
-      const uint4 y = b ? *reinterpret_cast<const uint4*>(b + k) : make_uint4(0u, 0u, 0u, 0u);
-      differ = ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) & (b ? 0xffffffffu : ABS);
-    }
-    if (__any_sync(0xffffffffu, differ != 0u)) return false;
-  }
-  return true;
-}
-
 // m_j = min(budgets[j] - s_j, n_v - s_j) and its exclusive prefix sum over the kept slots.  If
 // the total exceeds max_ctx, RIFT_EBIT_CAPACITY is set and every m_j is taken as 0 (no contextual
 // row is then written or read).
@@ -446,6 +429,7 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
   __shared__ int best_j[TB][2];
   __shared__ float inv_n[TB], row_ss[TB];
   __shared__ int far;              // a target's norm is below 2^-40
+  __shared__ int twin[TB], any_twin;  // an earlier target of the same norm, or -1
   __shared__ int n_all, all[TB];   // rows with all targets for candidates
   __shared__ double part_s[8];
   __shared__ int part_q[8];
@@ -472,6 +456,24 @@ __global__ void __launch_bounds__(256) merge_assign_kernel(const XT* __restrict_
       const double nn = b0 + tid < m ? tnorm[co + b0 + tid] : 0.0;
       inv_n[tid] = nn > 0.0 ? (float)(1.0 / nn) : 0.f;  // a zero target has similarity 0
       if (inv_n[tid] > 0x1p40f) far = 1;
+    }
+    // targets whose row is a copy of an earlier one's (blank parts of a tile): a tie never chooses them
+    if (tid == 0) any_twin = 0;
+    __syncthreads();
+    if (tid < TB) {
+      twin[tid] = -1;
+      const int q = b0 + tid;
+      for (int p = 0; q < m && p < q && twin[tid] < 0; ++p)
+        if (__double_as_longlong(tnorm[co + p]) == __double_as_longlong(tnorm[co + q])) twin[tid] = p;
+      if (twin[tid] >= 0) any_twin = 1;
+    }
+    __syncthreads();
+    if (any_twin) {
+      for (int q = tid >> 5; q < TB; q += 8)
+        if (twin[q] >= 0 && same_row(Xt + (size_t)ctx_target[co + twin[q]] * d, Xt + (size_t)ctx_target[co + b0 + q] * d, d,
+                                     tid & 31) &&
+            (tid & 31) == 0)
+          inv_n[q] = __int_as_float(0x7fffffff);  // NaN: no candidate
     }
     float acc[4][4] = {};
     // 64 rows x KC columns per operand and chunk: four 8-column groups per thread and operand,

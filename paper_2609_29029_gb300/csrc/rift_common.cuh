@@ -246,4 +246,21 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// Whether two rows hold the same bits (b null: whether the row is all zeros, of either sign), by one warp.
+template <typename XT>
+__device__ __forceinline__ bool same_row(const XT* a, const XT* b, int d, int lane) {
+  constexpr int W = 16 / sizeof(XT);  // elements of a 16-byte load
+  constexpr uint32_t ABS = sizeof(XT) == 2 ? 0x7fff7fffu : 0x7fffffffu;
+  for (int k = lane * W; k < (d + 32 * W - 1) / (32 * W) * (32 * W); k += 32 * W) {
+    uint32_t differ = 0u;
+    if (k < d) {
+      const uint4 x = *reinterpret_cast<const uint4*>(a + k);
+      const uint4 y = b ? *reinterpret_cast<const uint4*>(b + k) : make_uint4(0u, 0u, 0u, 0u);
+      differ = ((x.x ^ y.x) | (x.y ^ y.y) | (x.z ^ y.z) | (x.w ^ y.w)) & (b ? 0xffffffffu : ABS);
+    }
+    if (__any_sync(0xffffffffu, differ != 0u)) return false;
+  }
+  return true;
+}
+
 }  // namespace rift
