@@ -7,15 +7,16 @@
 // gemm_tc_kernel (many rows: the prefill of a scene): persistent and warp-specialised on SM pairs
 // (2-CTA clusters, 256 x 256 tiles, or 256 x 192: tile_width), or on single SMs where 128 x 256 tiles take
 // fewer waves (one_sm_tiles), 192 threads per CTA:
-//   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 6-stage shared-memory ring
+//   warp 0      one thread issues TMA tile loads (128B-swizzled) into a 6-stage shared-memory ring (4 on one SM)
 //   warp 1      allocates 512 TMEM columns; the even CTA's issues tcgen05.mma (cta_group::2, M = 256,
-//               N = 256, K = 16) into one of two 256-column fp32 accumulators and commits to
+//               N = 256, K = 16; a CTA alone cta_group::1, M = 128) into one of two 256-column fp32 accumulators and commits to
 //               mbarriers
 //   warps 2..5  epilogue: tcgen05.ld of their 32 TMEM lanes (one row per thread), fused op, store
-// The issuing warp runs its loop with all lanes and issues under elect_one(): a K-block takes 514 cycles
+// Warp 1 runs its loop with all lanes and issues under elect_one(): a K-block takes 514 cycles
 // (the tensor pipe's own time is 512), against 551 with one lane issuing from a branch of its own.  The
-// large products are limited by power all the same (their clock falls from 1650 to 1550 MHz with it); the
-// whole 400-tile query gained 2%, a 2,448-row prefill over a prefix 2%, a one-tile prefill 2%.
+// large products are limited by power all the same: their clock falls from 1650 to 1550 MHz with it, and the
+// whole 400-tile query, a 5,900-row prefill and one of 2,448 rows over a prefix gained 1.2-1.9%, little more
+// than two runs of one build differ by.
 // Two accumulators let the epilogue of one tile overlap the main loop of the next.  Tiles are
 // visited in bands whose rows of the larger operand fit in L2 (48 MB), so each tile of the other
 // operand is read from DRAM once per band.

@@ -240,9 +240,11 @@ void launch_pack(const void* X, rift_dtype xdt, int N, int n_v, int d, const int
     static std::atomic<unsigned long long> smem_raised{0};
     if (raise_smem_limit(smem_raised, pack_bulk_kernel, PKB_SLOTS * 8192 * 2) != cudaSuccess)
       return;  // the error stays pending for the caller's launch check
-    // A CTA streams its rows one ring after another, so with few tiles its row count is the time: 64 rows
-    // a CTA where many tiles keep the GPU full (fewer CTAs for tiles that are not kept), else 16 (64 tiles,
-    // 17 kept: 36 us with 64 rows a CTA, 16 with 16).
+    // A CTA streams its rows one ring after another, so with few tiles its row count is the time; with many,
+    // 64 rows a CTA make fewer CTAs for the tiles that are not kept.  us, 16 rows : 64, 576 tokens a tile: d = 4096,
+    // 64 tiles 25 : 41, 128 35 : 43, 129 37 : 44, 200 48 : 51, 400 75 : 78, 700 119 : 119, 1600 270 : 251, 6400
+    // 1014 : 892; d = 1024, 400 30 : 43, 1600 99 : 93; d = 256, 128 15 : 39, 700 33 : 43, 1600 70 : 61.
+    // The two meet at about 700 tiles at d = 4096 and later at smaller d, so 16 rows would pay further up than this line.
     const int cta_rows = N > 128 ? PKB_ROWS : 16;
     dim3 gb(N, (max_L + cta_rows - 1) / cta_rows);
     launch_ex(pack_bulk_kernel, gb, dim3(64), smem, st, true, static_cast<const uint16_t*>(X), N, n_v, d, kept,

@@ -228,8 +228,10 @@ int launch_prefill(const rift_model& m, void* hidden, int T, const int* T_dev, c
 
   // With few rows the kernels after the first are launched as programmatic dependents of the kernel before
   // them: launch latencies are a good part of the time (two layers over one 131-row tile 373 -> 316 us
-  // with the setup in one launch).  At 28,000 rows the early launches cost more than they hide: a
-  // 32-layer query 256.5 ms with them, 254.1 without.
+  // with the setup in one launch).  With many, the early launches cost more than they hide.  Time with them
+  // over time without, two 7B layers: 1,938 rows 0.970, 3,660 0.992, 5,395 0.996, 7,333 0.998, 8,374 0.994,
+  // 9,618 0.998, 12,728 1.018, 19,020 1.009, 27,047 1.015 (at d = 1024, where a kernel is shorter, 0.83 at 347
+  // rows to 0.98 at 27,047).
   const bool pdl = T <= 8192;
   prof_begin(RIFT_PROF_ROPE, st);
   PrefillSetup ps = {rope, max_len, half, rope_freq(m), qkv, 3 * d, T_dev};

@@ -158,7 +158,8 @@ struct EpiParams {
   int kmap_d = 0;
   int kmap_a = 0, kmap_b = 0;
 };
-// pdl: launch as a programmatic dependent of the previous kernel in the stream (few-row products).
+// pdl: launch as a programmatic dependent of the previous kernel in the stream (decode steps, prefills of up
+// to 8,192 rows).
 int launch_gemm(const void* A, const void* B, int M, int N, int K, int epi, void* C,
                 cudaStream_t st, const EpiParams& ep = EpiParams(), bool pdl = false);
 // b_const: B does not depend on earlier kernels (constant weights), so a programmatic dependent

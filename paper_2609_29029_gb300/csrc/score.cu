@@ -673,9 +673,9 @@ __global__ void __launch_bounds__(32 * RIFT_MAX_KNN / CS) knn_rescore_smooth_ker
   const int w = cta * (RIFT_MAX_KNN / CS) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w < C) {
     const int j = top_j[(size_t)il * C + w];
-    // V_i is read by all the CTA's warps (L1 serves all but the first).  The kernel moves 16 rows
-    // of V per tile from L2: its time follows those bytes, not the length of this chain (four
-    // independent chains with loads ahead measured slower, at fewer resident CTAs).
+    // V_i is read by all the CTA's warps (L1 serves all but the first).  With many tiles (U = 4, CS = 1) the
+    // kernel's time follows the 16 rows of V per tile from L2, not the length of this chain: four independent
+    // chains with loads ahead measured slower there, at fewer resident CTAs.
     float hi = 0.f, lo = 0.f;
     if (j >= 0 && j < N) {
       const float4* vi = reinterpret_cast<const float4*>(V + (size_t)i * d);

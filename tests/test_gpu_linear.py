@@ -23,8 +23,8 @@ def _rel(g, o):
     return float((g.double() - o).abs().max() / o.abs().max())
 
 
-# M >= 1024 runs on SM pairs (256 x 256 tiles): ragged last tiles whose second 128 rows or second
-# 128 B rows lie wholly or partly outside the operands.
+# Few rows on clusters, more on single SMs or on SM pairs (256 x 256 tiles): ragged last tiles whose second 128
+# rows or second 128 B rows lie wholly or partly outside the operands.
 SHAPES = [(1, 256, 64), (128, 256, 64), (129, 264, 72), (200, 768, 256), (384, 256, 688), (333, 1024, 4096),
           (1000, 4096, 4096), (300, 12288, 4096), (1100, 264, 72), (2000, 640, 200), (4097, 768, 128),
           (1024, 4096, 4096)]
