@@ -650,7 +650,9 @@ static_assert(MAX_BN * BM * 4 <= RING, "the partial product reuses the ring");
 // where all clusters of 3 or more would only just fit, some wait for a second round: a sixteenth is left free then
 // (two layers over 347 rows, whose W_o takes 96 tiles, 507 us with S = 3, of which 97 fit, 466 with S = 2; 20 decoded
 // tokens 472 : 459).  A quarter free is too much (524 rows 536 : 575), pairs need none (2,970 rows at d = 1024, 152 of
-// 152 pairs, 298 : 321), nor does a launch of its own (W_o at 384 rows 26.6 : 32.8).
+// 152 pairs, 298 : 321), nor does a launch of its own (W_o at 384 rows 26.6 : 32.8), nor do fewer than 8 rows, whose
+// norm before it takes as many CTAs (decode steps over 4 layers, without : with: 1 row 418 : 420, 3 418 : 424, 6 420 : 422,
+// 8 431 : 429, 16 453 : 441).
 // K too short to split (fewer than 16 K-blocks): row tiles of at most SHORT_BN instead, as long as they fit at
 // once; what a CTA takes is then its epilogue, a serial chain over its rows.  us, tiles of 160 rows, 48, and the
 // SM pairs, 300 rows: 256 x 256 + residual 22.5 : 12.3 : 20.5, 768 x 256 10.2 : 8.2 : 14.3, SwiGLU 1376 x 256
@@ -673,7 +675,7 @@ inline Plan plan(int M, int N, int K, int sms, const int* resident, bool gram, b
   const long long tiles = m_tiles * n_tiles;
   if (gram && tiles <= 2 && kt / MAX_S >= min_blocks) return {height(m_tiles), MAX_S, true};
   int S = gram && tiles > 32 ? 4 : PORTABLE_S;
-  auto fit = [&](int s) { return pdl && s > 2 ? resident[s] * 15 / 16 : resident[s]; };
+  auto fit = [&](int s) { return pdl && M >= 8 && s > 2 ? resident[s] * 15 / 16 : resident[s]; };
   while (S > 1 && (tiles > fit(S) || kt / S < min_blocks)) --S;
   return {height(m_tiles), S, S >= 2};
 }
